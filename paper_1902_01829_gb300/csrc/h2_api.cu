@@ -461,7 +461,6 @@ h2_status run_pass(h2_matrix_s* h, int nv, const double* x, int64_t ldx, double*
   using namespace h2;
   const int k = h->k, kp = h->kp, LR = h->lr;
   const unsigned wb = (unsigned)kWarps * 32;
-  auto grid = [](int64_t items) { return (unsigned)((items + kWarps - 1) / kWarps); };
   cudaError_t e = set_stream_smem<NVB>();
   if (e != cudaSuccess) return fail(H2_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
   constexpr int CW = dense_consumer_warps(NVB);
@@ -494,17 +493,26 @@ h2_status run_pass(h2_matrix_s* h, int nv, const double* x, int64_t ldx, double*
   k_vec_scale<<<kScaleBlocks, kScaleThreads, 0, st>>>(x, ldx, h->n, nv, h->vpart, h->vticket, h->vexp);
   k_upsweep_tree<RPL_K, NVB><<<tree_grid, tree_threads, 0, st>>>(T);
   if (me == cudaSuccess) me = mark(&h->prof, st);
+  CouplingParams C{};
+  C.S = h->smat;
+  C.Sco = h->Sco;
+  C.segs = static_cast<const CouplingSeg*>(h->csegs);
+  C.xhat = h->xhat;
+  C.yhat = h->yhat;
+  C.part = h->cpart;
+  C.ticket = h->cticket;
+  C.kkp = kkp;
+  C.k = k;
+  C.kp = kp;
+  C.LR = LR;
+  C.nv = nv;
+  const unsigned cgrid = (unsigned)h->ncsegs;
   if (h->pair_rows) {
     constexpr int CB = NVB <= 2 ? 4 : (NVB <= 4 ? 2 : 1);
-    if (h->s_tiny)
-      k_coupling<NVB, CB, true><<<grid(h->n_nodes), wb, 0, st>>>(h->smat, kkp, h->Srow, h->Sco, k, kp, h->n_nodes, nv,
-                                                                  h->xhat, h->yhat);
-    else
-      k_coupling<NVB, CB, false><<<grid(h->n_nodes), wb, 0, st>>>(h->smat, kkp, h->Srow, h->Sco, k, kp, h->n_nodes, nv,
-                                                                   h->xhat, h->yhat);
+    if (h->s_tiny) k_coupling<NVB, CB, true><<<cgrid, wb, 0, st>>>(C);
+    else k_coupling<NVB, CB, false><<<cgrid, wb, 0, st>>>(C);
   } else {
-    k_coupling_generic<RPL_K, NVB><<<grid(h->n_nodes), wb, 0, st>>>(h->smat, kkp, h->Srow, h->Sco, k, kp, LR, h->n_nodes,
-                                                                     nv, h->xhat, h->yhat);
+    k_coupling_generic<RPL_K, NVB><<<cgrid, wb, 0, st>>>(C);
   }
   if (me == cudaSuccess) me = mark(&h->prof, st);
   k_downsweep_tree<RPL_K, NVB><<<tree_grid, tree_threads, 0, st>>>(T);
@@ -555,6 +563,27 @@ h2_status matvec_device(h2_matrix_s* h, int nv, const double* x, int64_t ldx, do
     if (s != H2_OK) return s;
   }
   return H2_OK;
+}
+
+// The FP64 coupling phase's segments: the blocks of every node row, a long row cut into several
+// (one CTA each). A row is cut when it holds more than a quarter of an SM's share of all blocks,
+// into pieces of about a sixteenth of that share (at least 8192 entries, 64 KB): with fewer rows
+// than that the longest row sets the phase's time, with more the rows balance by themselves.
+// Returns the number of partial-sum slots.
+int64_t coupling_segments(const int32_t* Srow, int64_t n_nodes, int k, int grid, std::vector<h2::CouplingSeg>* out) {
+  const int64_t nS = Srow[n_nodes], least = std::max<int64_t>(4, 8192 / ((int64_t)k * k));
+  const int64_t piece = std::max(least, nS / (16 * (int64_t)grid)), limit = std::max(piece + piece / 2, nS / (4 * (int64_t)grid));
+  int64_t slots = 0;
+  for (int64_t r = 0; r < n_nodes; r++) {
+    const int64_t b0 = Srow[r], nb = Srow[r + 1] - b0;
+    const int64_t parts = nb > limit ? (nb + piece - 1) / piece : 1;
+    for (int64_t p = 0; p < parts; p++) {
+      const int64_t lo = nb * p / parts, hi = nb * (p + 1) / parts;
+      out->push_back(h2::CouplingSeg{(int)r, (int)(b0 + lo), (int)(hi - lo), parts > 1 ? (int)slots : 0, (int)p, (int)parts, {0, 0}});
+    }
+    if (parts > 1) slots += parts;
+  }
+  return slots;
 }
 
 // ------------------------------------------------------------------ device layout
@@ -700,6 +729,17 @@ h2_status build_device(h2_matrix_s* h, const h2_desc* d) {
     std::vector<int2> sco((size_t)h->nS);
     for (int64_t b = 0; b < h->nS; b++) sco[b] = make_int2(d->S_colidx[b], R.oS[b]);
     if ((st = upload(h, &h->Sco, (const int2*)sco.data(), h->nS)) != H2_OK) return st;
+  }
+  {
+    std::vector<h2::CouplingSeg> segs;
+    const int64_t slots = coupling_segments(d->S_rowptr, h->n_nodes, k, h->grid, &segs);
+    h2::CouplingSeg* ds = nullptr;
+    if ((st = upload(h, &ds, (const h2::CouplingSeg*)segs.data(), (int64_t)segs.size())) != H2_OK) return st;
+    h->csegs = ds;
+    h->ncsegs = (int64_t)segs.size();
+    if ((st = dalloc(h, &h->cpart, slots * kPassVectors * h->kp)) != H2_OK) return st;
+    if ((st = dalloc(h, &h->cticket, slots)) != H2_OK) return st;
+    CUDA_TRY(cudaMemset(h->cticket, 0, (size_t)std::max<int64_t>(slots, 1) * sizeof(int)));
   }
   if ((st = dalloc(h, &h->vexp, h2i::kPassVectors)) != H2_OK) return st;
   if ((st = dalloc(h, &h->vpart, (int64_t)h2::kScaleBlocks * 16)) != H2_OK) return st;

@@ -286,10 +286,19 @@ __global__ void __launch_bounds__(kTreeWarps * 32) k_downsweep_tree(TreeParams P
 }
 
 // ---------------------------------------------------------------- coupling, all levels
-// One warp per node row i: yhat_i = sum_{b in row i} S_b xhat_{col(b)}   (Eq. 3, Alg. 3)
+// yhat_i = sum_{b in row i} S_b xhat_{col(b)}   (Eq. 3, Alg. 3). A CTA of kWarps warps takes one
+// segment, a run of blocks of one node row, and its warps take the segment's blocks in turn; the
+// warps' sums meet in shared memory. Most rows are one segment. Where the matrix has few long rows
+// (3D, upper levels, small n) a row is cut into several segments (coupling_segments): each leaves
+// its partial sum in `part`, and the row's last segment to finish (ticket per row) adds them in
+// order, so the result does not depend on the order of arrival.
+// What bounds it: HBM at few vectors, as long as enough 16-byte loads are in flight. One warp per
+// row left 3D n = 2^14 (511 rows of up to 150 blocks of 32 KB) with 511 warps on the chip and the
+// longest row as the kernel's time: 972 us against 87 us of HBM time; split as above 180 us.
+//
 // k = 2H with H a power of two: lane = g * H + h owns rows 2h, 2h + 1 of every block,
 // read as one 16-byte load per column; column groups g = 0 .. G-1 (G = 32 / H)
-// take columns g, g + G, ... The row's blocks are walked in batches of CB
+// take columns g, g + G, ... The warp's blocks are walked in batches of CB
 // columns per lane, two batches in flight: the next batch's matrix and xhat
 // loads are issued before the current batch is multiplied. Blocks are padded
 // to kkp doubles; Sco[b] = (column node, exponent offset) of block b. Every node row
@@ -298,21 +307,81 @@ __global__ void __launch_bounds__(kTreeWarps * 32) k_downsweep_tree(TreeParams P
 // FP32 sum of the small parts never runs over a whole row.
 // SAFE: some coupling entry is zero or below 2^-103 after its offset (zero-safe split).
 constexpr int kFoldProducts = 64;
+
+struct __align__(16) CouplingSeg {
+  int row, b0, nb;  // node row; first block; blocks
+  int base;         // the row's first slot in `part` (and its ticket); unused when parts = 1
+  int seg, parts;   // this segment of the row, and how many the row has
+  int pad[2];
+};
+
+struct CouplingParams {
+  const double* S;
+  const int2* Sco;
+  const CouplingSeg* segs;
+  const float2* xhat;
+  float2* yhat;
+  float2* part;   // [slot][v][kp], the segments of split rows
+  int* ticket;    // per slot base, zero between products
+  int kkp, k, kp, LR, nv;
+};
+
+// the CTA's warps have left their sums in red[warp][v][64]: add them, then store the row (or add up
+// the row's segments when this is the last of them)
+template <int NVB>
+__device__ __forceinline__ void coupling_finish(const CouplingParams& P, const CouplingSeg& sg, float2 (*red)[NVB][64],
+                                                int* last) {
+  __syncthreads();
+  const int k = P.k, kp = P.kp, nv = P.nv;
+  float2* row = P.yhat + (int64_t)sg.row * nv * kp;
+  float2* mine = sg.parts == 1 ? row : P.part + (int64_t)(sg.base + sg.seg) * nv * kp;
+  for (int t = threadIdx.x; t < nv * k; t += kWarps * 32) {
+    const int v = t / k, r = t - v * k;
+    float s = 0.f, c = 0.f;
+#pragma unroll
+    for (int w = 0; w < kWarps; w++) df_add(s, c, red[w][v][r].x, red[w][v][r].y);
+    mine[v * kp + r] = df_norm(s, c);
+  }
+  if (sg.parts == 1) return;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    *last = atomicAdd(P.ticket + sg.base, 1) == sg.parts - 1;
+    if (*last) P.ticket[sg.base] = 0;  // every segment has arrived: reset for the next product
+  }
+  __syncthreads();
+  if (!*last) return;
+  __threadfence();
+  for (int t = threadIdx.x; t < nv * k; t += kWarps * 32) {
+    const int v = t / k, r = t - v * k;
+    const float2* src = P.part + (int64_t)sg.base * nv * kp + v * kp + r;
+    float s = 0.f, c = 0.f;
+#pragma unroll 4
+    for (int p = 0; p < sg.parts; p++) {
+      const float2 a = __ldcg(src + (int64_t)p * nv * kp);
+      df_add(s, c, a.x, a.y);
+    }
+    row[v * kp + r] = df_norm(s, c);
+  }
+}
+
 template <int NVB, int CB, bool SAFE>
-__global__ void __launch_bounds__(kWarps * 32) k_coupling(const double* __restrict__ S, int kkp,
-                                                        const int32_t* __restrict__ Srow, const int2* __restrict__ Sco,
-                                                        int k, int kp, int64_t n_nodes, int nv,
-                                                        const float2* __restrict__ xhat, float2* __restrict__ yhat) {
+__global__ void __launch_bounds__(kWarps * 32) k_coupling(CouplingParams P) {
+  __shared__ float2 red[kWarps][NVB][64];
+  __shared__ int last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t i = (int64_t)blockIdx.x * kWarps + warp;
-  if (i >= n_nodes) return;
+  const CouplingSeg sg = P.segs[blockIdx.x];
+  const int k = P.k, kp = P.kp, nv = P.nv;
+  const double* __restrict__ S = P.S;
+  const int2* __restrict__ Sco = P.Sco;
+  const float2* __restrict__ xhat = P.xhat;
   const int H = k >> 1, G = 32 / H;
   const int g = lane / H, h = lane - g * H;
   const bool active = g < G;            // lanes beyond G * H idle
   const int cpl = (k + G - 1) / G;      // columns per lane per block
   const int ncb = (cpl + CB - 1) / CB;  // batches per block
-  const int32_t b0 = Srow[i];
-  const int nbatch = (Srow[i + 1] - b0) * ncb;
+  const int b0 = sg.b0 + warp;          // this warp's blocks: b0, b0 + kWarps, ...
+  const int nbatch = warp < sg.nb ? ((sg.nb - warp + kWarps - 1) / kWarps) * ncb : 0;
   constexpr int FB = kFoldProducts / CB;  // batches per chain
   float s[2][NVB], c[2][NVB], S2[2][NVB], C2[2][NVB];
   acc_zero(s, c);
@@ -322,9 +391,9 @@ __global__ void __launch_bounds__(kWarps * 32) k_coupling(const double* __restri
   float2 x0[CB][NVB], x1[CB][NVB];
   int o0 = 0, o1 = 0;
   auto load = [&](int bt, double2(&a)[CB], float2(&xv)[CB][NVB], int& o) {
-    const int b = bt / ncb, cb = bt - b * ncb;
-    const double* A = S + (int64_t)(b0 + b) * kkp;
-    const int2 co = __ldg(Sco + b0 + b);
+    const int bl = bt / ncb, cb = bt - bl * ncb, b = b0 + kWarps * bl;
+    const double* A = S + (int64_t)b * P.kkp;
+    const int2 co = __ldg(Sco + b);
     const float2* X = xhat + (int64_t)co.x * nv * kp;
     o = co.y;
 #pragma unroll
@@ -382,44 +451,40 @@ __global__ void __launch_bounds__(kWarps * 32) k_coupling(const double* __restri
       }
   }
   if (g == 0) {
-    float2* dst = yhat + i * nv * kp;
 #pragma unroll
-    for (int v = 0; v < NVB; v++)
-      if (v < nv) {
-        if (2 * h < k) dst[v * kp + 2 * h] = df_norm(s[0][v], c[0][v]);
-        if (2 * h + 1 < k) dst[v * kp + 2 * h + 1] = df_norm(s[1][v], c[1][v]);
-      }
+    for (int v = 0; v < NVB; v++) {
+      red[warp][v][2 * h] = make_float2(s[0][v], c[0][v]);
+      red[warp][v][2 * h + 1] = make_float2(s[1][v], c[1][v]);
+    }
   }
+  coupling_finish<NVB>(P, sg, red, &last);
 }
 
 // Any other k: the generic row mapping of warp_mv, one block at a time (each
 // block's chain folded into the row's long-term pair).
 template <int RPL, int NVB>
-__global__ void __launch_bounds__(kWarps * 32) k_coupling_generic(const double* __restrict__ S, int kkp,
-                                                            const int32_t* __restrict__ Srow,
-                                                            const int2* __restrict__ Sco, int k, int kp, int LR,
-                                                            int64_t n_nodes, int nv, const float2* __restrict__ xhat,
-                                                            float2* __restrict__ yhat) {
+__global__ void __launch_bounds__(kWarps * 32) k_coupling_generic(CouplingParams P) {
+  __shared__ float2 red[kWarps][NVB][64];
+  __shared__ int last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t i = (int64_t)blockIdx.x * kWarps + warp;
-  if (i >= n_nodes) return;
+  const CouplingSeg sg = P.segs[blockIdx.x];
+  const int k = P.k, kp = P.kp, LR = P.LR, nv = P.nv;
   float s[RPL][NVB], c[RPL][NVB], S2[RPL][NVB], C2[RPL][NVB];
   acc_zero(s, c);
   acc_zero(S2, C2);
-  for (int32_t b = Srow[i]; b < Srow[i + 1]; b++) {
-    const int2 co = Sco[b];
-    warp_mv<RPL, NVB>(S + (int64_t)b * kkp, co.y, k, k, LR, xhat + (int64_t)co.x * nv * kp, kp, nv, s, c, lane);
+  for (int b = sg.b0 + warp; b < sg.b0 + sg.nb; b += kWarps) {
+    const int2 co = P.Sco[b];
+    warp_mv<RPL, NVB>(P.S + (int64_t)b * P.kkp, co.y, k, k, LR, P.xhat + (int64_t)co.x * nv * kp, kp, nv, s, c, lane);
     acc_fold(S2, C2, s, c);
   }
   group_reduce(S2, C2, LR);
+  if (lane < LR) {
 #pragma unroll
-  for (int r = 0; r < RPL; r++)
+    for (int r = 0; r < RPL; r++)
 #pragma unroll
-    for (int v = 0; v < NVB; v++) {
-      s[r][v] = S2[r][v];
-      c[r][v] = C2[r][v];
-    }
-  store_node<RPL, NVB, false>(yhat + i * nv * kp, k, kp, LR, nv, s, c, lane);
+      for (int v = 0; v < NVB; v++) red[warp][v][lane + 32 * r] = make_float2(S2[r][v], C2[r][v]);
+  }
+  coupling_finish<NVB>(P, sg, red, &last);
 }
 
 // ---------------------------------------------------------------- per-vector scale
