@@ -786,7 +786,6 @@ h2_status create_handle(const h2_desc* d, const h2_coupling_kernel* kc, h2_handl
   h->kf = kc != nullptr;
   if (kc) {
     h->kf_kind = kc->kernel;
-    h->kf_inv_ell = (float)(1.0 / kc->ell);
   }
   try {
     st = build_device(h, d);

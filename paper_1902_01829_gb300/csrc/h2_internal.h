@@ -51,7 +51,7 @@ struct MixedLaunch {
   void* mats = nullptr;              // device h2::MatDesc table
   const int2* jobs = nullptr;        // (matrix, subtree) per tree CTA
   int64_t njobs = 0;
-  const int4* chunks = nullptr;      // coupling row chunks {matrix, first row, rows, 0}
+  const int4* chunks = nullptr;      // coupling row chunks (mixed.cuh)
   int64_t nchunks = 0;
   const h2::StreamItem* items = nullptr;
   const int* cta_begin = nullptr;    // [grid + 1]
@@ -150,10 +150,12 @@ struct MixedData {
   std::vector<h2::StreamItem> items_host;  // the dense items (matrix index 0), kept for batches
   std::vector<int64_t> row_bytes;          // bytes each leaf row streams (load balance)
   std::vector<int64_t> row_item0;          // first item of each leaf row, [leaves + 1]
-  std::vector<int4> chunks_host;           // coupling row chunks (matrix index 0), current target
   std::vector<int32_t> srow_host;          // S_rowptr (to cut chunks for another target)
   int4* chunk_dev[3] = {nullptr, nullptr, nullptr};  // device chunk lists per target option
   int64_t chunk_n[3] = {0, 0, 0};
+  float* cpart = nullptr;                             // pieces of cut coupling rows: sums [slot][v][kp4]
+  int* cticket = nullptr;                             // [slot][4] counters, zero between products
+  int64_t cslots = 0;
   int2* jobs_dev[3] = {nullptr, nullptr, nullptr};    // tree jobs per subtree-level option
   int tree_opt = -1;                                  // subtree level L = default - tree_opt
 };
@@ -163,7 +165,8 @@ constexpr int kChunkOpts[3] = {64, 128, 256};  // coupling blocks per warp chunk
 constexpr int kTreeOpts[3] = {4, 5, 6};       // log2 of the leaves per tree CTA (batches)
 constexpr int kDefaultChunkOpt = 1, kDefaultTreeOpt = 2;
 constexpr int kDenseCW = 8;                   // dense-stream consumer warps (or twice as many)
-std::vector<int4> coupling_chunks(const int32_t* Srow, int64_t n_nodes, int64_t target);
+std::vector<int4> coupling_chunks(const int32_t* Srow, int64_t n_nodes, int64_t target, int k, int64_t total, int sms,
+                                  bool kf, int64_t* slots);
 
 // vector-count buckets of the precision-form kernels: bucket b runs the
 // variant for up to kBucketNV[b] vectors and takes counts kBucketLo[b] ..
@@ -184,7 +187,6 @@ struct h2_matrix_s {
   const double* gen_points = nullptr;      // while h2_create_generated builds the handle (host, n x dim)
   bool kf = false;                         // coupling blocks evaluated from the kernel
   int kf_kind = 0;
-  float kf_inv_ell = 0.f;
   int64_t paper_bytes = 0, device_bytes = 0;
   std::vector<void*> allocs;
   int64_t* leaf_off = nullptr;

@@ -151,9 +151,9 @@ h2::MatDesc fill_desc(const h2_matrix_s* h, int tree_L) {
   D.kf_chi = M.kf_chi;
   D.kf_clo = M.kf_clo;
   D.kf_off = M.kf_off;
-  D.kf_inv_ell = h->kf_inv_ell;
-  D.kf_kind = h->kf_kind;
   D.spanel = M.spanel ? 1 : 0;
+  D.cpart = M.cpart;
+  D.cticket = M.cticket;
   D.rjobs = static_cast<const h2::RowJob*>(M.rjobs);
   D.blk = static_cast<const h2::MixedBlock*>(M.dblk);
   return D;
@@ -318,19 +318,41 @@ h2_status audit_producer_batches(const std::vector<h2::StreamItem>& items, const
 
 namespace h2i {
 
-// coupling row chunks of one matrix: consecutive rows, at most kChunkRows rows
-// and (unless one row alone has more) about `target` coupling blocks each
-std::vector<int4> coupling_chunks(const int32_t* Srow, int64_t n_nodes, int64_t target) {
+// coupling row chunks of one matrix, one warp each: consecutive rows, at most kChunkRows rows and
+// (unless one row alone has more) about `piece` coupling blocks, and long rows in pieces of that many.
+// piece: `target` (the launch option), or less where the launch's `total` blocks would then give the
+// `sms` SMs fewer than 32 chunks each (64 where the blocks are evaluated, kf: that work is bound by
+// issue slots and wants an even split), but at least 4096 entries of work (four 64 x 64 blocks, 16 of
+// 16 x 16). A row is cut when it holds more than one and a half pieces and more than an eighth (kf:
+// a thirty-second) of an SM's share: below that the chunks balance by themselves and cutting only
+// adds partial sums (2D n = 2^17, one vector: coupling 16.6 us, 20.9 us with every row over 24
+// blocks cut; evaluated at 3D n = 2^16, 8 vectors: 900 us at an eighth, 441 us with this rule and
+// the shorter evaluation). *slots: partial-sum slots.
+std::vector<int4> coupling_chunks(const int32_t* Srow, int64_t n_nodes, int64_t target, int k, int64_t total, int sms,
+                                  bool kf, int64_t* slots) {
   std::vector<int4> out;
+  const int64_t least = std::max<int64_t>(4, 4096 / ((int64_t)k * k));
+  const int64_t piece = std::min(target, std::max(least, total / ((kf ? 64 : 32) * (int64_t)sms)));
+  const int64_t limit = std::max(piece + piece / 2, total / ((kf ? 32 : 8) * (int64_t)sms));
+  int64_t slot = 0;
   for (int64_t r = 0; r < n_nodes;) {
-    const int64_t r0 = r;
+    const int64_t r0 = r, nb = Srow[r + 1] - Srow[r];
+    if (nb > limit) {
+      const int64_t parts = std::min<int64_t>((nb + piece - 1) / piece, 4095);
+      for (int64_t p = 0; p < parts; p++)
+        out.push_back(make_int4(0, (int)r, (int)(1u | ((unsigned)parts << 8) | ((unsigned)p << 20)), (int)slot));
+      slot += parts;
+      r++;
+      continue;
+    }
     int64_t blocks = 0;
-    while (r < n_nodes && r - r0 < h2::kChunkRows && (r == r0 || blocks + (Srow[r + 1] - Srow[r]) <= target)) {
+    while (r < n_nodes && r - r0 < h2::kChunkRows && (r == r0 || blocks + (Srow[r + 1] - Srow[r]) <= piece)) {
       blocks += Srow[r + 1] - Srow[r];
       r++;
     }
     out.push_back(make_int4(0, (int)r0, (int)(r - r0), 0));
   }
+  *slots = slot;
   return out;
 }
 
@@ -361,12 +383,14 @@ h2_status mixed_configure(h2_matrix_s* h, int chunk_opt, int cw, int tree_opt) {
     M.tree_opt = tree_opt;
   }
   if (!M.chunk_dev[chunk_opt]) {
-    const std::vector<int4> c = coupling_chunks(M.srow_host.data(), h->n_nodes, kChunkOpts[chunk_opt]);
+    int64_t slots = 0;
+    const std::vector<int4> c =
+        coupling_chunks(M.srow_host.data(), h->n_nodes, kChunkOpts[chunk_opt], h->k, h->nS, h->grid, h->kf, &slots);
+    if (slots > M.cslots) return h2_fail(H2_ERR_INVALID, "internal: %lld coupling pieces exceed their slots", (long long)slots);
     h2_status st = upload(h, &M.chunk_dev[chunk_opt], c.data(), (int64_t)c.size());
     if (st != H2_OK) return st;
     M.chunk_n[chunk_opt] = (int64_t)c.size();
   }
-  M.chunks_host = coupling_chunks(M.srow_host.data(), h->n_nodes, kChunkOpts[chunk_opt]);
   M.launch.chunks = M.chunk_dev[chunk_opt];
   M.launch.nchunks = M.chunk_n[chunk_opt];
   M.launch.cw = cw;
@@ -521,9 +545,11 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
     // coupling blocks evaluated in the product from the kernel at the interpolation points
     // (Sec. 4.6): per node its centre c (midpoint of its Chebyshev nodes per dimension) as an
     // FP32 pair hi + lo, and its k points as FP32 offsets from c (tensor index, dimension 0
-    // slowest); unused dimensions are 0
+    // slowest), all times `unit`, which makes a distance the kernel's argument (base-2 exponent of
+    // exp(-r / ell), s of the Matern kernel); unused dimensions are 0
     const h2_coupling_kernel* kc = h->kc;
     const int dim = kc->dim, p = kc->p;
+    const double unit = (kc->kernel == H2_KERNEL_MATERN32 ? 1.7320508075688772 : 1.4426950408889634) / kc->ell;
     std::vector<float4> chi((size_t)nodes), clo((size_t)nodes), off((size_t)(nodes * k));
 #pragma omp parallel for schedule(static)
     for (int64_t n = 0; n < nodes; n++) {
@@ -537,8 +563,8 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
           b = std::max(b, cd[t]);
         }
         c[e] = 0.5 * (a + b);
-        hi[e] = (float)c[e];
-        lo[e] = (float)(c[e] - (double)hi[e]);
+        hi[e] = (float)(c[e] * unit);
+        lo[e] = (float)(c[e] * unit - (double)hi[e]);
       }
       chi[(size_t)n] = make_float4(hi[0], hi[1], hi[2], 0.f);
       clo[(size_t)n] = make_float4(lo[0], lo[1], lo[2], 0.f);
@@ -548,7 +574,7 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
         for (int e = dim - 1; e >= 0; e--) {
           const int a = rem % p;
           rem /= p;
-          o[e] = (float)(kc->cheb[(n * dim + e) * p + a] - c[e]);
+          o[e] = (float)((kc->cheb[(n * dim + e) * p + a] - c[e]) * unit);
         }
         off[(size_t)(n * k + nu)] = make_float4(o[0], o[1], o[2], 0.f);
       }
@@ -907,6 +933,13 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
   // tables of the table-driven kernels: this matrix alone
   MixedLaunch& L = M.launch;
   M.srow_host.assign(d->S_rowptr, d->S_rowptr + nodes + 1);
+  // the smallest target of this matrix alone cuts its rows into the most pieces
+  coupling_chunks(M.srow_host.data(), nodes, kChunkOpts[0], k, h->nS, h->grid, h->kf, &M.cslots);
+  if ((st = dalloc(h, &M.cpart, M.cslots * kPassVectors * M.kp4)) != H2_OK) return st;
+  if ((st = dalloc(h, &M.cticket, 4 * M.cslots)) != H2_OK) return st;
+  CUDA_TRY(cudaMemset(M.cticket, 0, (size_t)std::max<int64_t>(4 * M.cslots, 1) * sizeof(int)));
+  // entries k .. kp4 - 1 of a slot are summed into yhat's padding: zero
+  CUDA_TRY(cudaMemset(M.cpart, 0, (size_t)std::max<int64_t>(M.cslots * kPassVectors * M.kp4, 1) * sizeof(float)));
   L.items = M.dense_items.items;
   L.cta_begin = M.dense_items.cta_begin;
   L.blk = M.dblk;
@@ -1060,9 +1093,16 @@ h2_status batch_configure(h2_batch_s* b, int chunk_opt, int tree_opt, int cw) {
     return h2_fail(H2_ERR_INVALID, "internal: launch configuration out of range");
   if (!b->chunk_dev[chunk_opt]) {
     std::vector<int4> chunks;
+    int64_t total = 0;
+    for (const h2_matrix_s* h : b->hs) total += h->nS;
     for (int64_t i = 0; i < count; i++) {
       const h2_matrix_s* h = b->hs[(size_t)i];
-      for (int4 c : coupling_chunks(h->mx.srow_host.data(), h->n_nodes, kChunkOpts[chunk_opt])) {
+      int64_t slots = 0;
+      const std::vector<int4> own = coupling_chunks(h->mx.srow_host.data(), h->n_nodes, kChunkOpts[chunk_opt], h->k, total,
+                                                    h->grid, false, &slots);
+      if (slots > h->mx.cslots)
+        return h2_fail(H2_ERR_INVALID, "internal: %lld coupling pieces exceed their slots", (long long)slots);
+      for (int4 c : own) {
         c.x = (int)i;
         chunks.push_back(c);
       }

@@ -112,13 +112,14 @@ struct MatDesc {
   long long kk8, n_nodes;
   int k, kp, LR, q, L;
   int spanel;            // k = 64: coupling codes in the panel layout (8 panels of 8 rows, 1024 bytes apart)
-  // coupling blocks from the kernel (k_coupling_kf): node centres as FP32 high and low parts,
-  // the interpolation points' offsets from the centre, 1 / ell and the kernel kind
+  // coupling blocks from the kernel (k_coupling_kf), lengths in units of the kernel's argument
+  // (kf_unit): node centres as FP32 high and low parts, the interpolation points' offsets from them
   const float4* kf_chi;
   const float4* kf_clo;
   const float4* kf_off;
-  float kf_inv_ell;
-  int kf_kind;
+  // split coupling rows: partial sums [slot][v][kp] and a counter per (row's first slot, vector slice)
+  float* cpart;
+  int* cticket;
   // the leaf expansion done by the downsweep: the matrix's row jobs and the block records they index
   const RowJob* rjobs;
   const MixedBlock* blk;
@@ -563,11 +564,46 @@ __global__ void __launch_bounds__(kTreeWarpsM * 32) k_downsweep_tree_m(const Mat
 
 // ---------------------------------------------------------------- coupling, all levels
 // The coupling rows of all levels (Eq. 3) are cut into chunks of consecutive
-// rows of one matrix: int4 {matrix, first row, rows (1 .. 31), 0}, about the
-// same number of blocks each. One warp per chunk; a launch serves the
-// matrices whose vector count lies in [nvlo, nvhi] (the others' chunks return
-// at once), so a batch with mixed vector counts runs each count's variant.
+// rows of one matrix, or pieces of one long row, about the same number of blocks
+// each: int4 {matrix, first row, rows (1 .. 31) | parts << 8 | part << 20, slot}.
+// One warp per chunk; a launch serves the matrices whose vector count lies in
+// [nvlo, nvhi] (the others' chunks return at once), so a batch with mixed vector
+// counts runs each count's variant. A piece (parts > 1) leaves its sums in
+// slot + part of the matrix's cpart, and the row's last piece to finish adds the
+// pieces in order (split_finish). Without the pieces a matrix with few long rows
+// (3D, small n) ran on a few hundred warps, its longest row setting the time:
+// kernel-evaluated coupling at 3D n = 2^16, 8 vectors, 1420 us whole rows, 900 us in pieces.
 constexpr int kChunkRows = 31;
+__device__ __forceinline__ int chunk_parts(int4 ch) { return max(1, (ch.z >> 8) & 0xFFF); }
+__device__ __forceinline__ int chunk_part(int4 ch) { return (ch.z >> 20) & 0xFFF; }
+// where a chunk's row sums go: the row itself, or the piece's slot
+__device__ __forceinline__ float* chunk_dst(const MatDesc& D, int4 ch, int64_t row) {
+  return chunk_parts(ch) > 1 ? D.cpart + (int64_t)(ch.w + chunk_part(ch)) * D.nv * D.kp : D.yhat + row * D.nv * D.kp;
+}
+// this warp's piece (vectors vbase .. vbase + vcount - 1) is stored: the last of the row's pieces adds
+// them all in order. slice: the warp's vector slice (its own counter, at most four per row)
+__device__ __forceinline__ void split_finish(const MatDesc& D, int4 ch, int slice, int vbase, int vcount, int lane) {
+  const int parts = chunk_parts(ch);
+  int* ticket = D.cticket + 4 * (int64_t)ch.w + slice;
+  __threadfence();
+  __syncwarp();
+  int last = 0;
+  if (lane == 0) {
+    last = atomicAdd(ticket, 1) == parts - 1;
+    if (last) *ticket = 0;  // every piece is in: reset for the next product
+  }
+  if (!__shfl_sync(0xFFFFFFFFu, last, 0)) return;
+  __threadfence();
+  const int64_t stride = (int64_t)D.nv * D.kp;
+  const float* src = D.cpart + (int64_t)ch.w * stride + vbase * D.kp;
+  float* dst = D.yhat + ch.y * stride + vbase * D.kp;
+  for (int t = lane; t < vcount * D.kp; t += 32) {
+    float sum = 0.f;
+#pragma unroll 4
+    for (int p = 0; p < parts; p++) sum += __ldcg(src + p * stride + t);
+    dst[t] = sum;
+  }
+}
 
 // chunk state shared by both kernels: row pointers of the chunk in lanes 0 .. rows
 struct ChunkRows {
@@ -626,7 +662,7 @@ __global__ void __launch_bounds__(128) k_coupling_m(const MatDesc* __restrict__ 
   const int kp = D.kp;
   const float* __restrict__ xhat = D.xhat;
   float* __restrict__ yhat = D.yhat;
-  const int row0 = ch.y, rows = min(ch.z, kChunkRows);
+  const int row0 = ch.y, rows = min(ch.z & 0xFF, kChunkRows), parts = chunk_parts(ch), part = chunk_part(ch);
   const ChunkRows cr = chunk_rows(D.Srow, yhat, row0, rows, nv, kp, lane, vbase, min(NVW, nv - vbase));
   if (!cr.nonempty) return;
   const int m = lane % RG, cl = lane / RG;
@@ -715,7 +751,7 @@ __global__ void __launch_bounds__(128) k_coupling_m(const MatDesc* __restrict__ 
 #pragma unroll
         for (int v = 0; v < NVW; v++) acc[rr][v] += __shfl_xor_sync(0xFFFFFFFFu, acc[rr][v], off);
     if (cl == 0) {
-      float* dst = yhat + ((int64_t)(row0 + r) * nv + vbase) * kp + 8 * m;
+      float* dst = chunk_dst(D, ch, row0 + r) + vbase * kp + 8 * m;
 #pragma unroll
       for (int v = 0; v < NVW; v++)
         if (vbase + v < nv) {
@@ -739,7 +775,13 @@ __global__ void __launch_bounds__(128) k_coupling_m(const MatDesc* __restrict__ 
     c.r = __ffs(c.mask) - 1;
     c.bt = 0;
     c.b0 = __shfl_sync(0xFFFFFFFFu, cr.sr, c.r);
-    c.nslot = (__shfl_sync(0xFFFFFFFFu, cr.sr, c.r + 1) - c.b0) * SPB;
+    int nb = __shfl_sync(0xFFFFFFFFu, cr.sr, c.r + 1) - c.b0;
+    if (parts > 1) {  // a piece of the row (its only row)
+      const int lo = (int)((int64_t)nb * part / parts);
+      nb = (int)((int64_t)nb * (part + 1) / parts) - lo;
+      c.b0 += lo;
+    }
+    c.nslot = nb * SPB;
   };
   auto advance = [&](Cursor& c) -> bool {
     if ((c.bt + 1) * CB < c.nslot) {
@@ -794,6 +836,7 @@ __global__ void __launch_bounds__(128) k_coupling_m(const MatDesc* __restrict__ 
     if ((cc.bt + 1) * CB >= cc.nslot) flush(cc.r);
     if (!advance(cc)) break;
   }
+  if (parts > 1) split_finish(D, ch, warp % VG, vbase, min(NVW, nv - vbase), lane);
 }
 
 // any other k: the chunk's rows one after another, one block at a time
@@ -817,11 +860,16 @@ __global__ void __launch_bounds__(128) k_coupling_m_generic(const MatDesc* __res
   const int k = D.k, kp = D.kp, LR = D.LR;
   const float* __restrict__ xhat = D.xhat;
   float* __restrict__ yhat = D.yhat;
-  const int row0 = ch.y, rows = min(ch.z, kChunkRows);
+  const int row0 = ch.y, rows = min(ch.z & 0xFF, kChunkRows), parts = chunk_parts(ch), part = chunk_part(ch);
   const ChunkRows cr = chunk_rows(D.Srow, yhat, row0, rows, nv, kp, lane, 0, nv);
   for (unsigned m = cr.nonempty; m; m &= m - 1u) {
     const int r = __ffs(m) - 1;
-    const int32_t b0 = __shfl_sync(0xFFFFFFFFu, cr.sr, r), b1 = __shfl_sync(0xFFFFFFFFu, cr.sr, r + 1);
+    int32_t b0 = __shfl_sync(0xFFFFFFFFu, cr.sr, r), b1 = __shfl_sync(0xFFFFFFFFu, cr.sr, r + 1);
+    if (parts > 1) {  // a piece of the row
+      const int64_t nb = b1 - b0;
+      b1 = b0 + (int32_t)(nb * (part + 1) / parts);
+      b0 += (int32_t)(nb * part / parts);
+    }
     float acc[RPL][NVB];
 #pragma unroll
     for (int rr = 0; rr < RPL; rr++)
@@ -833,8 +881,9 @@ __global__ void __launch_bounds__(128) k_coupling_m_generic(const MatDesc* __res
       __syncwarp();
     }
     group_reduce_m(acc, LR);
-    store_node_m<RPL, NVB, false>(yhat + (int64_t)(row0 + r) * nv * kp, k, kp, LR, nv, acc, lane);
+    store_node_m<RPL, NVB, false>(chunk_dst(D, ch, row0 + r), k, kp, LR, nv, acc, lane);
   }
+  if (parts > 1) split_finish(D, ch, 0, 0, nv, lane);
 }
 
 // ---------------------------------------------------------------- coupling from the kernel
@@ -848,17 +897,27 @@ __global__ void __launch_bounds__(128) k_coupling_m_generic(const MatDesc* __res
 // (group g the blocks b0 + g, b0 + g + G, ...; GB <= G groups, so that their staged data fit),
 // each lane all k columns of its group's block in runs of four, so a vector's four entries are one
 // float4 read. A row's sums are reduced over the groups once, after its last block. Each group
-// stages its block's column points and vectors in the warp's shared memory; r = r2 * rsqrt(r2)
-// and exp(-t) = __expf(-t) (CUDA's fast intrinsics: relative errors of a few 1e-6 here, below the
-// form's FP32 accumulation bound).
-// 2^x by the special-function unit (PTX ex2.approx: relative error a few 2^-23)
+// stages its block's column points and vectors in the warp's shared memory. The points are stored
+// scaled (kf_unit: log2(e) / ell, or sqrt(3) / ell for Matern), so that a value is one distance
+// t = r2 * rsqrt(r2) and 2^-t, or (1 + t) 2^(-t log2 e): nine instructions, two of them on the
+// special-function unit, and one FMA per vector.
+// What bounds it: issue slots (3D n = 2^16, 8 vectors, 4.65e8 values: 28 instructions a value before
+// the scaling moved to the points and the vector loop lost its per-vector branches; with the finer
+// row split of coupling_chunks 900 -> 441 us).
+// 2^x and 1 / sqrt(x) by the special-function unit (PTX approx: relative errors of a few 2^-23; no
+// argument here is subnormal, so flushing those to zero changes nothing)
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 __device__ __forceinline__ float ex2_approx(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
 
-// KIND: H2_KERNEL_EXP (0) or H2_KERNEL_MATERN32 (1); the descriptor's kf_kind selects the instance
+// KIND: H2_KERNEL_EXP (0) or H2_KERNEL_MATERN32 (1)
 template <int RPL, int NVB, int KIND>
 __global__ void __launch_bounds__(128, RPL == 1 ? 6 : 4) k_coupling_kf(const MatDesc* __restrict__ mats,
                                                                      const int4* __restrict__ chunks, int64_t nchunks,
@@ -875,23 +934,25 @@ __global__ void __launch_bounds__(128, RPL == 1 ? 6 : 4) k_coupling_kf(const Mat
   const int k = min(D.k, 64), kp = D.kp, LR = D.LR, G = 32 / LR, g = lane / LR, rl = lane - g * LR;
   const int GB = max(1, min(G, 64 / kp));  // groups with a block: GB * kp <= 64 staged columns
   const bool active = g < GB;
-  float* wbuf = wstage[warp] + g * nv * kp;  // this group's block: vectors (nv x kp) and points (k)
+  float* wbuf = wstage[warp] + (active ? g : 0) * NVB * kp;  // this group's block: vectors (NVB x kp) and points (k)
   float4* obuf = ostage[warp] + g * kp;
   const float4* __restrict__ chi = D.kf_chi;
   const float4* __restrict__ clo = D.kf_clo;
   const float4* __restrict__ off = D.kf_off;
-  const float inv_ell = D.kf_inv_ell;
-  // exp: K = 2^(-r c), c = log2(e) / ell; Matern-3/2: t = r sqrt(3) / ell, K = (1 + t) 2^(-t log2(e))
-  const float tscale = KIND == 1 ? 1.7320508f * inv_ell : 1.4426950f * inv_ell;
   const int32_t* __restrict__ Scol = D.Scol;
   const float* __restrict__ xhat = D.xhat;
   float* __restrict__ yhat = D.yhat;
-  const int row0 = ch.y, rows = min(ch.z, kChunkRows);
+  const int row0 = ch.y, rows = min(ch.z & 0xFF, kChunkRows), parts = chunk_parts(ch), part = chunk_part(ch);
   const ChunkRows cr = chunk_rows(D.Srow, yhat, row0, rows, nv, kp, lane, 0, nv);
   for (unsigned m = cr.nonempty; m; m &= m - 1u) {
     const int r = __ffs(m) - 1;
     const int64_t i = row0 + r;
-    const int32_t b0 = __shfl_sync(0xFFFFFFFFu, cr.sr, r), b1 = __shfl_sync(0xFFFFFFFFu, cr.sr, r + 1);
+    int32_t b0 = __shfl_sync(0xFFFFFFFFu, cr.sr, r), b1 = __shfl_sync(0xFFFFFFFFu, cr.sr, r + 1);
+    if (parts > 1) {  // a piece of the row
+      const int64_t nb = b1 - b0;
+      b1 = b0 + (int32_t)(nb * (part + 1) / parts);
+      b0 += (int32_t)(nb * part / parts);
+    }
     float4 oi[RPL];
 #pragma unroll
     for (int rr = 0; rr < RPL; rr++) {
@@ -940,7 +1001,7 @@ __global__ void __launch_bounds__(128, RPL == 1 ? 6 : 4) k_coupling_kf(const Mat
             for (int rr = 0; rr < RPL; rr++) {
               const float dx = ax[rr] - oj.x, dy = ay[rr] - oj.y, dz = az[rr] - oj.z;
               const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-              const float t = (r2 * rsqrtf(r2)) * tscale;
+              const float t = r2 * rsqrt_approx(r2);
               float val;
               if constexpr (KIND == 1) {
                 const float ex = ex2_approx(-1.4426950f * t);
@@ -953,7 +1014,8 @@ __global__ void __launch_bounds__(128, RPL == 1 ? 6 : 4) k_coupling_kf(const Mat
           }
 #pragma unroll
           for (int v = 0; v < NVB; v++) {
-            if (v >= nv) break;
+            // tested every fourth vector only: a vector past nv multiplies what its slot holds, unused
+            if ((v & 3) == 0 && v >= nv) break;
             float4 xv = *reinterpret_cast<const float4*>(wbuf + v * kp + mu0);
             if (!FULL) {  // entries past k (the vectors' padding) take no part
               if (mu0 + 3 >= k) xv.w = 0.f;
@@ -973,8 +1035,9 @@ __global__ void __launch_bounds__(128, RPL == 1 ? 6 : 4) k_coupling_kf(const Mat
     }
     // the groups' partial sums: lanes rl, rl + LR, ... hold the same rows
     group_reduce_m(acc, LR);
-    store_node_m<RPL, NVB, false>(yhat + i * nv * kp, k, kp, LR, nv, acc, lane);
+    store_node_m<RPL, NVB, false>(chunk_dst(D, ch, i), k, kp, LR, nv, acc, lane);
   }
+  if (parts > 1) split_finish(D, ch, 0, 0, nv, lane);
 }
 
 // ---------------------------------------------------------------- dense near field + expansion (TMA stream)

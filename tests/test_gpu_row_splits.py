@@ -6,6 +6,10 @@ import torch
 
 import h2gen
 import oracle
+from fp32_tol import acc_tol, check
+from oracle import kernel_coupling, quant
+
+KERNEL_EVAL = 2e-6  # the evaluated blocks' own error (test_gpu_kernel_coupling.py)
 
 pytestmark = pytest.mark.gpu
 
@@ -36,4 +40,32 @@ def test_split_rows_fp64(h2, shape, nv):
     first = M.matvec(to_dev(x)).cpu().numpy()
     assert oracle.rel_l2(first, ref) <= 1e-12
     assert np.array_equal(M.matvec(to_dev(x)).cpu().numpy(), first)  # the tickets are back at zero, the order is fixed
+    M.close()
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("nv", [1, 3, 7, 16])
+def test_split_rows_scaled(h2, shape, nv):
+    A = h2gen.generate(**shape, kernel="exp", seed=32)
+    x = h2gen.vectors(720 + nv, A.n, nv)
+    M = h2.H2Matrix.from_generator(A, storage="int16", bases_fp32=True)
+    ref = oracle.matvec(A, x, **quant.dequantized_arrays(A, "int16", True))
+    first = M.matvec(to_dev(x)).cpu().numpy()
+    check(oracle.rel_l2(first, ref), acc_tol(A), ("split rows", A.k, nv))
+    assert np.array_equal(M.matvec(to_dev(x)).cpu().numpy(), first)
+    M.close()
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("nv", [1, 6, 16])
+@pytest.mark.parametrize("kernel", ["exp", "matern32"])
+def test_split_rows_evaluated(h2, shape, nv, kernel):
+    A = h2gen.generate(**shape, kernel=kernel, seed=33)
+    x = h2gen.vectors(740 + nv, A.n, nv)
+    M = h2.H2Matrix.from_generator(A, storage="int16", bases_fp32=True, coupling="kernel")
+    arrays = dict(quant.dequantized_arrays(A, "int16", True))
+    arrays["S_val"] = kernel_coupling.coupling_blocks(A.chebyshev_nodes(), A.kernel, A.ell, A.S_rowptr, A.S_colidx)
+    first = M.matvec(to_dev(x)).cpu().numpy()
+    check(oracle.rel_l2(first, oracle.matvec(A, x, **arrays)), acc_tol(A) + KERNEL_EVAL, ("split rows, evaluated", A.k, nv, kernel))
+    assert np.array_equal(M.matvec(to_dev(x)).cpu().numpy(), first)
     M.close()
