@@ -388,13 +388,13 @@ h2_status h2_batch_matvec(h2_batch b, const int32_t* nv, const double* const* x,
  * Autotuning of a batch: as h2_tune, over the candidates
  *   dense consumer warps:   8 or 16 (16 only when no member takes more than 8 vectors)
  *   coupling row chunks:    about 64, 128 or 256 coupling blocks per warp
- *   tree jobs:              subtrees of 16, 32 or 64 leaves per CTA
+ *   tree jobs:              subtrees of 16, 32 or 64 leaves per group of eight CTAs
  * (one warm-up and two timed batched products each, arguments as for
  * h2_batch_matvec), then the split of the dense work items over the CTAs:
  * each leaf row weighed by its bytes times (1 + beta nv/16), nv its member's
  * vectors per pass, beta in {0, 1, 2, 4} (the fastest kept). chosen[0]
- * consumer warps, chosen[1] chunk size, chosen[2] leaves per tree CTA.
- * Synchronizes `stream`.
+ * consumer warps, chosen[1] chunk size, chosen[2] leaves per group of
+ * eight tree CTAs. Synchronizes `stream`.
  */
 h2_status h2_batch_tune(h2_batch b, const int32_t* nv, const double* const* x, const int64_t* ldx,
                         double* const* y, const int64_t* ldy, void* stream, int32_t chosen[3]);

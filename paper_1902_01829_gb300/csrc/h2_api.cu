@@ -446,13 +446,15 @@ void profile_free(Profiler* p) {
 namespace {
 
 template <int NVB>
-cudaError_t set_stream_smem() {
-  static cudaError_t done = cudaErrorNotReady;
-  if (done == cudaErrorNotReady) {
+cudaError_t set_pass_smem() {
+  static const cudaError_t done = [] {
     constexpr int CW = h2::dense_consumer_warps(NVB);
-    done = cudaFuncSetAttribute(h2::k_dense_stream<NVB, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                h2::stream_smem_bytes(NVB, CW));
-  }
+    cudaError_t e = cudaFuncSetAttribute(h2::k_dense_stream<NVB, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         h2::stream_smem_bytes(NVB, CW));
+    for (const void* f : {(const void*)h2::k_upsweep_tree<NVB>, (const void*)h2::k_downsweep_tree<NVB>})
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, h2::kSmemLimit);
+    return e;
+  }();
   return done;
 }
 
@@ -461,7 +463,7 @@ h2_status run_pass(h2_matrix_s* h, int nv, const double* x, int64_t ldx, double*
   using namespace h2;
   const int k = h->k, kp = h->kp, LR = h->lr;
   const unsigned wb = (unsigned)kWarps * 32;
-  cudaError_t e = set_stream_smem<NVB>();
+  cudaError_t e = set_pass_smem<NVB>();
   if (e != cudaSuccess) return fail(H2_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
   constexpr int CW = dense_consumer_warps(NVB);
   constexpr int smem = stream_smem_bytes(NVB, CW);
@@ -469,7 +471,7 @@ h2_status run_pass(h2_matrix_s* h, int nv, const double* x, int64_t ldx, double*
   TreeParams T{};
   T.Vt = h->Vt;
   T.Ft = h->Ft;
-  T.E = h->E;
+  T.Et = h->E;
   T.leaf_off = h->leaf_off;
   T.xp_off = h->xp_off;
   T.x = x;
@@ -484,14 +486,15 @@ h2_status run_pass(h2_matrix_s* h, int nv, const double* x, int64_t ldx, double*
   T.vexp = h->vexp;
   T.k = k;
   T.kp = kp;
-  T.LR = LR;
+  T.kks = (int64_t)k * k;
   T.q = h->q;
   T.L = h->tree_L;
   T.nv = nv;
-  const unsigned tree_grid = 1u << h->tree_L, tree_threads = kTreeWarps * 32;
+  const unsigned tree_grid = 1u << h->tree_L, tree_threads = tree_warps<NVB>() * 32;
+  const unsigned tsm = tree_smem<TreeOp64, NVB>(k, tree_block_entries(k, T.kks, false), T.q - T.L).bytes;
   cudaError_t me = mark(&h->prof, st);
   k_vec_scale<<<kScaleBlocks, kScaleThreads, 0, st>>>(x, ldx, h->n, nv, h->vpart, h->vticket, h->vexp);
-  k_upsweep_tree<RPL_K, NVB><<<tree_grid, tree_threads, 0, st>>>(T);
+  k_upsweep_tree<NVB><<<std::max(tree_grid, (unsigned)kTreeCluster), tree_threads, tsm, st>>>(T);
   if (me == cudaSuccess) me = mark(&h->prof, st);
   CouplingParams C{};
   C.S = h->smat;
@@ -515,7 +518,7 @@ h2_status run_pass(h2_matrix_s* h, int nv, const double* x, int64_t ldx, double*
     k_coupling_generic<RPL_K, NVB><<<cgrid, wb, 0, st>>>(C);
   }
   if (me == cudaSuccess) me = mark(&h->prof, st);
-  k_downsweep_tree<RPL_K, NVB><<<tree_grid, tree_threads, 0, st>>>(T);
+  k_downsweep_tree<NVB><<<tree_grid, tree_threads, tsm, st>>>(T);
   if (me == cudaSuccess) me = mark(&h->prof, st);
   StreamParams P{};
   P.items = h->dense_items.items;
@@ -605,10 +608,11 @@ h2_status build_device(h2_matrix_s* h, const h2_desc* d) {
   CUDA_TRY(cudaMemset(h->err, 0, sizeof(int)));
   if ((st = dalloc(h, &h->ticket, h->n_nodes)) != H2_OK) return st;
   CUDA_TRY(cudaMemset(h->ticket, 0, (size_t)h->n_nodes * sizeof(int)));
-  // subtree roots of the fused tree kernels: at least two CTAs per SM when the tree is deep enough
-  int lmax = 0;
-  while (((int64_t)1 << lmax) < 2 * (int64_t)h->grid) lmax++;
-  h->tree_L = std::min(h->q, lmax);
+  // subtree roots of the tree kernels: up to 128 CTAs of one leaf; then four leaves per CTA, whose three
+  // inner steps cost less than two more climbed levels (2D n = 2^16, 16 vectors, up + down: four leaves
+  // 73 us, two 85, eight 94); from 2^13 leaves on the CTAs outnumber the SMs many times and each repeats
+  // the path from the root, so they take up to 16
+  h->tree_L = h->q <= 7 ? h->q : h->q <= 9 ? 7 : h->q <= 12 ? h->q - 2 : std::max(10, h->q - 4);
   if (h->storage != H2_FP64) return mixed_build(h, d);
 
   // padded leaf offsets of the split x

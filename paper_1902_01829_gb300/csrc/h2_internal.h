@@ -51,6 +51,7 @@ struct MixedLaunch {
   void* mats = nullptr;              // device h2::MatDesc table
   const int2* jobs = nullptr;        // (matrix, subtree) per tree CTA
   int64_t njobs = 0;
+  int tree_T = 0;                    // levels below the subtree roots of the deepest job
   const int4* chunks = nullptr;      // coupling row chunks (mixed.cuh)
   int64_t nchunks = 0;
   const h2::StreamItem* items = nullptr;
@@ -162,7 +163,7 @@ struct MixedData {
 
 // launch parameters the tuner chooses between (h2_tune, h2_batch_tune)
 constexpr int kChunkOpts[3] = {64, 128, 256};  // coupling blocks per warp chunk (target)
-constexpr int kTreeOpts[3] = {4, 5, 6};       // log2 of the leaves per tree CTA (batches)
+constexpr int kTreeOpts[3] = {1, 2, 3};       // log2 of the leaves per tree CTA (batches; a cluster of 8 CTAs: 16 .. 64)
 constexpr int kDefaultChunkOpt = 1, kDefaultTreeOpt = 2;
 constexpr int kDenseCW = 8;                   // dense-stream consumer warps (or twice as many)
 std::vector<int4> coupling_chunks(const int32_t* Srow, int64_t n_nodes, int64_t target, int k, int64_t total, int sms,

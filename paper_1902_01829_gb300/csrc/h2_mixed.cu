@@ -356,6 +356,12 @@ std::vector<int4> coupling_chunks(const int32_t* Srow, int64_t n_nodes, int64_t 
   return out;
 }
 
+// the tree jobs of matrix `mat` with subtrees at level L: one CTA each, filled up to whole clusters
+void tree_jobs(int mat, int L, std::vector<int2>* jobs) {
+  const int n = 1 << L;
+  for (int t = 0; t < std::max(n, h2::kTreeCluster); t++) jobs->push_back(make_int2(mat, t < n ? t : -1));
+}
+
 h2_status mixed_configure(h2_matrix_s* h, int chunk_opt, int cw, int tree_opt) {
   MixedData& M = h->mx;
   if (chunk_opt < 0 || chunk_opt > 2 || tree_opt < 0 || tree_opt > 2 ||
@@ -364,8 +370,8 @@ h2_status mixed_configure(h2_matrix_s* h, int chunk_opt, int cw, int tree_opt) {
   if (tree_opt != M.tree_opt) {  // subtree level of the tree jobs (in the descriptor and the job list)
     const int L = std::max(0, h->tree_L - tree_opt);
     if (!M.jobs_dev[tree_opt]) {
-      std::vector<int2> jobs((size_t)1 << L);
-      for (size_t t = 0; t < jobs.size(); t++) jobs[t] = make_int2(0, (int)t);
+      std::vector<int2> jobs;
+      tree_jobs(0, L, &jobs);
       h2_status st = upload(h, &M.jobs_dev[tree_opt], jobs.data(), (int64_t)jobs.size());
       if (st != H2_OK) return st;
     }
@@ -379,7 +385,8 @@ h2_status mixed_configure(h2_matrix_s* h, int chunk_opt, int cw, int tree_opt) {
       CUDA_TRY(cudaMemcpy(M.launch.mats, &D, sizeof(D), cudaMemcpyHostToDevice));
     }
     M.launch.jobs = M.jobs_dev[tree_opt];
-    M.launch.njobs = (int64_t)1 << L;
+    M.launch.tree_T = h->q - L;
+    M.launch.njobs = std::max<int64_t>((int64_t)1 << L, h2::kTreeCluster);
     M.tree_opt = tree_opt;
   }
   if (!M.chunk_dev[chunk_opt]) {
@@ -1114,8 +1121,7 @@ h2_status batch_configure(h2_batch_s* b, int chunk_opt, int tree_opt, int cw) {
   if (!b->jobs_dev[tree_opt]) {
     std::vector<int2> jobs;
     for (int64_t i = 0; i < count; i++) {
-      const int Li = std::max(0, b->hs[(size_t)i]->q - T);
-      for (int64_t t = 0; t < ((int64_t)1 << Li); t++) jobs.push_back(make_int2((int)i, (int)t));
+      tree_jobs((int)i, std::max(0, b->hs[(size_t)i]->q - T), &jobs);
     }
     if ((int64_t)jobs.size() >= INT32_MAX) return h2_fail(H2_ERR_UNSUPPORTED, "batch too large: %lld tree jobs", (long long)jobs.size());
     if ((st = balloc(b, &b->jobs_dev[tree_opt], (int64_t)jobs.size(), jobs.data())) != H2_OK) return st;
@@ -1139,6 +1145,7 @@ h2_status batch_configure(h2_batch_s* b, int chunk_opt, int tree_opt, int cw) {
   L.chunks = b->chunk_dev[chunk_opt];
   L.nchunks = b->chunk_n[chunk_opt];
   L.jobs = b->jobs_dev[tree_opt];
+  L.tree_T = T;
   L.njobs = b->jobs_n[tree_opt];
   L.cw = cw;
   b->chunk_opt = chunk_opt;
@@ -1225,16 +1232,17 @@ h2_status batch_build(h2_batch_s* b) {
   L.bases_fp32 = h0->mx.bases_fp32;
   L.prof = nullptr;
   b->n_items = (int64_t)items.size();
-  // defaults (h2_batch_tune may choose others): at most 64 leaves per tree CTA, fewer while the
-  // batch has under four tree CTAs per SM; 128 coupling blocks per chunk; 16 dense consumer warps
-  // when every member's leaves hold at most 32 points
+  // defaults (h2_batch_tune may choose others): eight leaves per tree CTA, four (two) while the batch has
+  // under eight tree CTAs per SM (32 matrices of 1024 .. 16384 points: 1046 us a product with eight, 1037
+  // with four, 1098 with two); 128 coupling blocks per chunk; 16 dense consumer warps when every
+  // member's leaves hold at most 32 points
   int tree_opt = kDefaultTreeOpt;
   auto jobs_for = [&](int T) {
     int64_t n = 0;
     for (const h2_matrix_s* h : b->hs) n += (int64_t)1 << std::max(0, h->q - T);
     return n;
   };
-  while (tree_opt > 0 && jobs_for(kTreeOpts[tree_opt]) < 4 * (int64_t)h0->grid) tree_opt--;
+  while (tree_opt > 0 && jobs_for(kTreeOpts[tree_opt]) < (tree_opt == 2 ? 8 : 4) * (int64_t)h0->grid) tree_opt--;
   bool small = true;
   for (const h2_matrix_s* h : b->hs) small = small && h->m_max <= 32;
   b->tree_opt = -1;
@@ -1428,7 +1436,7 @@ h2_status h2_batch_tune(h2_batch b, const int32_t* nv, const double* const* x, c
   }
   chosen[0] = best_cw;
   chosen[1] = kChunkOpts[best_c];
-  chosen[2] = 1 << kTreeOpts[best_t];
+  chosen[2] = h2::kTreeCluster << kTreeOpts[best_t];
   return H2_OK;
 }
 

@@ -10,20 +10,22 @@
 
 namespace h2i {
 
-template <int F, int NVB, int CW>
-cudaError_t set_mixed_smem() {
-  static cudaError_t done = cudaErrorNotReady;
-  if (done == cudaErrorNotReady)
-    done = cudaFuncSetAttribute(h2::k_dense_stream_m<F, NVB, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                h2::mixed_smem_bytes(NVB, CW));
-  return done;
-}
-
-// Kernels that run beside the dense stream prefer its L1 / shared memory split (the largest shared
-// part): an SM holds CTAs of one configuration at a time.
+// The dense stream and the kernels that run beside it prefer the largest shared part of the L1 / shared
+// memory split: an SM holds CTAs of one configuration at a time.
 template <class K>
 void prefer_max_shared(K kernel) {
   cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+}
+
+template <int F, int NVB, int CW>
+cudaError_t set_mixed_smem() {
+  static cudaError_t done = cudaErrorNotReady;
+  if (done == cudaErrorNotReady) {
+    done = cudaFuncSetAttribute(h2::k_dense_stream_m<F, NVB, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                h2::mixed_smem_bytes(NVB, CW));
+    prefer_max_shared(h2::k_dense_stream_m<F, NVB, CW>);
+  }
+  return done;
 }
 
 // the tree and coupling launches of one vector-count bucket (phase 0: upsweep, 1: coupling, 2: downsweep)
@@ -35,8 +37,14 @@ void bucket_phase(const MixedLaunch& L, int phase, int nvlo, cudaStream_t st, bo
   using namespace h2;
   static const bool carveout = [] {
     constexpr int NVW = NVB < 4 ? NVB : 4, VG = NVB / NVW;
-    prefer_max_shared(k_upsweep_tree_m<FB, RPL, NVB>);
-    prefer_max_shared(k_downsweep_tree_m<FB, RPL, NVB>);
+    prefer_max_shared(k_upsweep_tree_m<FB, NVB>);
+    prefer_max_shared(k_downsweep_tree_m<FB, NVB>);
+    if constexpr (NVB <= 4) {
+      prefer_max_shared(k_upsweep_tree_beside<FB, NVB>);
+      cudaFuncSetAttribute(k_upsweep_tree_beside<FB, NVB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+    }
+    cudaFuncSetAttribute(k_upsweep_tree_m<FB, NVB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+    cudaFuncSetAttribute(k_downsweep_tree_m<FB, NVB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     prefer_max_shared(k_coupling_kf<RPL, NVB, 0>);
     prefer_max_shared(k_coupling_kf<RPL, NVB, 1>);
     prefer_max_shared(k_coupling_m<F, 16, NVW, (NVW <= 2 ? 4 : 2), VG>);
@@ -47,9 +55,17 @@ void bucket_phase(const MixedLaunch& L, int phase, int nvlo, cudaStream_t st, bo
   }();
   (void)carveout;
   const MatDesc* mats = static_cast<const MatDesc*>(L.mats);
-  const unsigned tree_threads = kTreeWarpsM * 32;
+  const unsigned tree_threads = tree_warps<NVB>() * 32;
+  const int entries = tree_block_entries(L.k, round_up((int64_t)L.k * L.k, 8), FB != kFormF32);
+  const unsigned tsm = tree_smem<TreeOpM<FB>, NVB>(L.k, entries, L.tree_T).bytes;
   if (phase == 0 && L.njobs > 0) {
-    k_upsweep_tree_m<FB, RPL, NVB><<<(unsigned)L.njobs, tree_threads, 0, st>>>(mats, L.jobs, nvlo, NVB, convert ? 1 : 0);
+    if constexpr (NVB <= 4) {
+      if (!convert) {  // beside the dense stream
+        k_upsweep_tree_beside<FB, NVB><<<(unsigned)L.njobs, tree_threads, tsm, st>>>(mats, L.jobs, nvlo, NVB, L.tree_T, entries);
+        return;
+      }
+    }
+    k_upsweep_tree_m<FB, NVB><<<(unsigned)L.njobs, tree_threads, tsm, st>>>(mats, L.jobs, nvlo, NVB, convert ? 1 : 0, L.tree_T, entries);
   } else if (phase == 1 && L.nchunks > 0) {
     const unsigned cgrid = (unsigned)((L.nchunks + 3) / 4);
     const int k = L.k;
@@ -74,7 +90,7 @@ void bucket_phase(const MixedLaunch& L, int phase, int nvlo, cudaStream_t st, bo
       k_coupling_m_generic<F, RPL, NVB><<<cgrid, 128, 0, st>>>(mats, L.chunks, L.nchunks, nvlo, NVB);
     }
   } else if (phase == 2 && L.njobs > 0) {
-    k_downsweep_tree_m<FB, RPL, NVB><<<(unsigned)L.njobs, tree_threads, 0, st>>>(mats, L.jobs, nvlo, NVB, expand);
+    k_downsweep_tree_m<FB, NVB><<<(unsigned)L.njobs, tree_threads, tsm, st>>>(mats, L.jobs, nvlo, NVB, expand, L.tree_T, entries);
   }
 }
 

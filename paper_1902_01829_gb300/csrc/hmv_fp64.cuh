@@ -1,14 +1,14 @@
-// FP64 plain-form kernels for the tree phases of the H^2 matrix-vector
-// product (Sec. 4.2 and 4.4): leaf projection, upsweep and downsweep.
+// FP64 plain-form kernels of the H^2 matrix-vector product (Sec. 4.2 - 4.4): the tree phases
+// (tree.cuh with double-float arithmetic), the coupling phase and the per-vector scale.
 //
 // Each phase is a sum of column-major block products "rows += A_block * x_cols":
 //   leaf projection  xhat_j  = V_j^T x(j)            A = V_j^T (stored transposed)
 //   upsweep          xhat_p  = sum_c F_c^T xhat_c    A = F_c^T (stored transposed)   Eq. 2
+//   coupling         yhat_i  = sum_j S_ij xhat_j     A = S_ij                        Eq. 3
 //   downsweep        yhat_c += E_c yhat_p            A = E_c                         Eq. 5
-// One warp owns one output node: a lane owns output rows, consecutive lanes read
-// consecutive rows of a column (coalesced), the column's input entry is a
-// broadcast, and products accumulate in double-float. Loads of several columns
-// are issued before any of them is used, so a warp keeps many in flight.
+// A lane owns output rows, consecutive lanes read consecutive rows of a column (coalesced), the
+// column's input entry is a broadcast, and products accumulate in double-float. Loads of several
+// columns are issued before any of them is used, so a warp keeps many in flight.
 //
 // Range: every block is split with its exponent offset o (a' = a * 2^-o, see
 // df64.cuh) and x is scaled per vector by 2^-vexp[v], so that x, xhat and yhat
@@ -20,6 +20,7 @@
 //   yhat  same as xhat
 #pragma once
 #include "df64.cuh"
+#include "tree.cuh"
 
 namespace h2 {
 
@@ -28,8 +29,9 @@ constexpr int kWarps = 4;  // warps per CTA for the per-node kernels
 // Row mapping of a warp over an R-row block: lane = g * LR + rl owns rows
 // rl + 32 r (r < RPL) and columns col = g, g + G, ... with G = 32 / LR groups.
 // RPL = 2 requires LR = 32 (R <= 64); RPL = 1 allows LR = 1 .. 32 (R <= LR).
-template <int RPL, int NVB, bool CG = false>
-__device__ __forceinline__ void warp_mv_impl(const double* __restrict__ A, int o, int R, int C, int LR, const float2* xin,
+// xin is read with plain loads
+template <int RPL, int NVB>
+__device__ __forceinline__ void warp_mv(const double* __restrict__ A, int o, int R, int C, int LR, const float2* xin,
                                              int64_t xstride, int nv, float (&s)[RPL][NVB], float (&c)[RPL][NVB], int lane) {
   constexpr int UB = (NVB <= 2) ? 8 : (NVB <= 4 ? 4 : 2);  // columns whose loads are issued together
   const int G = 32 / LR;
@@ -47,8 +49,7 @@ __device__ __forceinline__ void warp_mv_impl(const double* __restrict__ A, int o
       }
 #pragma unroll
       for (int v = 0; v < NVB; v++)
-        xv[u][v] = (col < C && v < nv) ? (CG ? __ldcg(xin + v * xstride + col) : xin[v * xstride + col])
-                                       : make_float2(0.f, 0.f);
+        xv[u][v] = (col < C && v < nv) ? xin[v * xstride + col] : make_float2(0.f, 0.f);
     }
 #pragma unroll
     for (int u = 0; u < UB; u++) {
@@ -61,13 +62,6 @@ __device__ __forceinline__ void warp_mv_impl(const double* __restrict__ A, int o
       }
     }
   }
-}
-
-// xin is read with plain loads: it may have been written earlier in the same kernel by this CTA
-template <int RPL, int NVB>
-__device__ __forceinline__ void warp_mv(const double* __restrict__ A, int o, int R, int C, int LR, const float2* xin,
-                                        int64_t xstride, int nv, float (&s)[RPL][NVB], float (&c)[RPL][NVB], int lane) {
-  warp_mv_impl<RPL, NVB, false>(A, o, R, C, LR, xin, xstride, nv, s, c, lane);
 }
 
 // (S, C) += (s, c) elementwise, (s, c) = 0
@@ -103,37 +97,11 @@ __device__ __forceinline__ void group_reduce(float (&s)[RPL][NVB], float (&c)[RP
   }
 }
 
-// write a node's k x nv vector (stride kp per vector) from lanes of group 0; optionally add the old value
-template <int RPL, int NVB, bool ACCUM>
-__device__ __forceinline__ void store_node(float2* __restrict__ dst, int k, int kp, int LR, int nv, float (&s)[RPL][NVB],
-                                           float (&c)[RPL][NVB], int lane) {
-  if (lane >= LR) return;
-#pragma unroll
-  for (int r = 0; r < RPL; r++) {
-    const int row = lane + 32 * r;
-    if (row >= k) continue;
-#pragma unroll
-    for (int v = 0; v < NVB; v++) {
-      if (v >= nv) continue;
-      float ss = s[r][v], cc = c[r][v];
-      if (ACCUM) {
-        const float2 old = dst[v * kp + row];
-        df_add(ss, cc, old.x, old.y);
-      }
-      dst[v * kp + row] = df_norm(ss, cc);
-    }
-  }
-}
-
 // ---------------------------------------------------------------- tree phases, one launch each
-// CTA b owns the subtree rooted at node 2^L - 1 + b on level L (its T = q - L
-// levels below hold leaves [b 2^T, (b + 1) 2^T)). One warp computes one node.
-constexpr int kTreeWarps = 8;
-
 struct TreeParams {
   const double* Vt;        // leaf j: k x size_j (V_j^T)
   const double* Ft;        // node h >= 1: F_h^T
-  const double* E;         // node h >= 1: E_h
+  const double* Et;        // node h >= 1: E_h
   const int64_t* leaf_off;
   const int64_t* xp_off;
   const double* x;         // pass input, ldx
@@ -146,143 +114,80 @@ struct TreeParams {
   const int* oF;           // node h >= 1: exponent offset of F_h (upsweep into the parent)
   const int* oE;           // node h >= 1: exponent offset of E_h (downsweep from the parent)
   const int* vexp;         // per vector of the pass: x enters scaled by 2^-vexp[v]
-  int k, kp, LR, q, L, nv;
+  int64_t kks;             // doubles from a node's transfer matrix to the next node's
+  int k, kp, q, L, nv;
 };
 
-// leaf projection of leaf j: x2(j) = split(x(j)); xhat_j = V_j^T x(j)   (Alg. 2, first step)
-template <int RPL, int NVB>
-__device__ __forceinline__ void project_leaf(const TreeParams& P, int64_t j, int lane) {
-  const int64_t leaf0 = ((int64_t)1 << P.q) - 1;
-  const int64_t off = P.leaf_off[j];
-  const int sj = (int)(P.leaf_off[j + 1] - off);
-  const int spad = sj + (sj & 1);
-  float2* x2j = P.x2 + P.xp_off[j] * P.nv;
-  for (int v = 0; v < P.nv; v++) {
-    const int sv = P.vexp[v];
-    for (int a = lane; a < sj; a += 32) x2j[v * spad + a] = f64_to_df(scale2(P.x[v * P.ldx + off + a], -sv));
+// tree.cuh's arithmetic for the FP64 form: double-float vectors, FP64 entries split with their
+// block's exponent offset
+struct TreeOp64 {
+  using P = TreeParams;
+  using A = double;
+  using V = float2;
+  using Blk = int;
+  struct Acc {
+    float s, c;
+  };
+  static constexpr int kCopy = 8, kUnroll = 4;
+  static __device__ __forceinline__ double none() { return 0.0; }
+  static __device__ __forceinline__ float2 prep(double a, int o) {
+    float2 e;
+    split_f64(a, o, e.x, e.y);
+    return e;
   }
-  __syncwarp();
-  float s[RPL][NVB], c[RPL][NVB];
-  acc_zero(s, c);
-  warp_mv<RPL, NVB>(P.Vt + off * P.k, P.oV[j], P.k, sj, P.LR, x2j, spad, P.nv, s, c, lane);
-  group_reduce(s, c, P.LR);
-  store_node<RPL, NVB, false>(P.xhat + (leaf0 + j) * P.nv * P.kp, P.k, P.kp, P.LR, P.nv, s, c, lane);
+  static __device__ __forceinline__ void fma(Acc& p, float2 e, float2 x) { df_fma(p.s, p.c, e.x, e.y, x.x, x.y); }
+  static __device__ __forceinline__ void scale(Acc&, int) {}
+  static __device__ __forceinline__ void add(Acc& p, const Acc& q) { df_add(p.s, p.c, q.s, q.c); }
+  static __device__ __forceinline__ void add_value(Acc& p, float2 v) { df_add(p.s, p.c, v.x, v.y); }
+  static __device__ __forceinline__ Acc shfl_xor(const Acc& p, int off) {
+    return Acc{__shfl_xor_sync(0xFFFFFFFFu, p.s, off), __shfl_xor_sync(0xFFFFFFFFu, p.c, off)};
+  }
+  static __device__ __forceinline__ float2 value(const Acc& p) { return df_norm(p.s, p.c); }
+  static __device__ __forceinline__ int spad(int s) { return s + (s & 1); }
+  struct Leaf {
+    int64_t off, xp;  // first point; offset of the split x (per vector slot)
+    int s, bV, bU;    // points; exponent offset of V_j
+  };
+  static __device__ __forceinline__ Leaf leaf_v(const P& T, int64_t j) {
+    Leaf l;
+    l.off = T.leaf_off[j];
+    l.s = (int)(T.leaf_off[j + 1] - l.off);
+    l.xp = T.xp_off[j];
+    l.bV = T.oV[j];
+    l.bU = 0;
+    return l;
+  }
+  static __device__ __forceinline__ Leaf leaf_u(const P&, int64_t) { return Leaf{}; }
+  static __device__ __forceinline__ const double* Vt(const P& T, const Leaf& l) { return T.Vt + l.off * T.k; }
+  static __device__ __forceinline__ const double* Ft(const P& T, int64_t h) { return T.Ft + (h - 1) * T.kks; }
+  static __device__ __forceinline__ const double* E(const P& T, int64_t h) { return T.Et + (h - 1) * T.kks; }
+  static __device__ __forceinline__ int bF(const P& T, int64_t h) { return T.oF[h]; }
+  static __device__ __forceinline__ int bE(const P& T, int64_t h) { return T.oE[h]; }
+  using X = double;
+  static __device__ __forceinline__ double xload(const P& T, const Leaf& l, int v, int a, bool) {
+    return __ldg(T.x + v * T.ldx + l.off + a);
+  }
+  static __device__ __forceinline__ float2 xvalue(const P& T, double x, int v) { return f64_to_df(scale2(x, -T.vexp[v])); }
+  static __device__ __forceinline__ void xstore(const P& T, const Leaf& l, int sp, int v, int a, float2 x) {
+    T.x2[l.xp * T.nv + v * sp + a] = x;
+  }
+  static __device__ __forceinline__ int copy_bytes(int entries) { return 8 * entries; }
+  // (the leaf expansion is the dense stream's)
+  static __device__ __forceinline__ const double* U(const P&, const Leaf&) { return nullptr; }
+  static __device__ __forceinline__ int u_bytes(const P&, const Leaf&) { return 0; }
+  static __device__ __forceinline__ void u_layout(const P&, const Leaf&, int, int&, int&) {}
+  static __device__ __forceinline__ void ystore(const P&, int, int64_t, const Acc&, bool) {}
+};
+
+template <int NVB>
+__global__ void __cluster_dims__(kTreeCluster) __launch_bounds__(tree_warps<NVB>() * 32) k_upsweep_tree(TreeParams P) {
+  const bool active = (int64_t)blockIdx.x < ((int64_t)1 << P.L);
+  tree_up<TreeOp64, NVB, true>(P, active ? blockIdx.x : 0, active, true, P.q - P.L, tree_block_entries(P.k, P.kks, false));
 }
 
-// Eq. 2 at parent p: xhat_p = F_c1^T xhat_c1 + F_c2^T xhat_c2 (CG: read the children through L2)
-template <int RPL, int NVB, bool CG>
-__device__ __forceinline__ void up_node(const TreeParams& P, int64_t p, int lane) {
-  float s[RPL][NVB], c[RPL][NVB];
-  acc_zero(s, c);
-  for (int ci = 1; ci <= 2; ci++) {
-    const int64_t ch = 2 * p + ci;
-    warp_mv_impl<RPL, NVB, CG>(P.Ft + (ch - 1) * P.k * P.k, P.oF[ch], P.k, P.k, P.LR, P.xhat + ch * P.nv * P.kp, P.kp,
-                               P.nv, s, c, lane);
-  }
-  group_reduce(s, c, P.LR);
-  store_node<RPL, NVB, false>(P.xhat + p * P.nv * P.kp, P.k, P.kp, P.LR, P.nv, s, c, lane);
-}
-
-// Leaf projection and the whole upsweep (Alg. 2, Eq. 2) in one launch. Inside
-// a subtree the levels are separated by __syncthreads. Above level L, the
-// second CTA of a sibling pair to finish (atomic ticket) computes the parent,
-// so the climb needs no waiting: a CTA that arrives first simply stops.
-template <int RPL, int NVB>
-__global__ void __launch_bounds__(kTreeWarps * 32) k_upsweep_tree(TreeParams P) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int T = P.q - P.L;
-  const int64_t sub = blockIdx.x;
-  for (int64_t t = warp; t < ((int64_t)1 << T); t += kTreeWarps) project_leaf<RPL, NVB>(P, (sub << T) + t, lane);
-  __syncthreads();
-  for (int lvl = P.q - 1; lvl >= P.L; lvl--) {
-    const int64_t node0 = ((int64_t)1 << lvl) - 1 + (sub << (lvl - P.L));
-    for (int64_t t = warp; t < ((int64_t)1 << (lvl - P.L)); t += kTreeWarps) up_node<RPL, NVB, false>(P, node0 + t, lane);
-    __syncthreads();
-  }
-  __threadfence();  // every writer orders its xhat stores before the ticket below
-  __syncthreads();
-  if (warp != 0) return;
-  int64_t node = ((int64_t)1 << P.L) - 1 + sub;
-  while (node > 0) {
-    const int64_t par = (node - 1) / 2;
-    int second = 0;
-    if (lane == 0) {
-      second = atomicAdd(P.ticket + par, 1) == 1;
-      if (second) P.ticket[par] = 0;  // both arrivals are in: reset for the next product
-    }
-    second = __shfl_sync(0xFFFFFFFFu, second, 0);
-    if (!second) break;
-    __threadfence();  // order the sibling's xhat (published before its ticket) before our reads
-    up_node<RPL, NVB, true>(P, par, lane);
-    __threadfence();
-    __syncwarp();
-    node = par;
-  }
-}
-
-// Eq. 5 at node c: yhat_c += E_c yhat_parent (parent given explicitly)
-template <int RPL, int NVB>
-__device__ __forceinline__ void down_node(const TreeParams& P, int64_t ch, const float2* ypar, int lane) {
-  float s[RPL][NVB], c[RPL][NVB];
-  acc_zero(s, c);
-  warp_mv<RPL, NVB>(P.E + (ch - 1) * P.k * P.k, P.oE[ch], P.k, P.k, P.LR, ypar, P.kp, P.nv, s, c, lane);
-  group_reduce(s, c, P.LR);
-  store_node<RPL, NVB, true>(P.yhat + ch * P.nv * P.kp, P.k, P.kp, P.LR, P.nv, s, c, lane);
-}
-
-// The whole downsweep (Alg. 4, Eq. 5) in one launch. Warp 0 first carries the
-// parents' sums from the root down the path to this CTA's subtree root (the
-// path's nodes are shared with other CTAs, so their partial sums live only in
-// this CTA's shared memory; only the subtree root is written back). Then the
-// subtree is swept top-down, levels separated by __syncthreads.
-template <int RPL, int NVB>
-__global__ void __launch_bounds__(kTreeWarps * 32) k_downsweep_tree(TreeParams P) {
-  __shared__ float2 path[2][NVB][64];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t sub = blockIdx.x;
-  const int64_t root = ((int64_t)1 << P.L) - 1 + sub;
-  if (warp == 0 && P.L > 0) {
-    // path nodes a_0 = 0, ..., a_L = root: a_l = (root + 1) >> (L - l) minus 1
-    int cur = 0;
-    for (int v = 0; v < P.nv; v++)
-      for (int r = lane; r < P.k; r += 32) path[cur][v][r] = P.yhat[(int64_t)v * P.kp + r];  // node 0
-    __syncwarp();
-    for (int l = 1; l <= P.L; l++) {
-      const int64_t a = ((root + 1) >> (P.L - l)) - 1;
-      float s[RPL][NVB], c[RPL][NVB];
-      acc_zero(s, c);
-      warp_mv<RPL, NVB>(P.E + (a - 1) * P.k * P.k, P.oE[a], P.k, P.k, P.LR, &path[cur][0][0], 64, P.nv, s, c, lane);
-      group_reduce(s, c, P.LR);
-      if (lane < P.LR) {
-#pragma unroll
-        for (int rr = 0; rr < RPL; rr++) {
-          const int row = lane + 32 * rr;
-          if (row >= P.k) continue;
-#pragma unroll
-          for (int v = 0; v < NVB; v++) {
-            if (v >= P.nv) continue;
-            float ss = s[rr][v], cc = c[rr][v];
-            const float2 own = P.yhat[(a * P.nv + v) * P.kp + row];
-            df_add(ss, cc, own.x, own.y);
-            const float2 val = df_norm(ss, cc);
-            if (l == P.L) P.yhat[(a * P.nv + v) * P.kp + row] = val;
-            else path[cur ^ 1][v][row] = val;
-          }
-        }
-      }
-      __syncwarp();
-      cur ^= 1;
-    }
-  }
-  __syncthreads();
-  for (int lvl = P.L + 1; lvl <= P.q; lvl++) {
-    const int64_t node0 = ((int64_t)1 << lvl) - 1 + (sub << (lvl - P.L));
-    for (int64_t t = warp; t < ((int64_t)1 << (lvl - P.L)); t += kTreeWarps) {
-      const int64_t ch = node0 + t;
-      down_node<RPL, NVB>(P, ch, P.yhat + ((ch - 1) / 2) * P.nv * P.kp, lane);
-    }
-    __syncthreads();
-  }
+template <int NVB>
+__global__ void __launch_bounds__(tree_warps<NVB>() * 32) k_downsweep_tree(TreeParams P) {
+  tree_down<TreeOp64, NVB>(P, blockIdx.x, 0, P.q - P.L, tree_block_entries(P.k, P.kks, false));
 }
 
 // ---------------------------------------------------------------- coupling, all levels

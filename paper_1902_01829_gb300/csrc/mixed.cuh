@@ -16,6 +16,7 @@
 
 #include "stream_fp64.cuh"
 #include "tma.cuh"
+#include "tree.cuh"
 
 namespace h2 {
 
@@ -212,14 +213,14 @@ __device__ __forceinline__ void store_node_m(float* dst, int k, int kp, int LR, 
 }
 
 // ---------------------------------------------------------------- tree phases
-// Vt, Ft, E hold codes of the bases' format FB (16-bit codes, or FP32 entries)
+// Vt, Ft, Et hold codes of the bases' format (16-bit codes, or FP32 entries)
 struct TreeParamsM {
   const void* Vt;         // leaf j: k x size_j entries at vt_off[j]
   const float* vscale;
   const int64_t* vt_off;
-  const void* Ft;         // node h >= 1 at (h - 1) * kk8
+  const void* Ft;         // node h >= 1 at (h - 1) * kks
   const float* fscale;
-  const void* E;
+  const void* Et;
   const float* escale;
   const int64_t* leaf_off;
   const int64_t* xp4_off;
@@ -229,11 +230,10 @@ struct TreeParamsM {
   float* xhat;
   float* yhat;
   int* ticket;
-  int64_t kk8;
-  int k, kp, LR, q, L, nv, xy32;
+  int64_t kks;
+  int k, kp, q, L, nv, xy32;
+  const MatDesc* D;
 };
-
-constexpr int kTreeWarpsM = 8;
 
 __device__ __forceinline__ TreeParamsM tree_params(const MatDesc& D) {
   TreeParamsM P;
@@ -242,7 +242,7 @@ __device__ __forceinline__ TreeParamsM tree_params(const MatDesc& D) {
   P.vt_off = D.vt_off;
   P.Ft = D.Ft;
   P.fscale = D.fscale;
-  P.E = D.E;
+  P.Et = D.E;
   P.escale = D.escale;
   P.leaf_off = D.leaf_off;
   P.xp4_off = D.xp4_off;
@@ -252,314 +252,134 @@ __device__ __forceinline__ TreeParamsM tree_params(const MatDesc& D) {
   P.xhat = D.xhat;
   P.yhat = D.yhat;
   P.ticket = D.ticket;
-  P.kk8 = D.kk8;
+  P.kks = D.kk8;
   P.k = D.k;
   P.kp = D.kp;
-  P.LR = D.LR;
   P.q = D.q;
   P.L = D.L;
   P.nv = D.nv;
   P.xy32 = D.xy32;
+  P.D = &D;
   return P;
 }
 
-// copy n floats (n a multiple of 4, both ends 16-byte aligned) into the warp's staging buffer;
-// CG: read through L2 (the data was written by another CTA)
-template <bool CG>
+// tree.cuh's arithmetic for the scaled forms: FP32 vectors, entries of format F, a block's sum
+// multiplied by its scale once
+template <int F>
+struct TreeOpM {
+  using P = TreeParamsM;
+  using A = typename CodeT<F>::T;
+  using V = float;
+  using Blk = float;
+  using Acc = float;
+  static constexpr int kCopy = 16, kUnroll = 4;
+  static __device__ __forceinline__ A none() { return F == kFormInt16 ? (A)32768 : (A)0; }  // the code of zero
+  static __device__ __forceinline__ float prep(A a, float) { return code_to_f<F>(a); }
+  static __device__ __forceinline__ void fma(float& p, float e, float x) { p = fmaf(e, x, p); }
+  static __device__ __forceinline__ void scale(float& p, float sc) { p *= sc; }
+  static __device__ __forceinline__ void add(float& p, float q) { p += q; }
+  static __device__ __forceinline__ void add_value(float& p, float v) { p += v; }
+  static __device__ __forceinline__ float shfl_xor(float p, int off) { return __shfl_xor_sync(0xFFFFFFFFu, p, off); }
+  static __device__ __forceinline__ float value(float p) { return p; }
+  static __device__ __forceinline__ int spad(int s) { return (s + 3) & ~3; }
+  struct Leaf {
+    int64_t off, xp, vt;  // first point; offsets of x4 (per vector slot) and of V_j^T
+    int64_t uoff;         // U_j (size_j x k, column-major or in the panel layout) for the leaf expansion (Eq. 4)
+    int s, panel;
+    float bV, bU;
+  };
+  static __device__ __forceinline__ Leaf leaf_v(const P& T, int64_t j) {  // for the projection
+    Leaf l{};
+    l.off = T.leaf_off[j];
+    l.s = (int)(T.leaf_off[j + 1] - l.off);
+    l.xp = T.xp4_off[j];
+    l.vt = T.vt_off[j];
+    l.bV = T.vscale[j];
+    return l;
+  }
+  static __device__ __forceinline__ Leaf leaf_u(const P& T, int64_t j) {  // for the expansion
+    Leaf l{};
+    l.off = T.leaf_off[j];
+    l.s = (int)(T.leaf_off[j + 1] - l.off);
+    const RowJob J = T.D->rjobs[j];
+    const MixedBlock mb = T.D->blk[J.ublk];
+    l.uoff = J.uoff;
+    l.bU = mb.scale;
+    l.panel = (mb.src >> 2) & 1;
+    return l;
+  }
+  static __device__ __forceinline__ const A* Vt(const P& T, const Leaf& l) { return static_cast<const A*>(T.Vt) + l.vt; }
+  static __device__ __forceinline__ const A* F_(const void* p, const P& T, int64_t h) {
+    return static_cast<const A*>(p) + (h - 1) * T.kks;
+  }
+  static __device__ __forceinline__ const A* Ft(const P& T, int64_t h) { return F_(T.Ft, T, h); }
+  static __device__ __forceinline__ const A* E(const P& T, int64_t h) { return F_(T.Et, T, h); }
+  static __device__ __forceinline__ float bF(const P& T, int64_t h) { return T.fscale[h - 1]; }
+  static __device__ __forceinline__ float bE(const P& T, int64_t h) { return T.escale[h - 1]; }
+  using X = float;
+  static __device__ __forceinline__ float xload(const P& T, const Leaf& l, int v, int a, bool convert) {
+    return convert ? x_load(T.x, T.xy32, l.off + v * T.ldx + a) : T.x4[l.xp * T.nv + v * spad(l.s) + a];
+  }
+  static __device__ __forceinline__ float xvalue(const P&, float x, int) { return x; }
+  static __device__ __forceinline__ void xstore(const P& T, const Leaf& l, int sp, int v, int a, float x) {
+    T.x4[l.xp * T.nv + v * sp + a] = x;
+  }
+  static __device__ __forceinline__ int copy_bytes(int entries) { return (entries * (int)sizeof(A) + 15) & ~15; }
+  static __device__ __forceinline__ const char* U(const P& T, const Leaf& l) { return T.D->dmat + l.uoff; }
+  static __device__ __forceinline__ int u_bytes(const P& T, const Leaf& l) {
+    return l.panel ? panel_block_bytes(T.k) : copy_bytes(l.s * T.k);
+  }
+  static __device__ __forceinline__ void u_layout(const P& T, const Leaf& l, int row, int& roff, int& cs) {
+    if (l.panel) roff = (row >> 3) * (panel_stride(T.k) / 2) + (row & 7), cs = 8;
+  }
+  static __device__ __forceinline__ void ystore(const P& T, int v, int64_t i, float val, bool assign) {
+    y_store(T.D->y, T.xy32, v * T.D->ldy + i, val, assign);
+  }
+};
+
+// copy n floats (n a multiple of 4, both ends 16-byte aligned) into the warp's staging buffer
 __device__ __forceinline__ void stage_vectors(float* __restrict__ dst, const float* __restrict__ src, int n, int lane) {
   const float4* s4 = reinterpret_cast<const float4*>(src);
   float4* d4 = reinterpret_cast<float4*>(dst);
-  for (int i = lane; i < n / 4; i += 32) d4[i] = CG ? __ldcg(s4 + i) : s4[i];
+  for (int i = lane; i < n / 4; i += 32) d4[i] = s4[i];
   __syncwarp();
 }
 
-// Each warp stages the vector block it multiplies (a leaf's x chunk, a child's xhat, a
-// parent's yhat: nv x up to 64 floats) in its own shared-memory buffer wbuf, so that
-// warp_mv_m's many reads of it are shared-memory reads.
-// convert: x(j) is read in FP64 and its FP32 copy written to x4 here (products whose phases run
-// in order); else k_split_x4 wrote x4 before the launch
-template <int F, int RPL, int NVB>
-__device__ __forceinline__ void project_leaf_m(const TreeParamsM& P, int64_t j, int lane, float* wbuf, bool convert) {
-  const int64_t leaf0 = ((int64_t)1 << P.q) - 1;
-  const int64_t off = P.leaf_off[j];
-  const int sj = (int)(P.leaf_off[j + 1] - off);
-  const int spad = (sj + 3) & ~3;
-  float* xj = P.x4 + P.xp4_off[j] * P.nv;
-  if (convert) {
-    // every load of the chunk is issued before any store (the stores could alias x for the compiler)
-    float xr[NVB][2];
-#pragma unroll
-    for (int v = 0; v < NVB; v++)
-#pragma unroll
-      for (int h = 0; h < 2; h++) {
-        const int a = lane + 32 * h;
-        xr[v][h] = (v < P.nv && a < sj) ? x_load(P.x, P.xy32, off + v * P.ldx + a) : 0.f;  // padding is zero
-      }
-#pragma unroll
-    for (int v = 0; v < NVB; v++)
-#pragma unroll
-      for (int h = 0; h < 2; h++) {
-        const int a = lane + 32 * h;
-        if (v < P.nv && a < spad) {
-          xj[v * spad + a] = xr[v][h];
-          wbuf[v * spad + a] = xr[v][h];
-        }
-      }
-    __syncwarp();
-  } else {
-    stage_vectors<false>(wbuf, xj, P.nv * spad, lane);  // the FP32 copy of x(j), padding zero
-  }
-  float acc[RPL][NVB];
-#pragma unroll
-  for (int r = 0; r < RPL; r++)
-#pragma unroll
-    for (int v = 0; v < NVB; v++) acc[r][v] = 0.f;
-  warp_mv_m<F, RPL, NVB>(static_cast<const typename CodeT<F>::T*>(P.Vt) + P.vt_off[j], P.vscale[j], P.k, sj, P.LR, wbuf,
-                         spad, P.nv, acc, lane);
-  __syncwarp();
-  group_reduce_m(acc, P.LR);
-  store_node_m<RPL, NVB, false>(P.xhat + (leaf0 + j) * P.nv * P.kp, P.k, P.kp, P.LR, P.nv, acc, lane);
-}
-
-// parent p of the upsweep for vectors v0 .. v0 + nw - 1 (nw <= NVB)
-template <int F, int RPL, int NVB, bool CG>
-__device__ __forceinline__ void up_node_m(const TreeParamsM& P, int64_t p, int lane, float* wbuf, int v0, int nw) {
-  float acc[RPL][NVB];
-#pragma unroll
-  for (int r = 0; r < RPL; r++)
-#pragma unroll
-    for (int v = 0; v < NVB; v++) acc[r][v] = 0.f;
-  for (int ci = 1; ci <= 2; ci++) {
-    const int64_t ch = 2 * p + ci;
-    // CG: the sibling subtree was written by another CTA
-    stage_vectors<CG>(wbuf, P.xhat + (ch * P.nv + v0) * P.kp, nw * P.kp, lane);
-    warp_mv_m<F, RPL, NVB>(static_cast<const typename CodeT<F>::T*>(P.Ft) + (ch - 1) * P.kk8, P.fscale[ch - 1], P.k, P.k,
-                           P.LR, wbuf, P.kp, nw, acc, lane);
-    __syncwarp();
-  }
-  group_reduce_m(acc, P.LR);
-  store_node_m<RPL, NVB, false>(P.xhat + (p * P.nv + v0) * P.kp, P.k, P.kp, P.LR, nw, acc, lane);
-}
-
-// vectors per warp where the warps of a CTA split one node's vectors between them
-template <int NVB>
-__host__ __device__ constexpr int slice_vectors() { return NVB >= kTreeWarpsM ? NVB / kTreeWarpsM : 1; }
-
-// leaf projection + the whole upsweep in one launch (see k_upsweep_tree)
-// CTA b works on subtree jobs[b].y of matrix jobs[b].x
-template <int F, int RPL, int NVB>
-// (the matrices whose vector count lies outside [nvlo, nvhi] are left to another launch: all their CTAs return)
-__global__ void __launch_bounds__(kTreeWarpsM * 32) k_upsweep_tree_m(const MatDesc* __restrict__ mats,
-                                                                    const int2* __restrict__ jobs, int nvlo, int nvhi,
-                                                                    int convert) {
-  __shared__ __align__(16) float wstage[kTreeWarpsM][NVB * 64];
+// leaf projection + the whole upsweep in one launch: CTA b works on subtree jobs[b].y of matrix
+// jobs[b].x, a cluster on neighbouring subtrees of one matrix; jobs[b].y < 0 fills a cluster up (the
+// matrices whose vector count lies outside [nvlo, nvhi] are left to another launch: all their CTAs
+// return). T, entries: the launch's deepest subtree and largest block (its shared memory)
+template <int F, int NVB>
+__global__ void __cluster_dims__(kTreeCluster) __launch_bounds__(tree_warps<NVB>() * 32)
+    k_upsweep_tree_m(const MatDesc* __restrict__ mats, const int2* __restrict__ jobs, int nvlo, int nvhi, int convert, int T,
+                     int entries) {
   const int2 job = jobs[blockIdx.x];
   const TreeParamsM P = tree_params(mats[job.x]);
   if (P.nv < nvlo || P.nv > nvhi) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* wbuf = wstage[warp];
-  const int T = P.q - P.L;
-  const int64_t sub = job.y;
-  for (int64_t t = warp; t < ((int64_t)1 << T); t += kTreeWarpsM)
-    project_leaf_m<F, RPL, NVB>(P, (sub << T) + t, lane, wbuf, convert != 0);
-  __syncthreads();
-  constexpr int NVW = slice_vectors<NVB>();
-  for (int lvl = P.q - 1; lvl >= P.L; lvl--) {
-    const int64_t node0 = ((int64_t)1 << lvl) - 1 + (sub << (lvl - P.L));
-    const int nn = 1 << (lvl - P.L);
-    if (nn >= kTreeWarpsM || P.nv <= NVW) {  // a warp per node, all vectors
-      for (int t = warp; t < nn; t += kTreeWarpsM) up_node_m<F, RPL, NVB, false>(P, node0 + t, lane, wbuf, 0, P.nv);
-    } else {  // fewer nodes than warps: a warp per (node, slice of NVW vectors)
-      const int ns = (P.nv + NVW - 1) / NVW;
-      for (int u = warp; u < nn * ns; u += kTreeWarpsM) {
-        const int t = u % nn, v0 = (u / nn) * NVW;
-        up_node_m<F, RPL, NVW, false>(P, node0 + t, lane, wbuf, v0, min(NVW, P.nv - v0));
-      }
-    }
-    __syncthreads();
-  }
-  __threadfence();
-  __syncthreads();
-  // climb while this CTA arrives second at the parent; every warp takes a slice of the vectors
-  __shared__ int second;
-  const int v0 = warp * NVW, nw = min(NVW, P.nv - v0);
-  int64_t node = ((int64_t)1 << P.L) - 1 + sub;
-  while (node > 0) {
-    const int64_t par = (node - 1) / 2;
-    if (threadIdx.x == 0) {
-      const int s2 = atomicAdd(P.ticket + par, 1) == 1;
-      if (s2) P.ticket[par] = 0;
-      second = s2;
-    }
-    __syncthreads();
-    if (!second) break;
-    __threadfence();
-    if (nw > 0) up_node_m<F, RPL, NVW, true>(P, par, lane, wbuf, v0, nw);
-    __threadfence();
-    __syncthreads();
-    node = par;
-  }
+  tree_up<TreeOpM<F>, NVB, true>(P, max(job.y, 0), job.y >= 0, convert != 0, T, entries);
 }
 
-// the whole downsweep in one launch (see k_downsweep_tree)
-// Leaf expansion of leaf j (Eq. 4): y(j) = scale * U_j yhat_j (assign: the dense phase runs
-// afterwards and adds its part), or y(j) += scale * U_j yhat_j with FP64 atomic adds (the dense
-// phase adds its part the same way at the same time, both into a y zeroed before the product).
-// U_j is size_j x k, FP32 entries or 16-bit codes of format FB (column-major or panel layout);
-// its place and scale come from the matrix's row job and block record.
-template <int FB, int NVB>
-__device__ __forceinline__ void expand_leaf_m(const MatDesc& D, int64_t j, int lane, float* wbuf, bool assign) {
-  const RowJob J = D.rjobs[j];
-  const MixedBlock mb = D.blk[J.ublk];
-  const int nv = D.nv, k = D.k, kp = D.kp;
-  const int64_t off = D.leaf_off[j];
-  const int R = (int)(D.leaf_off[j + 1] - off);
-  stage_vectors<false>(wbuf, D.yhat + ((((int64_t)1 << D.q) - 1 + j) * nv) * kp, nv * kp, lane);
-  const bool f32 = (mb.src & 2) != 0, panel = (mb.src & 4) != 0;
-  const unsigned char* U = reinterpret_cast<const unsigned char*>(D.dmat) + J.uoff;
-  const int ps2 = panel_stride(k) / 2;
-  float acc[2][NVB];
-#pragma unroll
-  for (int r = 0; r < 2; r++)
-#pragma unroll
-    for (int v = 0; v < NVB; v++) acc[r][v] = 0.f;
-  for (int nu0 = 0; nu0 < k; nu0 += 8) {  // eight columns' loads before their use
-    float u[8][2];
-#pragma unroll
-    for (int c = 0; c < 8; c++)
-#pragma unroll
-      for (int r = 0; r < 2; r++) {
-        const int row = lane + 32 * r, nu = nu0 + c;
-        u[c][r] = 0.f;
-        if (row < R && nu < k) {
-          if (f32) u[c][r] = __ldg(reinterpret_cast<const float*>(U) + row + R * nu);
-          else
-            u[c][r] = code_to_f<FB>(__ldg(reinterpret_cast<const uint16_t*>(U) +
-                                          (panel ? (row >> 3) * ps2 + 8 * nu + (row & 7) : row + R * nu)));
-        }
-      }
-#pragma unroll
-    for (int c = 0; c < 8; c++) {
-      if (nu0 + c >= k) break;
-#pragma unroll
-      for (int v = 0; v < NVB; v++) {
-        const float yv = v < nv ? wbuf[v * kp + nu0 + c] : 0.f;
-        acc[0][v] = fmaf(u[c][0], yv, acc[0][v]);
-        acc[1][v] = fmaf(u[c][1], yv, acc[1][v]);
-      }
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < 2; r++) {
-    const int row = lane + 32 * r;
-    if (row >= R) continue;
-#pragma unroll
-    for (int v = 0; v < NVB; v++)
-      if (v < nv) {
-        y_store(D.y, D.xy32, v * D.ldy + off + row, mb.scale * acc[r][v], assign);
-      }
-  }
-  __syncwarp();  // wbuf is reused by the warp's next leaf
-}
-
-template <int F, int RPL, int NVB>
-__global__ void __launch_bounds__(kTreeWarpsM * 32) k_downsweep_tree_m(const MatDesc* __restrict__ mats,
-                                                                      const int2* __restrict__ jobs, int nvlo,
-                                                                      int nvhi, int expand) {  // 0 none, 1 add, 2 assign
-  __shared__ float path[2][NVB][64];
-  __shared__ __align__(16) float wstage[kTreeWarpsM][NVB * 64];
+// the same beside the dense stream: no clusters, and registers for several CTAs next to its CTA
+template <int F, int NVB>
+__global__ void __launch_bounds__(tree_warps<NVB>() * 32, 24 / tree_warps<NVB>())
+    k_upsweep_tree_beside(const MatDesc* __restrict__ mats, const int2* __restrict__ jobs, int nvlo, int nvhi, int T, int entries) {
   const int2 job = jobs[blockIdx.x];
   const TreeParamsM P = tree_params(mats[job.x]);
-  if (P.nv < nvlo || P.nv > nvhi) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* wbuf = wstage[warp];
-  const int64_t sub = job.y;
-  const int64_t root = ((int64_t)1 << P.L) - 1 + sub;
-  // the path from the root to the subtree root, recomputed by every CTA; every warp takes a
-  // slice of the vectors (the slices are independent)
-  constexpr int NVW = slice_vectors<NVB>();
-  const int v0 = warp * NVW, nw = min(NVW, P.nv - v0);
-  if (P.L > 0 && nw > 0) {
-    int cur = 0;
-    for (int v = v0; v < v0 + nw; v++)
-      for (int r = lane; r < P.k; r += 32) path[cur][v][r] = P.yhat[(int64_t)v * P.kp + r];
-    __syncwarp();
-    for (int l = 1; l <= P.L; l++) {
-      const int64_t a = ((root + 1) >> (P.L - l)) - 1;
-      float acc[RPL][NVW];
-#pragma unroll
-      for (int r = 0; r < RPL; r++)
-#pragma unroll
-        for (int v = 0; v < NVW; v++) acc[r][v] = 0.f;
-      warp_mv_m<F, RPL, NVW>(static_cast<const typename CodeT<F>::T*>(P.E) + (a - 1) * P.kk8, P.escale[a - 1], P.k, P.k,
-                             P.LR, &path[cur][v0][0], 64, nw, acc, lane);
-      group_reduce_m(acc, P.LR);
-      if (lane < P.LR) {
-#pragma unroll
-        for (int rr = 0; rr < RPL; rr++) {
-          const int row = lane + 32 * rr;
-          if (row >= P.k) continue;
-#pragma unroll
-          for (int v = 0; v < NVW; v++) {
-            if (v >= nw) continue;
-            const int64_t at = (a * P.nv + v0 + v) * P.kp + row;
-            const float val = acc[rr][v] + P.yhat[at];
-            if (l == P.L) P.yhat[at] = val;
-            else path[cur ^ 1][v0 + v][row] = val;
-          }
-        }
-      }
-      __syncwarp();
-      cur ^= 1;
-    }
-  }
-  __syncthreads();
-  for (int lvl = P.L + 1; lvl <= P.q; lvl++) {
-    const int64_t node0 = ((int64_t)1 << lvl) - 1 + (sub << (lvl - P.L));
-    const int nn = 1 << (lvl - P.L);
-    if (nn >= kTreeWarpsM || P.nv <= NVW) {  // a warp per node, all vectors
-      for (int t = warp; t < nn; t += kTreeWarpsM) {
-        const int64_t ch = node0 + t;
-        float acc[RPL][NVB];
-#pragma unroll
-        for (int r = 0; r < RPL; r++)
-#pragma unroll
-          for (int v = 0; v < NVB; v++) acc[r][v] = 0.f;
-        stage_vectors<false>(wbuf, P.yhat + ((ch - 1) / 2) * P.nv * P.kp, P.nv * P.kp, lane);
-        warp_mv_m<F, RPL, NVB>(static_cast<const typename CodeT<F>::T*>(P.E) + (ch - 1) * P.kk8, P.escale[ch - 1], P.k,
-                               P.k, P.LR, wbuf, P.kp, P.nv, acc, lane);
-        __syncwarp();
-        group_reduce_m(acc, P.LR);
-        store_node_m<RPL, NVB, true>(P.yhat + ch * P.nv * P.kp, P.k, P.kp, P.LR, P.nv, acc, lane);
-      }
-    } else {  // fewer nodes than warps: a warp per (node, slice of NVW vectors)
-      const int ns = (P.nv + NVW - 1) / NVW;
-      for (int u = warp; u < nn * ns; u += kTreeWarpsM) {
-        const int64_t ch = node0 + u % nn;
-        const int s0 = (u / nn) * NVW, sw = min(NVW, P.nv - s0);
-        float acc[RPL][NVW];
-#pragma unroll
-        for (int r = 0; r < RPL; r++)
-#pragma unroll
-          for (int v = 0; v < NVW; v++) acc[r][v] = 0.f;
-        stage_vectors<false>(wbuf, P.yhat + (((ch - 1) / 2) * P.nv + s0) * P.kp, sw * P.kp, lane);
-        warp_mv_m<F, RPL, NVW>(static_cast<const typename CodeT<F>::T*>(P.E) + (ch - 1) * P.kk8, P.escale[ch - 1], P.k,
-                               P.k, P.LR, wbuf, P.kp, sw, acc, lane);
-        __syncwarp();
-        group_reduce_m(acc, P.LR);
-        store_node_m<RPL, NVW, true>(P.yhat + (ch * P.nv + s0) * P.kp, P.k, P.kp, P.LR, sw, acc, lane);
-      }
-    }
-    __syncthreads();
-  }
-  // leaf expansion (Eq. 4) of the subtree's leaves: their yhat is final (written by this CTA
-  // above, or by the coupling phase when the subtree root is the root and a leaf)
-  if (expand) {
-    const MatDesc& D = mats[job.x];
-    const int T = P.q - P.L;
-    for (int64_t t = warp; t < ((int64_t)1 << T); t += kTreeWarpsM)
-      expand_leaf_m<F, NVB>(D, (sub << T) + t, lane, wbuf, expand == 2);
-  }
+  if (P.nv < nvlo || P.nv > nvhi || job.y < 0) return;
+  tree_up<TreeOpM<F>, NVB, false>(P, job.y, true, false, T, entries);
+}
+
+// the whole downsweep in one launch, ending with the leaf expansion y(j) = scale * U_j yhat_j (expand 2:
+// assigned, the dense phase runs afterwards and adds its part; 1: added with atomics, the dense phase
+// adds its part the same way at the same time, both into a y zeroed before the product; 0: none)
+template <int F, int NVB>
+__global__ void __launch_bounds__(tree_warps<NVB>() * 32)
+    k_downsweep_tree_m(const MatDesc* __restrict__ mats, const int2* __restrict__ jobs, int nvlo, int nvhi, int expand, int T,
+                       int entries) {
+  const int2 job = jobs[blockIdx.x];
+  const TreeParamsM P = tree_params(mats[job.x]);
+  if (P.nv < nvlo || P.nv > nvhi || job.y < 0) return;
+  tree_down<TreeOpM<F>, NVB>(P, job.y, expand, T, entries);
 }
 
 // ---------------------------------------------------------------- coupling, all levels
@@ -876,7 +696,7 @@ __global__ void __launch_bounds__(128) k_coupling_m_generic(const MatDesc* __res
 #pragma unroll
       for (int v = 0; v < NVB; v++) acc[rr][v] = 0.f;
     for (int32_t b = b0; b < b1; b++) {  // the column node's vectors staged in shared memory
-      stage_vectors<false>(wbuf, xhat + (int64_t)Scol[b] * nv * kp, nv * kp, lane);
+      stage_vectors(wbuf, xhat + (int64_t)Scol[b] * nv * kp, nv * kp, lane);
       warp_mv_m<F, RPL, NVB>(S + (int64_t)b * kk8, sscale[b], k, k, LR, wbuf, kp, nv, acc, lane);
       __syncwarp();
     }
@@ -1058,9 +878,12 @@ __host__ __device__ constexpr int mixed_red_bytes(int nvb, int cw) { return (nvb
 // them (U_i, not streamed) -- at most 32 (kMixedMaxBlocks + 1) records
 constexpr int kMixedBatchBlocks = 32 * (kMixedMaxBlocks + 1);
 constexpr int kMixedBlkBuf = kMixedBatchBlocks * 16;
+// passes of up to four vectors leave kTreeReserve bytes of an SM's shared memory to the tree kernels
+// that run beside the dense stream: four or five stages of 32 KB still keep more than 128 KB in flight
+constexpr int kTreeReserve = 40960;
 __host__ __device__ constexpr int mixed_stages(int nvb, int cw) {
-  return (kSmemLimit - 256 - kMixedBlkBuf - mixed_red_bytes(nvb, cw)) / mixed_stage_bytes(nvb) < 6
-             ? (kSmemLimit - 256 - kMixedBlkBuf - mixed_red_bytes(nvb, cw)) / mixed_stage_bytes(nvb)
+  return (kSmemLimit - (nvb <= 4 ? kTreeReserve : 0) - 256 - kMixedBlkBuf - mixed_red_bytes(nvb, cw)) / mixed_stage_bytes(nvb) < 6
+             ? (kSmemLimit - (nvb <= 4 ? kTreeReserve : 0) - 256 - kMixedBlkBuf - mixed_red_bytes(nvb, cw)) / mixed_stage_bytes(nvb)
              : 6;
 }
 __host__ __device__ constexpr int mixed_smem_bytes(int nvb, int cw) {
