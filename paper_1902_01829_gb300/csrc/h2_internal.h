@@ -56,6 +56,7 @@ struct MixedLaunch {
   int64_t nchunks = 0;
   const h2::StreamItem* items = nullptr;
   const int* cta_begin = nullptr;    // [grid + 1]
+  const int* mma_begin = nullptr;    // the same for passes of more than four vectors (k_dense_mma)
   const void* blk = nullptr;         // h2::MixedBlock records
   int grid = 0;
   int* err = nullptr;
@@ -126,6 +127,7 @@ struct MixedData {
   float* escale = nullptr;
   int64_t* xp4_off = nullptr; // leaf offsets of the FP32 x copy, padded to multiples of 4
   float* x4 = nullptr;        // FP32 copy of the pass's x (padded leaf layout)
+  unsigned char* xp = nullptr;  // the same as 16-bit parts (mixed.cuh), for passes of more than four vectors
   float* xhat = nullptr;      // [node][v][kp4]
   float* yhat = nullptr;
   int kp4 = 0;                // k rounded up to a multiple of 4
@@ -149,7 +151,8 @@ struct MixedData {
   // the table-driven kernels' tables for this matrix alone (a batch of one)
   MixedLaunch launch;
   std::vector<h2::StreamItem> items_host;  // the dense items (matrix index 0), kept for batches
-  std::vector<int64_t> row_bytes;          // bytes each leaf row streams (load balance)
+  int* mma_begin = nullptr;                // the items' split over the CTAs in k_dense_mma
+  std::vector<int64_t> row_bytes, row_mma;  // each leaf row's weight: bytes streamed; cycles in k_dense_mma
   std::vector<int64_t> row_item0;          // first item of each leaf row, [leaves + 1]
   std::vector<int32_t> srow_host;          // S_rowptr (to cut chunks for another target)
   int4* chunk_dev[3] = {nullptr, nullptr, nullptr};  // device chunk lists per target option

@@ -102,7 +102,7 @@ struct CallChunk {
   long long ldx[kCallChunk];
   long long ldy[kCallChunk];
   int nv[kCallChunk];
-  int xy32;
+  int xy32, xp_on;
 };
 static_assert(sizeof(CallChunk) < 32000, "kernel parameter space");
 
@@ -116,6 +116,7 @@ __global__ void k_set_calls(h2::MatDesc* mats, CallChunk c) {
     D.ldy = c.ldy[i];
     D.nv = c.nv[i];
     D.xy32 = c.xy32;
+    D.xp_on = c.xp_on;
   }
 }
 
@@ -153,6 +154,9 @@ h2::MatDesc fill_desc(const h2_matrix_s* h, int tree_L) {
   D.kf_off = M.kf_off;
   D.spanel = M.spanel ? 1 : 0;
   D.cpart = M.cpart;
+  D.xp = M.xp;
+  D.xks = (h->m_max + 15) / 16;
+  D.code_form = form_of(h->storage);
   D.cticket = M.cticket;
   D.rjobs = static_cast<const h2::RowJob*>(M.rjobs);
   D.blk = static_cast<const h2::MixedBlock*>(M.dblk);
@@ -161,11 +165,12 @@ h2::MatDesc fill_desc(const h2_matrix_s* h, int tree_L) {
 
 // write the fields of one product pass into a matrix table (entries [0, count))
 h2_status set_calls(h2::MatDesc* mats, int64_t count, const int* nv, const double* const* x, const int64_t* ldx,
-                    double* const* y, const int64_t* ldy, cudaStream_t st, int xy32 = 0) {
+                    double* const* y, const int64_t* ldy, cudaStream_t st, int xp_on, int xy32 = 0) {
   for (int64_t c0 = 0; c0 < count; c0 += kCallChunk) {
     CallChunk c{};
     c.first = (int)c0;
     c.xy32 = xy32;
+    c.xp_on = xp_on;
     c.count = (int)std::min<int64_t>(kCallChunk, count - c0);
     for (int i = 0; i < c.count; i++) {
       c.x[i] = x[c0 + i];
@@ -675,7 +680,8 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
           } else {
             m.scale = quantize(d->D_val + doff[b], si * sj, form, reinterpret_cast<uint16_t*>(base + boff[g]));
           }
-          m.voff = xp4[j];
+          m.voff = (uint64_t)xp4[j];
+          m.leaf = (uint64_t)j;
           m.cols = (unsigned short)sj;
           m.vs = (unsigned char)round_up(sj, 4);
           m.src = panel ? 4 : 0;
@@ -696,7 +702,8 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
           m.scale = quantize(d->U + lo[i] * k, si * k, form, reinterpret_cast<uint16_t*>(ub));
           m.src = 1;
         }
-        m.voff = (h->leaf0 + i) * M.kp4;
+        m.voff = (uint64_t)((h->leaf0 + i) * M.kp4);
+        m.leaf = 0;
         m.cols = (unsigned short)k;
         m.vs = (unsigned char)M.kp4;
       }
@@ -784,6 +791,8 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
     // phase does not wait for the tree phases.
     std::vector<h2::StreamItem> items;
     std::vector<int64_t> row_bytes((size_t)leaves), row_item0((size_t)leaves + 1);
+    // a row's cost in k_dense_mma (SM cycles): its blocks' K steps (per half of a 64-row block) and its end
+    std::vector<int64_t> row_mma((size_t)leaves, 1000);
     std::vector<h2::RowJob> rj((size_t)leaves);
     for (int64_t i = 0; i < leaves; i++) {
       row_item0[i] = (int64_t)items.size();
@@ -791,11 +800,13 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
       rj[i] = h2::RowJob{boff[g1], 0, (int)i, (int)g1, g1 > g0 ? 1 : 0, {0, 0}};
       int64_t bytes = 0;
       for (int64_t g = g0; g < g1;) {
-        int64_t e = g, mb = 0, vc = 0;
+        int64_t e = g, mb = 0, vc = 0, xb = 0;
+        auto parts = [&](int64_t b) { return h2::xp_chunk_bytes((blk[b].cols + 15) / 16, 2); };
         while (e < g1 && e - g < h2::kMixedMaxBlocks && mb + (boff[e + 1] - boff[e]) <= h2::kStageMat &&
-               vc + blk[e].vs <= h2::kMixedVecCols) {
+               vc + blk[e].vs <= h2::kMixedVecCols && mb + (boff[e + 1] - boff[e]) + xb + parts(e) <= h2::kMmaArea) {
           mb += boff[e + 1] - boff[e];
           vc += blk[e].vs;
+          xb += parts(e);
           e++;
         }
         h2::StreamItem it{};
@@ -810,10 +821,14 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
         g = e;
       }
       row_bytes[i] = bytes;
+      for (int64_t g = g0; g < g1; g++) row_mma[i] += (lo[i + 1] - lo[i] > 32 ? 2 : 1) * (70 * ((blk[g].cols + 15) / 16) + 50);
     }
     row_item0[leaves] = (int64_t)items.size();
-    const std::vector<int> begin = balance(row_bytes, row_item0, h->grid);
+    const std::vector<int> begin = balance(row_bytes, row_item0, h->grid), mbegin = balance(row_mma, row_item0, h->grid);
     if ((st = audit_producer_batches(items, begin)) != H2_OK) return st;
+    if ((st = audit_producer_batches(items, mbegin)) != H2_OK) return st;
+    for (size_t c = 0; c + 1 < mbegin.size(); c++)
+      if (mbegin[c] > mbegin[c + 1]) return h2_fail(H2_ERR_INVALID, "internal: item ranges not monotone");
     // audit: every copy in bounds, 16-byte aligned, and within its stage slot
     for (size_t c = 0; c + 1 < begin.size(); c++)
       if (begin[c] > begin[c + 1]) return h2_fail(H2_ERR_INVALID, "internal: item ranges not monotone");
@@ -822,14 +837,16 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
       const int nb = (int)((it.shape >> 8) & 0xFF);
       bool ok = it.m_off % 16 == 0 && it.m_bytes % 16 == 0 && it.m_bytes > 0 && it.m_bytes <= h2::kStageMat &&
                 it.m_off + it.m_bytes <= total && nb >= 1 && nb <= h2::kMixedMaxBlocks && it.v_off + nb <= nblk;
-      int64_t vc = 0;
+      int64_t vc = 0, xb = 0;
       for (int u = 0; ok && u < nb; u++) {
         const h2::MixedBlock& m = blk[it.v_off + u];
         const int64_t lim = (m.src & 1) ? nodes * M.kp4 : xp4[leaves];
-        ok = m.vs % 4 == 0 && m.vs >= m.cols && m.vs <= 64 && m.voff % 4 == 0 && m.voff + m.vs <= lim;
+        ok = m.vs % 4 == 0 && m.vs >= m.cols && m.vs <= 64 && m.voff % 4 == 0 && (int64_t)m.voff + m.vs <= lim &&
+             ((m.src & 1) || (int64_t)m.leaf < leaves);
         vc += m.vs;
+        xb += h2::xp_chunk_bytes((m.cols + 15) / 16, 2);
       }
-      ok = ok && vc <= h2::kMixedVecCols;
+      ok = ok && vc <= h2::kMixedVecCols && it.m_bytes + xb <= h2::kMmaArea;
       if (!ok) return h2_fail(H2_ERR_INVALID, "internal: precision-form work item %lld fails the layout audit", (long long)t);
     }
     if (M.panel) {
@@ -898,7 +915,7 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
         r[0] = nb | ((it.flags >> h2::kTcPairShift) << 8);
         for (int u = 0; u < nb; u++) {
           const h2::MixedBlock& m = blk[it.v_off + u];
-          if (m.voff < 0 || m.voff > INT32_MAX)
+          if ((int64_t)m.voff > INT32_MAX)
             return h2_fail(H2_ERR_UNSUPPORTED, "vector offset %lld exceeds the tensor-core records", (long long)m.voff);
           r[1 + 3 * u] = (int32_t)m.voff;
           r[2 + 3 * u] = h2::panel_cols(m.cols) | ((m.src & 1) << 16);
@@ -914,6 +931,8 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
     if ((st = upload(h, &M.dense_items.items, items.data(), (int64_t)items.size())) != H2_OK) return st;
     if ((st = upload(h, &M.dense_items.cta_begin, begin.data(), (int64_t)begin.size())) != H2_OK) return st;
     M.dense_items.count = (int64_t)items.size();
+    if ((st = upload(h, &M.mma_begin, mbegin.data(), (int64_t)mbegin.size())) != H2_OK) return st;
+    M.row_mma = std::move(row_mma);
     M.nblk = nblk;
     M.items_host = std::move(items);
     h2::RowJob* drj = nullptr;
@@ -925,6 +944,7 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
     M.row_item0 = std::move(row_item0);
   }
   if ((st = dalloc(h, &M.x4, xp4[leaves] * kPassVectors)) != H2_OK) return st;
+  if ((st = dalloc(h, &M.xp, leaves * h2::xp_chunk_bytes((h->m_max + 15) / 16, 2))) != H2_OK) return st;
   if ((st = dalloc(h, &M.xhat, nodes * kPassVectors * M.kp4)) != H2_OK) return st;
   if ((st = dalloc(h, &M.yhat, nodes * kPassVectors * M.kp4)) != H2_OK) return st;
   // entries k .. kp4 - 1 of every node vector are padding that no kernel writes except with
@@ -949,6 +969,7 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
   CUDA_TRY(cudaMemset(M.cpart, 0, (size_t)std::max<int64_t>(M.cslots * kPassVectors * M.kp4, 1) * sizeof(float)));
   L.items = M.dense_items.items;
   L.cta_begin = M.dense_items.cta_begin;
+  L.mma_begin = M.mma_begin;
   L.blk = M.dblk;
   L.grid = h->grid;
   L.err = h->err;
@@ -987,11 +1008,13 @@ h2_status mixed_pass(h2_matrix_s* h, int nv, const void* xv, int64_t ldx, void* 
   L.prof = &h->prof;
   cudaError_t me = mark(&h->prof, st);
   if (me != cudaSuccess) return h2_fail(H2_ERR_CUDA, "profiling event: %s", cudaGetErrorString(me));
-  h2_status s = set_calls(static_cast<h2::MatDesc*>(L.mats), 1, &nv, &x, &ldx, &y, &ldy, st, xy32);
-  if (s != H2_OK) return s;
   const MixedData& M = h->mx;
   const bool fp16 = h->storage == H2_FP16_SCALED;
   const bool tc_ok = nv >= kTcMinVectors && h->storage != H2_INT16_SCALED;
+  // passes of more than four vectors whose dense phase is not k_dense_tc's run k_dense_mma
+  const int xp_on = bucket_of(nv) > 2 && !(M.panel && tc_ok);
+  h2_status s = set_calls(static_cast<h2::MatDesc*>(L.mats), 1, &nv, &x, &ldx, &y, &ldy, st, xp_on, xy32);
+  if (s != H2_OK) return s;
   TcCall T, TS;
   TcPass P;
   // set_calls, upsweep, coupling, downsweep (+ expansion), dense; the split of x when the dense phase
@@ -1159,7 +1182,7 @@ h2_status batch_build(h2_batch_s* b) {
   MixedLaunch& L = b->launch;
   h2_status st;
   std::vector<h2::StreamItem> items;
-  std::vector<int64_t> row_bytes, row_item0;
+  std::vector<int64_t> row_bytes, row_item0, row_mma;
   std::vector<h2::RowJob> rjobs;
   int64_t blk0 = 0;
   for (int64_t i = 0; i < count; i++) {
@@ -1182,6 +1205,7 @@ h2_status batch_build(h2_batch_s* b) {
     for (size_t r = 0; r + 1 < M.row_item0.size(); r++) {
       row_item0.push_back(item0 + M.row_item0[r]);
       row_bytes.push_back(M.row_bytes[r]);
+      row_mma.push_back(M.row_mma[r]);
       b->row_mat.push_back((int32_t)i);
     }
     blk0 += M.nblk;
@@ -1189,10 +1213,12 @@ h2_status batch_build(h2_batch_s* b) {
   row_item0.push_back((int64_t)items.size());
   if ((int64_t)items.size() >= INT32_MAX)
     return h2_fail(H2_ERR_UNSUPPORTED, "batch too large: %lld dense items", (long long)items.size());
-  const std::vector<int> begin = balance(row_bytes, row_item0, h0->grid);
+  const std::vector<int> begin = balance(row_bytes, row_item0, h0->grid), mbegin = balance(row_mma, row_item0, h0->grid);
   if ((st = audit_producer_batches(items, begin)) != H2_OK) return st;
+  if ((st = audit_producer_batches(items, mbegin)) != H2_OK) return st;
   for (size_t c = 0; c + 1 < begin.size(); c++)
-    if (begin[c] > begin[c + 1]) return h2_fail(H2_ERR_INVALID, "internal: item ranges not monotone");
+    if (begin[c] > begin[c + 1] || mbegin[c] > mbegin[c + 1])
+      return h2_fail(H2_ERR_INVALID, "internal: item ranges not monotone");
   for (const h2::StreamItem& it : items)  // the member audits hold; only the block index moved
     if (it.v_off < 0 || it.v_off + ((it.shape >> 8) & 0xFF) > blk0)
       return h2_fail(H2_ERR_INVALID, "internal: batched work item outside the block records");
@@ -1202,6 +1228,9 @@ h2_status batch_build(h2_batch_s* b) {
   int* db = nullptr;
   if ((st = balloc(b, &db, (int64_t)begin.size(), begin.data())) != H2_OK) return st;
   b->cta_begin_dev = db;
+  int* dmb = nullptr;
+  if ((st = balloc(b, &dmb, (int64_t)mbegin.size(), mbegin.data())) != H2_OK) return st;
+  L.mma_begin = dmb;
   b->row_bytes = row_bytes;
   b->row_item0 = row_item0;
   b->items_host = items;
@@ -1355,7 +1384,7 @@ h2_status h2_batch_matvec(h2_batch b, const int32_t* nv, const double* const* x,
     cudaError_t me = mark(&b->prof, st);
     if (me != cudaSuccess) return h2_fail(H2_ERR_CUDA, "profiling event: %s", cudaGetErrorString(me));
     h2_status s = set_calls(static_cast<h2::MatDesc*>(L.mats), count, pnv.data(), px.data(), pldx.data(), py.data(),
-                            pldy.data(), st);
+                            pldy.data(), st, 31 - __builtin_clz(buckets | 1u) > 2);
     if (s != H2_OK) return s;
     b->prof.launches += (count + kCallChunk - 1) / kCallChunk + 3 * bucket_count(buckets) + 1 +
                         (31 - __builtin_clz(buckets | 1u) <= 2 && !b->prof.on ? 1 : 0);

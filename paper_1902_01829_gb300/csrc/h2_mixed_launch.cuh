@@ -6,6 +6,7 @@
 #include <algorithm>
 #include "h2_internal.h"
 #include "mixed.cuh"
+#include "mma_dense.cuh"
 #include "tc_dense.cuh"
 
 namespace h2i {
@@ -123,12 +124,29 @@ h2_status dense_launch_cw(const MixedLaunch& L, cudaStream_t st) {
 
 // consumer warps of the dense stream: rows of at most 32 points give each warp little
 // arithmetic per item, and twice the warps hide more latency (measured: 163 -> 134 us on a
-// 2^17-point matrix with 32-point leaves); 64-point rows run faster with 8. With 16 vectors
-// per pass the 16-warp variant fits 96 registers a thread (a few spilled).
+// 2^17-point matrix with 32-point leaves); 64-point rows run faster with 8. (Passes of more than
+// four vectors take k_dense_mma, which has no such choice.)
 template <int F, int NVB>
 h2_status dense_launch(const MixedLaunch& L, cudaStream_t st) {
   if (L.cw == 2 * h2::kMixedCW) return dense_launch_cw<F, NVB, 2 * h2::kMixedCW>(L, st);
   return dense_launch_cw<F, NVB, h2::kMixedCW>(L, st);
+}
+
+// the dense phase of a pass of more than four vectors
+template <int F>
+h2_status mma_launch(const MixedLaunch& L, cudaStream_t st) {
+  using namespace h2;
+  static const cudaError_t attr = cudaFuncSetAttribute(k_dense_mma<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMmaSmem);
+  if (attr != cudaSuccess) return h2_fail(H2_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(attr));
+  MixedStreamParams P{};
+  P.items = L.items;
+  P.cta_begin = L.mma_begin;
+  P.blk = static_cast<const MixedBlock*>(L.blk);
+  P.mats = static_cast<const MatDesc*>(L.mats);
+  P.err = L.err;
+  P.budget = L.budget;
+  k_dense_mma<F><<<L.grid, (kMmaWarps + 1) * 32, kMmaSmem, st>>>(P);
+  return H2_OK;
 }
 
 // a phase on the tensor cores (the dense phase, or the coupling phase): per-vector scales, then the
@@ -211,8 +229,7 @@ h2_status mixed_pass_t(const MixedLaunch& L, unsigned buckets, cudaStream_t st, 
            : top == 0 ? dense_launch<F, 1>(L, ds)
            : top == 1 ? dense_launch<F, 2>(L, ds)
            : top == 2 ? dense_launch<F, 4>(L, ds)
-           : top == 3 ? dense_launch<F, 8>(L, ds)
-                      : dense_launch<F, 16>(L, ds);
+                      : mma_launch<F>(L, ds);
   };
   // passes of more than four vectors keep the phases in order: their tree kernels' shared memory does
   // not fit beside the dense stream's, and the dense phase is bound by arithmetic there (measured)

@@ -171,6 +171,7 @@ struct TreeOp64 {
   static __device__ __forceinline__ void xstore(const P& T, const Leaf& l, int sp, int v, int a, float2 x) {
     T.x2[l.xp * T.nv + v * sp + a] = x;
   }
+  static constexpr bool kParts = false;
   static __device__ __forceinline__ int copy_bytes(int entries) { return 8 * entries; }
   // (the leaf expansion is the dense stream's)
   static __device__ __forceinline__ const double* U(const P&, const Leaf&) { return nullptr; }

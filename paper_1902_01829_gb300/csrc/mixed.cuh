@@ -12,6 +12,7 @@
 // strides rounded up to multiples of 4 (16-byte chunks for the bulk copies).
 #pragma once
 #include <type_traits>
+#include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
 #include "stream_fp64.cuh"
@@ -68,7 +69,8 @@ struct __align__(16) RowJob {
   int pad[2];
 };
 struct __align__(16) MixedBlock {
-  long long voff;       // vector chunk offset, in floats per vector slot
+  unsigned long long voff : 40;  // vector chunk offset, in floats per vector slot
+  unsigned long long leaf : 24;  // column leaf (dense blocks)
   float scale;
   unsigned short cols;  // C
   unsigned char vs;     // vector stride (>= C, multiple of 4)
@@ -86,6 +88,14 @@ constexpr int kPanelPad = 16;
 __host__ __device__ constexpr int panel_cols(int C) { return (C + 15) & ~15; }
 __host__ __device__ constexpr int panel_stride(int C) { return 16 * panel_cols(C) + kPanelPad; }  // bytes
 __host__ __device__ constexpr int panel_block_bytes(int C) { return 8 * panel_stride(C); }
+
+// The vectors of a leaf as 16-bit parts in the A-fragment order of mma.sync m16n8k16 (k_dense_mma): 16 scale
+// floats (per vector), then per K step of 16 points and half of eight vectors three parts of 256 bytes, lane
+// (g, t)'s entries (vector g + 8 half; points t, t + 4, t + 8, t + 12 as k = 2t, 2t + 1, 2t + 8, 2t + 9) at
+// 8 (4 g + t). Every leaf's chunk
+// has the same number of K steps (the matrix's xks).
+constexpr int kXpScale = 64, kXpStep = 768;
+__host__ __device__ constexpr int xp_chunk_bytes(int ksteps, int halves) { return kXpScale + ksteps * halves * kXpStep; }
 
 // ---------------------------------------------------------------- per-matrix descriptor
 // One entry per matrix of a batch (a single product is a batch of one); the
@@ -121,6 +131,10 @@ struct MatDesc {
   // split coupling rows: partial sums [slot][v][kp] and a counter per (row's first slot, vector slice)
   float* cpart;
   int* cticket;
+  // the pass's vectors as 16-bit parts, xks K steps per leaf
+  unsigned char* xp;
+  int xks;
+  int code_form;  // kFormFp16, kFormBf16 or kFormInt16 (the dense codes')
   // the leaf expansion done by the downsweep: the matrix's row jobs and the block records they index
   const RowJob* rjobs;
   const MixedBlock* blk;
@@ -130,6 +144,7 @@ struct MatDesc {
   double* y;
   long long ldy;
   int nv, xy32;   // xy32: x and y are FP32 (else FP64)
+  int xp_on;      // the dense phase reads the vectors as 16-bit parts (k_dense_mma): the upsweep writes them
 };
 
 // x and y are FP64 or, for products that ask for it, FP32 (MatDesc::xy32)
@@ -324,6 +339,53 @@ struct TreeOpM {
   static __device__ __forceinline__ void xstore(const P& T, const Leaf& l, int sp, int v, int a, float x) {
     T.x4[l.xp * T.nv + v * sp + a] = x;
   }
+  static constexpr bool kParts = true;
+  // leaf j's vectors xs ([point][vector], stride VS) as 16-bit parts; vmax: float bits of max |x| per vector
+  template <int VS, int TH>
+  static __device__ __forceinline__ void parts(const P& T, int64_t j, int s, const float* xs, const unsigned* vmax) {
+    const int nh = T.nv > 8 ? 2 : 1;
+    unsigned char* chunk = T.D->xp + j * xp_chunk_bytes(T.D->xks, nh);
+    const bool bf = T.D->code_form == kFormBf16;
+    // x = 2^(e - 14) (hi + mid + lo); e from the exponent bits, at least -110 so that 2^(14 - e) is finite
+    auto shift = [&](int v) { return bf ? 0 : 14 - max((int)(vmax[v] >> 23) - 126, -110); };
+    for (int i = threadIdx.x; i < ((s + 15) >> 4) * 32 * nh; i += TH) {
+      const int ln = i & 31, u = i >> 5, ks = nh == 2 ? u >> 1 : u, half = nh == 2 ? u & 1 : 0;
+      const int v = (ln >> 2) + 8 * half, c0 = 16 * ks + (ln & 3);
+      const float up = __int_as_float((127 + (v < T.nv ? shift(v) : 0)) << 23);
+      float x[4];
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        const int c = c0 + 4 * q;
+        x[q] = (v < T.nv && c < s) ? xs[c * VS + v] * up : 0.f;
+      }
+      uint2* dst = reinterpret_cast<uint2*>(chunk + kXpScale + u * 768 + ln * 8);
+#pragma unroll
+      for (int p = 0; p < 3; p++) {
+        uint32_t w[2];
+#pragma unroll
+        for (int q = 0; q < 2; q++) {
+          if (bf) {
+            const __nv_bfloat162 b = __floats2bfloat162_rn(x[2 * q], x[2 * q + 1]);
+            x[2 * q] -= __low2float(b);
+            x[2 * q + 1] -= __high2float(b);
+            w[q] = *reinterpret_cast<const uint32_t*>(&b);
+          } else {
+            const __half2 b = __floats2half2_rn(x[2 * q], x[2 * q + 1]);
+            x[2 * q] -= __low2float(b);
+            x[2 * q + 1] -= __high2float(b);
+            w[q] = *reinterpret_cast<const uint32_t*>(&b);
+          }
+        }
+        dst[32 * p] = make_uint2(w[0], w[1]);
+      }
+    }
+    if (threadIdx.x < 16) {
+      const int v = threadIdx.x;
+      reinterpret_cast<float*>(chunk)[v] = v < T.nv ? __int_as_float((127 - shift(v)) << 23) : 0.f;
+    }
+  }
+  static __device__ __forceinline__ bool want_parts(const P& T) { return T.D->xp_on != 0; }
+  static __device__ __forceinline__ unsigned abs_bits(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
   static __device__ __forceinline__ int copy_bytes(int entries) { return (entries * (int)sizeof(A) + 15) & ~15; }
   static __device__ __forceinline__ const char* U(const P& T, const Leaf& l) { return T.D->dmat + l.uoff; }
   static __device__ __forceinline__ int u_bytes(const P& T, const Leaf& l) {
@@ -871,25 +933,30 @@ constexpr int kMixedVecCols = 256;   // vector columns of one work item (sum of 
 constexpr int kMixedHeader = 256;
 __host__ __device__ constexpr int mixed_vec_area(int nvb) { return kMixedVecCols * nvb * 4; }
 __host__ __device__ constexpr int mixed_stage_bytes(int nvb) { return kMixedHeader + kStageMat + mixed_vec_area(nvb); }
-// row partials [warp][vector][64 rows]; passes of at most four vectors double-buffer them by row
-// parity (rows end without a CTA-wide barrier, see k_dense_stream_m)
-__host__ __device__ constexpr int mixed_red_bytes(int nvb, int cw) { return (nvb <= 4 ? 2 : 1) * cw * nvb * 64 * 4; }
+// row partials [warp][vector][64 rows], double-buffered by row parity (rows end without a CTA-wide
+// barrier, see k_dense_stream_m)
+__host__ __device__ constexpr int mixed_red_bytes(int nvb, int cw) { return 2 * cw * nvb * 64 * 4; }
 // block records of one producer batch of 32 items: their blocks, plus one record per row between
 // them (U_i, not streamed) -- at most 32 (kMixedMaxBlocks + 1) records
 constexpr int kMixedBatchBlocks = 32 * (kMixedMaxBlocks + 1);
 constexpr int kMixedBlkBuf = kMixedBatchBlocks * 16;
-// passes of up to four vectors leave kTreeReserve bytes of an SM's shared memory to the tree kernels
+// the dense stream leaves kTreeReserve bytes of an SM's shared memory to the tree kernels
 // that run beside the dense stream: four or five stages of 32 KB still keep more than 128 KB in flight
 constexpr int kTreeReserve = 40960;
 __host__ __device__ constexpr int mixed_stages(int nvb, int cw) {
-  return (kSmemLimit - (nvb <= 4 ? kTreeReserve : 0) - 256 - kMixedBlkBuf - mixed_red_bytes(nvb, cw)) / mixed_stage_bytes(nvb) < 6
-             ? (kSmemLimit - (nvb <= 4 ? kTreeReserve : 0) - 256 - kMixedBlkBuf - mixed_red_bytes(nvb, cw)) / mixed_stage_bytes(nvb)
+  return (kSmemLimit - kTreeReserve - 256 - kMixedBlkBuf - mixed_red_bytes(nvb, cw)) / mixed_stage_bytes(nvb) < 6
+             ? (kSmemLimit - kTreeReserve - 256 - kMixedBlkBuf - mixed_red_bytes(nvb, cw)) / mixed_stage_bytes(nvb)
              : 6;
 }
 __host__ __device__ constexpr int mixed_smem_bytes(int nvb, int cw) {
   return mixed_stages(nvb, cw) * mixed_stage_bytes(nvb) + 256 + mixed_red_bytes(nvb, cw) + kMixedBlkBuf;
 }
 constexpr int kMixedCW = 8;
+// codes and vector parts of a work item in passes of more than four vectors (k_dense_mma's stage: four
+// 64 x 64 blocks, eight of 32 x 32 and their parts fit; items of odd shapes are cut to it)
+constexpr int kMmaArea = kStageMat + 4 * xp_chunk_bytes(4, 2) + 256;
+static_assert(8 * 32 * 32 * 2 + 8 * xp_chunk_bytes(2, 2) <= kMmaArea && 4 * panel_block_bytes(64) + 4 * xp_chunk_bytes(4, 2) > kMmaArea,
+              "a stage holds eight 32 x 32 blocks; panel blocks go three to an item");
 
 // items: m_off (in the matrix's dmat), m_bytes, shape = R | nb << 8, v_off = first block (batch-wide
 // index into blk), row = y offset, flags = last-of-row | matrix index << 8
@@ -1055,21 +1122,17 @@ __device__ __forceinline__ void mixed_produce(const MixedStreamParams& P, const 
     }
 }
 
-// One work item of the dense stream for up to NV2 vectors (NV2 <= NVB): every
-// block's products are added, scaled by the block's scale, into acc (lane:
-// rows r0, r0 + 1 of the item's row, summed over the warps at the row end).
-// Rows of more than 32: warp w takes columns C w / CW .. C (w + 1) / CW of each
-// block (full 64 x 64 blocks of codes on a branch-free path). Rows of at most
-// 32: lanes l and l + 16 own rows 2 (l & 15), +1, and the 16 half-warps take
-// the item's 4-column units (block, columns 4u .. 4u + 3) in turn, reading the
+// One work item of the dense stream, rows of at most 32 points, for up to NV2 vectors (NV2 <= NVB):
+// every block's products are added, scaled by the block's scale, into acc (lane: rows r0, r0 + 1 of
+// the item's row, summed over the warps at the row end). Lanes l and l + 16 own rows 2 (l & 15), +1,
+// and the half-warps take the item's 4-column units (block, columns 4u .. 4u + 3) in turn, reading the
 // four vector entries of a unit as one 16-byte load.
 template <int F, int NV2, int NVB, int CW>
 __device__ __forceinline__ void consume_item(const unsigned char* stage, const int* hd, int nb, int R, int warp, int lane,
                                              float (&acc)[2][NVB]) {
   constexpr int VAREA = mixed_vec_area(NVB);
-  constexpr int SETS = NV2 == 1 ? 4 : (NV2 == 2 ? 2 : 1);
   constexpr bool kScaleCodes = NV2 >= 4;  // scale the codes once instead of per-vector partial sums
-  if (R <= 32) {
+  {
     constexpr int HW = 2 * CW;  // half-warps
     const int r0 = 2 * (lane & 15), hw = warp * 2 + (lane >> 4);
     const bool even = (R & 1) == 0;
@@ -1136,85 +1199,6 @@ __device__ __forceinline__ void consume_item(const unsigned char* stage, const i
           }
       }
     }
-    return;
-  }
-  const int r0 = 2 * lane;
-  for (int t = 0; t < nb; t++) {
-    const int cw = hd[8 + 4 * t];
-    const bool f32 = (cw >> 16) & 1, panel = (cw >> 17) & 1;
-    const int C = min(cw & 0xFFFF, 64), vs = min(hd[9 + 4 * t], 64);
-    // codes of rows r0, r0 + 1 in column c: lbase + cstr * c (16-bit units)
-    const int lbase = panel ? (r0 >> 3) * (panel_stride(C) / 2) + (r0 & 7) : r0;
-    const int cstr = panel ? 8 : R;
-    const int moff = min(hd[10 + 4 * t], kStageMat - 16) & ~15;
-    const float scale = __int_as_float(hd[11 + 4 * t]);
-    const int voff = min(hd[kHdVoff + t], VAREA - 16) & ~15;
-    const uint16_t* A = reinterpret_cast<const uint16_t*>(stage + kMixedHeader + moff);
-    const float* A32 = reinterpret_cast<const float*>(stage + kMixedHeader + moff);
-    const float* X = reinterpret_cast<const float*>(stage + kMixedHeader + kStageMat + voff);
-    const int c0 = (C * warp) / CW, c1 = (C * (warp + 1)) / CW;
-    float p[SETS][2][NV2];
-#pragma unroll
-    for (int u = 0; u < SETS; u++)
-#pragma unroll
-      for (int r = 0; r < 2; r++)
-#pragma unroll
-        for (int v = 0; v < NV2; v++) p[u][r][v] = 0.f;
-    if (!f32 && R == 64 && C == 64 && vs == 64) {
-      // full 64 x 64 block of codes: fixed strides, every column loaded up front
-      constexpr int CPW = 64 / CW;
-      const uint32_t* Aw = reinterpret_cast<const uint32_t*>(A + lbase + cstr * c0);
-      uint32_t w[CPW];
-#pragma unroll
-      for (int u = 0; u < CPW; u++) w[u] = Aw[(cstr >> 1) * u];
-#pragma unroll
-      for (int v = 0; v < NV2; v++) {
-        float xv[CPW];
-#pragma unroll
-        for (int u = 0; u < CPW; u += 4) {
-          const float4 t4 = *reinterpret_cast<const float4*>(X + v * 64 + c0 + u);
-          xv[u] = t4.x;
-          xv[u + 1] = t4.y;
-          xv[u + 2] = t4.z;
-          xv[u + 3] = t4.w;
-        }
-#pragma unroll
-        for (int u = 0; u < CPW; u++) {
-          const float2 a = codes_to_f2<F>(w[u]);
-          p[u % SETS][0][v] = fmaf(a.x, xv[u], p[u % SETS][0][v]);
-          p[u % SETS][1][v] = fmaf(a.y, xv[u], p[u % SETS][1][v]);
-        }
-      }
-    } else if (r0 < R) {
-      const bool pair = panel || (R & 1) == 0;  // rows r0, r0 + 1 adjacent: one 4-byte load
-      for (int col = c0; col < c1; col++) {
-        float2 a;
-        if (f32) {
-          a.x = A32[r0 + R * col];
-          a.y = (r0 + 1 < R) ? A32[r0 + 1 + R * col] : 0.f;
-        } else if (pair) {
-          a = codes_to_f2<F>(*reinterpret_cast<const uint32_t*>(A + lbase + cstr * col));
-        } else {
-          a.x = code_to_f<F>(A[r0 + R * col]);
-          a.y = (r0 + 1 < R) ? code_to_f<F>(A[r0 + 1 + R * col]) : 0.f;
-        }
-#pragma unroll
-        for (int v = 0; v < NV2; v++) {
-          const float xv = X[v * vs + col];
-          p[0][0][v] = fmaf(a.x, xv, p[0][0][v]);
-          p[0][1][v] = fmaf(a.y, xv, p[0][1][v]);
-        }
-      }
-    }
-#pragma unroll
-    for (int v = 0; v < NV2; v++)
-#pragma unroll
-      for (int r = 0; r < 2; r++) {
-        float sum = p[0][r][v];
-#pragma unroll
-        for (int u = 1; u < SETS; u++) sum += p[u][r][v];
-        acc[r][v] = fmaf(scale, sum, acc[r][v]);
-      }
   }
 }
 
@@ -1343,22 +1327,21 @@ __global__ void __launch_bounds__((CW + 1) * 32, 1) k_dense_stream_m(MixedStream
   static_assert(NST >= 2, "at least two stages");
   extern __shared__ __align__(1024) unsigned char smem[];
   const StreamShared S = stream_shared<NST, SB>(smem);
-  // kAsyncRows (passes of at most four vectors): rows end without a CTA-wide barrier. Every warp
+  // Rows end without a CTA-wide barrier. Every warp
   // writes its partial sums into the row's half of the double-buffered red area and counts
   // itself in (cnt[row parity]); the warp that completes the count sums the partials, writes y,
   // resets the count and arrives on rowfree2[parity] (count 1), which a warp waits for before
-  // it writes that half again. Wider passes share the row's sum among all warps between the
-  // rowfull and rowfree barriers (count CW each).
-  constexpr bool kAsyncRows = NVB <= 4;
-  uint64_t* rowfree2 = S.rowfull;  // kAsyncRows: rowfree2[0], rowfree2[1] (the stream's two row barriers)
+  // it writes that half again.
+  static_assert(NVB <= 4, "wider passes take k_dense_mma");
+  uint64_t* rowfree2 = S.rowfull;  // rowfree2[0], rowfree2[1] (the stream's two row barriers)
   int* cnt = const_cast<int*>(S.abort_flag) + 1;
   if (threadIdx.x == 0) {
     for (int s = 0; s < NST; s++) {
       mbar_init(S.full + s, 1);
       mbar_init(S.empty + s, CW);
     }
-    mbar_init(S.rowfull, kAsyncRows ? 1 : CW);
-    mbar_init(S.rowfree, kAsyncRows ? 1 : CW);
+    mbar_init(S.rowfull, 1);
+    mbar_init(S.rowfree, 1);
     *S.abort_flag = 0;
     cnt[0] = cnt[1] = 0;
     fence_mbar_init();
@@ -1376,10 +1359,9 @@ __global__ void __launch_bounds__((CW + 1) * 32, 1) k_dense_stream_m(MixedStream
   W.err = P.err;
   W.budget = P.budget;
   float* red = reinterpret_cast<float*>(S.red);
-  // kEight: rows of more than 32 points use the eight-rows-per-lane layout (consume_item8); the
-  // other layouts keep their sums in the first two rows of acc
-  constexpr bool kEight = NVB <= 4;
-  constexpr int AR = kEight ? 8 : 2;
+  // rows of more than 32 points use the eight-rows-per-lane layout (consume_item8); shorter ones
+  // keep their sums in the first two rows of acc
+  constexpr int AR = 8;
   float acc[AR][NVB];
 #pragma unroll
   for (int r = 0; r < AR; r++)
@@ -1398,8 +1380,8 @@ __global__ void __launch_bounds__((CW + 1) * 32, 1) k_dense_stream_m(MixedStream
     const bool y32 = hd[kHdXy32] != 0;
     const long long ldy = *reinterpret_cast<const long long*>(hd + kHdLdy);
     // the variant for the item's vector count (a matrix of a batch may take fewer than NVB)
-    const bool eight = kEight && R > 32;
-    if constexpr (kEight) {
+    const bool eight = R > 32;
+    {
       const int uni = hd[4];
       if (eight && (uni == 1 || uni == 2) && nb * 64 * nv <= kMixedVecCols * NVB) {
         const bool pnl = uni == 2;
@@ -1413,9 +1395,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, 1) k_dense_stream_m(MixedStream
       }
     }
     if (!eight) {
-      if (NVB >= 16 && nv > 8) consume_item<F, (NVB >= 16 ? 16 : 1), NVB, CW>(stage, hd, nb, R, warp, lane, acc2);
-      else if (NVB >= 8 && nv > 4) consume_item<F, (NVB >= 8 ? 8 : 1), NVB, CW>(stage, hd, nb, R, warp, lane, acc2);
-      else if (NVB >= 4 && nv > 2) consume_item<F, (NVB >= 4 ? 4 : 1), NVB, CW>(stage, hd, nb, R, warp, lane, acc2);
+      if (NVB >= 4 && nv > 2) consume_item<F, (NVB >= 4 ? 4 : 1), NVB, CW>(stage, hd, nb, R, warp, lane, acc2);
       else if (NVB >= 2 && nv > 1) consume_item<F, (NVB >= 2 ? 2 : 1), NVB, CW>(stage, hd, nb, R, warp, lane, acc2);
       else consume_item<F, 1, NVB, CW>(stage, hd, nb, R, warp, lane, acc2);
     }
@@ -1438,13 +1418,9 @@ __global__ void __launch_bounds__((CW + 1) * 32, 1) k_dense_stream_m(MixedStream
 #pragma unroll
           for (int v = 0; v < NVB; v++) acc[r][v] += __shfl_xor_sync(0xFFFFFFFFu, acc[r][v], 16);
       }
-      const int par = kAsyncRows ? rows_done & 1 : 0;
-      if (kAsyncRows) {
-        // the half of red this row uses was last summed for row rows_done - 2
-        if (rows_done >= 2 && !warp_wait(rowfree2 + par, ((rows_done >> 1) - 1) & 1, W, S.abort_flag)) break;
-      } else if (rows_done > 0 && !warp_wait(S.rowfree, (rows_done - 1) & 1, W, S.abort_flag)) {
-        break;
-      }
+      const int par = rows_done & 1;
+      // the half of red this row uses was last summed for row rows_done - 2
+      if (rows_done >= 2 && !warp_wait(rowfree2 + par, ((rows_done >> 1) - 1) & 1, W, S.abort_flag)) break;
       float* redp = red + par * (CW * NVB * 64);
       if (eight) {
         if (lane < 8)
@@ -1467,21 +1443,6 @@ __global__ void __launch_bounds__((CW + 1) * 32, 1) k_dense_stream_m(MixedStream
 #pragma unroll
         for (int v = 0; v < NVB; v++) acc[r][v] = 0.f;
       __syncwarp();
-      if (!kAsyncRows) {
-        if (lane == 0) mbar_arrive(S.rowfull);
-        if (!warp_wait(S.rowfull, rows_done & 1, W, S.abort_flag)) break;
-        for (int idx = threadIdx.x; idx < R * nv; idx += CW * 32) {
-          const int r = idx % R, v = idx / R;
-          float sum = 0.f;
-#pragma unroll
-          for (int w = 0; w < CW; w++) sum += red[(w * NVB + v) * 64 + r];
-          y_store(ydst, y32, v * ldy + row + r, sum, false);  // y was zeroed or assigned; the other part adds too
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(S.rowfree);
-        rows_done++;
-        continue;
-      }
       int last = 0;
       if (lane == 0) {
         __threadfence_block();

@@ -48,8 +48,8 @@ template <int NVB>
 __host__ __device__ constexpr int tree_area(int k) { return (k * tree_vstride<NVB>() + 3) & ~3; }
 
 // Dynamic shared memory of a tree CTA: nbuf block buffers of `block` bytes, two vector areas of 64 rows
-// (a leaf's points, a pair of children, a path node), then 2 + T vector areas of k rows, the leaf table
-// and a flag.
+// (a leaf's points, a pair of children, a path node), then 2 + T vector areas of k rows, the leaf table,
+// the leaves' maxima and a flag.
 struct TreeSmem {
   int block, nbuf, table, bytes;
 };
@@ -61,7 +61,7 @@ __host__ __device__ inline TreeSmem tree_smem(int k, int block_entries, int T) {
   // vectors, would not fit beside the dense stream's CTA (kTreeReserve)
   S.nbuf = S.block <= (NVB >= 8 ? 32768 : 10240) ? 2 : 1;
   S.table = (S.nbuf * S.block + (2 * 64 * tree_vstride<NVB>() + (2 + T) * tree_area<NVB>(k)) * (int)sizeof(typename Op::V) + 15) & ~15;
-  S.bytes = S.table + (1 << T) * (int)sizeof(typename Op::Leaf) + 16;
+  S.bytes = S.table + (((1 << T) * (int)sizeof(typename Op::Leaf) + 15) & ~15) + 16 + 3 * 64;
   return S;
 }
 // i / k for i < 4096, k <= 64, as a multiplication (m = div_magic(k))
@@ -172,12 +172,15 @@ __device__ __forceinline__ void tree_up(const typename Op::P& P, int64_t sub, bo
   V* nodes = xbuf + 2 * 64 * VS;                                // right results (by depth parity), then left ones by depth
   Leaf* table = reinterpret_cast<Leaf*>(tree_dyn + S.table);
   int* won_s = reinterpret_cast<int*>(tree_dyn + S.bytes - 16);
+  unsigned* vmax = reinterpret_cast<unsigned*>(tree_dyn + S.bytes - 16 - 3 * 64);  // max |x| per vector of a leaf, three leaves in turn
   const int warp = threadIdx.x >> 5, rl = threadIdx.x & 7, g = (threadIdx.x >> 3) & 3;
   const int64_t j0 = sub << T, leaf0 = ((int64_t)1 << P.q) - 1, vs = (int64_t)nv * P.kp;
   const int kr = (k + 7) / 8, krl = 32 - __clz(kr - 1), ns = (nv + VW - 1) / VW, nt = ns << krl;
   const unsigned kdiv = div_magic(k);
   const int AS = tree_area<NVB>(k);
 
+  bool parts = false;  // the dense phase wants the vectors as 16-bit parts too
+  if constexpr (Op::kParts) parts = convert && Op::want_parts(P);
   typename Op::X xr[XN];  // the next leaf's x: point tid % 64 of vectors tid / 64 + (TH / 64) i
   const int xa = threadIdx.x & 63, xv0 = threadIdx.x >> 6;
   int buf = 0;
@@ -271,6 +274,7 @@ __device__ __forceinline__ void tree_up(const typename Op::P& P, int64_t sub, bo
 
   if (active) {
     for (int i = threadIdx.x; i < (1 << T); i += TH) table[i] = Op::leaf_v(P, j0 + i);
+    if (threadIdx.x < 48) vmax[threadIdx.x] = 0u;
     __syncthreads();
   }
   int t = 0, d = 0;
@@ -294,12 +298,20 @@ __device__ __forceinline__ void tree_up(const typename Op::P& P, int64_t sub, bo
 #pragma unroll
         for (int i = 0; i < XN; i++) {
           const int v = xv0 + (TH / 64) * i;
-          if (v < nv) {
+          if (v < nv) {  // (the same for the whole warp)
             const V val = Op::xvalue(P, xr[i], v);
             if (xa < lf.s) xs[xa * VS + v] = val;
             if (convert && xa < sp) Op::xstore(P, lf, sp, v, xa, val);  // (the padding is zero)
+            if constexpr (Op::kParts) {
+              if (parts) {
+                const unsigned m = __reduce_max_sync(0xFFFFFFFFu, xa < lf.s ? Op::abs_bits(val) : 0u);
+                if ((threadIdx.x & 31) == 0) atomicMax(vmax + 16 * (t % 3) + v, m);
+              }
+            }
           }
         }
+        // cleared for the next leaf: its last reader was the leaf before the last one, a barrier ago
+        if (parts && threadIdx.x < 16) vmax[16 * ((t + 1) % 3) + threadIdx.x] = 0u;
         x0 = x1 = xs;
         C = lf.s;
         NB = 1;
@@ -352,6 +364,9 @@ __device__ __forceinline__ void tree_up(const typename Op::P& P, int64_t sub, bo
       }
     };
     if (S.nbuf == 2) fetch_next(buf = cur ^ 1);
+    if constexpr (Op::kParts) {
+      if (parts && !climbing && d == 0) Op::template parts<VS, TH>(P, j0 + t, C, x0, vmax + 16 * (t % 3));
+    }
     const typename Op::A* A = reinterpret_cast<const typename Op::A*>(tree_dyn + cur * S.block);
 #pragma unroll 1
     for (int u = warp; u < nt; u += TW) {
