@@ -87,6 +87,7 @@ bool values_ok(const double* v, int64_t count, int64_t* bad, bool fp32_range = t
 struct BlockStat {
   double lnorm = -HUGE_VAL;  // log2 of the largest row sum of |a| (-inf for a zero block)
   int emax = 0;              // frexp exponent of the largest |a| (0 for a zero block)
+  double mmax = 0.0;         // and its frexp fraction
   int emin = 0;              // frexp exponent of the smallest nonzero normal |a|
   bool zero = false;         // some entry is zero or an FP64 subnormal
 };
@@ -106,7 +107,7 @@ BlockStat block_stat(const double* a, int64_t rows, int64_t cols, int64_t rs, in
     st.zero = true;
     return st;
   }
-  std::frexp(mx, &st.emax);
+  st.mmax = std::frexp(mx, &st.emax);
   std::frexp(mn, &st.emin);
   double best = 0.0;
   for (int64_t r = 0; r < rows; r++) {
@@ -139,6 +140,8 @@ bool needs_safe_split(const BlockStat& st, int o) { return st.zero || st.emin - 
 struct Fp64Ranges {
   std::vector<int32_t> oV, oF, oE, oS, oD, oU, eY;
   std::vector<char> d_safe;
+  std::vector<int32_t> d_exp;  // each dense block's exponent ea for k_dense_oz
+  bool d_narrow = true;         // every dense block's nonzero entries lie within 2^10
   bool s_tiny = false;
 };
 
@@ -199,6 +202,7 @@ Fp64Ranges fp64_ranges(const h2_desc* d, int64_t leaves, int64_t n_nodes, int64_
   R.oS.resize((size_t)nS);
   R.oD.resize((size_t)nD);
   R.d_safe.resize((size_t)nD);
+  R.d_exp.resize((size_t)nD);
   for (int64_t j = 0; j < leaves; j++) {
     R.eY[j] = exp_of_bound(bY[j]);
     R.oV[j] = block_offset(ex[leaf0 + j], sV[j]);
@@ -217,6 +221,9 @@ Fp64Ranges fp64_ranges(const h2_desc* d, int64_t leaves, int64_t n_nodes, int64_
   for (int64_t b = 0; b < nD; b++) {
     R.oD[b] = block_offset(R.eY[drow[b]], sD[b]);
     R.d_safe[b] = needs_safe_split(sD[b], R.oD[b]);
+    // |a| 2^(46 - ea) <= 0x7F7F7F7F7F7F, the digits' range: one less than the frexp exponent where that fits
+    R.d_exp[b] = sD[b].emax - (sD[b].mmax < 0.99 ? 1 : 0);
+    if (sD[b].lnorm != -HUGE_VAL && sD[b].emax - sD[b].emin > 10) R.d_narrow = false;
   }
   (void)q;
   return R;
@@ -451,6 +458,8 @@ cudaError_t set_pass_smem() {
     constexpr int CW = h2::dense_consumer_warps(NVB);
     cudaError_t e = cudaFuncSetAttribute(h2::k_dense_stream<NVB, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          h2::stream_smem_bytes(NVB, CW));
+    if (e == cudaSuccess && NVB > 4)
+      e = cudaFuncSetAttribute(h2::k_dense_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, h2::kOzSmem);
     for (const void* f : {(const void*)h2::k_upsweep_tree<NVB>, (const void*)h2::k_downsweep_tree<NVB>})
       if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, h2::kSmemLimit);
     return e;
@@ -490,6 +499,16 @@ h2_status run_pass(h2_matrix_s* h, int nv, const double* x, int64_t ldx, double*
   T.q = h->q;
   T.L = h->tree_L;
   T.nv = nv;
+  const bool oz = NVB > 4 && h->oz;
+  T.oz = oz;
+  T.xks = (h->m_max + 15) / 16;
+  T.xd = h->xd;
+  T.dmat = h->dmat;
+  T.u_off = h->u_off;
+  T.oU = h->oU;
+  T.eY = h->eY;
+  T.y = y;
+  T.ldy = ldy;
   const unsigned tree_grid = 1u << h->tree_L, tree_threads = tree_warps<NVB>() * 32;
   const unsigned tsm = tree_smem<TreeOp64, NVB>(k, tree_block_entries(k, T.kks, false), T.q - T.L).bytes;
   cudaError_t me = mark(&h->prof, st);
@@ -533,7 +552,26 @@ h2_status run_pass(h2_matrix_s* h, int nv, const double* x, int64_t ldx, double*
   P.err = h->err;
   P.budget = h->budget;
   P.inject = h->inject;
-  k_dense_stream<NVB, CW><<<h->grid, (CW + 1) * 32, smem, st>>>(P);
+  if (oz) {
+    OzParams O{};
+    O.items = P.items;
+    O.cta_begin = P.cta_begin;
+    O.item_exp = h->item_exp;
+    O.item_leaf = h->item_leaf;
+    O.mat = P.mat;
+    O.xd = h->xd;
+    O.xks = T.xks;
+    O.nv = nv;
+    O.y = y;
+    O.ldy = ldy;
+    O.vexp = h->vexp;
+    O.err = h->err;
+    O.budget = h->budget;
+    O.inject = h->inject;
+    k_dense_oz<<<h->grid, (kOzWarps + 1) * 32, kOzSmem, st>>>(O);
+  } else {
+    k_dense_stream<NVB, CW><<<h->grid, (CW + 1) * 32, smem, st>>>(P);
+  }
   if (h->inject >= 0) {  // the test hook applies to one product only
     h->inject = -1;
     h->budget = kWaitBudget;
@@ -704,6 +742,25 @@ h2_status build_device(h2_matrix_s* h, const h2_desc* d) {
       row_bytes[i] = bytes + it.m_bytes + 8 * h->kp + 16 * si;
     }
     row_item0[h->leaves] = (int64_t)items.size();
+    // the digits' tables (see mma_fp64.cuh)
+    h->oz = R.d_narrow && h->nD > 0;
+    if (h->oz) {
+      std::vector<int32_t> iexp(items.size(), 0), ileaf(items.size(), 0);
+      std::vector<int64_t> uo((size_t)h->leaves);
+      for (int64_t i = 0, b = 0, t = 0; i < h->leaves; i++, t++) {
+        for (; b < d->D_rowptr[i + 1]; b++, t++) {
+          iexp[(size_t)t] = R.d_exp[(size_t)b];
+          ileaf[(size_t)t] = d->D_colidx[b];
+        }
+        uo[(size_t)i] = (dtot + upo[i]) * 8;
+      }
+      if ((st = upload(h, &h->item_exp, iexp.data(), (int64_t)iexp.size())) != H2_OK) return st;
+      if ((st = upload(h, &h->item_leaf, ileaf.data(), (int64_t)ileaf.size())) != H2_OK) return st;
+      if ((st = upload(h, &h->u_off, (const int64_t*)uo.data(), h->leaves)) != H2_OK) return st;
+      if ((st = upload(h, &h->oU, R.oU.data(), h->leaves)) != H2_OK) return st;
+      if ((st = upload(h, &h->eY, R.eY.data(), h->leaves)) != H2_OK) return st;
+      if ((st = dalloc(h, &h->xd, h->leaves * h2::xd_chunk_bytes((h->m_max + 15) / 16, 2))) != H2_OK) return st;
+    }
     const std::vector<int> begin = balance(row_bytes, row_item0, h->grid);
     // vector sources per slot: split x (padded leaf layout) and yhat (n_nodes x kp)
     if ((st = audit_items(items, begin, total * 8, xp[h->leaves], h->n_nodes * h->kp)) != H2_OK) return st;

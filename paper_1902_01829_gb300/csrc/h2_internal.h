@@ -208,6 +208,14 @@ struct h2_matrix_s {
   int32_t* oF = nullptr;
   int32_t* oE = nullptr;
   int2* Sco = nullptr;
+  // passes of more than four vectors: the dense phase by digits (k_dense_oz), if no dense block spans more than 2^10
+  bool oz = false;
+  int* item_exp = nullptr;            // per dense item: its block's exponent and column leaf
+  int* item_leaf = nullptr;
+  unsigned char* xd = nullptr;        // digits of the pass's vectors
+  int64_t* u_off = nullptr;           // per leaf: byte offset of U_j in dmat, its exponent offset, the rows' exponent
+  int* oU = nullptr;
+  int* eY = nullptr;
   const void* csegs = nullptr;        // coupling segments (h2::CouplingSeg), and the split rows' partial sums
   int64_t ncsegs = 0;
   float2* cpart = nullptr;            // [slot][v][kp]

@@ -20,6 +20,7 @@
 //   yhat  same as xhat
 #pragma once
 #include "df64.cuh"
+#include "mma_fp64.cuh"
 #include "tree.cuh"
 
 namespace h2 {
@@ -116,6 +117,16 @@ struct TreeParams {
   const int* vexp;         // per vector of the pass: x enters scaled by 2^-vexp[v]
   int64_t kks;             // doubles from a node's transfer matrix to the next node's
   int k, kp, q, L, nv;
+  // passes whose dense phase is k_dense_oz: the vectors' digits (xks K steps per leaf), and the leaf expansion
+  // by the downsweep: U_j at dmat + u_off[j], its exponent offset, the rows' output exponent
+  int oz, xks;
+  unsigned char* xd;
+  const char* dmat;
+  const int64_t* u_off;
+  const int* oU;
+  const int* eY;
+  double* y;
+  int64_t ldy;
 };
 
 // tree.cuh's arithmetic for the FP64 form: double-float vectors, FP64 entries split with their
@@ -145,19 +156,26 @@ struct TreeOp64 {
   static __device__ __forceinline__ float2 value(const Acc& p) { return df_norm(p.s, p.c); }
   static __device__ __forceinline__ int spad(int s) { return s + (s & 1); }
   struct Leaf {
-    int64_t off, xp;  // first point; offset of the split x (per vector slot)
-    int s, bV, bU;    // points; exponent offset of V_j
+    int64_t off, xp, uoff;  // first point; offsets of the split x (per vector slot) and of U_j
+    int s, bV, bU, eY;      // points; exponent offsets of V_j and U_j; the rows' output exponent
   };
   static __device__ __forceinline__ Leaf leaf_v(const P& T, int64_t j) {
-    Leaf l;
+    Leaf l{};
     l.off = T.leaf_off[j];
     l.s = (int)(T.leaf_off[j + 1] - l.off);
     l.xp = T.xp_off[j];
     l.bV = T.oV[j];
-    l.bU = 0;
     return l;
   }
-  static __device__ __forceinline__ Leaf leaf_u(const P&, int64_t) { return Leaf{}; }
+  static __device__ __forceinline__ Leaf leaf_u(const P& T, int64_t j) {
+    Leaf l{};
+    l.off = T.leaf_off[j];
+    l.s = (int)(T.leaf_off[j + 1] - l.off);
+    l.uoff = T.u_off[j];
+    l.bU = T.oU[j];
+    l.eY = T.eY[j];
+    return l;
+  }
   static __device__ __forceinline__ const double* Vt(const P& T, const Leaf& l) { return T.Vt + l.off * T.k; }
   static __device__ __forceinline__ const double* Ft(const P& T, int64_t h) { return T.Ft + (h - 1) * T.kks; }
   static __device__ __forceinline__ const double* E(const P& T, int64_t h) { return T.Et + (h - 1) * T.kks; }
@@ -171,13 +189,46 @@ struct TreeOp64 {
   static __device__ __forceinline__ void xstore(const P& T, const Leaf& l, int sp, int v, int a, float2 x) {
     T.x2[l.xp * T.nv + v * sp + a] = x;
   }
-  static constexpr bool kParts = false;
+  static constexpr bool kParts = true;
+  static __device__ __forceinline__ bool want_parts(const P& T) { return T.oz != 0; }
+  static __device__ __forceinline__ unsigned abs_bits(float2 x) { return __float_as_uint(x.x) & 0x7FFFFFFFu; }
+  // leaf j's vectors xs ([point][vector], stride VS) as digits (mma_fp64.cuh); vmax: float bits of max |x| per vector
+  template <int VS, int TH>
+  static __device__ __forceinline__ void parts(const P& T, int64_t j, int s, const float2* xs, const unsigned* vmax) {
+    const int nh = T.nv > 8 ? 2 : 1;
+    unsigned char* chunk = T.xd + j * xd_chunk_bytes(T.xks, nh);
+    // |x| 2^(46 - ex) <= 0x7F7F7F7F7F7F, the digits' range: the exponent of the largest |x|, one more where its
+    // fraction leaves no room; a chunk below 2^-80 of its vector's largest entry keeps that unit
+    auto ex = [&](int v) { return max((int)(vmax[v] >> 23) - ((vmax[v] & 0x7FFFFFu) < 0x7D0000u ? 127 : 126), -80); };
+    for (int i = threadIdx.x; i < ((s + 15) >> 4) * 32 * nh; i += TH) {
+      const int ln = i & 31, u = i >> 5, ks = nh == 2 ? u >> 1 : u, half = nh == 2 ? u & 1 : 0;
+      const int v = (ln >> 2) + 8 * half, c0 = 16 * ks + (ln & 3);
+      const float up = __int_as_float((127 + 46 - (v < T.nv ? ex(v) : 0)) << 23);
+      uint32_t lo[4], hi[4];
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        const int c = c0 + 4 * q;
+        const float2 x = (v < T.nv && c < s) ? xs[c * VS + v] : make_float2(0.f, 0.f);
+        const long long n = __float2ll_rn(x.x * up) + __float2ll_rn(x.y * up) + 0x808080808080LL;
+        lo[q] = (uint32_t)n;
+        hi[q] = (uint32_t)((unsigned long long)n >> 32);
+      }
+      uint32_t d0[6], d1[6];
+      digit_pairs(lo[0], hi[0], lo[1], hi[1], d0);
+      digit_pairs(lo[2], hi[2], lo[3], hi[3], d1);
+      uint2* dst = reinterpret_cast<uint2*>(chunk + kXdScale + u * kXdStep + ln * 8);
+#pragma unroll
+      for (int p = 0; p < 6; p++) dst[32 * p] = make_uint2(d0[p], d1[p]);
+    }
+    if (threadIdx.x < 16) reinterpret_cast<int*>(chunk)[threadIdx.x] = threadIdx.x < T.nv ? ex(threadIdx.x) : -80;
+  }
   static __device__ __forceinline__ int copy_bytes(int entries) { return 8 * entries; }
-  // (the leaf expansion is the dense stream's)
-  static __device__ __forceinline__ const double* U(const P&, const Leaf&) { return nullptr; }
-  static __device__ __forceinline__ int u_bytes(const P&, const Leaf&) { return 0; }
+  static __device__ __forceinline__ const char* U(const P& T, const Leaf& l) { return T.dmat + l.uoff; }
+  static __device__ __forceinline__ int u_bytes(const P& T, const Leaf& l) { return 8 * l.s * T.k; }
   static __device__ __forceinline__ void u_layout(const P&, const Leaf&, int, int&, int&) {}
-  static __device__ __forceinline__ void ystore(const P&, int, int64_t, const Acc&, bool) {}
+  static __device__ __forceinline__ void ystore(const P& T, const Leaf& l, int v, int row, const Acc& a, bool) {
+    T.y[v * T.ldy + l.off + row] = scale2(df_to_f64(a.s, a.c), l.eY + T.vexp[v]);
+  }
 };
 
 template <int NVB>
@@ -188,7 +239,7 @@ __global__ void __cluster_dims__(kTreeCluster) __launch_bounds__(tree_warps<NVB>
 
 template <int NVB>
 __global__ void __launch_bounds__(tree_warps<NVB>() * 32) k_downsweep_tree(TreeParams P) {
-  tree_down<TreeOp64, NVB>(P, blockIdx.x, 0, P.q - P.L, tree_block_entries(P.k, P.kks, false));
+  tree_down<TreeOp64, NVB>(P, blockIdx.x, P.oz ? 2 : 0, P.q - P.L, tree_block_entries(P.k, P.kks, false));
 }
 
 // ---------------------------------------------------------------- coupling, all levels

@@ -394,8 +394,8 @@ struct TreeOpM {
   static __device__ __forceinline__ void u_layout(const P& T, const Leaf& l, int row, int& roff, int& cs) {
     if (l.panel) roff = (row >> 3) * (panel_stride(T.k) / 2) + (row & 7), cs = 8;
   }
-  static __device__ __forceinline__ void ystore(const P& T, int v, int64_t i, float val, bool assign) {
-    y_store(T.D->y, T.xy32, v * T.D->ldy + i, val, assign);
+  static __device__ __forceinline__ void ystore(const P& T, const Leaf& l, int v, int row, float val, bool assign) {
+    y_store(T.D->y, T.xy32, v * T.D->ldy + l.off + row, val, assign);
   }
 };
 

@@ -514,7 +514,7 @@ __device__ __forceinline__ void tree_down(const typename Op::P& P, int64_t sub, 
       if (g < VW && row < rows && v < nv) {
         typename Op::Acc r = tree_pick<Op, VW>(acc, g);
         if (ex) {
-          Op::ystore(P, v, table[j].off + row, r, expand == 2);
+          Op::ystore(P, table[j], v, row, r, expand == 2);
         } else {
           Op::add_value(r, ow[row * VS + v]);
           const V val = Op::value(r);

@@ -80,3 +80,26 @@ def test_batch_with_fewer_vectors(h2):
     for A, x, y in zip(As, xs, ys):
         check(oracle.rel_l2(y.cpu().numpy(), oracle.matvec(A, x, **quant.dequantized_arrays(A, "int16"))), acc_tol(A), (A.n, x.shape[1]))
     B.close()
+
+
+@pytest.mark.parametrize("sizes", [SIZES, [32] * 8, [64] * 4 + [49] * 4, [29, 30] * 4, [5]])
+@pytest.mark.parametrize("span", ["narrow", "wide"])
+def test_fp64_digits(h2, sizes, span):
+    """FP64: blocks whose nonzero entries lie within 2^10 (the digits' path for more than four vectors; zeros,
+    exact powers of two and block magnitudes 2^-200 .. 2^200 among them) and blocks that do not."""
+    A = dense_matrix(50 + len(sizes), sizes)
+    rng = np.random.default_rng(5)
+    if span == "narrow":
+        D = np.sign(A.D_val) * rng.uniform(2.0 ** -9, 1.0, A.D_val.size)
+        D[rng.random(D.size) < 0.05] = 0.0
+        D[rng.random(D.size) < 0.05] = 1.0
+        nb = A.D_valoff.size - 1
+        A.D_val = D * np.repeat(np.ldexp(1.0, np.where(rng.random(nb) < 0.1, rng.integers(-200, 201, nb), 0)), np.diff(A.D_valoff))
+    M = handle(h2, A, "fp64")
+    for nv in (5, 8, 9, 16, 22):
+        x = h2gen.vectors(820 + nv, A.n, nv) * np.ldexp(1.0, 20 * np.arange(nv) - 160)[None, :]
+        x[rng.random(x.shape) < 0.05] = 0.0
+        x[: A.leaf_offset[1]] *= 2.0 ** -60  # a leaf far below the vector's largest entry
+        assert oracle.rel_l2(M.matvec(to_dev(x)).cpu().numpy(), oracle.matvec(A, x)) <= 1e-12
+    M.check()
+    M.close()
