@@ -528,13 +528,14 @@ h2_status run_pass(h2_matrix_s* h, int nv, const double* x, int64_t ldx, double*
   C.kp = kp;
   C.LR = LR;
   C.nv = nv;
-  const unsigned cgrid = (unsigned)h->ncsegs;
+  constexpr int CV = NVB < 4 ? NVB : 4;  // vectors per CTA
+  const dim3 cgrid((unsigned)h->ncsegs, (unsigned)((nv + CV - 1) / CV));
   if (h->pair_rows) {
-    constexpr int CB = NVB <= 2 ? 4 : (NVB <= 4 ? 2 : 1);
-    if (h->s_tiny) k_coupling<NVB, CB, true><<<cgrid, wb, 0, st>>>(C);
-    else k_coupling<NVB, CB, false><<<cgrid, wb, 0, st>>>(C);
+    constexpr int CB = CV <= 2 ? 4 : 2;
+    if (h->s_tiny) k_coupling<CV, CB, true><<<cgrid, wb, 0, st>>>(C);
+    else k_coupling<CV, CB, false><<<cgrid, wb, 0, st>>>(C);
   } else {
-    k_coupling_generic<RPL_K, NVB><<<cgrid, wb, 0, st>>>(C);
+    k_coupling_generic<RPL_K, CV><<<cgrid, wb, 0, st>>>(C);
   }
   if (me == cudaSuccess) me = mark(&h->prof, st);
   k_downsweep_tree<NVB><<<tree_grid, tree_threads, tsm, st>>>(T);
@@ -799,8 +800,8 @@ h2_status build_device(h2_matrix_s* h, const h2_desc* d) {
     h->csegs = ds;
     h->ncsegs = (int64_t)segs.size();
     if ((st = dalloc(h, &h->cpart, slots * kPassVectors * h->kp)) != H2_OK) return st;
-    if ((st = dalloc(h, &h->cticket, slots)) != H2_OK) return st;
-    CUDA_TRY(cudaMemset(h->cticket, 0, (size_t)std::max<int64_t>(slots, 1) * sizeof(int)));
+    if ((st = dalloc(h, &h->cticket, 4 * slots)) != H2_OK) return st;
+    CUDA_TRY(cudaMemset(h->cticket, 0, (size_t)std::max<int64_t>(4 * slots, 1) * sizeof(int)));
   }
   if ((st = dalloc(h, &h->vexp, h2i::kPassVectors)) != H2_OK) return st;
   if ((st = dalloc(h, &h->vpart, (int64_t)h2::kScaleBlocks * 16)) != H2_OK) return st;

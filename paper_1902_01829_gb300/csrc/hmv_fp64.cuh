@@ -220,7 +220,10 @@ struct TreeOp64 {
 #pragma unroll
       for (int p = 0; p < 6; p++) dst[32 * p] = make_uint2(d0[p], d1[p]);
     }
-    if (threadIdx.x < 16) reinterpret_cast<int*>(chunk)[threadIdx.x] = threadIdx.x < T.nv ? ex(threadIdx.x) : -80;
+    // (a chunk with an infinity or NaN: kXdNaN makes its vector's sums NaN)
+    if (threadIdx.x < 16)
+      reinterpret_cast<int*>(chunk)[threadIdx.x] =
+          threadIdx.x >= T.nv ? -80 : vmax[threadIdx.x] >= 0x7F800000u ? kXdNaN : ex(threadIdx.x);
   }
   static __device__ __forceinline__ int copy_bytes(int entries) { return 8 * entries; }
   static __device__ __forceinline__ const char* U(const P& T, const Leaf& l) { return T.dmat + l.uoff; }
@@ -262,6 +265,8 @@ __global__ void __launch_bounds__(tree_warps<NVB>() * 32) k_downsweep_tree(TreeP
 // is written (zero when it has no blocks). A lane's products form chains of
 // at most 64 (kFoldProducts) that are folded into a long-term pair, so the
 // FP32 sum of the small parts never runs over a whole row.
+// Passes of more than four vectors run slices of four (grid y): 16 vectors in one warp took 255 registers and
+// left 8 warps an SM; four slices split every entry four times but hold twice the warps (COUPSLICE).
 // SAFE: some coupling entry is zero or below 2^-103 after its offset (zero-safe split).
 constexpr int kFoldProducts = 64;
 
@@ -279,7 +284,7 @@ struct CouplingParams {
   const float2* xhat;
   float2* yhat;
   float2* part;   // [slot][v][kp], the segments of split rows
-  int* ticket;    // per slot base, zero between products
+  int* ticket;    // [slot base][4], a counter per vector slice, zero between products
   int kkp, k, kp, LR, nv;
 };
 
@@ -289,9 +294,10 @@ template <int NVB>
 __device__ __forceinline__ void coupling_finish(const CouplingParams& P, const CouplingSeg& sg, float2 (*red)[NVB][64],
                                                 int* last) {
   __syncthreads();
-  const int k = P.k, kp = P.kp, nv = P.nv;
-  float2* row = P.yhat + (int64_t)sg.row * nv * kp;
-  float2* mine = sg.parts == 1 ? row : P.part + (int64_t)(sg.base + sg.seg) * nv * kp;
+  const int k = P.k, kp = P.kp, v0 = blockIdx.y * NVB, nv = min(P.nv - v0, NVB);
+  const int64_t stride = (int64_t)P.nv * kp;
+  float2* row = P.yhat + sg.row * stride + v0 * kp;
+  float2* mine = sg.parts == 1 ? row : P.part + (sg.base + sg.seg) * stride + v0 * kp;
   for (int t = threadIdx.x; t < nv * k; t += kWarps * 32) {
     const int v = t / k, r = t - v * k;
     float s = 0.f, c = 0.f;
@@ -303,19 +309,20 @@ __device__ __forceinline__ void coupling_finish(const CouplingParams& P, const C
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
-    *last = atomicAdd(P.ticket + sg.base, 1) == sg.parts - 1;
-    if (*last) P.ticket[sg.base] = 0;  // every segment has arrived: reset for the next product
+    int* ticket = P.ticket + 4 * (int64_t)sg.base + blockIdx.y;
+    *last = atomicAdd(ticket, 1) == sg.parts - 1;
+    if (*last) *ticket = 0;  // every segment has arrived: reset for the next product
   }
   __syncthreads();
   if (!*last) return;
   __threadfence();
   for (int t = threadIdx.x; t < nv * k; t += kWarps * 32) {
     const int v = t / k, r = t - v * k;
-    const float2* src = P.part + (int64_t)sg.base * nv * kp + v * kp + r;
+    const float2* src = P.part + sg.base * stride + (v0 + v) * kp + r;
     float s = 0.f, c = 0.f;
 #pragma unroll 4
     for (int p = 0; p < sg.parts; p++) {
-      const float2 a = __ldcg(src + (int64_t)p * nv * kp);
+      const float2 a = __ldcg(src + p * stride);
       df_add(s, c, a.x, a.y);
     }
     row[v * kp + r] = df_norm(s, c);
@@ -328,7 +335,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_coupling(CouplingParams P) {
   __shared__ int last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const CouplingSeg sg = P.segs[blockIdx.x];
-  const int k = P.k, kp = P.kp, nv = P.nv;
+  const int k = P.k, kp = P.kp, v0 = blockIdx.y * NVB, nv = min(P.nv - v0, NVB);  // this CTA's vectors
   const double* __restrict__ S = P.S;
   const int2* __restrict__ Sco = P.Sco;
   const float2* __restrict__ xhat = P.xhat;
@@ -351,7 +358,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_coupling(CouplingParams P) {
     const int bl = bt / ncb, cb = bt - bl * ncb, b = b0 + kWarps * bl;
     const double* A = S + (int64_t)b * P.kkp;
     const int2 co = __ldg(Sco + b);
-    const float2* X = xhat + (int64_t)co.x * nv * kp;
+    const float2* X = xhat + ((int64_t)co.x * P.nv + v0) * kp;
     o = co.y;
 #pragma unroll
     for (int u = 0; u < CB; u++) {
@@ -425,13 +432,13 @@ __global__ void __launch_bounds__(kWarps * 32) k_coupling_generic(CouplingParams
   __shared__ int last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const CouplingSeg sg = P.segs[blockIdx.x];
-  const int k = P.k, kp = P.kp, LR = P.LR, nv = P.nv;
+  const int k = P.k, kp = P.kp, LR = P.LR, v0 = blockIdx.y * NVB, nv = min(P.nv - v0, NVB);
   float s[RPL][NVB], c[RPL][NVB], S2[RPL][NVB], C2[RPL][NVB];
   acc_zero(s, c);
   acc_zero(S2, C2);
   for (int b = sg.b0 + warp; b < sg.b0 + sg.nb; b += kWarps) {
     const int2 co = P.Sco[b];
-    warp_mv<RPL, NVB>(P.S + (int64_t)b * P.kkp, co.y, k, k, LR, P.xhat + (int64_t)co.x * nv * kp, kp, nv, s, c, lane);
+    warp_mv<RPL, NVB>(P.S + (int64_t)b * P.kkp, co.y, k, k, LR, P.xhat + ((int64_t)co.x * P.nv + v0) * kp, kp, nv, s, c, lane);
     acc_fold(S2, C2, s, c);
   }
   group_reduce(S2, C2, LR);

@@ -358,10 +358,12 @@ struct TreeOpM {
         const int c = c0 + 4 * q;
         x[q] = (v < T.nv && c < s) ? xs[c * VS + v] * up : 0.f;
       }
+      const bool finite = v >= T.nv || vmax[v] < 0x7F800000u;
       uint2* dst = reinterpret_cast<uint2*>(chunk + kXpScale + u * 768 + ln * 8);
 #pragma unroll
       for (int p = 0; p < 3; p++) {
         uint32_t w[2];
+        if (p == 1 && !finite) x[0] = x[1] = x[2] = x[3] = 0.f;  // an infinity is its high part alone
 #pragma unroll
         for (int q = 0; q < 2; q++) {
           if (bf) {

@@ -34,6 +34,7 @@ namespace h2 {
 // digits of a leaf's vectors: 16 exponents ex (ints), then per K step of 16 points and half of eight vectors six
 // digits of 256 bytes, lane (g, t)'s entries (vector g + 8 half; points t, t + 4, t + 8, t + 12) at 8 (4 g + t)
 constexpr int kXdScale = 64, kXdStep = 6 * 256;
+constexpr int kXdNaN = 1 << 20;  // as an exponent: the chunk's vector has an entry that is not finite
 __host__ __device__ constexpr int xd_chunk_bytes(int ksteps, int halves) { return kXdScale + ksteps * halves * kXdStep; }
 
 constexpr int kOzWarps = 12;  // a multiple of 1 .. 4: a warp keeps to one 16-row quarter of the rows
@@ -287,7 +288,7 @@ __global__ void __launch_bounds__((kOzWarps + 1) * 32, 1) k_dense_oz(OzParams P)
 #pragma unroll
         for (int b = 0; b < 2; b++) {
           const int n = ea - shift + ex[g + 8 * b] - 28;
-          f[b] = n < -126 ? 0.f : __int_as_float((min(n, 127) + 127) << 23);
+          f[b] = n < -126 ? 0.f : __int_as_float(n > 127 ? 0x7FC00000 : (n + 127) << 23);  // (n > 127: kXdNaN)
         }
 #pragma unroll
         for (int i = 0; i < 2; i++)

@@ -103,3 +103,20 @@ def test_fp64_digits(h2, sizes, span):
         assert oracle.rel_l2(M.matvec(to_dev(x)).cpu().numpy(), oracle.matvec(A, x)) <= 1e-12
     M.check()
     M.close()
+
+
+@pytest.mark.parametrize("form", ["fp64", "int16", "fp16", "bf16"])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_not_finite_entries(h2, form, bad):
+    """An infinity or NaN in one vector reaches every row of that vector and no other vector."""
+    A = dense_matrix(70, [32] * 4 + [49] * 4)
+    A.D_val = np.sign(A.D_val) * np.maximum(np.abs(A.D_val), 2.0 ** -7 * np.max(np.abs(A.D_val)))
+    M = handle(h2, A, form)
+    x = h2gen.vectors(840, A.n, 9)
+    clean = M.matvec(to_dev(x)).cpu().numpy()
+    x[17, 3] = bad
+    y = M.matvec(to_dev(x)).cpu().numpy()
+    assert not np.isfinite(y[:, 3]).any()
+    keep = [v for v in range(9) if v != 3]
+    assert np.array_equal(y[:, keep], clean[:, keep])
+    M.close()
