@@ -381,9 +381,8 @@ namespace {
 // its stage slot and be 16-byte aligned; checked once on the host so that a
 // layout bug is an error here, never an out-of-bounds bulk copy on the device.
 //   mat_bytes   size of the matrix buffer the items index
-//   v0, v1      float2 counts per vector slot of the two vector sources
-h2_status audit_items(const std::vector<h2::StreamItem>& items, const std::vector<int>& begin, int64_t mat_bytes,
-                      int64_t v0, int64_t v1) {
+//   lim         float2 count per vector slot of the vector source
+h2_status audit_items(const std::vector<h2::StreamItem>& items, const std::vector<int>& begin, int64_t mat_bytes, int64_t lim) {
   for (size_t c = 0; c + 1 < begin.size(); c++)
     if (begin[c] > begin[c + 1]) return fail(H2_ERR_INVALID, "internal: item ranges not monotone");
   if (begin.front() != 0 || begin.back() != (int)items.size()) return fail(H2_ERR_INVALID, "internal: item ranges do not cover the list");
@@ -391,7 +390,6 @@ h2_status audit_items(const std::vector<h2::StreamItem>& items, const std::vecto
     const h2::StreamItem& it = items[i];
     const int64_t R = it.shape & 0xFF, C = (it.shape >> 8) & 0xFF, vs = (it.shape >> 16) & 0xFF, nb = (it.shape >> 24) & 0xFF;
     // vector chunk: nv * vs float2 at v_off * nv, nv <= kPassVectors; stage slot: 512 * NVB bytes >= 64 * nv * 8
-    const int64_t lim = (it.flags & h2::kItemFlagSrc1) ? v1 : v0;
     const bool ok = it.m_off >= 0 && it.m_off % 16 == 0 && it.m_bytes >= 16 && it.m_bytes % 16 == 0 &&
                     it.m_bytes <= h2::kStageMat && it.m_off + it.m_bytes <= mat_bytes && R >= 1 && R <= 64 && C >= 1 &&
                     C <= 64 && vs >= C && vs <= 64 && vs % 2 == 0 && nb == 1 && it.v_off >= 0 && it.v_off % 2 == 0 &&
@@ -462,6 +460,13 @@ cudaError_t set_pass_smem() {
       e = cudaFuncSetAttribute(h2::k_dense_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, h2::kOzSmem);
     for (const void* f : {(const void*)h2::k_upsweep_tree<NVB>, (const void*)h2::k_downsweep_tree<NVB>})
       if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, h2::kSmemLimit);
+    // kernels that run beside one another prefer the same (largest) shared part of the L1 / shared memory split
+    constexpr int CV = NVB < 4 ? NVB : 4;
+    for (const void* f : {(const void*)h2::k_downsweep_tree<NVB>, (const void*)h2::k_dense_stream<NVB, CW>,
+                          (const void*)h2::k_coupling<CV, (CV <= 2 ? 4 : 2), true>, (const void*)h2::k_coupling<CV, (CV <= 2 ? 4 : 2), false>,
+                          (const void*)h2::k_coupling_generic<1, CV>, (const void*)h2::k_coupling_generic<2, CV>})
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
     return e;
   }();
   return done;
@@ -500,6 +505,11 @@ h2_status run_pass(h2_matrix_s* h, int nv, const double* x, int64_t ldx, double*
   T.L = h->tree_L;
   T.nv = nv;
   const bool oz = NVB > 4 && h->oz;
+  // Passes of up to four vectors stream the dense blocks on the caller's stream beside the coupling phase and the
+  // downsweep on the handle's side stream (the upsweep, which splits x, runs before both); k_vec_scale zeroes y,
+  // and the dense phase and the leaf expansion add into it. Wider passes and profiled ones run in order.
+  const bool beside = NVB <= 4 && !h->prof.on;
+  T.add = beside;
   T.oz = oz;
   T.xks = (h->m_max + 15) / 16;
   T.xd = h->xd;
@@ -511,10 +521,52 @@ h2_status run_pass(h2_matrix_s* h, int nv, const double* x, int64_t ldx, double*
   T.ldy = ldy;
   const unsigned tree_grid = 1u << h->tree_L, tree_threads = tree_warps<NVB>() * 32;
   const unsigned tsm = tree_smem<TreeOp64, NVB>(k, tree_block_entries(k, T.kks, false), T.q - T.L).bytes;
+  const unsigned dsm = tree_smem<TreeOp64, NVB>(k, tree_down_entries(k, T.kks, false), T.q - T.L).bytes;
   cudaError_t me = mark(&h->prof, st);
-  k_vec_scale<<<kScaleBlocks, kScaleThreads, 0, st>>>(x, ldx, h->n, nv, h->vpart, h->vticket, h->vexp);
+  k_vec_scale<<<kScaleBlocks, kScaleThreads, 0, st>>>(x, ldx, h->n, nv, h->vpart, h->vticket, h->vexp, beside ? y : nullptr, ldy);
   k_upsweep_tree<NVB><<<std::max(tree_grid, (unsigned)kTreeCluster), tree_threads, tsm, st>>>(T);
   if (me == cudaSuccess) me = mark(&h->prof, st);
+  cudaStream_t ts = st;  // the coupling phase's and the downsweep's
+  auto launch_dense = [&] {
+    StreamParams P{};
+    P.items = h->dense_items.items;
+    P.cta_begin = h->dense_items.cta_begin;
+    P.mat = h->dmat;
+    P.vsrc0 = h->x2;
+    P.nv = nv;
+    P.y = y;
+    P.ldy = ldy;
+    P.vexp = h->vexp;
+    P.err = h->err;
+    P.budget = h->budget;
+    P.inject = h->inject;
+    if (oz) {
+      OzParams O{};
+      O.items = P.items;
+      O.cta_begin = P.cta_begin;
+      O.item_exp = h->item_exp;
+      O.item_leaf = h->item_leaf;
+      O.mat = P.mat;
+      O.xd = h->xd;
+      O.xks = T.xks;
+      O.nv = nv;
+      O.y = y;
+      O.ldy = ldy;
+      O.vexp = h->vexp;
+      O.err = h->err;
+      O.budget = h->budget;
+      O.inject = h->inject;
+      k_dense_oz<<<h->grid, (kOzWarps + 1) * 32, kOzSmem, st>>>(O);
+    } else {
+      k_dense_stream<NVB, CW><<<h->grid, (CW + 1) * 32, smem, st>>>(P);
+    }
+  };
+  if (beside) {
+    ts = h->side;
+    if ((e = cudaEventRecord(h->ev_fork, st)) == cudaSuccess) e = cudaStreamWaitEvent(ts, h->ev_fork, 0);
+    if (e != cudaSuccess) return fail(H2_ERR_CUDA, "fork to the side stream: %s", cudaGetErrorString(e));
+    launch_dense();
+  }
   CouplingParams C{};
   C.S = h->smat;
   C.Sco = h->Sco;
@@ -532,46 +584,19 @@ h2_status run_pass(h2_matrix_s* h, int nv, const double* x, int64_t ldx, double*
   const dim3 cgrid((unsigned)h->ncsegs, (unsigned)((nv + CV - 1) / CV));
   if (h->pair_rows) {
     constexpr int CB = CV <= 2 ? 4 : 2;
-    if (h->s_tiny) k_coupling<CV, CB, true><<<cgrid, wb, 0, st>>>(C);
-    else k_coupling<CV, CB, false><<<cgrid, wb, 0, st>>>(C);
+    if (h->s_tiny) k_coupling<CV, CB, true><<<cgrid, wb, 0, ts>>>(C);
+    else k_coupling<CV, CB, false><<<cgrid, wb, 0, ts>>>(C);
   } else {
-    k_coupling_generic<RPL_K, CV><<<cgrid, wb, 0, st>>>(C);
+    k_coupling_generic<RPL_K, CV><<<cgrid, wb, 0, ts>>>(C);
   }
-  if (me == cudaSuccess) me = mark(&h->prof, st);
-  k_downsweep_tree<NVB><<<tree_grid, tree_threads, tsm, st>>>(T);
-  if (me == cudaSuccess) me = mark(&h->prof, st);
-  StreamParams P{};
-  P.items = h->dense_items.items;
-  P.cta_begin = h->dense_items.cta_begin;
-  P.mat = h->dmat;
-  P.vsrc0 = h->x2;
-  P.vsrc1 = h->yhat;
-  P.nv = nv;
-  P.y = y;
-  P.ldy = ldy;
-  P.vexp = h->vexp;
-  P.err = h->err;
-  P.budget = h->budget;
-  P.inject = h->inject;
-  if (oz) {
-    OzParams O{};
-    O.items = P.items;
-    O.cta_begin = P.cta_begin;
-    O.item_exp = h->item_exp;
-    O.item_leaf = h->item_leaf;
-    O.mat = P.mat;
-    O.xd = h->xd;
-    O.xks = T.xks;
-    O.nv = nv;
-    O.y = y;
-    O.ldy = ldy;
-    O.vexp = h->vexp;
-    O.err = h->err;
-    O.budget = h->budget;
-    O.inject = h->inject;
-    k_dense_oz<<<h->grid, (kOzWarps + 1) * 32, kOzSmem, st>>>(O);
+  if (me == cudaSuccess) me = mark(&h->prof, ts);
+  k_downsweep_tree<NVB><<<tree_grid, tree_threads, dsm, ts>>>(T);
+  if (me == cudaSuccess) me = mark(&h->prof, ts);
+  if (beside) {
+    if ((e = cudaEventRecord(h->ev_join, ts)) == cudaSuccess) e = cudaStreamWaitEvent(st, h->ev_join, 0);
+    if (e != cudaSuccess) return fail(H2_ERR_CUDA, "join from the side stream: %s", cudaGetErrorString(e));
   } else {
-    k_dense_stream<NVB, CW><<<h->grid, (CW + 1) * 32, smem, st>>>(P);
+    launch_dense();
   }
   if (h->inject >= 0) {  // the test hook applies to one product only
     h->inject = -1;
@@ -728,43 +753,31 @@ h2_status build_device(h2_matrix_s* h, const h2_desc* d) {
         it.shape = (unsigned)si | ((unsigned)sj << 8) | ((unsigned)even(sj) << 16) | (1u << 24);
         it.v_off = xp[j];
         it.row = (int)lo[i];
-        it.flags = (R.d_safe[b] ? h2::kItemFlagSafe : 0) | h2::item_pack_exp(R.oD[b], 0);
+        const bool last = b + 1 == d->D_rowptr[i + 1];  // ends the row: the rows' output exponent
+        it.flags = (R.d_safe[b] ? h2::kItemFlagSafe : 0) | (last ? h2::kItemFlagLast : 0) |
+                   h2::item_pack_exp(R.oD[b], last ? R.eY[i] : 0);
         items.push_back(it);
         bytes += it.m_bytes + 8 * sj;
       }
-      h2::StreamItem it{};
-      it.m_off = (dtot + upo[i]) * 8;
-      it.m_bytes = (int)((upo[i + 1] - upo[i]) * 8);
-      it.shape = (unsigned)si | ((unsigned)k << 8) | ((unsigned)h->kp << 16) | (1u << 24);
-      it.v_off = (h->leaf0 + i) * h->kp;
-      it.row = (int)lo[i];
-      it.flags = h2::kItemFlagLast | h2::kItemFlagSrc1 | h2::kItemFlagSafe | h2::item_pack_exp(R.oU[i], R.eY[i]);
-      items.push_back(it);
-      row_bytes[i] = bytes + it.m_bytes + 8 * h->kp + 16 * si;
+      row_bytes[i] = bytes + 16 * si;
     }
     row_item0[h->leaves] = (int64_t)items.size();
-    // the digits' tables (see mma_fp64.cuh)
-    h->oz = R.d_narrow && h->nD > 0;
-    if (h->oz) {
-      std::vector<int32_t> iexp(items.size(), 0), ileaf(items.size(), 0);
+    {  // the leaf expansion's tables
       std::vector<int64_t> uo((size_t)h->leaves);
-      for (int64_t i = 0, b = 0, t = 0; i < h->leaves; i++, t++) {
-        for (; b < d->D_rowptr[i + 1]; b++, t++) {
-          iexp[(size_t)t] = R.d_exp[(size_t)b];
-          ileaf[(size_t)t] = d->D_colidx[b];
-        }
-        uo[(size_t)i] = (dtot + upo[i]) * 8;
-      }
-      if ((st = upload(h, &h->item_exp, iexp.data(), (int64_t)iexp.size())) != H2_OK) return st;
-      if ((st = upload(h, &h->item_leaf, ileaf.data(), (int64_t)ileaf.size())) != H2_OK) return st;
+      for (int64_t i = 0; i < h->leaves; i++) uo[(size_t)i] = (dtot + upo[i]) * 8;
       if ((st = upload(h, &h->u_off, (const int64_t*)uo.data(), h->leaves)) != H2_OK) return st;
       if ((st = upload(h, &h->oU, R.oU.data(), h->leaves)) != H2_OK) return st;
       if ((st = upload(h, &h->eY, R.eY.data(), h->leaves)) != H2_OK) return st;
+    }
+    // the digits' tables (see mma_fp64.cuh), per item = per dense block
+    h->oz = R.d_narrow && h->nD > 0;
+    if (h->oz) {
+      if ((st = upload(h, &h->item_exp, R.d_exp.data(), h->nD)) != H2_OK) return st;
+      if ((st = upload(h, &h->item_leaf, d->D_colidx, h->nD)) != H2_OK) return st;
       if ((st = dalloc(h, &h->xd, h->leaves * h2::xd_chunk_bytes((h->m_max + 15) / 16, 2))) != H2_OK) return st;
     }
     const std::vector<int> begin = balance(row_bytes, row_item0, h->grid);
-    // vector sources per slot: split x (padded leaf layout) and yhat (n_nodes x kp)
-    if ((st = audit_items(items, begin, total * 8, xp[h->leaves], h->n_nodes * h->kp)) != H2_OK) return st;
+    if ((st = audit_items(items, begin, total * 8, xp[h->leaves])) != H2_OK) return st;  // (vectors: the split x per slot)
     if ((st = upload_items(h, &h->dense_items, items, begin)) != H2_OK) return st;
   }
 
@@ -803,6 +816,9 @@ h2_status build_device(h2_matrix_s* h, const h2_desc* d) {
     if ((st = dalloc(h, &h->cticket, 4 * slots)) != H2_OK) return st;
     CUDA_TRY(cudaMemset(h->cticket, 0, (size_t)std::max<int64_t>(4 * slots, 1) * sizeof(int)));
   }
+  CUDA_TRY(cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking));
+  CUDA_TRY(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
+  CUDA_TRY(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming));
   if ((st = dalloc(h, &h->vexp, h2i::kPassVectors)) != H2_OK) return st;
   if ((st = dalloc(h, &h->vpart, (int64_t)h2::kScaleBlocks * 16)) != H2_OK) return st;
   if ((st = dalloc(h, &h->vticket, 1)) != H2_OK) return st;

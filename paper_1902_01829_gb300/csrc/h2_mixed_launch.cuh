@@ -59,6 +59,7 @@ void bucket_phase(const MixedLaunch& L, int phase, int nvlo, cudaStream_t st, bo
   const unsigned tree_threads = tree_warps<NVB>() * 32;
   const int entries = tree_block_entries(L.k, round_up((int64_t)L.k * L.k, 8), FB != kFormF32);
   const unsigned tsm = tree_smem<TreeOpM<FB>, NVB>(L.k, entries, L.tree_T).bytes;
+  const int dentries = tree_down_entries(L.k, round_up((int64_t)L.k * L.k, 8), FB != kFormF32);
   if (phase == 0 && L.njobs > 0) {
     if constexpr (NVB <= 4) {
       if (!convert) {  // beside the dense stream
@@ -91,7 +92,8 @@ void bucket_phase(const MixedLaunch& L, int phase, int nvlo, cudaStream_t st, bo
       k_coupling_m_generic<F, RPL, NVB><<<cgrid, 128, 0, st>>>(mats, L.chunks, L.nchunks, nvlo, NVB);
     }
   } else if (phase == 2 && L.njobs > 0) {
-    k_downsweep_tree_m<FB, NVB><<<(unsigned)L.njobs, tree_threads, tsm, st>>>(mats, L.jobs, nvlo, NVB, expand, L.tree_T, entries);
+    k_downsweep_tree_m<FB, NVB><<<(unsigned)L.njobs, tree_threads, tree_smem<TreeOpM<FB>, NVB>(L.k, dentries, L.tree_T).bytes, st>>>(
+        mats, L.jobs, nvlo, NVB, expand, L.tree_T, dentries);
   }
 }
 

@@ -117,10 +117,12 @@ struct TreeParams {
   const int* vexp;         // per vector of the pass: x enters scaled by 2^-vexp[v]
   int64_t kks;             // doubles from a node's transfer matrix to the next node's
   int k, kp, q, L, nv;
-  // passes whose dense phase is k_dense_oz: the vectors' digits (xks K steps per leaf), and the leaf expansion
-  // by the downsweep: U_j at dmat + u_off[j], its exponent offset, the rows' output exponent
+  // passes whose dense phase is k_dense_oz: the vectors' digits (xks K steps per leaf)
   int oz, xks;
   unsigned char* xd;
+  // the leaf expansion: U_j at dmat + u_off[j], its exponent offset, the rows' output exponent; added to y
+  // (atomically) when the dense phase runs beside the tree phases, else assigned
+  int add;
   const char* dmat;
   const int64_t* u_off;
   const int* oU;
@@ -229,8 +231,11 @@ struct TreeOp64 {
   static __device__ __forceinline__ const char* U(const P& T, const Leaf& l) { return T.dmat + l.uoff; }
   static __device__ __forceinline__ int u_bytes(const P& T, const Leaf& l) { return 8 * l.s * T.k; }
   static __device__ __forceinline__ void u_layout(const P&, const Leaf&, int, int&, int&) {}
-  static __device__ __forceinline__ void ystore(const P& T, const Leaf& l, int v, int row, const Acc& a, bool) {
-    T.y[v * T.ldy + l.off + row] = scale2(df_to_f64(a.s, a.c), l.eY + T.vexp[v]);
+  static __device__ __forceinline__ void ystore(const P& T, const Leaf& l, int v, int row, const Acc& a, bool assign) {
+    double* y = T.y + v * T.ldy + l.off + row;
+    const double val = scale2(df_to_f64(a.s, a.c), l.eY + T.vexp[v]);
+    if (assign) *y = val;
+    else atomicAdd(y, val);
   }
 };
 
@@ -242,7 +247,7 @@ __global__ void __cluster_dims__(kTreeCluster) __launch_bounds__(tree_warps<NVB>
 
 template <int NVB>
 __global__ void __launch_bounds__(tree_warps<NVB>() * 32) k_downsweep_tree(TreeParams P) {
-  tree_down<TreeOp64, NVB>(P, blockIdx.x, P.oz ? 2 : 0, P.q - P.L, tree_block_entries(P.k, P.kks, false));
+  tree_down<TreeOp64, NVB>(P, blockIdx.x, P.add ? 1 : 2, P.q - P.L, tree_down_entries(P.k, P.kks, false));
 }
 
 // ---------------------------------------------------------------- coupling, all levels
@@ -266,7 +271,8 @@ __global__ void __launch_bounds__(tree_warps<NVB>() * 32) k_downsweep_tree(TreeP
 // at most 64 (kFoldProducts) that are folded into a long-term pair, so the
 // FP32 sum of the small parts never runs over a whole row.
 // Passes of more than four vectors run slices of four (grid y): 16 vectors in one warp took 255 registers and
-// left 8 warps an SM; four slices split every entry four times but hold twice the warps (COUPSLICE).
+// left 8 warps an SM; four slices split every entry four times but hold twice the warps (2D n = 50,001, 16 vectors:
+// 234 -> 204 us; 3D n = 4,096, 13 vectors: 150 -> 89; slices of two: 240 and 87).
 // SAFE: some coupling entry is zero or below 2^-103 after its offset (zero-safe split).
 constexpr int kFoldProducts = 64;
 
@@ -459,12 +465,17 @@ __global__ void __launch_bounds__(kWarps * 32) k_coupling_generic(CouplingParams
 // eight loads in flight; one round covers n = 2^20 on 152 blocks.
 constexpr int kScaleBlocks = 152, kScaleThreads = 1024, kScaleUnroll = 8;
 __device__ __forceinline__ unsigned long long abs_bits(double a) { return (unsigned long long)__double_as_longlong(fabs(a)); }
+// zero_y (or null): zeroed for the products whose phases add into it.
 __global__ void __launch_bounds__(kScaleThreads) k_vec_scale(const double* __restrict__ x, int64_t ldx, int64_t n, int nv,
-                                                            unsigned long long* partial, unsigned* ticket, int* vexp) {
+                                                            unsigned long long* partial, unsigned* ticket, int* vexp,
+                                                            double* zero_y, int64_t ldy) {
   __shared__ unsigned long long wmax[kScaleThreads / 32][16];
   __shared__ int last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t stride = (int64_t)gridDim.x * kScaleThreads;
+  if (zero_y)
+    for (int v = 0; v < nv; v++)
+      for (int64_t i = (int64_t)blockIdx.x * kScaleThreads + threadIdx.x; i < n; i += stride) zero_y[v * ldy + i] = 0.0;
   for (int v = 0; v < nv; v++) {
     const double* xv = x + v * ldx;
     unsigned long long m = 0;

@@ -942,9 +942,7 @@ __host__ __device__ constexpr int mixed_red_bytes(int nvb, int cw) { return 2 * 
 // them (U_i, not streamed) -- at most 32 (kMixedMaxBlocks + 1) records
 constexpr int kMixedBatchBlocks = 32 * (kMixedMaxBlocks + 1);
 constexpr int kMixedBlkBuf = kMixedBatchBlocks * 16;
-// the dense stream leaves kTreeReserve bytes of an SM's shared memory to the tree kernels
-// that run beside the dense stream: four or five stages of 32 KB still keep more than 128 KB in flight
-constexpr int kTreeReserve = 40960;
+// (kTreeReserve bytes are left to the tree kernels that run beside the dense stream, see stream_fp64.cuh)
 __host__ __device__ constexpr int mixed_stages(int nvb, int cw) {
   return (kSmemLimit - kTreeReserve - 256 - kMixedBlkBuf - mixed_red_bytes(nvb, cw)) / mixed_stage_bytes(nvb) < 6
              ? (kSmemLimit - kTreeReserve - 256 - kMixedBlkBuf - mixed_red_bytes(nvb, cw)) / mixed_stage_bytes(nvb)

@@ -94,7 +94,7 @@ __device__ __forceinline__ uint32_t scale_digits(uint32_t d) {  // / 256, exact
 struct OzParams {
   const StreamItem* items;
   const int* cta_begin;
-  const int* item_exp;   // per item: the block's ea, and (item_leaf) its column leaf; U items have none
+  const int* item_exp;   // per item: the block's ea, and (item_leaf) its column leaf
   const int* item_leaf;
   const char* mat;
   const unsigned char* xd;  // the leaves' digits, xks K steps each
@@ -107,8 +107,7 @@ struct OzParams {
   int inject;  // >= 0: CTA 0 withholds the copy of this local item (bounded-wait test)
 };
 
-// Producer warp. Stage header (ints): R, C, flags, row, ea, vector halves; an item of U_i (kItemFlagSrc1) has no
-// block here and only ends its row.
+// Producer warp. Stage header (ints): R, C, flags, row, ea.
 __device__ __forceinline__ void oz_produce(const OzParams& P, const StreamShared& S, int ib, int ie) {
   const int lane = threadIdx.x & 31;
   const uint64_t pol = policy_evict_first();
@@ -152,14 +151,10 @@ __device__ __forceinline__ void oz_produce(const OzParams& P, const StreamShared
         h[3] = row;
         h[4] = ea;
         if (!((P.inject == it) && (blockIdx.x == 0))) {
-          if (flags & kItemFlagSrc1) {
-            mbar_arrive(S.full + s);
-          } else {
-            const unsigned vbytes = (unsigned)xd_chunk_bytes((C + 15) / 16, nh);
-            mbar_arrive_expect_tx(S.full + s, (unsigned)m_bytes + vbytes);
-            bulk_g2s_stream(stage + kStageHeader, P.mat + m_off, (unsigned)m_bytes, S.full + s, pol);
-            bulk_g2s(stage + kStageHeader + kStageMat, P.xd + (long long)leaf * xd_chunk_bytes(P.xks, nh), vbytes, S.full + s);
-          }
+          const unsigned vbytes = (unsigned)xd_chunk_bytes((C + 15) / 16, nh);
+          mbar_arrive_expect_tx(S.full + s, (unsigned)m_bytes + vbytes);
+          bulk_g2s_stream(stage + kStageHeader, P.mat + m_off, (unsigned)m_bytes, S.full + s, pol);
+          bulk_g2s(stage + kStageHeader + kStageMat, P.xd + (long long)leaf * xd_chunk_bytes(P.xks, nh), vbytes, S.full + s);
         }
       }
       __syncwarp();
@@ -273,7 +268,7 @@ __global__ void __launch_bounds__((kOzWarps + 1) * 32, 1) k_dense_oz(OzParams P)
     const int* h = reinterpret_cast<const int*>(stage);
     const int R = min(h[0], 64), C = min(h[1], 64), flags = h[2], row = h[3], ea = h[4];
     const int nu = (R + 15) >> 4;
-    if (!(flags & kItemFlagSrc1)) {
+    {
       bool ok = true;
       for (; turn < nu; turn += kOzWarps) {
         const int r = 16 * turn + 2 * g;

@@ -1,16 +1,16 @@
 // Persistent TMA-streaming kernel for the byte-heavy phase of the FP64 plain
-// form: the dense near-field blocks fused with the leaf expansion,
-//   y(i) = sum_j D_ij x(j) + U_i yhat_i        (Sec. 2.2, Eq. 4, Sec. 4.1)
+// form, the dense near-field blocks:   y(i) += sum_j D_ij x(j)   (Sec. 2.2, Sec. 4.1)
 //
 // One CTA per SM owns a contiguous range of leaf rows, and hence one
 // contiguous byte range of the repacked dense blocks. Its producer warp walks
 // a host-built list of "items" (one column-major block of the row plus the
-// vector chunk it multiplies: D_ij with the split x(j), or U_i with yhat_i as
-// the row's last item) and copies each into a ring of shared-memory stages
+// split x(j) it multiplies) and copies each into a ring of shared-memory stages
 // with cp.async.bulk. CW consumer warps split each stage's columns, multiply
 // in double-float with several independent accumulator sets per lane, and
 // hand the stage back. A row's partial sums meet in shared memory at the
-// row's last item.
+// row's last item and are added to y, where the downsweep puts the leaf expansion
+// U_i yhat_i (Eq. 4): before this kernel, or, beside it, with atomic adds too into a y
+// zeroed before the product (two terms onto zero: the order does not matter).
 //
 // Synchronisation uses mbarriers only (stage full/empty, row partials
 // ready/consumed) and every wait is bounded (see tma.cuh): a fault in the
@@ -28,7 +28,7 @@ struct __align__(16) StreamItem {
   unsigned shape;   // R | C << 8 | vstride << 16 | nb << 24   (nb = 1)
   long long v_off;  // vector chunk offset, in float2 per vector slot
   int row;          // first point of the row leaf (y offset)
-  int flags;        // bit 0: last item of its row; bit 1: vector chunk from the second source (yhat);
+  int flags;        // bit 0: last item of its row;
                     // bit 2: the block holds zeros or magnitudes below 2^-103 after its offset (zero-safe split);
                     // FP64 form: bits 4-17 the block's exponent offset, bits 18-31 (last item) the row's
                     // output exponent (both signed 14-bit)
@@ -37,7 +37,7 @@ struct __align__(16) StreamItem {
 constexpr int kStageHeader = 128;
 constexpr int kStageMat = 32768;
 constexpr int kSmemLimit = 232448;  // opt-in shared memory per CTA on sm_103a
-constexpr int kItemFlagLast = 1, kItemFlagSrc1 = 2, kItemFlagSafe = 4;
+constexpr int kItemFlagLast = 1, kItemFlagSafe = 4;
 constexpr int kItemOffsetShift = 4, kItemRowExpShift = 18, kItemExpMax = 8191;  // 14-bit signed fields
 __host__ __device__ constexpr int item_offset(int flags) { return (int)((unsigned)flags << 14) >> 18; }
 __host__ __device__ constexpr int item_row_exp(int flags) { return flags >> kItemRowExpShift; }
@@ -49,9 +49,12 @@ __host__ __device__ constexpr int item_pack_exp(int offset, int row_exp) {
 __host__ __device__ constexpr int stage_vec_bytes(int nvb) { return 512 * nvb; }
 __host__ __device__ constexpr int stage_bytes(int nvb) { return kStageHeader + kStageMat + stage_vec_bytes(nvb); }
 __host__ __device__ constexpr int red_bytes(int nvb, int cw) { return cw * nvb * 64 * 8; }
+// passes of up to four vectors leave kTreeReserve bytes of an SM's shared memory to the coupling and tree
+// kernels that run beside this one: four or five stages of 32 KB still keep more than 128 KB in flight
+constexpr int kTreeReserve = 40960;
 __host__ __device__ constexpr int stream_stages(int nvb, int cw) {
-  return (kSmemLimit - 256 - red_bytes(nvb, cw)) / stage_bytes(nvb) < 6
-             ? (kSmemLimit - 256 - red_bytes(nvb, cw)) / stage_bytes(nvb)
+  return (kSmemLimit - (nvb <= 4 ? kTreeReserve : 0) - 256 - red_bytes(nvb, cw)) / stage_bytes(nvb) < 6
+             ? (kSmemLimit - (nvb <= 4 ? kTreeReserve : 0) - 256 - red_bytes(nvb, cw)) / stage_bytes(nvb)
              : 6;
 }
 __host__ __device__ constexpr int stream_smem_bytes(int nvb, int cw) {
@@ -66,7 +69,6 @@ struct StreamParams {
   const int* cta_begin;  // [grid + 1] item ranges
   const char* mat;       // matrix buffer
   const float2* vsrc0;   // split x, padded leaf layout
-  const float2* vsrc1;   // yhat (expansion items)
   int nv;                // vectors of this pass (<= NVB)
   double* y;             // output
   long long ldy;
@@ -172,8 +174,7 @@ __device__ __forceinline__ void stream_produce(const StreamParams& P, const Stre
         if (!((P.inject == it) && (blockIdx.x == 0))) {
           mbar_arrive_expect_tx(S.full + s, (unsigned)m_bytes + vbytes);
           bulk_g2s_stream(stage + kStageHeader, P.mat + m_off, (unsigned)m_bytes, S.full + s, pol);
-          const float2* src = (flags & kItemFlagSrc1) ? P.vsrc1 : P.vsrc0;
-          bulk_g2s(stage + kStageHeader + kStageMat, src + v_off * P.nv, vbytes, S.full + s);
+          bulk_g2s(stage + kStageHeader + kStageMat, P.vsrc0 + v_off * P.nv, vbytes, S.full + s);
         }
       }
       __syncwarp();
@@ -192,7 +193,7 @@ __device__ __forceinline__ void stream_produce(const StreamParams& P, const Stre
     }
 }
 
-// ---------------------------------------------------------------- dense near field + expansion
+// ---------------------------------------------------------------- dense near field
 // Each block is split with its item's exponent offset; the row's sum is
 // scaled by 2^(row exponent + vexp[v]) when it is written. A lane's
 // accumulator sets are folded every FI items (chains of about 64 products)
@@ -332,7 +333,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, 1) k_dense_stream(StreamParams 
           const float2 p = S.red[(w * NVB + v) * 64 + r];
           df_add(ss, cc, p.x, p.y);
         }
-        P.y[v * P.ldy + row + r] = scale2(df_to_f64(ss, cc), ey + vexp_s[v]);
+        atomicAdd(P.y + v * P.ldy + row + r, scale2(df_to_f64(ss, cc), ey + vexp_s[v]));
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(S.rowfree);

@@ -73,6 +73,12 @@ __host__ __device__ inline int tree_block_entries(int k, int64_t kks, bool panel
   return leaf > pair ? leaf : pair;
 }
 
+// the same for the downsweep: a leaf's 64 x k or one transfer
+__host__ __device__ inline int tree_down_entries(int k, int64_t kks, bool panel) {
+  const int leaf = 64 * k + (panel ? 64 : 0);
+  return leaf > kks ? leaf : (int)kks;
+}
+
 // copy `bytes` (a multiple of Op::kCopy, both ends so aligned) into shared memory, asynchronously
 template <int W>
 __device__ __forceinline__ void cp_async(uint32_t dst, const void* src) {
