@@ -260,13 +260,13 @@ __global__ void __launch_bounds__(256) k_gen_dense(GenDense a) {
     for (int w = 1; w < 8; w++) m = fmax(m, wmax[w]);
     const float sigma = F == h2::kFormInt16 ? (float)(m / 32767.0) : (float)m;
     uint16_t* dst = reinterpret_cast<uint16_t*>(a.dmat + a.bbyte[t]);
-    const int ps2 = h2::panel_stride(sj) / 2;
+    const int ps2 = h2::panel_stride(sj) / 2, cs = h2::code_stride(si);
 #pragma unroll
     for (int u = 0; u < 16; u++) {
       const int e = threadIdx.x + 256 * u;
       if (e < si * sj) {
         const int r = e % si, c = e / si;
-        dst[a.panel ? (r >> 3) * ps2 + 8 * c + (r & 7) : r + si * c] = gen_code<F>(v[u], sigma);
+        dst[a.panel ? (r >> 3) * ps2 + 8 * c + (r & 7) : r + cs * c] = gen_code<F>(v[u], sigma);
       }
     }
     if (threadIdx.x == 0) a.blk[a.bglob[t]].scale = sigma;
@@ -638,7 +638,7 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
       for (; b < d->D_rowptr[i + 1]; b++) {
         const int64_t sj = lo[d->D_colidx[b] + 1] - lo[d->D_colidx[b]], sz = si * sj;
         doff[b + 1] = doff[b] + sz;
-        boff[b + i + 1] = boff[b + i] + (panel ? h2::panel_block_bytes((int)sj) : round_up(sz * 2, 16));
+        boff[b + i + 1] = boff[b + i] + (panel ? h2::panel_block_bytes((int)sj) : round_up(h2::code_stride((int)si) * sj * 2, 16));
       }
       boff[b + i + 1] = boff[b + i] + (panel ? h2::panel_block_bytes(k) : round_up(si * k * ubytes, 16));  // U_i
     }
@@ -678,7 +678,10 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
             m.scale = quantize(d->D_val + doff[b], si * sj, form, tmp.data());
             to_panels(sj, reinterpret_cast<uint16_t*>(base + boff[g]));
           } else {
-            m.scale = quantize(d->D_val + doff[b], si * sj, form, reinterpret_cast<uint16_t*>(base + boff[g]));
+            uint16_t* dst = reinterpret_cast<uint16_t*>(base + boff[g]);
+            m.scale = quantize(d->D_val + doff[b], si * sj, form, dst);
+            const int64_t cs = h2::code_stride((int)si);  // spread the columns, the last first
+            for (int64_t c = sj - 1; cs != si && c > 0; c--) std::memmove(dst + c * cs, dst + c * si, (size_t)si * 2);
           }
           m.voff = (uint64_t)xp4[j];
           m.leaf = (uint64_t)j;

@@ -89,6 +89,12 @@ __host__ __device__ constexpr int panel_cols(int C) { return (C + 15) & ~15; }
 __host__ __device__ constexpr int panel_stride(int C) { return 16 * panel_cols(C) + kPanelPad; }  // bytes
 __host__ __device__ constexpr int panel_block_bytes(int C) { return 8 * panel_stride(C); }
 
+// Column stride (codes) of a dense block outside the panel layout: rows of more than 32 are padded to a multiple
+// of eight, so that eight rows of a column are one aligned 16-byte load (ragged 33- to 64-point leaves were
+// read code by code: 3D n = 12,952, bf16, two vectors, dense phase 131 us, 86 so; the pad is 6% of the bytes
+// on average). The pad's codes are unspecified, its rows never stored.
+__host__ __device__ constexpr int code_stride(int R) { return R > 32 ? (R + 7) & ~7 : R; }
+
 // The vectors of a leaf as 16-bit parts in the A-fragment order of mma.sync m16n8k16 (k_dense_mma): 16 scale
 // floats (per vector), then per K step of 16 points and half of eight vectors three parts of 256 bytes, lane
 // (g, t)'s entries (vector g + 8 half; points t, t + 4, t + 8, t + 12 as k = 2t, 2t + 1, 2t + 8, 2t + 9) at
@@ -1055,9 +1061,8 @@ __device__ __forceinline__ void mixed_produce(const MixedStreamParams& P, const 
       MixedBlock mb{};
       const long long bi = b0 - bfirst + lane;
       if (lane < nb && bi >= 0 && bi < nbatch) mb = blkbuf[bi];
-      const int esize = (mb.src & 2) ? 4 : 2;
       const int codes = (mb.src & 4) ? panel_block_bytes(mb.cols)                   // padded bytes of this block
-                                     : (R * (int)mb.cols * esize + 15) & ~15;
+                                     : (code_stride(R) * (int)mb.cols * 2 + 15) & ~15;
       int moff = codes;  // inclusive prefix of the blocks' padded byte counts
 #pragma unroll
       for (int d = 1; d < kMixedMaxBlocks; d <<= 1) {
@@ -1218,14 +1223,14 @@ __device__ __forceinline__ void consume_item8(const unsigned char* stage, const 
   const int g = lane & 7, j = lane >> 3;
   for (int t = 0; t < nb; t++) {
     const int4 bh = *reinterpret_cast<const int4*>(hd + 8 + 4 * t);  // cols | flags, vs, matrix offset, scale
-    const bool f32 = (bh.x >> 16) & 1, panel = (bh.x >> 17) & 1;
+    const bool panel = (bh.x >> 17) & 1;
     const int C = min(bh.x & 0xFFFF, 64), vs = min(bh.y, 64);
     const int moff = min(bh.z, kStageMat - 16) & ~15;
     const float scale = __int_as_float(bh.w);
     const int voff = min(hd[kHdVoff + t], VAREA - 16) & ~15;
     const unsigned char* A = stage + kMixedHeader + moff;
     const float* X = reinterpret_cast<const float*>(stage + kMixedHeader + kStageMat + voff);
-    if (!f32 && R == 64 && C == 64 && vs == 64) {
+    if (R == 64 && C == 64 && vs == 64) {
       const int gb = panel ? g * panel_stride(64) : 16 * g;  // bytes: rows 8g .. 8g + 7
       const int cb = panel ? 16 : 128;                        // bytes per column
 #pragma unroll
@@ -1247,27 +1252,25 @@ __device__ __forceinline__ void consume_item8(const unsigned char* stage, const 
           acc[7][v] = fmaf(q3.y, xs, acc[7][v]);
         }
       }
-    } else {
-      // any other block: element (row, col) at 16-bit unit row + R col (column-major) or
-      // (row / 8) (panel stride / 2) + 8 col + row % 8 (panel layout); FP32 entries column-major
-      const uint16_t* A16 = reinterpret_cast<const uint16_t*>(A);
-      const float* A32 = reinterpret_cast<const float*>(A);
-      const int c0 = (C * warp) / CW, c1 = (C * (warp + 1)) / CW;
-      const int ps2 = panel_stride(C) / 2;
-      for (int col = c0 + j; col < c1; col += 4) {
-        float q[8];
-#pragma unroll
-        for (int i = 0; i < 8; i++) {
-          const int row = 8 * g + i;
-          q[i] = 0.f;
-          if (row < R)
-            q[i] = f32 ? A32[row + R * col] : code_to_f<F>(A16[panel ? g * ps2 + 8 * col + i : row + R * col]);
-        }
+    } else if (8 * g < R) {
+      // any other block: the lane's eight rows of a column are 16 bytes (column-major with the padded stride, or
+      // the panel layout); rows past R are not stored
+      const unsigned char* col0 = A + (panel ? g * panel_stride(C) : 16 * g);
+      const int cb = panel ? 16 : 2 * code_stride(R);
+      for (int col = 4 * warp + j; col < C; col += 4 * CW) {
+        const uint4 w = *reinterpret_cast<const uint4*>(col0 + cb * col);
+        const float2 q0 = codes_to_f2<F>(w.x), q1 = codes_to_f2<F>(w.y), q2 = codes_to_f2<F>(w.z), q3 = codes_to_f2<F>(w.w);
 #pragma unroll
         for (int v = 0; v < NV2; v++) {
           const float xs = scale * X[v * vs + col];
-#pragma unroll
-          for (int i = 0; i < 8; i++) acc[i][v] = fmaf(q[i], xs, acc[i][v]);
+          acc[0][v] = fmaf(q0.x, xs, acc[0][v]);
+          acc[1][v] = fmaf(q0.y, xs, acc[1][v]);
+          acc[2][v] = fmaf(q1.x, xs, acc[2][v]);
+          acc[3][v] = fmaf(q1.y, xs, acc[3][v]);
+          acc[4][v] = fmaf(q2.x, xs, acc[4][v]);
+          acc[5][v] = fmaf(q2.y, xs, acc[5][v]);
+          acc[6][v] = fmaf(q3.x, xs, acc[6][v]);
+          acc[7][v] = fmaf(q3.y, xs, acc[7][v]);
         }
       }
     }

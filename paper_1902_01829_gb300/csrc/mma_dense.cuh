@@ -126,7 +126,7 @@ __device__ __forceinline__ void mma_produce(const MixedStreamParams& P, const St
       MixedBlock mb{};
       const long long bi = b0 - bfirst + lane;
       if (lane < nb && bi >= 0 && bi < nbatch) mb = blkbuf[bi];
-      const int codes = (mb.src & 4) ? panel_block_bytes(mb.cols) : (R * (int)mb.cols * 2 + 15) & ~15;
+      const int codes = (mb.src & 4) ? panel_block_bytes(mb.cols) : (code_stride(R) * (int)mb.cols * 2 + 15) & ~15;
       const int vbytes = (lane < nb && nv > 0) ? xp_chunk_bytes((mb.cols + 15) / 16, nh) : 0;
       int moff = codes, voff = vbytes;  // inclusive prefixes of the blocks' bytes
 #pragma unroll
@@ -195,9 +195,10 @@ __device__ __forceinline__ uint32_t lds16(uint32_t addr) {
 // 2t + 1, 2t + 8, 2t + 9 of the fragments here and in the parts (neighbouring lanes read neighbouring columns:
 // with 32 rows half the bank conflicts). Codes at `base`, a column `cb` bytes on (shared-memory addresses); tile i holds row + i. run[i]: vectors g (0, 1) and g + 8
 // (2, 3), the rows of lanes g = 2t and 2t + 1. (Four tiles with two accumulators each fit the registers of 13
-// warps; the halves of a 64-row block go to two warps.) FULL: C is a multiple of 16 and a column's four rows are
-// one aligned 8-byte load; else every code is tested and loaded by itself.
-template <int F, bool FULL>
+// warps; the halves of a 64-row block go to two warps.) LOAD 2: C is a multiple of 16 and a column's four
+// rows are one aligned 8-byte load; 1: the same with the last K step's columns tested (tested in every case, 64-point
+// blocks took 318 us for 301: 2D n = 65,536, 64 vectors); 0: every code is tested and loaded by itself.
+template <int F, int LOAD>
 __device__ __forceinline__ void mma_block(uint32_t base, int cb, uint32_t X, int C, int rows, float scale, int nh,
                                           float (&run)[4][4]) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -217,13 +218,15 @@ __device__ __forceinline__ void mma_block(uint32_t base, int cb, uint32_t X, int
 #pragma unroll
     for (int q = 0; q < 4; q++) {
       w[q][0] = w[q][1] = 0u;
-      if constexpr (FULL) {
-        const uint2 u = lds64(col[q]);
-        w[q][0] = u.x, w[q][1] = u.y;
-      } else if (k0 + t + 4 * q < C) {
+      if (LOAD == 2 || k0 + t + 4 * q < C) {
+        if constexpr (LOAD > 0) {
+          const uint2 u = lds64(col[q]);
+          w[q][0] = u.x, w[q][1] = u.y;
+        } else {
 #pragma unroll
-        for (int i = 0; i < 4; i++)
-          if (i < rows) w[q][i / 2] |= lds16(col[q] + 2 * i) << (16 * (i & 1));
+          for (int i = 0; i < 4; i++)
+            if (i < rows) w[q][i / 2] |= lds16(col[q] + 2 * i) << (16 * (i & 1));
+        }
       }
       col[q] += 16 * cb;
     }
@@ -316,11 +319,13 @@ __global__ void __launch_bounds__((kMmaWarps + 1) * 32, 1) k_dense_mma(MixedStre
         const bool panel = (bh.x >> 17) & 1;
         const uint32_t codes = smem_addr(stage + kMixedHeader) + (min(bh.z, kStageMat - 16) & ~15);
         const uint32_t X = smem_addr(stage + kMixedHeader) + (min(bh.y, kMmaArea - xp_chunk_bytes(1, 1)) & ~15);
-        const int r = two ? 8 * g + 4 * (turn & 1) : 4 * g, cb = panel ? 16 : 2 * R;
+        const int r = two ? 8 * g + 4 * (turn & 1) : 4 * g, cb = panel ? 16 : 2 * code_stride(R);
         // (in the column-major layout the last lanes' rows may lie past R: they read what follows, unused)
         const uint32_t base = codes + (panel ? (r >> 3) * panel_stride(C) + 2 * (r & 7) : 2 * r);
-        if ((C & 15) == 0 && (panel || (R & 3) == 0)) mma_block<F, true>(base, cb, X, C, 4, __int_as_float(bh.w), nh, run);
-        else mma_block<F, false>(base, cb, X, C, R - r, __int_as_float(bh.w), nh, run);
+        const bool wide = panel || (code_stride(R) & 3) == 0;
+        if (wide && (C & 15) == 0) mma_block<F, 2>(base, cb, X, C, 4, __int_as_float(bh.w), nh, run);
+        else if (wide) mma_block<F, 1>(base, cb, X, C, 4, __int_as_float(bh.w), nh, run);
+        else mma_block<F, 0>(base, cb, X, C, R - r, __int_as_float(bh.w), nh, run);
       }
       turn -= nb << two;
     }

@@ -120,3 +120,16 @@ def test_not_finite_entries(h2, form, bad):
     keep = [v for v in range(9) if v != 3]
     assert np.array_equal(y[:, keep], clean[:, keep])
     M.close()
+
+
+@pytest.mark.parametrize("form", ["int16", "fp16", "bf16"])
+@pytest.mark.parametrize("sizes", [SIZES, [33, 39, 40, 41, 55, 57, 63, 64]])
+def test_leaf_sizes_up_to_four_vectors(h2, form, sizes):
+    """The columns of leaves of more than 32 points are padded to eight rows: every remainder, streamed."""
+    A = dense_matrix(sum(sizes), sizes)
+    M = handle(h2, A, form)
+    arrays = quant.dequantized_arrays(A, form)
+    for nv in (1, 2, 4):
+        x = h2gen.vectors(830 + nv, A.n, nv)
+        check(oracle.rel_l2(M.matvec(to_dev(x)).cpu().numpy(), oracle.matvec(A, x, **arrays)), acc_tol(A), (form, nv))
+    M.close()
