@@ -463,7 +463,10 @@ cudaError_t set_pass_smem() {
     // kernels that run beside one another prefer the same (largest) shared part of the L1 / shared memory split
     constexpr int CV = NVB < 4 ? NVB : 4;
     for (const void* f : {(const void*)h2::k_downsweep_tree<NVB>, (const void*)h2::k_dense_stream<NVB, CW>,
-                          (const void*)h2::k_coupling<CV, (CV <= 2 ? 4 : 2), true>, (const void*)h2::k_coupling<CV, (CV <= 2 ? 4 : 2), false>,
+                          (const void*)h2::k_coupling_small<CV, true>, (const void*)h2::k_coupling_small<CV, false>,
+                          (const void*)h2::k_coupling<16, CV, true>, (const void*)h2::k_coupling<16, CV, false>,
+                          (const void*)h2::k_coupling<32, CV, true>, (const void*)h2::k_coupling<32, CV, false>,
+                          (const void*)h2::k_coupling<64, CV, true>, (const void*)h2::k_coupling<64, CV, false>,
                           (const void*)h2::k_coupling_generic<1, CV>, (const void*)h2::k_coupling_generic<2, CV>})
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
@@ -583,9 +586,15 @@ h2_status run_pass(h2_matrix_s* h, int nv, const double* x, int64_t ldx, double*
   constexpr int CV = NVB < 4 ? NVB : 4;  // vectors per CTA
   const dim3 cgrid((unsigned)h->ncsegs, (unsigned)((nv + CV - 1) / CV));
   if (h->pair_rows) {
-    constexpr int CB = CV <= 2 ? 4 : 2;
-    if (h->s_tiny) k_coupling<CV, CB, true><<<cgrid, wb, 0, ts>>>(C);
-    else k_coupling<CV, CB, false><<<cgrid, wb, 0, ts>>>(C);
+    auto launch = [&](auto safe) {
+      constexpr bool SAFE = decltype(safe)::value;
+      if (k == 16) k_coupling<16, CV, SAFE><<<cgrid, wb, 0, ts>>>(C);
+      else if (k == 32) k_coupling<32, CV, SAFE><<<cgrid, wb, 0, ts>>>(C);
+      else if (k == 64) k_coupling<64, CV, SAFE><<<cgrid, wb, 0, ts>>>(C);
+      else k_coupling_small<CV, SAFE><<<cgrid, wb, 0, ts>>>(C);
+    };
+    if (h->s_tiny) launch(std::true_type{});
+    else launch(std::false_type{});
   } else {
     k_coupling_generic<RPL_K, CV><<<cgrid, wb, 0, ts>>>(C);
   }

@@ -259,11 +259,11 @@ __global__ void __launch_bounds__(tree_warps<NVB>() * 32) k_downsweep_tree(TreeP
 // order, so the result does not depend on the order of arrival.
 // What bounds it: HBM at few vectors, as long as enough 16-byte loads are in flight. One warp per
 // row left 3D n = 2^14 (511 rows of up to 150 blocks of 32 KB) with 511 warps on the chip and the
-// longest row as the kernel's time: 972 us against 87 us of HBM time; split as above 180 us.
+// longest row as the kernel's time: 972 us against 87 us of HBM time; split as above 180 us, and 146 as below.
 //
 // k = 2H with H a power of two: lane = g * H + h owns rows 2h, 2h + 1 of every block,
 // read as one 16-byte load per column; column groups g = 0 .. G-1 (G = 32 / H)
-// take columns g, g + G, ... The warp's blocks are walked in batches of CB
+// take a run of columns each (xhat in pairs). The warp's blocks are walked in batches of CB
 // columns per lane, two batches in flight: the next batch's matrix and xhat
 // loads are issued before the current batch is multiplied. Blocks are padded
 // to kkp doubles; Sco[b] = (column node, exponent offset) of block b. Every node row
@@ -335,8 +335,122 @@ __device__ __forceinline__ void coupling_finish(const CouplingParams& P, const C
   }
 }
 
-template <int NVB, int CB, bool SAFE>
+// k = K = 16, 32 or 64: nothing to test, since the lanes' columns fill the block. From K = 32 on the four warps take a
+// quarter of every block's columns each (a block to a warp left them waiting for the one with a block more, a
+// sixth of the kernel's time); at 16 a block is one or two batches, and a warp takes it whole. Bound by issue slots
+// (about 0.6 of them used, 12 operations of each product in double-float): with k known only at run time, a column of
+// 3D n = 2^14 took 80 instructions; phase 180 -> 146 us, n = 10,004 with four vectors 406 -> 256, 2D n = 50,001
+// with 16 vectors 204 -> 150.
+template <int K, int NVB, bool SAFE>
 __global__ void __launch_bounds__(kWarps * 32) k_coupling(CouplingParams P) {
+  constexpr int CB = NVB <= 2 ? 4 : 2, H = K / 2, G = 32 / H, CW = K >= 32 ? K / kWarps : K, CPL = CW / G, NCB = CPL / CB;
+  constexpr int STEP = K >= 32 ? 1 : kWarps;  // from a warp's block to its next
+  constexpr int FB = kFoldProducts / CB;      // batches per chain
+  static_assert(G * H == 32 && CPL * G == CW && NCB * CB == CPL && FB % 2 == 0, "k_coupling: column split");
+  __shared__ float2 red[kWarps][NVB][64];
+  __shared__ int last;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const CouplingSeg sg = P.segs[blockIdx.x];
+  const int v0 = blockIdx.y * NVB, nv = min(P.nv - v0, NVB);  // this CTA's vectors
+  const int g = lane / H, h = lane % H;
+  const int col0 = g * CPL + (K >= 32 ? warp * CW : 0);  // the lane's first column
+  const int first = sg.b0 + (K >= 32 ? 0 : warp), end = sg.b0 + sg.nb;
+  const int nbatch = first < end ? (end - first + STEP - 1) / STEP * NCB : 0;
+  float s[2][NVB], c[2][NVB], S2[2][NVB], C2[2][NVB];
+  acc_zero(s, c);
+  acc_zero(S2, C2);
+  int xo[NVB];  // (a slice's missing vectors repeat its last one; their sums are not stored)
+#pragma unroll
+  for (int v = 0; v < NVB; v++) xo[v] = (v0 + min(v, nv - 1)) * K + col0;
+  // the next batch's place: block b, columns cb CB ..; the block's column node and offset are read a block ahead
+  int b = first, cb = 0;
+  int2 co = nbatch > 0 ? __ldg(P.Sco + b) : make_int2(0, 0), cn = b + STEP < end ? __ldg(P.Sco + b + STEP) : co;
+  const double* A = P.S + (int64_t)b * (K * K) + 2 * h + K * col0;
+  const float2* X = P.xhat + (int64_t)co.x * P.nv * K;
+
+  double2 a0[CB], a1[CB];
+  float4 x0[CB / 2][NVB], x1[CB / 2][NVB];
+  int o0 = 0, o1 = 0;
+  auto load = [&](double2(&a)[CB], float4(&xv)[CB / 2][NVB], int& o) {
+    o = co.y;
+#pragma unroll
+    for (int u = 0; u < CB; u++) a[u] = __ldg(reinterpret_cast<const double2*>(A + K * u));
+#pragma unroll
+    for (int u = 0; u < CB / 2; u++)
+#pragma unroll
+      for (int v = 0; v < NVB; v++) xv[u][v] = __ldg(reinterpret_cast<const float4*>(X + xo[v] + 2 * u));
+    A += K * CB;
+    X += CB;
+    if (++cb == NCB) {
+      cb = 0;
+      b += STEP;
+      A += STEP * K * K - CPL * K;
+      co = cn;
+      if (b + STEP < end) cn = __ldg(P.Sco + b + STEP);
+      X = P.xhat + (int64_t)co.x * P.nv * K;
+    }
+  };
+  auto compute = [&](const double2(&a)[CB], const float4(&xv)[CB / 2][NVB], int o) {
+#pragma unroll
+    for (int u = 0; u < CB; u++) {
+      float h0, l0, h1, l1;
+      if (SAFE) {
+        split_f64(a[u].x, o, h0, l0);
+        split_f64(a[u].y, o, h1, l1);
+      } else {
+        split_f64_fast(a[u].x, o, h0, l0);
+        split_f64_fast(a[u].y, o, h1, l1);
+      }
+#pragma unroll
+      for (int v = 0; v < NVB; v++) {
+        const float4 x = xv[u / 2][v];
+        const float xh = u % 2 ? x.z : x.x, xl = u % 2 ? x.w : x.y;
+        df_fma(s[0][v], c[0][v], h0, l0, xh, xl);
+        df_fma(s[1][v], c[1][v], h1, l1, xh, xl);
+      }
+    }
+  };
+  if (nbatch > 0) load(a0, x0, o0);
+  for (int bt = 0; bt < nbatch; bt += 2) {
+    if (bt + 1 < nbatch) load(a1, x1, o1);
+    compute(a0, x0, o0);
+    if (bt + 2 < nbatch) load(a0, x0, o0);
+    if (bt + 1 < nbatch) compute(a1, x1, o1);
+    if ((bt + 2) % FB == 0) acc_fold(S2, C2, s, c);
+  }
+  acc_fold(S2, C2, s, c);
+#pragma unroll
+  for (int r = 0; r < 2; r++)
+#pragma unroll
+    for (int v = 0; v < NVB; v++) {
+      s[r][v] = S2[r][v];
+      c[r][v] = C2[r][v];
+    }
+  // sum the column groups (lanes h, h + H, ...)
+  for (int off = H; off < 32; off <<= 1) {
+#pragma unroll
+    for (int r = 0; r < 2; r++)
+#pragma unroll
+      for (int v = 0; v < NVB; v++) {
+        const float s2 = __shfl_xor_sync(0xFFFFFFFFu, s[r][v], off);
+        const float c2 = __shfl_xor_sync(0xFFFFFFFFu, c[r][v], off);
+        df_add(s[r][v], c[r][v], s2, c2);
+      }
+  }
+  if (g == 0) {
+#pragma unroll
+    for (int v = 0; v < NVB; v++) {
+      red[warp][v][2 * h] = make_float2(s[0][v], c[0][v]);
+      red[warp][v][2 * h + 1] = make_float2(s[1][v], c[1][v]);
+    }
+  }
+  coupling_finish<NVB>(P, sg, red, &last);
+}
+
+// k = 2, 4 or 8: columns g, g + G, ... with lanes beyond k columns idle; every bound is tested
+template <int NVB, bool SAFE>
+__global__ void __launch_bounds__(kWarps * 32) k_coupling_small(CouplingParams P) {
+  constexpr int CB = NVB <= 2 ? 4 : 2;
   __shared__ float2 red[kWarps][NVB][64];
   __shared__ int last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
