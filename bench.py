@@ -151,27 +151,28 @@ class ClockSampler:
 
 
 # DRAM bytes (read + write) of one dense-stream launch over its algorithmic bytes, from full ncu captures
-# of the 2D n=2^18 workload (FP64, and int16 codes with FP32 bases); the traffic grows with the leaf
-# count, so the ratio carries over to the n=2^20 launch
+# of the 2D n=2^18 workload (FP64 with the leaf bases still in the stream, and int16 codes with FP32
+# bases); the traffic grows with the leaf count, so the ratio carries over to the n=2^20 launch
 TRAFFIC_RATIO = {("fp64", False): 3184266039 / 3178496000, ("int16", True): 794616064 / 788584800}
 TRAFFIC_KERNEL = {("fp64", False): "k_dense_stream", ("int16", True): "k_dense_stream_m"}  # the kernel those counters belong to
 
-# FP32 instructions per double-float product a * x (split entry times split vector entry): the exact
-# product p, e (2), the two cross terms (2), TwoSum of the running sum (6), the small-part sum (2)
-DF_FP32_OPS = 12
-FP32_LANES_PER_SM = 128
+# digit products per product of two FP64 entries in the FP64 form's dense phase at more than four vectors
+# (six 8-bit digits each: the 21 pairs of weight <= 5 and the five of weight 6)
+DIGIT_PAIRS = 26
+# mma.sync FP16 rate of the chip, TFLOP/s (a loop of m16n8k16: 8 cycles each per SM quarter)
+MMA_SYNC_TFLOPS = 600.0
 
 
 def dense_kernel_bytes(info: dict, A, nv: int, storage: str = "fp64", bases_fp32: bool = False) -> int:
-    """Algorithmic bytes of one launch of the dense phase's kernel. FP64 form (D blocks and the fused
-    leaf expansion): D and U once, x read once, y written once (8 bytes), the leaf yhat read once.
-    Precision form on the CUDA cores (D blocks only; the expansion runs in the downsweep): D codes
-    and one 4-byte scale per block, x once (FP32), y written once (8 bytes). Tensor-core pass (D
-    blocks with the fused expansion): D codes and U codes with their scales, x once, y once, yhat."""
+    """Algorithmic bytes of one launch of the dense phase's kernel. The leaf expansion runs in the
+    downsweep, except in the tcgen05 passes. FP64 form: D, x read once, y written once (8 bytes).
+    Precision form: D codes and one 4-byte scale per block, x once (FP32), y written once (8 bytes).
+    tcgen05 pass (D blocks with the fused expansion): D codes and U codes with their scales, x once,
+    y once, yhat."""
     nDval = int(A.D_valoff[-1])
     if storage == "fp64":
-        return 8 * (nDval + A.n * A.k) + 8 * A.n * nv * 2 + 8 * A.leaves * A.k * nv
-    if dense_kernel_name(A, nv, storage, bases_fp32) == "k_dense_stream_m":
+        return 8 * nDval + 8 * A.n * nv * 2
+    if dense_kernel_name(A, nv, storage, bases_fp32) != "k_dense_tc":
         return 2 * nDval + 4 * A.nD + 4 * A.n * nv + 8 * A.n * nv
     u_bytes = 4 if bases_fp32 else 2
     return (2 * nDval + u_bytes * A.n * A.k + 4 * (A.nD + A.leaves) + 4 * A.n * nv + 8 * A.n * nv
@@ -182,17 +183,6 @@ def sm_count(dev) -> int:
     import torch
 
     return int(torch.cuda.get_device_properties(dev).multi_processor_count)
-
-
-def df_peak_products(dev) -> float:
-    """Peak double-float products per second on the FP32 pipes: 128 FP32 lanes per SM x SMs x the
-    measured maximum SM clock / 12 FP32 instructions per product."""
-    p = os.path.join(ROOT, "MEASURED_PEAKS.json")
-    mhz = 2070.0
-    if os.path.exists(p):
-        with open(p) as f:
-            mhz = float(json.load(f).get("sm_max_mhz", mhz))
-    return FP32_LANES_PER_SM * sm_count(dev) * mhz * 1e6 / DF_FP32_OPS
 
 
 FP64_FMA_PER_SM_CYCLE = 2   # GB300: 152 SMs x 2 FP64 FMA per cycle x 2.07 GHz x 2 = 1.26 TFLOP/s (nominal 1.25)
@@ -482,14 +472,15 @@ def construction_line(h2, A, values=("U", "E", "S", "D")) -> dict:
 
 
 def dense_kernel_name(A, nv: int, storage: str, bases_fp32: bool) -> str:
-    """The kernel of the dense phase: the FP64 stream, or in the precision form the tensor-core
-    kernel (16-bit fp16 / bf16 codes and bases, k a multiple of 16, every leaf 64 points, 8 or
-    more vectors) or else the CUDA-core stream."""
+    """The kernel of the dense phase: for up to four vectors the streams; for more, in the FP64 form
+    the digit kernel (unless a dense block spans more than 2^10), in the precision form the tcgen05
+    kernel (16-bit fp16 / bf16 codes and bases, k a multiple of 16, every leaf 64 points, 8 or more
+    vectors) or else the MMA tiles."""
     if storage == "fp64":
-        return "k_dense_stream"
+        return "k_dense_stream" if nv <= 4 else "k_dense_oz"
     panel = (storage in ("fp16", "bf16") and not bases_fp32 and A.k % 16 == 0 and A.k <= 64
              and bool(np.all(np.diff(np.asarray(A.leaf_offset)) == 64)))
-    return "k_dense_tc" if panel and nv >= 8 else "k_dense_stream_m"
+    return "k_dense_tc" if panel and nv >= 8 else "k_dense_stream_m" if nv <= 4 else "k_dense_mma"
 
 
 def run_oracle_baseline(A, x, budget_s: float = 12.0):
@@ -584,12 +575,8 @@ def main():
             dist.barrier()
         torch.cuda.synchronize()
 
-    # The FP64 form runs its phases in order: per-phase events inside the timed region give the dense
-    # kernel's duration live. A scaled form runs its dense phase beside the tree phases (events
-    # between phases would serialize them), so it is timed plain and its phases are timed after.
-    live_phases = args.storage == "fp64"
-    M.profile(live_phases)
-    M.profile_read()
+    # Products of up to four vectors run the dense phase beside the far field (events between phases
+    # would serialize them), so the product is timed plain and its phases are timed after.
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     with ClockSampler(dev.index) as clk:
         barrier()
@@ -598,33 +585,28 @@ def main():
             step()
         e1.record(stream)
         barrier()
-    if live_phases:
-        phase_ms, launches = M.profile_read()
-        M.profile(False)
-    else:
-        M.profile(True)
-        M.profile_read()
-        for _ in range(args.steps):
-            step()
-        phase_ms, launches = M.profile_read()
-        M.profile(False)
+    M.profile(True)
+    M.profile_read()
+    for _ in range(args.steps):
+        step()
+    phase_ms, launches = M.profile_read()
+    M.profile(False)
     ms = max_over_ranks(e0.elapsed_time(e1), dist, dev)
     ms_step = ms / args.steps
     gbs = job_rate(info["paper_bytes"], world, ms_step * 1e-3) / 1e9
     vps = job_rate(nv, world, ms_step * 1e-3)
 
-    # roofline of the dominant kernel (dense blocks + leaf expansion), timed live above
+    # roofline of the dominant kernel (dense blocks)
     dense_ms = phase_ms["dense_expand"] / args.steps
     dbytes = dense_kernel_bytes(info, A, nv, args.storage, args.bases_fp32)
     achieved = dbytes / (dense_ms * 1e-3) / 1e9
     kname = dense_kernel_name(A, nv, args.storage, args.bases_fp32)
-    roofline = {"kernel": kname + " (dense blocks + leaf expansion)", "bound": "hbm", "achieved": round(achieved, 1), "peak": hbm,
+    roofline = {"kernel": kname + (" (dense blocks + leaf expansion)" if kname == "k_dense_tc" else " (dense blocks)"), "bound": "hbm", "achieved": round(achieved, 1), "peak": hbm,
                 "peak_kind": peak_kind, "unit": "GB/s", "frac": round(achieved / hbm, 4),
                 "traffic": (round(TRAFFIC_RATIO[(args.storage, args.bases_fp32)] * dbytes)
                             if (args.storage, args.bases_fp32) in TRAFFIC_RATIO and nv == 1
                             and TRAFFIC_KERNEL[(args.storage, args.bases_fp32)] == kname else None),
-                "duration_source": ("CUDA events between phases inside the timed region" if live_phases else
-                                    "CUDA events between phases, separate run of the same steps"),
+                "duration_source": "CUDA events between phases, separate run of the same steps (phases in order)",
                 "bytes_per_launch": dbytes,
                 "phase_share": {k: round(v / max(sum(phase_ms.values()), 1e-9), 4) for k, v in phase_ms.items()}}
 
@@ -683,8 +665,8 @@ def main():
                        "GBs": round(info["paper_bytes"] * world / (ms16 * 1e-3) / 1e9, 1),
                        "rel_err_vs_oracle": oracle.rel_l2(y16.cpu().numpy(), oracle.matvec(A, x16_np))}
         if args.storage == "fp64":
-            # at 16 vectors the FP64 form's dense phase is bound by double-float arithmetic on the FP32
-            # pipes, not by HBM: products per second of its kernel against that peak
+            # at 16 vectors the FP64 form's dense phase is digit products on the tensor cores: their rate
+            # against that of mma.sync
             M.profile(True)
             M.profile_read()
             for _ in range(steps16):
@@ -692,17 +674,14 @@ def main():
             ph16, _ = M.profile_read()
             M.profile(False)
             d16_ms = ph16["dense_expand"] / steps16
-            prods = 16 * (int(A.D_valoff[-1]) + A.n * A.k)
-            peak = df_peak_products(dev)
-            ach = prods / (d16_ms * 1e-3)
+            flops = 2 * DIGIT_PAIRS * 16 * int(A.D_valoff[-1])
+            ach = flops / (d16_ms * 1e-3) / 1e12
             hbm_frac = dense_kernel_bytes(info, A, 16) / (d16_ms * 1e-3) / 1e9 / hbm
             out["nv16"]["roofline"] = {
-                "kernel": "k_dense_stream (dense blocks + leaf expansion, 16 vectors)", "bound": "alu",
-                "achieved": round(ach / 1e12, 4), "peak": round(peak / 1e12, 4), "unit": "T double-float products/s",
-                "frac": round(ach / peak, 4), "hbm_frac": round(hbm_frac, 4),
-                "peak_derivation": f"{FP32_LANES_PER_SM} FP32 lanes x {sm_count(dev)} SMs x max SM clock / "
-                                   f"{DF_FP32_OPS} FP32 instructions per product",
-                "products_per_launch": prods, "kernel_ms": round(d16_ms, 4)}
+                "kernel": "k_dense_oz (dense blocks, 16 vectors)", "bound": "tensor", "achieved": round(ach, 2),
+                "peak": MMA_SYNC_TFLOPS, "unit": "TFLOP/s of digit products", "frac": round(ach / MMA_SYNC_TFLOPS, 4),
+                "hbm_frac": round(hbm_frac, 4), "peak_derivation": "measured rate of mma.sync m16n8k16 FP16",
+                "flops_per_launch": flops, "kernel_ms": round(d16_ms, 4)}
 
         # precision form (per-block scaled 16-bit S and D; U, V, E, F in FP32 or 16-bit) at several vector counts
         out["mixed"] = mixed_lines(h2, A, info, dev, stream, y_ref, x_np, args.steps, world, rank)

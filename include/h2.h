@@ -206,7 +206,10 @@ h2_status h2_create_generated(const h2_desc* d, const h2_coupling_kernel* kc, co
  * tensor cores (vector operands split into two 16-bit parts, so the result
  * keeps the FP32 accumulation accuracy of the other path). With fp16 or bf16
  * codes and k = 64, such a pass also runs the coupling blocks (Eq. 3) on the
- * tensor cores, whatever the leaves and bases.
+ * tensor cores, whatever the leaves and bases. Other passes of more than four
+ * vectors run the dense blocks on MMA tiles: the scaled forms with the vectors
+ * split into three 16-bit parts, the FP64 form by exact products of 8-bit
+ * digits if no dense block's nonzero entries span more than 2^10.
  * Errors: H2_ERR_INVALID (NULL, nv < 1, ld < n), H2_ERR_CUDA (launch failed).
  */
 h2_status h2_matvec(h2_handle h, int32_t nv, const double* x, int64_t ldx, double* y, int64_t ldy, void* stream);
@@ -264,9 +267,10 @@ h2_status h2_info(h2_handle h, int64_t info[8]);
  * phases; h2_profile_read waits for the last recorded event, returns the
  * summed milliseconds of each phase since profiling was enabled (or last
  * read), the number of kernel launches, and starts a new sum.
- * Phases: 0 leaf projection + upsweep, 1 coupling, 2 downsweep,
- * 3 dense blocks + leaf expansion. Disabled by default; enabling costs one
- * event record per phase boundary.
+ * Phases: 0 leaf projection + upsweep, 1 coupling, 2 downsweep + leaf
+ * expansion, 3 dense blocks (with the expansion in passes of 8 or more vectors
+ * on panel-layout handles). Disabled by default; enabling costs one event
+ * record per phase boundary and keeps the phases in order.
  */
 #define H2_NPHASES 4
 h2_status h2_profile(h2_handle h, int32_t enable);
@@ -319,7 +323,8 @@ h2_status h2_matvec_static_check(void* stream);
  * product y = A^H x with each candidate configuration (one warm-up and three
  * timed products, CUDA events on `stream`) and keeps the fastest for later
  * calls on this handle:
- *   dense consumer warps:   8 or 16 (16 only for passes of at most 8 vectors)
+ *   dense consumer warps:   8 or 16 (they matter in passes of up to four vectors;
+ *                           16 only for passes of at most 8 vectors)
  *   coupling row chunks:    about 64, 128 or 256 coupling blocks per warp
  *   tree jobs:              subtrees at the default level (2^L >= twice the SMs)
  *                           or one or two levels higher (fewer, larger subtrees)
