@@ -361,10 +361,11 @@ std::vector<int4> coupling_chunks(const int32_t* Srow, int64_t n_nodes, int64_t 
   return out;
 }
 
-// the tree jobs of matrix `mat` with subtrees at level L: one CTA each, filled up to whole clusters
+// the tree jobs of matrix `mat` with subtrees at level L: one CTA each, filled up to whole clusters (fewer
+// subtrees than a cluster's CTAs lie tree_spread apart)
 void tree_jobs(int mat, int L, std::vector<int2>* jobs) {
-  const int n = 1 << L;
-  for (int t = 0; t < std::max(n, h2::kTreeCluster); t++) jobs->push_back(make_int2(mat, t < n ? t : -1));
+  const int spread = h2::tree_spread(L);
+  for (int t = 0; t < 1 << (L + spread); t++) jobs->push_back(make_int2(mat, (t & ((1 << spread) - 1)) ? -1 : t >> spread));
 }
 
 h2_status mixed_configure(h2_matrix_s* h, int chunk_opt, int cw, int tree_opt) {

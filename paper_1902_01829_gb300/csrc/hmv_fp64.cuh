@@ -241,8 +241,9 @@ struct TreeOp64 {
 
 template <int NVB>
 __global__ void __cluster_dims__(kTreeCluster) __launch_bounds__(tree_warps<NVB>() * 32) k_upsweep_tree(TreeParams P) {
-  const bool active = (int64_t)blockIdx.x < ((int64_t)1 << P.L);
-  tree_up<TreeOp64, NVB, true>(P, active ? blockIdx.x : 0, active, true, P.q - P.L, tree_block_entries(P.k, P.kks, false));
+  const int spread = tree_spread(P.L);
+  const bool active = (blockIdx.x & ((1 << spread) - 1)) == 0;
+  tree_up<TreeOp64, NVB, true>(P, active ? blockIdx.x >> spread : 0, active, true, P.q - P.L, tree_block_entries(P.k, P.kks, false));
 }
 
 template <int NVB>

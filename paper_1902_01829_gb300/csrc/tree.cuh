@@ -34,6 +34,10 @@ namespace cg = cooperative_groups;
 
 constexpr int kTreeClusterLog = 3, kTreeCluster = 1 << kTreeClusterLog;  // CTAs (subtrees) per cluster of the upsweep
 
+// With fewer subtrees (2^L) than a cluster has CTAs, subtree s is on rank s << tree_spread(L): a level of nn
+// nodes is climbed on ranks 0, 8 / nn, ..., the subtrees' roots like the levels above them.
+__host__ __device__ constexpr int tree_spread(int L) { return L < kTreeClusterLog ? kTreeClusterLog - L : 0; }
+
 // warps per CTA: a step has (rows / 8) x (vectors / 4) tasks of a warp
 template <int NVB>
 __host__ __device__ constexpr int tree_warps() { return NVB >= 4 ? 8 : 4; }
@@ -151,7 +155,8 @@ __device__ __forceinline__ typename Op::Acc tree_pick(const typename Op::Acc (&a
 }
 
 // Leaf projection and the whole upsweep (Alg. 2, Eq. 2) of subtree `sub` (active: this CTA has one; a CTA
-// without passes its cluster's first subtree and takes part in the barriers only). The subtree's steps
+// without passes its cluster's first subtree and takes part in the barriers only). Subtrees are on the
+// clusters' ranks in order, eight to a cluster (fewer in all: tree_spread). The subtree's steps
 // follow a binary counter: leaf, leaf, their parent, leaf, ... convert: x(j) is copied into the product's
 // own layout and type here (else a kernel before this one did it).
 // CLUSTER false: the CTA climbs alone, with a ticket per level. A cluster needs room on eight SMs of a GPC at
