@@ -141,6 +141,7 @@ struct MixedData {
   float4* kf_chi = nullptr;      // coupling from the kernel: node centres (FP32 high parts, x y z 0)
   float4* kf_clo = nullptr;      // and their low parts
   float4* kf_off = nullptr;      // [node][k] offsets of the interpolation points from the centre
+  float kf_scale = 1.f;          // a distance of those points times this is the kernel's argument
   int4* tc_brec = nullptr;       // and the builders' records of those items
   bool spanel = false;           // coupling codes in the panel layout, unpadded (fp16 / bf16, k = 64)
   float smax = 0.f;              // largest coupling block scale

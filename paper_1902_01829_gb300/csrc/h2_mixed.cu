@@ -152,6 +152,7 @@ h2::MatDesc fill_desc(const h2_matrix_s* h, int tree_L) {
   D.kf_chi = M.kf_chi;
   D.kf_clo = M.kf_clo;
   D.kf_off = M.kf_off;
+  D.kf_scale = M.kf_scale;
   D.spanel = M.spanel ? 1 : 0;
   D.cpart = M.cpart;
   D.xp = M.xp;
@@ -559,10 +560,22 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
     // (Sec. 4.6): per node its centre c (midpoint of its Chebyshev nodes per dimension) as an
     // FP32 pair hi + lo, and its k points as FP32 offsets from c (tensor index, dimension 0
     // slowest), all times `unit`, which makes a distance the kernel's argument (base-2 exponent of
-    // exp(-r / ell), s of the Matern kernel); unused dimensions are 0
+    // exp(-r / ell), s of the Matern kernel); unused dimensions are 0. Where a coordinate times unit
+    // exceeds 2^60 the points are held 2^-m as large (coordinates up to 2^30) and the distance is multiplied by
+    // 2^m: squares stay finite, and the argument too (m <= 95: above that a distance of 2^-63 is 2^32 of
+    // the kernel's argument, K = 0, all the same).
     const h2_coupling_kernel* kc = h->kc;
     const int dim = kc->dim, p = kc->p;
-    const double unit = (kc->kernel == H2_KERNEL_MATERN32 ? 1.7320508075688772 : 1.4426950408889634) / kc->ell;
+    double unit = (kc->kernel == H2_KERNEL_MATERN32 ? 1.7320508075688772 : 1.4426950408889634) / kc->ell;
+    {
+      double ext = 0.0;
+      for (int64_t t = 0; t < nodes * dim * p; t++) ext = std::max(ext, std::fabs(kc->cheb[t]));
+      int e = 0;
+      std::frexp(ext * unit, &e);
+      const int m = e > 60 ? e - 30 : 0;
+      unit = std::ldexp(unit, -m);
+      M.kf_scale = std::ldexp(1.f, std::min(m, 95));
+    }
     std::vector<float4> chi((size_t)nodes), clo((size_t)nodes), off((size_t)(nodes * k));
 #pragma omp parallel for schedule(static)
     for (int64_t n = 0; n < nodes; n++) {

@@ -129,11 +129,12 @@ struct MatDesc {
   long long kk8, n_nodes;
   int k, kp, LR, q, L;
   int spanel;            // k = 64: coupling codes in the panel layout (8 panels of 8 rows, 1024 bytes apart)
-  // coupling blocks from the kernel (k_coupling_kf), lengths in units of the kernel's argument
-  // (kf_unit): node centres as FP32 high and low parts, the interpolation points' offsets from them
+  // coupling blocks from the kernel (k_coupling_kf): node centres as FP32 high and low parts, the interpolation
+  // points' offsets from them; a distance in their units times kf_scale is the kernel's argument
   const float4* kf_chi;
   const float4* kf_clo;
   const float4* kf_off;
+  float kf_scale;
   // split coupling rows: partial sums [slot][v][kp] and a counter per (row's first slot, vector slice)
   float* cpart;
   int* cticket;
@@ -788,17 +789,19 @@ __global__ void __launch_bounds__(128) k_coupling_m_generic(const MatDesc* __res
 // each lane all k columns of its group's block in runs of four, so a vector's four entries are one
 // float4 read. A row's sums are reduced over the groups once, after its last block. Each group
 // stages its block's column points and vectors in the warp's shared memory. The points are stored
-// scaled (kf_unit: log2(e) / ell, or sqrt(3) / ell for Matern), so that a value is one distance
-// t = r2 * rsqrt(r2) and 2^-t, or (1 + t) 2^(-t log2 e): nine instructions, two of them on the
-// special-function unit, and one FMA per vector.
+// scaled (by log2(e) / ell, or sqrt(3) / ell for Matern), so that a value is one distance
+// t = kf_scale sqrt(r2) and 2^-t, or (1 + t) 2^(-t log2 e): nine instructions, two of them on the
+// special-function unit, and one FMA per vector. kf_scale is 1 unless some coordinate in those units exceeds 2^60
+// (mixed_build: the points are then held 2^-m as large and kf_scale is 2^m), so r2 stays finite for any points and
+// ell; an r2 that underflows gives t = 0, K = 1, as t below 2^-63 does.
 // What bounds it: issue slots (3D n = 2^16, 8 vectors, 4.65e8 values: 28 instructions a value before
 // the scaling moved to the points and the vector loop lost its per-vector branches; with the finer
 // row split of coupling_chunks 900 -> 441 us).
-// 2^x and 1 / sqrt(x) by the special-function unit (PTX approx: relative errors of a few 2^-23; no
-// argument here is subnormal, so flushing those to zero changes nothing)
-__device__ __forceinline__ float rsqrt_approx(float x) {
+// 2^x and sqrt(x) by the special-function unit (PTX approx: relative errors of a few 2^-23; subnormals count as
+// zero, sqrt(0) = 0)
+__device__ __forceinline__ float sqrt_approx(float x) {
   float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -829,6 +832,7 @@ __global__ void __launch_bounds__(128, RPL == 1 ? 6 : 4) k_coupling_kf(const Mat
   const float4* __restrict__ chi = D.kf_chi;
   const float4* __restrict__ clo = D.kf_clo;
   const float4* __restrict__ off = D.kf_off;
+  const float arg_scale = D.kf_scale, to_exp2 = KIND == 1 ? -1.4426950f * arg_scale : -arg_scale;
   const int32_t* __restrict__ Scol = D.Scol;
   const float* __restrict__ xhat = D.xhat;
   float* __restrict__ yhat = D.yhat;
@@ -872,7 +876,7 @@ __global__ void __launch_bounds__(128, RPL == 1 ? 6 : 4) k_coupling_kf(const Mat
         // row point minus the column centre, once per block: a coordinate difference is then one
         // subtraction. The clusters of a coupling block are separated (their boxes' distance is
         // positive and at least their diameter / eta), so the difference does not cancel and
-        // keeps FP32 relative precision, and r^2 > 0.
+        // keeps FP32 relative precision.
         float ax[RPL], ay[RPL], az[RPL];
 #pragma unroll
         for (int rr = 0; rr < RPL; rr++) {
@@ -891,13 +895,13 @@ __global__ void __launch_bounds__(128, RPL == 1 ? 6 : 4) k_coupling_kf(const Mat
             for (int rr = 0; rr < RPL; rr++) {
               const float dx = ax[rr] - oj.x, dy = ay[rr] - oj.y, dz = az[rr] - oj.z;
               const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-              const float t = r2 * rsqrt_approx(r2);
+              const float dist = sqrt_approx(r2);
               float val;
               if constexpr (KIND == 1) {
-                const float ex = ex2_approx(-1.4426950f * t);
-                val = fmaf(t, ex, ex);
+                const float ex = ex2_approx(to_exp2 * dist);
+                val = fmaf(arg_scale * dist, ex, ex);
               } else {
-                val = ex2_approx(-t);
+                val = ex2_approx(to_exp2 * dist);
               }
               sv[rr][e] = (FULL || mu0 + e < k) ? val : 0.f;
             }
