@@ -323,8 +323,8 @@ h2_status h2_matvec_static_check(void* stream);
  * product y = A^H x with each candidate configuration (one warm-up and three
  * timed products, CUDA events on `stream`) and keeps the fastest for later
  * calls on this handle:
- *   dense consumer warps:   8 or 16 (they matter in passes of up to four vectors;
- *                           16 only for passes of at most 8 vectors)
+ *   dense consumer warps:   8 or 16 (the handle's own number where no pass of the
+ *                           product takes up to four vectors: only such passes use them)
  *   coupling row chunks:    about 64, 128 or 256 coupling blocks per warp
  *   tree jobs:              subtrees at the default level (2^L >= twice the SMs)
  *                           or one or two levels higher (fewer, larger subtrees)
@@ -391,13 +391,15 @@ h2_status h2_batch_matvec(h2_batch b, const int32_t* nv, const double* const* x,
 
 /*
  * Autotuning of a batch: as h2_tune, over the candidates
- *   dense consumer warps:   8 or 16 (16 only when no member takes more than 8 vectors)
+ *   dense consumer warps:   8 or 16 (the batch's own number where no pass takes up to
+ *                           four vectors)
  *   coupling row chunks:    about 64, 128 or 256 coupling blocks per warp
  *   tree jobs:              subtrees of 16, 32 or 64 leaves per group of eight CTAs
  * (one warm-up and two timed batched products each, arguments as for
  * h2_batch_matvec), then the split of the dense work items over the CTAs:
- * each leaf row weighed by its bytes times (1 + beta nv/16), nv its member's
- * vectors per pass, beta in {0, 1, 2, 4} (the fastest kept). chosen[0]
+ * each leaf row weighed by its bytes (its cycles in passes of more than four
+ * vectors) times (1 + beta nv/16), nv its member's vectors per pass, beta in
+ * {0, 1, 2, 4} (the fastest kept). chosen[0]
  * consumer warps, chosen[1] chunk size, chosen[2] leaves per group of
  * eight tree CTAs. Synchronizes `stream`.
  */

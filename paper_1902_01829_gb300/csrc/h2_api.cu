@@ -1005,8 +1005,8 @@ h2_status h2_tune(h2_handle h, int32_t nv, const double* x, int64_t ldx, double*
   cudaEvent_t e0, e1;
   CUDA_TRY(cudaEventCreate(&e0));
   CUDA_TRY(cudaEventCreate(&e1));
-  // 16 dense consumer warps exist for passes of at most 8 vectors
-  const int ncw = 2;  // 8 or 16 dense consumer warps
+  // 8 or 16 dense consumer warps, where some pass streams its dense blocks
+  const int ncw = h2i::tune_warps(nv) ? 2 : 1, cw0 = h->mx.launch.cw;
   float best = 3.4e38f;
   int best_opt = kDefaultChunkOpt, best_cw = h->mx.launch.cw, best_tree = 0;
   h2_status s = H2_OK;
@@ -1014,7 +1014,7 @@ h2_status h2_tune(h2_handle h, int32_t nv, const double* x, int64_t ldx, double*
   for (int c = 0; c < ncw && s == H2_OK; c++)
     for (int opt = 0; opt < 3 && s == H2_OK; opt++)
       for (int tr = 0; tr < ntree && s == H2_OK; tr++) {
-      const int cw = c ? 2 * kDenseCW : kDenseCW;
+      const int cw = ncw == 1 ? cw0 : c ? 2 * kDenseCW : kDenseCW;
       if ((s = mixed_configure(h, opt, cw, tr)) != H2_OK) break;
       if ((s = matvec_device(h, nv, x, ldx, y, ldy, st)) != H2_OK) break;  // warm-up
       cudaEventRecord(e0, st);

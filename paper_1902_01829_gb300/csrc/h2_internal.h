@@ -170,6 +170,9 @@ constexpr int kChunkOpts[3] = {64, 128, 256};  // coupling blocks per warp chunk
 constexpr int kTreeOpts[3] = {1, 2, 3};       // log2 of the leaves per tree CTA (batches; a cluster of 8 CTAs: 16 .. 64)
 constexpr int kDefaultChunkOpt = 1, kDefaultTreeOpt = 2;
 constexpr int kDenseCW = 8;                   // dense-stream consumer warps (or twice as many)
+// whether a product of nv vectors has a pass that streams its dense blocks (up to four vectors: its last),
+// the only one that the number of consumer warps is for
+constexpr bool tune_warps(int nv) { return (nv - 1) % 16 < 4; }
 std::vector<int4> coupling_chunks(const int32_t* Srow, int64_t n_nodes, int64_t target, int k, int64_t total, int sms,
                                   bool kf, int64_t* slots);
 
@@ -316,7 +319,8 @@ struct h2_batch_s {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   // the dense items' split over the CTAs (h2_batch_tune weighs each row by its member's vector count)
   std::vector<h2::StreamItem> items_host;
-  std::vector<int64_t> row_bytes, row_item0;
+  std::vector<int64_t> row_bytes, row_mma, row_item0;
   std::vector<int32_t> row_mat;
   int* cta_begin_dev = nullptr;
+  int* mma_begin_dev = nullptr;
 };

@@ -1247,8 +1247,9 @@ h2_status batch_build(h2_batch_s* b) {
   b->cta_begin_dev = db;
   int* dmb = nullptr;
   if ((st = balloc(b, &dmb, (int64_t)mbegin.size(), mbegin.data())) != H2_OK) return st;
-  L.mma_begin = dmb;
+  L.mma_begin = b->mma_begin_dev = dmb;
   b->row_bytes = row_bytes;
+  b->row_mma = std::move(row_mma);
   b->row_item0 = row_item0;
   b->items_host = items;
   h2::MixedBlock* blk = nullptr;
@@ -1347,22 +1348,27 @@ h2_status h2_batch_create(const h2_handle* hs, int32_t count, h2_batch* out) {
 
 namespace {
 
-// The dense items' split over the CTAs for the vector counts nv (nullptr: bytes alone): row r of
-// member i weighs bytes_r (1 + beta nv_i / 16), since a row's arithmetic grows with its vectors
-// while its bytes do not; the split is uploaded after `stream` has drained (no product reads it).
+// The dense items' splits over the CTAs for the vector counts nv (nullptr: the defaults): row r of member i
+// weighs w_r (1 + beta nv_i / 16), with w_r its bytes in the streams' split (k_dense_stream_m) and its cycles
+// in that of k_dense_mma: a row's arithmetic, vectors and output grow with its member's vectors, and a member
+// of none costs little. The splits are uploaded after `stream` has drained (no product reads them).
 h2_status batch_rebalance(h2_batch b, const int32_t* nv, float beta, cudaStream_t stream) {
-  std::vector<int64_t> w(b->row_bytes.size());
-  for (size_t r = 0; r < w.size(); r++) {
-    const int v = nv ? std::max(0, std::min(nv[b->row_mat[r]], kPassVectors)) : 0;
-    w[r] = (int64_t)((double)b->row_bytes[r] * (1.0 + beta * v / kPassVectors));
+  std::vector<int> begin[2];
+  for (int m = 0; m < 2; m++) {
+    std::vector<int64_t> w = m ? b->row_mma : b->row_bytes;
+    for (size_t r = 0; r < w.size(); r++) {
+      const int v = nv ? std::max(0, std::min(nv[b->row_mat[r]], kPassVectors)) : 0;
+      w[r] = (int64_t)((double)w[r] * (1.0 + beta * v / kPassVectors));
+    }
+    begin[m] = balance(w, b->row_item0, b->launch.grid);
+    h2_status st = audit_producer_batches(b->items_host, begin[m]);
+    if (st != H2_OK) return st;
+    for (size_t c = 0; c + 1 < begin[m].size(); c++)
+      if (begin[m][c] > begin[m][c + 1]) return h2_fail(H2_ERR_INVALID, "internal: item ranges not monotone");
   }
-  const std::vector<int> begin = balance(w, b->row_item0, b->launch.grid);
-  h2_status st = audit_producer_batches(b->items_host, begin);
-  if (st != H2_OK) return st;
-  for (size_t c = 0; c + 1 < begin.size(); c++)
-    if (begin[c] > begin[c + 1]) return h2_fail(H2_ERR_INVALID, "internal: item ranges not monotone");
   CUDA_TRY(cudaStreamSynchronize(stream));
-  CUDA_TRY(cudaMemcpy(b->cta_begin_dev, begin.data(), begin.size() * sizeof(int), cudaMemcpyHostToDevice));
+  CUDA_TRY(cudaMemcpy(b->cta_begin_dev, begin[0].data(), begin[0].size() * sizeof(int), cudaMemcpyHostToDevice));
+  CUDA_TRY(cudaMemcpy(b->mma_begin_dev, begin[1].data(), begin[1].size() * sizeof(int), cudaMemcpyHostToDevice));
   return H2_OK;
 }
 
@@ -1422,14 +1428,16 @@ h2_status h2_batch_tune(h2_batch b, const int32_t* nv, const double* const* x, c
   cudaEvent_t e0, e1;
   CUDA_TRY(cudaEventCreate(&e0));
   CUDA_TRY(cudaEventCreate(&e1));
-  const int ncw = 2;  // 8 or 16 dense consumer warps
+  // 8 or 16 dense consumer warps, where some pass streams its dense blocks (tune_warps)
+  const int ncw = nvmax > 0 && tune_warps(nvmax) ? 2 : 1;
+  const int cw0 = b->launch.cw;
   float best = 3.4e38f;
   int best_c = b->chunk_opt, best_t = b->tree_opt, best_cw = b->launch.cw;
   h2_status s = H2_OK;
   for (int c = 0; c < ncw && s == H2_OK; c++)
     for (int co = 0; co < 3 && s == H2_OK; co++)
       for (int to = 0; to < 3 && s == H2_OK; to++) {
-        const int cw = c ? 2 * h2::kMixedCW : h2::kMixedCW;
+        const int cw = ncw == 1 ? cw0 : c ? 2 * h2::kMixedCW : h2::kMixedCW;
         if ((s = batch_configure(b, co, to, cw)) != H2_OK) break;
         if ((s = h2_batch_matvec(b, nv, x, ldx, y, ldy, stream)) != H2_OK) break;  // warm-up (validates)
         cudaEventRecord(e0, st);
