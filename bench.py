@@ -157,8 +157,8 @@ TRAFFIC_RATIO = {("fp64", False): 3184266039 / 3178496000, ("int16", True): 7946
 TRAFFIC_KERNEL = {("fp64", False): "k_dense_stream", ("int16", True): "k_dense_stream_m"}  # the kernel those counters belong to
 
 # digit products per product of two FP64 entries in the FP64 form's dense phase at more than four vectors
-# (six 8-bit digits each: the 21 pairs of weight <= 5 and the five of weight 6)
-DIGIT_PAIRS = 26
+# (seven 8-bit digits each: the 21 pairs of weight <= 5 and the seven of weight 6)
+DIGIT_PAIRS = 28
 # mma.sync FP16 rate of the chip, TFLOP/s (a loop of m16n8k16: 8 cycles each per SM quarter)
 MMA_SYNC_TFLOPS = 600.0
 
@@ -473,7 +473,7 @@ def construction_line(h2, A, values=("U", "E", "S", "D")) -> dict:
 
 def dense_kernel_name(A, nv: int, storage: str, bases_fp32: bool) -> str:
     """The kernel of the dense phase: for up to four vectors the streams; for more, in the FP64 form
-    the digit kernel (unless a dense block spans more than 2^10), in the precision form the tcgen05
+    the digit kernel, in the precision form the tcgen05
     kernel (16-bit fp16 / bf16 codes and bases, k a multiple of 16, every leaf 64 points, 8 or more
     vectors) or else the MMA tiles."""
     if storage == "fp64":

@@ -209,7 +209,12 @@ h2_status h2_create_generated(const h2_desc* d, const h2_coupling_kernel* kc, co
  * tensor cores, whatever the leaves and bases. Other passes of more than four
  * vectors run the dense blocks on MMA tiles: the scaled forms with the vectors
  * split into three 16-bit parts, the FP64 form by exact products of 8-bit
- * digits if no dense block's nonzero entries span more than 2^10.
+ * digits where a dense block has no zeros and its entries span less than 2^9,
+ * else in double-float. Digits hold a block's entries to 2^-55 of its largest
+ * and a vector's to 2^-54 of the largest of its leaf (double-float: each to
+ * 2^-46 of itself): the error of a row stays below 2^-38 of sum_j |a_ij||x_j|
+ * for any vector and near 2^-46 of it where a row's entries are alike, and the
+ * last bits of a column may differ between a call of four vectors and of five.
  * Errors: H2_ERR_INVALID (NULL, nv < 1, ld < n), H2_ERR_CUDA (launch failed).
  */
 h2_status h2_matvec(h2_handle h, int32_t nv, const double* x, int64_t ldx, double* y, int64_t ldy, void* stream);

@@ -141,7 +141,7 @@ struct Fp64Ranges {
   std::vector<int32_t> oV, oF, oE, oS, oD, oU, eY;
   std::vector<char> d_safe;
   std::vector<int32_t> d_exp;  // each dense block's exponent ea for k_dense_oz
-  bool d_narrow = true;         // every dense block's nonzero entries lie within 2^10
+  std::vector<char> d_wide;     // its entries don't lie within 2^9 of the digits' range, or some are zero
   bool s_tiny = false;
 };
 
@@ -203,6 +203,7 @@ Fp64Ranges fp64_ranges(const h2_desc* d, int64_t leaves, int64_t n_nodes, int64_
   R.oD.resize((size_t)nD);
   R.d_safe.resize((size_t)nD);
   R.d_exp.resize((size_t)nD);
+  R.d_wide.resize((size_t)nD);
   for (int64_t j = 0; j < leaves; j++) {
     R.eY[j] = exp_of_bound(bY[j]);
     R.oV[j] = block_offset(ex[leaf0 + j], sV[j]);
@@ -221,9 +222,9 @@ Fp64Ranges fp64_ranges(const h2_desc* d, int64_t leaves, int64_t n_nodes, int64_
   for (int64_t b = 0; b < nD; b++) {
     R.oD[b] = block_offset(R.eY[drow[b]], sD[b]);
     R.d_safe[b] = needs_safe_split(sD[b], R.oD[b]);
-    // |a| 2^(46 - ea) <= 0x7F7F7F7F7F7F, the digits' range: one less than the frexp exponent where that fits
+    // |a| 2^(54 - ea) <= 0x7F7F7F7F7F7F7F, the digits' range: one less than the frexp exponent where that fits
     R.d_exp[b] = sD[b].emax - (sD[b].mmax < 0.99 ? 1 : 0);
-    if (sD[b].lnorm != -HUGE_VAL && sD[b].emax - sD[b].emin > 10) R.d_narrow = false;
+    R.d_wide[b] = sD[b].zero || R.d_exp[b] + 1 - sD[b].emin > 9;
   }
   (void)q;
   return R;
@@ -454,16 +455,21 @@ template <int NVB>
 cudaError_t set_pass_smem() {
   static const cudaError_t done = [] {
     constexpr int CW = h2::dense_consumer_warps(NVB);
-    cudaError_t e = cudaFuncSetAttribute(h2::k_dense_stream<NVB, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         h2::stream_smem_bytes(NVB, CW));
-    if (e == cudaSuccess && NVB > 4)
+    cudaError_t e = cudaSuccess;
+    if constexpr (NVB > 4) {
       e = cudaFuncSetAttribute(h2::k_dense_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, h2::kOzSmem);
+    } else {
+      e = cudaFuncSetAttribute(h2::k_dense_stream<NVB, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               h2::stream_smem_bytes(NVB, CW));
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(h2::k_dense_stream<NVB, CW>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 (int)cudaSharedmemCarveoutMaxShared);
+    }
     for (const void* f : {(const void*)h2::k_upsweep_tree<NVB>, (const void*)h2::k_downsweep_tree<NVB>})
       if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, h2::kSmemLimit);
     // kernels that run beside one another prefer the same (largest) shared part of the L1 / shared memory split
     constexpr int CV = NVB < 4 ? NVB : 4;
-    for (const void* f : {(const void*)h2::k_downsweep_tree<NVB>, (const void*)h2::k_dense_stream<NVB, CW>,
-                          (const void*)h2::k_coupling_small<CV, true>, (const void*)h2::k_coupling_small<CV, false>,
+    for (const void* f : {(const void*)h2::k_downsweep_tree<NVB>, (const void*)h2::k_coupling_small<CV, true>, (const void*)h2::k_coupling_small<CV, false>,
                           (const void*)h2::k_coupling<16, CV, true>, (const void*)h2::k_coupling<16, CV, false>,
                           (const void*)h2::k_coupling<32, CV, true>, (const void*)h2::k_coupling<32, CV, false>,
                           (const void*)h2::k_coupling<64, CV, true>, (const void*)h2::k_coupling<64, CV, false>,
@@ -483,7 +489,6 @@ h2_status run_pass(h2_matrix_s* h, int nv, const double* x, int64_t ldx, double*
   cudaError_t e = set_pass_smem<NVB>();
   if (e != cudaSuccess) return fail(H2_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
   constexpr int CW = dense_consumer_warps(NVB);
-  constexpr int smem = stream_smem_bytes(NVB, CW);
   const int kkp = (int)even((int64_t)k * k);
   TreeParams T{};
   T.Vt = h->Vt;
@@ -507,13 +512,12 @@ h2_status run_pass(h2_matrix_s* h, int nv, const double* x, int64_t ldx, double*
   T.q = h->q;
   T.L = h->tree_L;
   T.nv = nv;
-  const bool oz = NVB > 4 && h->oz;
   // Passes of up to four vectors stream the dense blocks on the caller's stream beside the coupling phase and the
   // downsweep on the handle's side stream (the upsweep, which splits x, runs before both); k_vec_scale zeroes y,
   // and the dense phase and the leaf expansion add into it. Wider passes and profiled ones run in order.
   const bool beside = NVB <= 4 && !h->prof.on;
   T.add = beside;
-  T.oz = oz;
+  T.oz = NVB > 4;
   T.xks = (h->m_max + 15) / 16;
   T.xd = h->xd;
   T.dmat = h->dmat;
@@ -531,37 +535,32 @@ h2_status run_pass(h2_matrix_s* h, int nv, const double* x, int64_t ldx, double*
   if (me == cudaSuccess) me = mark(&h->prof, st);
   cudaStream_t ts = st;  // the coupling phase's and the downsweep's
   auto launch_dense = [&] {
-    StreamParams P{};
-    P.items = h->dense_items.items;
-    P.cta_begin = h->dense_items.cta_begin;
-    P.mat = h->dmat;
-    P.vsrc0 = h->x2;
-    P.nv = nv;
-    P.y = y;
-    P.ldy = ldy;
-    P.vexp = h->vexp;
-    P.err = h->err;
-    P.budget = h->budget;
-    P.inject = h->inject;
-    if (oz) {
-      OzParams O{};
-      O.items = P.items;
-      O.cta_begin = P.cta_begin;
-      O.item_exp = h->item_exp;
-      O.item_leaf = h->item_leaf;
-      O.mat = P.mat;
-      O.xd = h->xd;
-      O.xks = T.xks;
-      O.nv = nv;
-      O.y = y;
-      O.ldy = ldy;
-      O.vexp = h->vexp;
-      O.err = h->err;
-      O.budget = h->budget;
-      O.inject = h->inject;
-      k_dense_oz<<<h->grid, (kOzWarps + 1) * 32, kOzSmem, st>>>(O);
+    auto common = [&](auto& P) {
+      P.items = h->dense_items.items;
+      P.cta_begin = h->dense_items.cta_begin;
+      P.mat = h->dmat;
+      P.nv = nv;
+      P.y = y;
+      P.ldy = ldy;
+      P.vexp = h->vexp;
+      P.err = h->err;
+      P.budget = h->budget;
+      P.inject = h->inject;
+    };
+    if constexpr (NVB > 4) {
+      OzParams P{};
+      common(P);
+      P.item_exp = h->item_exp;
+      P.item_leaf = h->item_leaf;
+      P.xd = h->xd;
+      P.x2 = h->x2;
+      P.xks = T.xks;
+      k_dense_oz<<<h->grid, (kOzWarps + 1) * 32, kOzSmem, st>>>(P);
     } else {
-      k_dense_stream<NVB, CW><<<h->grid, (CW + 1) * 32, smem, st>>>(P);
+      StreamParams P{};
+      common(P);
+      P.vsrc0 = h->x2;
+      k_dense_stream<NVB, CW><<<h->grid, (CW + 1) * 32, stream_smem_bytes(NVB, CW), st>>>(P);
     }
   };
   if (beside) {
@@ -764,7 +763,7 @@ h2_status build_device(h2_matrix_s* h, const h2_desc* d) {
         it.v_off = xp[j];
         it.row = (int)lo[i];
         const bool last = b + 1 == d->D_rowptr[i + 1];  // ends the row: the rows' output exponent
-        it.flags = (R.d_safe[b] ? h2::kItemFlagSafe : 0) | (last ? h2::kItemFlagLast : 0) |
+        it.flags = (R.d_safe[b] ? h2::kItemFlagSafe : 0) | (R.d_wide[b] ? h2::kItemFlagWide : 0) | (last ? h2::kItemFlagLast : 0) |
                    h2::item_pack_exp(R.oD[b], last ? R.eY[i] : 0);
         items.push_back(it);
         bytes += it.m_bytes + 8 * sj;
@@ -780,12 +779,9 @@ h2_status build_device(h2_matrix_s* h, const h2_desc* d) {
       if ((st = upload(h, &h->eY, R.eY.data(), h->leaves)) != H2_OK) return st;
     }
     // the digits' tables (see mma_fp64.cuh), per item = per dense block
-    h->oz = R.d_narrow && h->nD > 0;
-    if (h->oz) {
-      if ((st = upload(h, &h->item_exp, R.d_exp.data(), h->nD)) != H2_OK) return st;
-      if ((st = upload(h, &h->item_leaf, d->D_colidx, h->nD)) != H2_OK) return st;
-      if ((st = dalloc(h, &h->xd, h->leaves * h2::xd_chunk_bytes((h->m_max + 15) / 16, 2))) != H2_OK) return st;
-    }
+    if ((st = upload(h, &h->item_exp, R.d_exp.data(), h->nD)) != H2_OK) return st;
+    if ((st = upload(h, &h->item_leaf, d->D_colidx, h->nD)) != H2_OK) return st;
+    if ((st = dalloc(h, &h->xd, h->leaves * h2::xd_chunk_bytes((h->m_max + 15) / 16, 2))) != H2_OK) return st;
     const std::vector<int> begin = balance(row_bytes, row_item0, h->grid);
     if ((st = audit_items(items, begin, total * 8, xp[h->leaves])) != H2_OK) return st;  // (vectors: the split x per slot)
     if ((st = upload_items(h, &h->dense_items, items, begin)) != H2_OK) return st;

@@ -212,8 +212,7 @@ struct h2_matrix_s {
   int32_t* oF = nullptr;
   int32_t* oE = nullptr;
   int2* Sco = nullptr;
-  // passes of more than four vectors: the dense phase by digits (k_dense_oz), if no dense block spans more than 2^10
-  bool oz = false;
+  // passes of more than four vectors: the dense phase by digits (k_dense_oz)
   int* item_exp = nullptr;            // per dense item: its block's exponent and column leaf
   int* item_leaf = nullptr;
   unsigned char* xd = nullptr;        // digits of the pass's vectors

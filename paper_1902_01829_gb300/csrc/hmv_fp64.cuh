@@ -199,33 +199,33 @@ struct TreeOp64 {
   static __device__ __forceinline__ void parts(const P& T, int64_t j, int s, const float2* xs, const unsigned* vmax) {
     const int nh = T.nv > 8 ? 2 : 1;
     unsigned char* chunk = T.xd + j * xd_chunk_bytes(T.xks, nh);
-    // |x| 2^(46 - ex) <= 0x7F7F7F7F7F7F, the digits' range: the exponent of the largest |x|, one more where its
-    // fraction leaves no room; a chunk below 2^-80 of its vector's largest entry keeps that unit
-    auto ex = [&](int v) { return max((int)(vmax[v] >> 23) - ((vmax[v] & 0x7FFFFFu) < 0x7D0000u ? 127 : 126), -80); };
+    // |x| 2^(54 - ex) <= 0x7F7F7F7F7F7F7F, the digits' range: the exponent of the largest |x|, one more where its
+    // fraction leaves no room
+    auto ex = [&](int v) { return max((int)(vmax[v] >> 23) - ((vmax[v] & 0x7FFFFFu) < 0x7D0000u ? 127 : 126), kXdMinExp); };
     for (int i = threadIdx.x; i < ((s + 15) >> 4) * 32 * nh; i += TH) {
       const int ln = i & 31, u = i >> 5, ks = nh == 2 ? u >> 1 : u, half = nh == 2 ? u & 1 : 0;
       const int v = (ln >> 2) + 8 * half, c0 = 16 * ks + (ln & 3);
-      const float up = __int_as_float((127 + 46 - (v < T.nv ? ex(v) : 0)) << 23);
+      const float up = __int_as_float((127 - (v < T.nv ? ex(v) : 0)) << 23);  // 2^-ex; 2^(54 - ex) may be no float
       uint32_t lo[4], hi[4];
 #pragma unroll
       for (int q = 0; q < 4; q++) {
         const int c = c0 + 4 * q;
         const float2 x = (v < T.nv && c < s) ? xs[c * VS + v] : make_float2(0.f, 0.f);
-        const long long n = __float2ll_rn(x.x * up) + __float2ll_rn(x.y * up) + 0x808080808080LL;
+        const long long n = __float2ll_rn(x.x * up * 0x1p54f) + __float2ll_rn(x.y * up * 0x1p54f) + 0x80808080808080LL;
         lo[q] = (uint32_t)n;
         hi[q] = (uint32_t)((unsigned long long)n >> 32);
       }
-      uint32_t d0[6], d1[6];
+      uint32_t d0[kXdDigits], d1[kXdDigits];
       digit_pairs(lo[0], hi[0], lo[1], hi[1], d0);
       digit_pairs(lo[2], hi[2], lo[3], hi[3], d1);
       uint2* dst = reinterpret_cast<uint2*>(chunk + kXdScale + u * kXdStep + ln * 8);
 #pragma unroll
-      for (int p = 0; p < 6; p++) dst[32 * p] = make_uint2(d0[p], d1[p]);
+      for (int p = 0; p < kXdDigits; p++) dst[32 * p] = make_uint2(d0[p], d1[p]);
     }
     // (a chunk with an infinity or NaN: kXdNaN makes its vector's sums NaN)
     if (threadIdx.x < 16)
       reinterpret_cast<int*>(chunk)[threadIdx.x] =
-          threadIdx.x >= T.nv ? -80 : vmax[threadIdx.x] >= 0x7F800000u ? kXdNaN : ex(threadIdx.x);
+          threadIdx.x >= T.nv ? kXdMinExp : vmax[threadIdx.x] >= 0x7F800000u ? kXdNaN : ex(threadIdx.x);
   }
   static __device__ __forceinline__ int copy_bytes(int entries) { return 8 * entries; }
   static __device__ __forceinline__ const char* U(const P& T, const Leaf& l) { return T.dmat + l.uoff; }

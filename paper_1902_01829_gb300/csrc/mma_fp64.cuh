@@ -1,25 +1,30 @@
 // Dense near field of the FP64 plain form for passes of more than four vectors, on the tensor cores:
 //   y(i) += sum_j D_ij x(j)     (Sec. 2.2; y(i) holds U_i yhat_i from the downsweep)
 // by integer slicing (the Ozaki scheme: Ozaki, Ogita, Oishi, Rump, "Error-free transformations of matrix
-// multiplication by using fast routines of matrix multiplication", 2012): every entry becomes six signed
+// multiplication by using fast routines of matrix multiplication", 2012): every entry becomes seven signed
 // 8-bit digits, digit products are exact in FP16 MMAs, and their sums are exact in the FP32 accumulators.
 //
-//   a = 2^(ea - 46) sum_i d_i 2^(8 (5 - i)),  |a| <= 0x7F7F7F7F7F7F 2^(ea - 46) over the block,   i = 0 .. 5
-//   x = 2^(ex - 46) sum_j e_j 2^(8 (5 - j)),  the same over a leaf's chunk of one vector
-// so both are held to 2^-47 or 2^-48 of the largest entry of their block (chunk) -- the double-float kernel cuts each
-// entry at 2^-47 of itself, so a handle takes this path only if no dense block spans more than 2^10
-// (nonzero entries) and rows of smaller entries keep 2^-37. The 21 products with i + j <= 5 are summed by
-// weight: |d e| <= 2^14, 64 columns and at most 6 pairs stay below 2^23, exact for every weight; the five of
-// weight 6 (2^-44 of a typical sum) join weight 5's at 2^-8. A block's six sums are joined in double-float
-// (the upper four exactly) and added to the row's running pairs, so blocks of any magnitude meet as in the
-// double-float kernel.
+//   a = 2^(ea - 54) sum_i d_i 2^(8 (6 - i)),  |a| <= 0x7F7F7F7F7F7F7F 2^(ea - 54) over the block,   i = 0 .. 6
+//   x = 2^(ex - 54) sum_j e_j 2^(8 (6 - j)),  the same over a leaf's chunk of one vector
+// so a block's entries are held to 2^-55 of its largest, where the double-float kernel cuts each at 2^-46 of
+// itself: a block takes this form if it has no zeros and its entries lie within 2^9 of 2^(ea + 1), and none of them
+// is then held in fewer bits. Any other block ("wide") is multiplied in double-float by the same warps
+// (oz_wide_block), so that an entry far below its block's largest, in a row that sees no other, keeps its bits.
+// The vectors' entries are held to 2^-54 of their chunk's largest, whatever they span: without zeros every row
+// of a digit block weighs that largest entry with 2^-9 of the block's at least, so the cut is below
+// 64 2^9 2^-54 of sum_j |a_ij| |x_j|, and 2^-50 of it where a row's entries are alike. The 21 products with
+// i + j <= 5 are summed by weight: |d e| <= 2^14, 64 columns and at most 6 pairs stay below 2^23, exact for every
+// weight; the seven of weight 6 join weight 5's at 2^-8, the rest (2^-56 of the largest product each) is left out.
+// A block's six sums are joined in double-float (the upper four exactly) and added to the row's running pairs, so
+// blocks of any magnitude meet as in the double-float kernel.
 //
 // What bounds it: at 16 vectors a 64 x 64 block cost the FP32 pipes 65,536 double-float products of 11
-// instructions, 8,800 cycles an SM; 832 MMAs take 1,664, slicing its 4,096 entries about 800 issue slots,
-// and its 32 KB 1,400 at the copy bandwidth. Measured, 2D n = 50,001 (48- and 49-point
-// leaves), 16 vectors: dense phase 837 -> 404 us, error against 64 bits 2.6e-14 -> 2.1e-14 (weight 6 left out:
-// 7e-14; the sums joined without the third exact step: 1e-13). 5,000 cycles a block are still the chain of
-// slicing, loads and MMAs of three warps a scheduler, not a pipe.
+// instructions, 8,800 cycles an SM (which a wide block still takes); 896 MMAs take 1,792, slicing its 4,096 entries
+// about 800 issue slots, and its 32 KB 1,400 at the copy bandwidth. Measured, 2D n = 50,001 (48- and 49-point leaves),
+// 16 vectors: six digits 837 -> 404 us in the dense phase, error against 64 bits 2.6e-14 -> 2.1e-14 (weight 6 left
+// out: 7e-14; the sums joined without the third exact step: 1e-13); seven digits with the vectors' fragments loaded
+// one at a time (76 bytes of spills less) 682 -> 669 us in the product, error 2.0e-14. About 5,000 cycles a block are
+// still the chain of slicing, loads and MMAs of three warps a scheduler, not a pipe.
 //
 // Y^T = X^T D^T as in mma_dense.cuh: the vectors' digits are the A operand, written in fragment order by
 // the upsweep; a lane slices the entries it loads from the item's stage into B fragments. The dense
@@ -31,9 +36,10 @@
 
 namespace h2 {
 
-// digits of a leaf's vectors: 16 exponents ex (ints), then per K step of 16 points and half of eight vectors six
+// digits of a leaf's vectors: 16 exponents ex (ints), then per K step of 16 points and half of eight vectors seven
 // digits of 256 bytes, lane (g, t)'s entries (vector g + 8 half; points t, t + 4, t + 8, t + 12) at 8 (4 g + t)
-constexpr int kXdScale = 64, kXdStep = 6 * 256;
+constexpr int kXdScale = 64, kXdDigits = 7, kXdStep = kXdDigits * 256;
+constexpr int kXdMinExp = -120;   // smallest ex: a chunk further below its vector's largest entry keeps this unit
 constexpr int kXdNaN = 1 << 20;  // as an exponent: the chunk's vector has an entry that is not finite
 __host__ __device__ constexpr int xd_chunk_bytes(int ksteps, int halves) { return kXdScale + ksteps * halves * kXdStep; }
 
@@ -46,22 +52,21 @@ constexpr int kOzSmem = kOzStages * kOzStage + 256 + kOzRed;
 static_assert(kOzStages >= 3, "at least three stages");
 static_assert(kOzStage % 16 == 0, "stage alignment");
 
-// v = (a as an integer multiple of 2^(ea - 46), rounded to nearest) + 0x808080808080: the digits are its
-// bytes minus 128. E = ea + 1022: the biased FP64 exponent of the block's largest entry, or one less. lo: low 32 bits, hi: the rest.
-// The block's nonzero normal entries lie within 2^10 of its largest; zeros and subnormals give 0.
+// v = (a as an integer multiple of 2^(ea - 54), rounded to nearest) + 0x80808080808080: the digits are its
+// bytes minus 128. E = ea + 1031: |a| < 2^(ea + 1) has a biased FP64 exponent of ea + 1023 at most. lo: low 32
+// bits, hi: the rest. The block's entries are normal; a zero (a column or row past the block) gives digits
+// of no meaning, which meet zeros or are not stored.
 __device__ __forceinline__ void slice_f64(double a, int E, uint32_t& lo, uint32_t& hi) {
   const uint32_t h = (uint32_t)__double2hiint(a), l = (uint32_t)__double2loint(a);
-  const int ef = (int)((h >> 20) & 0x7FFu);
-  const int s = min(E - ef + 6, 31);  // |a| 2^47 / 2^ea: the value with one bit below the unit (s >= 5)
-  uint32_t mh = (h & 0xFFFFFu) | 0x100000u, ml = l;
-  if (ef == 0) mh = ml = 0u;
+  const int s = min(E - (int)((h >> 20) & 0x7FFu), 31);  // |a| 2^(55 - ea): the value with one bit below the unit (s >= 8)
+  const uint32_t mh = __funnelshift_l(l, h, 11) | 0x80000000u, ml = l << 11;
   uint32_t vl = __funnelshift_r(ml, mh, s), vh = mh >> s;
   // round: (v + 1) >> 1, then the sign, then the digits' bias
   asm("add.cc.u32 %0, %0, 1;\n\taddc.u32 %1, %1, 0;" : "+r"(vl), "+r"(vh));
   vl = __funnelshift_r(vl, vh, 1);
   vh >>= 1;
   if (h >> 31) asm("sub.cc.u32 %0, 0, %0;\n\tsubc.u32 %1, 0, %1;" : "+r"(vl), "+r"(vh));
-  asm("add.cc.u32 %0, %0, 0x80808080;\n\taddc.u32 %1, %1, 0x8080;" : "+r"(vl), "+r"(vh));
+  asm("add.cc.u32 %0, %0, 0x80808080;\n\taddc.u32 %1, %1, 0x808080;" : "+r"(vl), "+r"(vh));
   lo = vl;
   hi = vh;
 }
@@ -75,15 +80,17 @@ __device__ __forceinline__ uint32_t digit_pair(uint32_t p) {
   return *reinterpret_cast<const uint32_t*>(&r);
 }
 
-// the six digits (from the top) of two sliced values as fp16 pairs
-__device__ __forceinline__ void digit_pairs(uint32_t l0, uint32_t h0, uint32_t l1, uint32_t h1, uint32_t (&d)[6]) {
-  const uint32_t p0 = __byte_perm(l0, l1, 0x5140), p1 = __byte_perm(l0, l1, 0x7362), p2 = __byte_perm(h0, h1, 0x5140);
-  d[5] = digit_pair<0>(p0);
-  d[4] = digit_pair<1>(p0);
-  d[3] = digit_pair<0>(p1);
-  d[2] = digit_pair<1>(p1);
-  d[1] = digit_pair<0>(p2);
-  d[0] = digit_pair<1>(p2);
+// the seven digits (from the top) of two sliced values as fp16 pairs
+__device__ __forceinline__ void digit_pairs(uint32_t l0, uint32_t h0, uint32_t l1, uint32_t h1, uint32_t (&d)[kXdDigits]) {
+  const uint32_t p0 = __byte_perm(l0, l1, 0x5140), p1 = __byte_perm(l0, l1, 0x7362), p2 = __byte_perm(h0, h1, 0x5140),
+                 p3 = __byte_perm(h0, h1, 0x7362);
+  d[6] = digit_pair<0>(p0);
+  d[5] = digit_pair<1>(p0);
+  d[4] = digit_pair<0>(p1);
+  d[3] = digit_pair<1>(p1);
+  d[2] = digit_pair<0>(p2);
+  d[1] = digit_pair<1>(p2);
+  d[0] = digit_pair<0>(p3);
 }
 
 __device__ __forceinline__ uint32_t scale_digits(uint32_t d) {  // / 256, exact
@@ -98,6 +105,7 @@ struct OzParams {
   const int* item_leaf;
   const char* mat;
   const unsigned char* xd;  // the leaves' digits, xks K steps each
+  const float2* x2;         // split x, padded leaf layout: the wide blocks' vectors
   int xks, nv;
   double* y;
   long long ldy;
@@ -107,7 +115,7 @@ struct OzParams {
   int inject;  // >= 0: CTA 0 withholds the copy of this local item (bounded-wait test)
 };
 
-// Producer warp. Stage header (ints): R, C, flags, row, ea.
+// Producer warp. Stage header (ints): R, C, flags, row, ea, vector stride of a wide block.
 __device__ __forceinline__ void oz_produce(const OzParams& P, const StreamShared& S, int ib, int ie) {
   const int lane = threadIdx.x & 31;
   const uint64_t pol = policy_evict_first();
@@ -140,21 +148,26 @@ __device__ __forceinline__ void oz_produce(const OzParams& P, const StreamShared
       const int m_bytes = __shfl_sync(0xFFFFFFFFu, mine.m_bytes, t), row = __shfl_sync(0xFFFFFFFFu, mine.row, t);
       const unsigned shape = __shfl_sync(0xFFFFFFFFu, mine.shape, t);
       const int flags = __shfl_sync(0xFFFFFFFFu, mine.flags, t);
+      const long long v_off = __shfl_sync(0xFFFFFFFFu, mine.v_off, t);
       const int ea = __shfl_sync(0xFFFFFFFFu, l_exp, t), leaf = __shfl_sync(0xFFFFFFFFu, l_leaf, t);
       if (lane == 0) {
         unsigned char* stage = S.stage0 + s * kOzStage;
         int* h = reinterpret_cast<int*>(stage);
-        const int C = (int)((shape >> 8) & 0xFF);
+        const int C = (int)((shape >> 8) & 0xFF), vs = (int)((shape >> 16) & 0xFF);
+        const bool wide = (flags & kItemFlagWide) != 0;
         h[0] = (int)(shape & 0xFF);
         h[1] = C;
         h[2] = flags;
         h[3] = row;
         h[4] = ea;
+        h[5] = vs;
         if (!((P.inject == it) && (blockIdx.x == 0))) {
-          const unsigned vbytes = (unsigned)xd_chunk_bytes((C + 15) / 16, nh);
+          const unsigned vbytes = wide ? 8u * (unsigned)(vs * P.nv) : (unsigned)xd_chunk_bytes((C + 15) / 16, nh);
+          const void* vsrc = wide ? static_cast<const void*>(P.x2 + v_off * P.nv)
+                                  : P.xd + (long long)leaf * xd_chunk_bytes(P.xks, nh);
           mbar_arrive_expect_tx(S.full + s, (unsigned)m_bytes + vbytes);
           bulk_g2s_stream(stage + kStageHeader, P.mat + m_off, (unsigned)m_bytes, S.full + s, pol);
-          bulk_g2s(stage + kStageHeader + kStageMat, P.xd + (long long)leaf * xd_chunk_bytes(P.xks, nh), vbytes, S.full + s);
+          bulk_g2s(stage + kStageHeader + kStageMat, vsrc, vbytes, S.full + s);
         }
       }
       __syncwarp();
@@ -207,17 +220,7 @@ __device__ __forceinline__ void oz_block(const double* A, uint32_t X, int R, int
   load(0);
 #pragma unroll 1
   for (int k0 = 0; k0 < C; k0 += 16) {
-    uint32_t a[6][4];
-#pragma unroll
-    for (int p = 0; p < 6; p++) {
-      const uint2 u = lds64(xa + 256 * p), v = lds64(xa + 256 * p + half);
-      a[p][0] = u.x;
-      a[p][1] = v.x;
-      a[p][2] = u.y;
-      a[p][3] = v.y;
-    }
-    xa += xstep;
-    uint32_t d[2][2][6];
+    uint32_t d[2][2][kXdDigits];
 #pragma unroll
     for (int i = 0; i < 2; i++) {
       uint32_t l[4], h[4];
@@ -227,17 +230,55 @@ __device__ __forceinline__ void oz_block(const double* A, uint32_t X, int R, int
       digit_pairs(l[2], h[2], l[3], h[3], d[i][1]);
     }
     if (k0 + 16 < C) load(k0 + 16);
+    // the vectors' digits in turn, the next one's fragment loaded ahead (all seven at once do not fit the registers)
+    uint32_t a[2][4];
+    auto load_digit = [&](int j, uint32_t(&f)[4]) {
+      const uint2 u = lds64(xa + 256 * j), v = lds64(xa + 256 * j + half);
+      f[0] = u.x;
+      f[1] = v.x;
+      f[2] = u.y;
+      f[3] = v.y;
+    };
+    load_digit(0, a[0]);
 #pragma unroll
-    for (int p = 0; p < 6; p++)
+    for (int j = 0; j < kXdDigits; j++) {
+      if (j + 1 < kXdDigits) load_digit(j + 1, a[(j + 1) & 1]);
 #pragma unroll
-      for (int j = 0; j < 6 - p; j++)
+      for (int p = 0; p < 6 - j; p++)
 #pragma unroll
-        for (int i = 0; i < 2; i++) mma_m16n8k16(acc[i][p + j], a[j], d[i][0][p], d[i][1][p], false);
-    // weight 6, the matrix digits / 256, with weight 5's sums
+        for (int i = 0; i < 2; i++) mma_m16n8k16(acc[i][p + j], a[j & 1], d[i][0][p], d[i][1][p], false);
+      // weight 6, the matrix digit / 256, with weight 5's sums
 #pragma unroll
-    for (int p = 1; p < 6; p++)
+      for (int i = 0; i < 2; i++) mma_m16n8k16(acc[i][5], a[j & 1], scale_digits(d[i][0][6 - j]), scale_digits(d[i][1][6 - j]), false);
+    }
+    xa += xstep;
+  }
+}
+
+// The same quarter of a wide block in double-float: the block split with its offset o, the vectors' pairs X
+// ([vector][vs points]); acc[i][e] of rows r = 16 quarter + 4 t + 2 (e & 1) + i and vectors g (e < 2) and g + 8.
+__device__ __forceinline__ void oz_wide_block(const double* A, const float2* X, int R, int C, int vs, int r, int o, int nv,
+                                              float2 (&acc)[2][4]) {
+  const int g = (threadIdx.x & 31) >> 2;
 #pragma unroll
-      for (int i = 0; i < 2; i++) mma_m16n8k16(acc[i][5], a[6 - p], scale_digits(d[i][0][p]), scale_digits(d[i][1][p]), false);
+  for (int i = 0; i < 2; i++)
+#pragma unroll
+    for (int e = 0; e < 4; e++) acc[i][e] = make_float2(0.f, 0.f);
+#pragma unroll 1
+  for (int c = 0; c < C; c++) {
+    float2 x[2];
+#pragma unroll
+    for (int b = 0; b < 2; b++) x[b] = g + 8 * b < nv ? X[(g + 8 * b) * vs + c] : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      float h, l;
+      split_f64(r + q < R ? A[r + q + R * c] : 0.0, o, h, l);
+#pragma unroll
+      for (int b = 0; b < 2; b++) {
+        float2& p = acc[q & 1][(q >> 1) + 2 * b];
+        df_fma(p.x, p.y, h, l, x[b].x, x[b].y);
+      }
+    }
   }
 }
 
@@ -271,34 +312,50 @@ __global__ void __launch_bounds__((kOzWarps + 1) * 32, 1) k_dense_oz(OzParams P)
     {
       bool ok = true;
       for (; turn < nu; turn += kOzWarps) {
-        const int r = 16 * turn + 2 * g;
-        const uint32_t X = smem_addr(stage + kStageHeader + kStageMat);
-        float acc[2][6][4];
-        oz_block(reinterpret_cast<const double*>(stage + kStageHeader), X, R, C, r, ea + 1022, nh, acc);
-        if (fresh && !(ok = open_row())) break;
-        // 2^(ea + ex - 28 - row exponent): the sums below are in units of 2^64 2^-92
-        const int* ex = reinterpret_cast<const int*>(stage + kStageHeader + kStageMat);
         const int shift = item_offset(flags);  // the row's output exponent (o of its blocks)
+        const double* A = reinterpret_cast<const double*>(stage + kStageHeader);
+        const unsigned char* xs = stage + kStageHeader + kStageMat;
+        // the lane's sums are added to its slots: tile i, element e are row 4 t + 2 (e & 1) + i, vector g + 8 (e >> 1)
+        auto put = [&](int i, int e, float s, float c) {
+          float2* slot = mine + (g + 8 * (e >> 1)) * kOzRedStride + 2 * (2 * t + (e & 1)) + i;
+          float2 p = fresh ? make_float2(0.f, 0.f) : *slot;
+          df_add(p.x, p.y, s, c);
+          *slot = p;
+        };
+        if (flags & kItemFlagWide) {
+          float2 acc[2][4];
+          oz_wide_block(A, reinterpret_cast<const float2*>(xs), R, C, min(h[5], 64), 16 * turn + 4 * t, shift, nv, acc);
+          if (fresh && !(ok = open_row())) break;
+#pragma unroll
+          for (int i = 0; i < 2; i++)
+#pragma unroll
+            for (int e = 0; e < 4; e++) put(i, e, acc[i][e].x, acc[i][e].y);
+          fresh = false;
+          continue;
+        }
+        float acc[2][6][4];
+        oz_block(A, smem_addr(xs), R, C, 16 * turn + 2 * g, ea + 1031, nh, acc);
+        if (fresh && !(ok = open_row())) break;
+        // the sums below are in units of 2^(96 - 16 + 38) (weight 2 times 2^-38), so that a contribution down to 2^-126 of
+        // the row's bound is a float, as in double-float
+        const int* ex = reinterpret_cast<const int*>(xs);
         float f[2];
 #pragma unroll
         for (int b = 0; b < 2; b++) {
-          const int n = ea - shift + ex[g + 8 * b] - 28;
+          const int n = ea - shift + ex[g + 8 * b] + 10;
           f[b] = n < -126 ? 0.f : __int_as_float(n > 127 ? 0x7FC00000 : (n + 127) << 23);  // (n > 127: kXdNaN)
         }
 #pragma unroll
         for (int i = 0; i < 2; i++)
 #pragma unroll
           for (int e = 0; e < 4; e++) {
-            const float tail = fmaf(acc[i][5][e], 0.00390625f, acc[i][4][e]) * 0x1p-16f;
+            const float tail = fmaf(acc[i][5][e], 0.00390625f, acc[i][4][e]) * 0x1p-54f;
             float s1, e1, s2, e2, s3, e3;
-            two_sum(acc[i][0][e] * 65536.f, acc[i][1][e] * 256.f, s1, e1);
-            two_sum(s1, acc[i][2][e], s2, e2);
-            two_sum(s2, acc[i][3][e] * 0.00390625f, s3, e3);
-            const float fb = f[e >> 1], s = s3 * fb, c = (((e1 + e2) + e3) + tail) * fb;
-            float2* slot = mine + (g + 8 * (e >> 1)) * kOzRedStride + 2 * (2 * t + (e & 1)) + i;
-            float2 p = fresh ? make_float2(0.f, 0.f) : *slot;
-            df_add(p.x, p.y, s, c);
-            *slot = p;
+            two_sum(acc[i][0][e] * 0x1p-22f, acc[i][1][e] * 0x1p-30f, s1, e1);
+            two_sum(s1, acc[i][2][e] * 0x1p-38f, s2, e2);
+            two_sum(s2, acc[i][3][e] * 0x1p-46f, s3, e3);
+            const float fb = f[e >> 1];
+            put(i, e, s3 * fb, (((e1 + e2) + e3) + tail) * fb);
           }
         fresh = false;
       }

@@ -28,7 +28,7 @@ struct __align__(16) StreamItem {
   unsigned shape;   // R | C << 8 | vstride << 16 | nb << 24   (nb = 1)
   long long v_off;  // vector chunk offset, in float2 per vector slot
   int row;          // first point of the row leaf (y offset)
-  int flags;        // bit 0: last item of its row;
+  int flags;        // bit 0: last item of its row; bit 1 (FP64 form): a wide block (mma_fp64.cuh);
                     // bit 2: the block holds zeros or magnitudes below 2^-103 after its offset (zero-safe split);
                     // FP64 form: bits 4-17 the block's exponent offset, bits 18-31 (last item) the row's
                     // output exponent (both signed 14-bit)
@@ -37,7 +37,7 @@ struct __align__(16) StreamItem {
 constexpr int kStageHeader = 128;
 constexpr int kStageMat = 32768;
 constexpr int kSmemLimit = 232448;  // opt-in shared memory per CTA on sm_103a
-constexpr int kItemFlagLast = 1, kItemFlagSafe = 4;
+constexpr int kItemFlagLast = 1, kItemFlagWide = 2, kItemFlagSafe = 4;
 constexpr int kItemOffsetShift = 4, kItemRowExpShift = 18, kItemExpMax = 8191;  // 14-bit signed fields
 __host__ __device__ constexpr int item_offset(int flags) { return (int)((unsigned)flags << 14) >> 18; }
 __host__ __device__ constexpr int item_row_exp(int flags) { return flags >> kItemRowExpShift; }
