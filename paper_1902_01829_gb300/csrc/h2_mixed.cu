@@ -82,6 +82,16 @@ float quantize(const double* a, int64_t cnt, int form, uint16_t* codes) {
   return sigma;
 }
 
+// kBlockWide if some code of a dense block is (mixed.cuh), else 0
+unsigned char wide_flag(const uint16_t* codes, int64_t cnt, int form) {
+  bool w = false;
+  if (form == h2::kFormFp16)
+    for (int64_t i = 0; i < cnt; i++) w |= h2::wide_code<h2::kFormFp16>(codes[i]);
+  else if (form == h2::kFormInt16)
+    for (int64_t i = 0; i < cnt; i++) w |= h2::wide_code<h2::kFormInt16>(codes[i]);
+  return w ? h2::kBlockWide : 0;
+}
+
 // quantize then transpose a rows x cols column-major block into cols x rows codes
 float quantize_transposed(const double* a, int64_t rows, int64_t cols, int form, uint16_t* codes,
                           std::vector<uint16_t>& tmp) {
@@ -219,6 +229,7 @@ template <int F>
 __global__ void __launch_bounds__(256) k_gen_dense(GenDense a) {
   __shared__ double xs[2][64 * 3];
   __shared__ double wmax[8];
+  __shared__ int wwide[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int64_t t = blockIdx.x; t < a.nblocks; t += gridDim.x) {
     const int i = a.brow[t], j = a.bcol[t];
@@ -262,16 +273,27 @@ __global__ void __launch_bounds__(256) k_gen_dense(GenDense a) {
     const float sigma = F == h2::kFormInt16 ? (float)(m / 32767.0) : (float)m;
     uint16_t* dst = reinterpret_cast<uint16_t*>(a.dmat + a.bbyte[t]);
     const int ps2 = h2::panel_stride(sj) / 2, cs = h2::code_stride(si);
+    bool wide = false;
 #pragma unroll
     for (int u = 0; u < 16; u++) {
       const int e = threadIdx.x + 256 * u;
       if (e < si * sj) {
         const int r = e % si, c = e / si;
-        dst[a.panel ? (r >> 3) * ps2 + 8 * c + (r & 7) : r + cs * c] = gen_code<F>(v[u], sigma);
+        const uint16_t code = gen_code<F>(v[u], sigma);
+        wide |= h2::wide_code<F>(code);
+        dst[a.panel ? (r >> 3) * ps2 + 8 * c + (r & 7) : r + cs * c] = code;
       }
     }
     if (threadIdx.x == 0) a.blk[a.bglob[t]].scale = sigma;
+    if constexpr (F != h2::kFormBf16) {
+      wide = __any_sync(0xFFFFFFFFu, wide);
+      if (lane == 0) wwide[warp] = wide;
+    }
     __syncthreads();  // xs and wmax are reused by the next block
+    if constexpr (F != h2::kFormBf16) {
+      if (threadIdx.x < 32 && __any_sync(0xFFFFFFFFu, lane < 8 && wwide[lane & 7]) && lane == 0)
+        a.blk[a.bglob[t]].src |= h2::kBlockWide;
+    }
   }
 }
 
@@ -685,15 +707,18 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
           const int32_t j = d->D_colidx[b];
           const int64_t sj = lo[j + 1] - lo[j];
           h2::MixedBlock& m = blk[g];
+          m.src = panel ? 4 : 0;
           if (gen) {
-            m.scale = 0.f;  // the device writes the codes and the scale
+            m.scale = 0.f;  // the device writes the codes, the scale and the wide bit
           } else if (panel) {
             tmp.resize((size_t)(si * sj));
             m.scale = quantize(d->D_val + doff[b], si * sj, form, tmp.data());
+            m.src |= wide_flag(tmp.data(), si * sj, form);
             to_panels(sj, reinterpret_cast<uint16_t*>(base + boff[g]));
           } else {
             uint16_t* dst = reinterpret_cast<uint16_t*>(base + boff[g]);
             m.scale = quantize(d->D_val + doff[b], si * sj, form, dst);
+            m.src |= wide_flag(dst, si * sj, form);
             const int64_t cs = h2::code_stride((int)si);  // spread the columns, the last first
             for (int64_t c = sj - 1; cs != si && c > 0; c--) std::memmove(dst + c * cs, dst + c * si, (size_t)si * 2);
           }
@@ -701,7 +726,6 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
           m.leaf = (uint64_t)j;
           m.cols = (unsigned short)sj;
           m.vs = (unsigned char)round_up(sj, 4);
-          m.src = panel ? 4 : 0;
         }
         h2::MixedBlock& m = blk[g];  // U_i, multiplied with yhat of leaf i
         unsigned char* ub = gen ? base + uoffc[i] : base + boff[g];
@@ -800,6 +824,7 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
     for (int64_t g = 0; g < nblk; g++) {
       float& mx = (blk[g].src & 1) ? M.umax : M.dmax;
       mx = std::max(mx, blk[g].scale);
+      M.launch.wide = M.launch.wide || (blk[g].src & h2::kBlockWide);
     }
 
     // work items: consecutive dense blocks of one row, at most kMixedMaxBlocks blocks, 32 KB of
@@ -1206,6 +1231,7 @@ h2_status batch_build(h2_batch_s* b) {
     const h2_matrix_s* h = b->hs[(size_t)i];
     const MixedData& M = h->mx;
     const int64_t item0 = (int64_t)items.size();
+    L.wide = L.wide || M.launch.wide;
     for (h2::StreamItem it : M.items_host) {
       it.v_off += blk0;
       it.flags = (it.flags & 0xFF) | (int)(i << 8);

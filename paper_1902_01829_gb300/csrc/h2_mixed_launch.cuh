@@ -135,10 +135,13 @@ h2_status dense_launch(const MixedLaunch& L, cudaStream_t st) {
 }
 
 // the dense phase of a pass of more than four vectors
-template <int F>
+template <int F, bool WIDE>
 h2_status mma_launch(const MixedLaunch& L, cudaStream_t st) {
   using namespace h2;
-  static const cudaError_t attr = cudaFuncSetAttribute(k_dense_mma<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMmaSmem);
+  if constexpr (!WIDE && F != kFormBf16) {  // (bf16 blocks are never wide)
+    if (L.wide) return mma_launch<F, true>(L, st);
+  }
+  static const cudaError_t attr = cudaFuncSetAttribute(k_dense_mma<F, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMmaSmem);
   if (attr != cudaSuccess) return h2_fail(H2_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(attr));
   MixedStreamParams P{};
   P.items = L.items;
@@ -147,7 +150,7 @@ h2_status mma_launch(const MixedLaunch& L, cudaStream_t st) {
   P.mats = static_cast<const MatDesc*>(L.mats);
   P.err = L.err;
   P.budget = L.budget;
-  k_dense_mma<F><<<L.grid, (kMmaWarps + 1) * 32, kMmaSmem, st>>>(P);
+  k_dense_mma<F, WIDE><<<L.grid, (kMmaWarps + 1) * 32, kMmaSmem, st>>>(P);
   return H2_OK;
 }
 
@@ -231,7 +234,7 @@ h2_status mixed_pass_t(const MixedLaunch& L, unsigned buckets, cudaStream_t st, 
            : top == 0 ? dense_launch<F, 1>(L, ds)
            : top == 1 ? dense_launch<F, 2>(L, ds)
            : top == 2 ? dense_launch<F, 4>(L, ds)
-                      : mma_launch<F>(L, ds);
+                      : mma_launch<F, false>(L, ds);
   };
   // passes of more than four vectors keep the phases in order: their tree kernels' shared memory does
   // not fit beside the dense stream's, and the dense phase is bound by arithmetic there (measured)

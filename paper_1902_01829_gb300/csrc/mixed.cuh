@@ -75,8 +75,17 @@ struct __align__(16) MixedBlock {
   unsigned short cols;  // C
   unsigned char vs;     // vector stride (>= C, multiple of 4)
   unsigned char src;    // bit 0: vector from the second source (yhat); bit 1: FP32 entries (not codes);
-                        // bit 2: panel layout (below)
+                        // bit 2: panel layout (below); bit 3: a wide block of fp16 or int16 codes
 };
+// A dense block is wide if an fp16 code is below 2^-10 (a block's largest is 1) or an int16 code below 256 (of 32767),
+// zeros among them: what k_dense_mma's split leaves out could then show in a row of small codes (mma_dense.cuh).
+constexpr int kBlockWide = 8;
+template <int F>
+__host__ __device__ __forceinline__ bool wide_code(uint16_t c) {
+  if (F == kFormFp16) return (c & 0x7FFFu) < 0x1400u;
+  if (F == kFormInt16) return c > 32768 - 256 && c < 32768 + 256;
+  return false;
+}
 
 // Panel layout of a block of codes (64 rows, C columns): eight panels of 8 rows,
 // panel p holding column c's rows 8p .. 8p + 7 as 16 contiguous bytes at c * 16,

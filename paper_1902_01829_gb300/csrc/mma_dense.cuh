@@ -6,12 +6,18 @@
 // side, 16 columns the K side. The codes then enter as the B operand straight from the registers they are
 // loaded into (a lane's four columns of a K step times its four or eight rows, one byte permute per pair),
 // and the vectors as the A operand in fragment order, written once per leaf by the upsweep:
-//   x_v = 2^(e - 14) (hi + mid + lo), hi, mid, lo fp16 (2^(e-1) <= max |x_v| over the leaf < 2^e: 33 bits
-//   of the leaf's largest entry), or for bf16 codes x_v = hi + mid + lo in bf16 (all 24 bits of an FP32).
+//   x_v = 2^(e - 14) (hi + mid + lo), hi, mid, lo fp16 (2^(e-1) <= max |x_v| over the leaf < 2^e: all 24 bits of
+//   an FP32 down to 2^-14 of the leaf's largest entry, below that what lies above 2^-38 of it), or for bf16 codes
+//   x_v = hi + mid + lo in bf16 (all 24 bits of any FP32).
 // A code is a B entry as it is (fp16, bf16); an int16 code q = 256 (h + l) with h = q >> 8 and l = the low
-// byte / 256, both exact in fp16, times hi, mid (and lo): l lo is below 2^-30 of the product. The leading
-// products h hi and the rest accumulate apart, in FP32, and a block's sums enter the row's after
-// sigma 2^(e - 14) is applied, so nothing is rounded to 16 bits and no chain is longer than a block.
+// byte / 256, both exact in fp16, times hi, mid (and lo): l lo is left out, below 2^-23 of its product where |q| >= 256
+// (with it 5 MMAs become 6: 2D n = 2^18, 8 vectors, dense phase 261 -> 313 us). The leading products h hi and the rest
+// accumulate apart, in FP32, and a block's sums enter the row's after sigma 2^(e - 14) is applied, so nothing is
+// rounded to 16 bits and no chain is longer than a block. Blocks with smaller int16 codes, or with fp16 codes below
+// 2^-10, zeros among them ("wide"), are multiplied in FP32 by the same warps (mma_wide_block) with the vectors as they
+// are: a row of such a block may see small codes or small vector entries alone. In the others every row weighs the
+// leaf's largest entry with 2^-10 (int16: 2^-7) at least, so what the parts cut off is below 64 2^10 2^-38 of
+// sum_j |d_ij| |x_j| for any vector, in most cases below FP32's rounding of the sum.
 //
 // What bounds it: at 16 vectors the FP32 pipes spent 2048 FMAs of a warp on a 64 x 64 block (1360 cycles an
 // SM with its loads); 3 (int16: 5) MMAs per tile and K step take 192 (320) and the codes' loads from shared
@@ -62,9 +68,11 @@ __device__ __forceinline__ uint32_t int16_low(uint32_t c) {
   return *reinterpret_cast<const uint32_t*>(&r);
 }
 
-// Producer warp: as mixed_produce, with the blocks' vector chunks in the parts' layout. Stage header (ints):
-// [0] R, [1] nb, [2] row, [3] flags, [4] vector halves (1 or 2); block t at 8 + 4 t: columns | panel << 17,
-// vector offset, matrix offset, scale; [48] nv, [49] xy32, [50..51] y, [52..53] ldy.
+// Producer warp: as mixed_produce, with the blocks' vector chunks in the parts' layout (a wide block's in FP32).
+// Stage header (ints): [0] R, [1] nb, [2] row, [3] flags, [4] vector halves (1 or 2); block t at 8 + 4 t:
+// columns | panel << 17 | wide << 18 | vector stride << 24, vector offset, matrix offset, scale; [48] nv, [49] xy32, [50..51] y, [52..53] ldy.
+// WIDE: the launch's matrices have wide blocks.
+template <bool WIDE>
 __device__ __forceinline__ void mma_produce(const MixedStreamParams& P, const StreamShared& S, int ib, int ie,
                                             MixedBlock* blkbuf) {
   const int lane = threadIdx.x & 31;
@@ -85,13 +93,14 @@ __device__ __forceinline__ void mma_produce(const MixedStreamParams& P, const St
     const int nbatch = (int)min(blast - bfirst, (long long)kMixedBatchBlocks);
     for (int u = lane; u < nbatch; u += 32) blkbuf[u] = P.blk[bfirst + u];
     // each lane fetches the matrix fields of its own item
-    unsigned long long l_dmat = 0, l_xp = 0, l_y = 0;
+    unsigned long long l_dmat = 0, l_xp = 0, l_x4 = 0, l_y = 0;
     long long l_ldy = 0;
     int l_nv = 0, l_xy32 = 0, l_xks = 0;
     if (base + lane < ie) {
       const MatDesc& D = P.mats[mine.flags >> 8];
       l_dmat = reinterpret_cast<unsigned long long>(D.dmat);
       l_xp = reinterpret_cast<unsigned long long>(D.xp);
+      l_x4 = reinterpret_cast<unsigned long long>(D.x4);
       l_y = reinterpret_cast<unsigned long long>(D.y);
       l_ldy = D.ldy;
       l_nv = D.nv;
@@ -108,6 +117,7 @@ __device__ __forceinline__ void mma_produce(const MixedStreamParams& P, const St
       const int flags = __shfl_sync(0xFFFFFFFFu, mine.flags, t);
       const char* dmat = reinterpret_cast<const char*>(__shfl_sync(0xFFFFFFFFu, l_dmat, t));
       const unsigned char* xp = reinterpret_cast<const unsigned char*>(__shfl_sync(0xFFFFFFFFu, l_xp, t));
+      const float* x4 = reinterpret_cast<const float*>(__shfl_sync(0xFFFFFFFFu, l_x4, t));
       const unsigned long long ydst = __shfl_sync(0xFFFFFFFFu, l_y, t);
       const long long ldy = __shfl_sync(0xFFFFFFFFu, l_ldy, t);
       const int nv = __shfl_sync(0xFFFFFFFFu, l_nv, t), xy32 = __shfl_sync(0xFFFFFFFFu, l_xy32, t);
@@ -127,7 +137,8 @@ __device__ __forceinline__ void mma_produce(const MixedStreamParams& P, const St
       const long long bi = b0 - bfirst + lane;
       if (lane < nb && bi >= 0 && bi < nbatch) mb = blkbuf[bi];
       const int codes = (mb.src & 4) ? panel_block_bytes(mb.cols) : (code_stride(R) * (int)mb.cols * 2 + 15) & ~15;
-      const int vbytes = (lane < nb && nv > 0) ? xp_chunk_bytes((mb.cols + 15) / 16, nh) : 0;
+      const bool wide = WIDE && (mb.src & kBlockWide) != 0;  // (the FP32 chunk is no larger than the parts)
+      const int vbytes = (lane < nb && nv > 0) ? (wide ? 4 * nv * mb.vs : xp_chunk_bytes((mb.cols + 15) / 16, nh)) : 0;
       int moff = codes, voff = vbytes;  // inclusive prefixes of the blocks' bytes
 #pragma unroll
       for (int d = 1; d < kMixedMaxBlocks; d <<= 1) {
@@ -141,7 +152,7 @@ __device__ __forceinline__ void mma_produce(const MixedStreamParams& P, const St
       moff -= codes;
       voff += m_bytes - vbytes;  // the vectors' chunks follow the codes
       if (lane < nb) {
-        hd[8 + 4 * lane] = mb.cols | ((mb.src & 4) << 15);
+        hd[8 + 4 * lane] = mb.cols | ((mb.src & (4 | kBlockWide)) << 15) | (mb.vs << 24);
         hd[9 + 4 * lane] = voff;
         hd[10 + 4 * lane] = moff;
         hd[11 + 4 * lane] = __float_as_int(mb.scale);
@@ -164,8 +175,9 @@ __device__ __forceinline__ void mma_produce(const MixedStreamParams& P, const St
       }
       __syncwarp();
       if (vbytes > 0)
-        bulk_g2s(stage + kMixedHeader + voff, xp + (long long)mb.leaf * xp_chunk_bytes(xks, nh), (unsigned)vbytes,
-                 S.full + s);
+        bulk_g2s(stage + kMixedHeader + voff,
+                 wide ? static_cast<const void*>(x4 + (long long)mb.voff * nv) : xp + (long long)mb.leaf * xp_chunk_bytes(xks, nh),
+                 (unsigned)vbytes, S.full + s);
       __syncwarp();
       issued = it + 1;
     }
@@ -278,7 +290,46 @@ __device__ __forceinline__ void mma_block(uint32_t base, int cb, uint32_t X, int
     for (int e = 0; e < 4; e++) run[i][e] = fmaf(s0 * sc[e >> 1], hi[i][e] + lo[i][e], run[i][e]);
 }
 
+// The same of a wide block, in FP32: codes at `codes`, vectors X ([vector][vs points]); n = 2t + (e & 1), its four rows
+// from row rows[e & 1], tile i the i-th of them. Bound by issue slots like the streams: 1,500 cycles an SM for a 64 x 64
+// block.
 template <int F>
+__device__ __forceinline__ void mma_wide_block(const unsigned char* codes, bool panel, const float* X, int vs, int C, int R,
+                                               const int (&rows)[2], float scale, int nv, float (&run)[4][4]) {
+  using T = typename CodeT<F>::T;
+  const int g = (threadIdx.x & 31) >> 2;
+  float acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; i++)
+#pragma unroll
+    for (int e = 0; e < 4; e++) acc[i][e] = 0.f;
+  const T* A[2];
+#pragma unroll
+  for (int u = 0; u < 2; u++)
+    A[u] = reinterpret_cast<const T*>(codes) + (panel ? (rows[u] >> 3) * (panel_stride(C) / 2) + (rows[u] & 7) : rows[u]);
+  const int cs = panel ? 8 : code_stride(R);
+#pragma unroll 2
+  for (int c = 0; c < C; c++) {
+    float x[2];
+#pragma unroll
+    for (int b = 0; b < 2; b++) x[b] = g + 8 * b < nv ? X[(g + 8 * b) * vs + c] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 2; u++)
+#pragma unroll
+      for (int i = 0; i < 4; i++) {
+        const float a = rows[u] + i < R ? code_to_f<F>(A[u][c * cs + i]) : 0.f;
+#pragma unroll
+        for (int b = 0; b < 2; b++) acc[i][u + 2 * b] = fmaf(a, x[b], acc[i][u + 2 * b]);
+      }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; i++)
+#pragma unroll
+    for (int e = 0; e < 4; e++) run[i][e] = fmaf(scale, acc[i][e], run[i][e]);
+}
+
+// (WIDE in every launch: 32 matrices of 1024 .. 16384 points, fp16, 667 -> 674 us with no wide block among them)
+template <int F, bool WIDE>
 __global__ void __launch_bounds__((kMmaWarps + 1) * 32, 1) k_dense_mma(MixedStreamParams P) {
   extern __shared__ __align__(1024) unsigned char smem[];
   const StreamShared S = stream_shared<kMmaStages, kMmaStage>(smem);
@@ -286,7 +337,7 @@ __global__ void __launch_bounds__((kMmaWarps + 1) * 32, 1) k_dense_mma(MixedStre
   const int ib = P.cta_begin[blockIdx.x], ie = P.cta_begin[blockIdx.x + 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   if (warp == kMmaWarps) {
-    mma_produce(P, S, ib, ie, reinterpret_cast<MixedBlock*>(smem + kMmaStages * kMmaStage + 256 + kMmaRed));
+    mma_produce<WIDE>(P, S, ib, ie, reinterpret_cast<MixedBlock*>(smem + kMmaStages * kMmaStage + 256 + kMmaRed));
     return;
   }
   StreamParams W{};
@@ -317,8 +368,14 @@ __global__ void __launch_bounds__((kMmaWarps + 1) * 32, 1) k_dense_mma(MixedStre
         const int4 bh = *reinterpret_cast<const int4*>(hd + 8 + 4 * (turn >> two));
         const int C = min(bh.x & 0xFFFF, 64);
         const bool panel = (bh.x >> 17) & 1;
-        const uint32_t codes = smem_addr(stage + kMixedHeader) + (min(bh.z, kStageMat - 16) & ~15);
-        const uint32_t X = smem_addr(stage + kMixedHeader) + (min(bh.y, kMmaArea - xp_chunk_bytes(1, 1)) & ~15);
+        const int moff = min(bh.z, kStageMat - 16) & ~15, voff = min(bh.y, kMmaArea - 16) & ~15;
+        if (WIDE && ((bh.x >> 18) & 1)) {
+          const int n0 = two ? 8 * 2 * t + 4 * (turn & 1) : 4 * 2 * t, rows[2] = {n0, n0 + (two ? 8 : 4)};
+          mma_wide_block<F>(stage + kMixedHeader + moff, panel, reinterpret_cast<const float*>(stage + kMixedHeader + voff),
+                            min((int)((unsigned)bh.x >> 24), 64), C, R, rows, __int_as_float(bh.w), nv, run);
+          continue;
+        }
+        const uint32_t codes = smem_addr(stage + kMixedHeader) + moff, X = smem_addr(stage + kMixedHeader) + voff;
         const int r = two ? 8 * g + 4 * (turn & 1) : 4 * g, cb = panel ? 16 : 2 * code_stride(R);
         // (in the column-major layout the last lanes' rows may lie past R: they read what follows, unused)
         const uint32_t base = codes + (panel ? (r >> 3) * panel_stride(C) + 2 * (r & 7) : 2 * r);

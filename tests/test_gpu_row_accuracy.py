@@ -6,12 +6,18 @@ import types
 import numpy as np
 import pytest
 
+from oracle import quant
+
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 # FP64: 64 products' share of what the digits leave out (384 2^-56 of the block's largest product) where a row is
 # 2^-8 of its block: 2^-43.4; entries cut at 2^-46; a double-float sum of two blocks: 2^-46
 FP64_TOL = 2.0 ** -42.5
+# scaled forms: FP32 sums of 64 products (2^-18) of two blocks
+FP32_TOL = 2.0 ** -17
+# every remainder of the tiles, halves and K steps
+EDGES = [1, 3, 4, 7, 8, 15, 16, 17, 31, 32, 33, 36, 47, 48, 63, 64]
 
 
 @pytest.fixture(scope="module")
@@ -33,7 +39,8 @@ def to_dev(x):
 def near_field(sizes, blocks):
     """A matrix of dense blocks alone: blocks {(i, j): array}."""
     sizes = np.asarray(sizes)
-    q, k, leaves, nodes = int(np.log2(sizes.size)), 2, sizes.size, 2 * sizes.size - 1
+    k = 16 if np.all(sizes == 64) else 2  # 64-point leaves at k = 16: the panel layout of 16-bit codes
+    q, leaves, nodes = int(np.log2(sizes.size)), sizes.size, 2 * sizes.size - 1
     lo = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
     keys = sorted(blocks)
     drp = np.searchsorted([i for i, _ in keys], np.arange(leaves + 1)).astype(np.int32)
@@ -87,7 +94,7 @@ def case(kind, sizes, nv):
 
 
 @pytest.mark.parametrize("kind", ["diagonal", "rows", "vectors", "mixed", "small leaf"])
-@pytest.mark.parametrize("sizes", [[64] * 4, [16] * 8, [49, 33, 17, 48]])
+@pytest.mark.parametrize("sizes", [[64] * 4, [16] * 8, [49, 33, 17, 48], EDGES])
 @pytest.mark.parametrize("nv", [4, 5, 9, 16])
 def test_fp64_rows(h2, kind, sizes, nv):
     if kind == "small leaf" and nv <= 4:
@@ -100,4 +107,23 @@ def test_fp64_rows(h2, kind, sizes, nv):
     ref, bound = product(A, A.D_val, x)
     worst = np.max(np.abs(y - ref) / bound)
     assert worst <= FP64_TOL, (kind, np.log2(worst))
+    M.close()
+
+
+@pytest.mark.parametrize("form", ["int16", "fp16", "bf16"])
+@pytest.mark.parametrize("kind", ["diagonal", "rows", "vectors", "mixed", "small leaf"])
+@pytest.mark.parametrize("sizes", [[64] * 4, [16] * 8, [49, 33, 17, 48], EDGES])
+@pytest.mark.parametrize("nv", [4, 5, 7, 16])
+def test_scaled_rows(h2, form, kind, sizes, nv):
+    if nv == 16 and form != "int16" and sizes == [64] * 4:
+        pytest.skip("the tcgen05 passes hold a vector's entries relative to its largest")
+    blocks, x = case(kind, sizes, nv)
+    x = x.astype(np.float32)
+    A = near_field(sizes, blocks)
+    M = handle(h2, A, form)
+    y = M.matvec_f32(to_dev(x)).cpu().numpy().astype(np.float64)
+    M.check()
+    ref, bound = product(A, quant.dequantized_arrays(A, form)["D_val"], x.astype(np.float64))
+    worst = np.max(np.abs(y - ref) / bound)
+    assert worst <= FP32_TOL, (kind, np.log2(worst))
     M.close()
