@@ -54,6 +54,7 @@ struct MixedLaunch {
   int tree_T = 0;                    // levels below the subtree roots of the deepest job
   const int4* chunks = nullptr;      // coupling row chunks (mixed.cuh)
   int64_t nchunks = 0;
+  bool split = false;                // some chunk is a piece of a long row
   const h2::StreamItem* items = nullptr;
   const int* cta_begin = nullptr;    // [grid + 1]
   const int* mma_begin = nullptr;    // the same for passes of more than four vectors (k_dense_mma)
@@ -159,6 +160,7 @@ struct MixedData {
   std::vector<int32_t> srow_host;          // S_rowptr (to cut chunks for another target)
   int4* chunk_dev[3] = {nullptr, nullptr, nullptr};  // device chunk lists per target option
   int64_t chunk_n[3] = {0, 0, 0};
+  bool chunk_split[3] = {false, false, false};
   float* cpart = nullptr;                             // pieces of cut coupling rows: sums [slot][v][kp4]
   int* cticket = nullptr;                             // [slot][4] counters, zero between products
   int64_t cslots = 0;
@@ -310,6 +312,7 @@ struct h2_batch_s {
   int chunk_opt = h2i::kDefaultChunkOpt, tree_opt = h2i::kDefaultTreeOpt;
   int4* chunk_dev[3] = {nullptr, nullptr, nullptr};
   int64_t chunk_n[3] = {0, 0, 0};
+  bool chunk_split[3] = {false, false, false};
   int2* jobs_dev[3] = {nullptr, nullptr, nullptr};
   int64_t jobs_n[3] = {0, 0, 0};
   h2i::Profiler prof;

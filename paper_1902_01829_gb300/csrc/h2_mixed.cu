@@ -426,9 +426,11 @@ h2_status mixed_configure(h2_matrix_s* h, int chunk_opt, int cw, int tree_opt) {
     h2_status st = upload(h, &M.chunk_dev[chunk_opt], c.data(), (int64_t)c.size());
     if (st != H2_OK) return st;
     M.chunk_n[chunk_opt] = (int64_t)c.size();
+    M.chunk_split[chunk_opt] = slots > 0;
   }
   M.launch.chunks = M.chunk_dev[chunk_opt];
   M.launch.nchunks = M.chunk_n[chunk_opt];
+  M.launch.split = M.chunk_split[chunk_opt];
   M.launch.cw = cw;
   return H2_OK;
 }
@@ -1174,6 +1176,7 @@ h2_status batch_configure(h2_batch_s* b, int chunk_opt, int tree_opt, int cw) {
                                                     h->grid, false, &slots);
       if (slots > h->mx.cslots)
         return h2_fail(H2_ERR_INVALID, "internal: %lld coupling pieces exceed their slots", (long long)slots);
+      b->chunk_split[chunk_opt] = b->chunk_split[chunk_opt] || slots > 0;
       for (int4 c : own) {
         c.x = (int)i;
         chunks.push_back(c);
@@ -1209,6 +1212,7 @@ h2_status batch_configure(h2_batch_s* b, int chunk_opt, int tree_opt, int cw) {
   }
   L.chunks = b->chunk_dev[chunk_opt];
   L.nchunks = b->chunk_n[chunk_opt];
+  L.split = b->chunk_split[chunk_opt];
   L.jobs = b->jobs_dev[tree_opt];
   L.tree_T = T;
   L.njobs = b->jobs_n[tree_opt];

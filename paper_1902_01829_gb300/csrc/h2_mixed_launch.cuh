@@ -48,9 +48,12 @@ void bucket_phase(const MixedLaunch& L, int phase, int nvlo, cudaStream_t st, bo
     cudaFuncSetAttribute(k_downsweep_tree_m<FB, NVB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     prefer_max_shared(k_coupling_kf<RPL, NVB, 0>);
     prefer_max_shared(k_coupling_kf<RPL, NVB, 1>);
-    prefer_max_shared(k_coupling_m<F, 16, NVW, (NVW <= 2 ? 4 : 2), VG>);
-    prefer_max_shared(k_coupling_m<F, 32, NVW, (NVW <= 1 ? 2 : 1), VG>);
-    prefer_max_shared(k_coupling_m<F, 64, NVW, (NVW <= 1 ? 2 : 1), VG>);
+    prefer_max_shared(k_coupling_m<F, 16, NVW, (NVW <= 2 ? 4 : 2), VG, true>);
+    prefer_max_shared(k_coupling_m<F, 16, NVW, (NVW <= 2 ? 4 : 2), VG, false>);
+    prefer_max_shared(k_coupling_m<F, 32, NVW, (NVW <= 1 ? 2 : 1), VG, true>);
+    prefer_max_shared(k_coupling_m<F, 32, NVW, (NVW <= 1 ? 2 : 1), VG, false>);
+    prefer_max_shared(k_coupling_m<F, 64, NVW, (NVW <= 1 ? 2 : 1), VG, true>);
+    prefer_max_shared(k_coupling_m<F, 64, NVW, (NVW <= 1 ? 2 : 1), VG, false>);
     prefer_max_shared(k_coupling_m_generic<F, RPL, NVB>);
     return true;
   }();
@@ -78,16 +81,15 @@ void bucket_phase(const MixedLaunch& L, int phase, int nvlo, cudaStream_t st, bo
       // up to four vectors per warp; 8 and 16 vectors take two and four warps per chunk
       constexpr int NVW = NVB < 4 ? NVB : 4, VG = NVB / NVW;
       const unsigned grid = (unsigned)((L.nchunks * VG + 3) / 4);
-      if (k == 16) {
-        constexpr int CB = NVW <= 2 ? 4 : 2;
-        k_coupling_m<F, 16, NVW, CB, VG><<<grid, 128, 0, st>>>(mats, L.chunks, L.nchunks, nvlo, NVB);
-      } else if (k == 32) {
-        constexpr int CB = NVW <= 1 ? 2 : 1;
-        k_coupling_m<F, 32, NVW, CB, VG><<<grid, 128, 0, st>>>(mats, L.chunks, L.nchunks, nvlo, NVB);
-      } else {
-        constexpr int CB = NVW <= 1 ? 2 : 1;
-        k_coupling_m<F, 64, NVW, CB, VG><<<grid, 128, 0, st>>>(mats, L.chunks, L.nchunks, nvlo, NVB);
-      }
+      auto launch = [&](auto split) {
+        constexpr bool SPLIT = decltype(split)::value;
+        constexpr int CB16 = NVW <= 2 ? 4 : 2, CB = NVW <= 1 ? 2 : 1;
+        if (k == 16) k_coupling_m<F, 16, NVW, CB16, VG, SPLIT><<<grid, 128, 0, st>>>(mats, L.chunks, L.nchunks, nvlo, NVB);
+        else if (k == 32) k_coupling_m<F, 32, NVW, CB, VG, SPLIT><<<grid, 128, 0, st>>>(mats, L.chunks, L.nchunks, nvlo, NVB);
+        else k_coupling_m<F, 64, NVW, CB, VG, SPLIT><<<grid, 128, 0, st>>>(mats, L.chunks, L.nchunks, nvlo, NVB);
+      };
+      if (L.split) launch(std::true_type{});
+      else launch(std::false_type{});
     } else {
       k_coupling_m_generic<F, RPL, NVB><<<cgrid, 128, 0, st>>>(mats, L.chunks, L.nchunks, nvlo, NVB);
     }

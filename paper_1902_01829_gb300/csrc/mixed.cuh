@@ -538,7 +538,9 @@ __device__ __forceinline__ ChunkRows chunk_rows(const int32_t* __restrict__ Srow
 // in flight; after a row's last batch its sums are reduced over the lanes of
 // the same row group and stored. VG warps of a CTA share a chunk, warp w taking
 // vectors (w % VG) * NVW .. + NVW - 1 (the later ones read the blocks from L1).
-template <int F, int K, int NVW, int CB, int VG>
+// SPLIT: the launch has pieces of long rows (their state costs registers: K = 16, NVW = 4, VG = 2 goes from 128 to 156
+// and from four CTAs an SM to three; 2D n = 2^20, where no row is cut, 8 vectors: 417 us with it, 336 without).
+template <int F, int K, int NVW, int CB, int VG, bool SPLIT>
 __global__ void __launch_bounds__(128) k_coupling_m(const MatDesc* __restrict__ mats, const int4* __restrict__ chunks,
                                                    int64_t nchunks, int nvlo, int nvhi) {
   static_assert(K == 16 || K == 32 || K == 64, "octet layout");
@@ -562,7 +564,7 @@ __global__ void __launch_bounds__(128) k_coupling_m(const MatDesc* __restrict__ 
   const int kp = D.kp;
   const float* __restrict__ xhat = D.xhat;
   float* __restrict__ yhat = D.yhat;
-  const int row0 = ch.y, rows = min(ch.z & 0xFF, kChunkRows), parts = chunk_parts(ch), part = chunk_part(ch);
+  const int row0 = ch.y, rows = min(ch.z & 0xFF, kChunkRows), parts = SPLIT ? chunk_parts(ch) : 1, part = SPLIT ? chunk_part(ch) : 0;
   const ChunkRows cr = chunk_rows(D.Srow, yhat, row0, rows, nv, kp, lane, vbase, min(NVW, nv - vbase));
   if (!cr.nonempty) return;
   const int m = lane % RG, cl = lane / RG;
@@ -651,7 +653,7 @@ __global__ void __launch_bounds__(128) k_coupling_m(const MatDesc* __restrict__ 
 #pragma unroll
         for (int v = 0; v < NVW; v++) acc[rr][v] += __shfl_xor_sync(0xFFFFFFFFu, acc[rr][v], off);
     if (cl == 0) {
-      float* dst = chunk_dst(D, ch, row0 + r) + vbase * kp + 8 * m;
+      float* dst = SPLIT ? chunk_dst(D, ch, row0 + r) + vbase * kp + 8 * m : yhat + ((int64_t)(row0 + r) * nv + vbase) * kp + 8 * m;
 #pragma unroll
       for (int v = 0; v < NVW; v++)
         if (vbase + v < nv) {
@@ -676,7 +678,7 @@ __global__ void __launch_bounds__(128) k_coupling_m(const MatDesc* __restrict__ 
     c.bt = 0;
     c.b0 = __shfl_sync(0xFFFFFFFFu, cr.sr, c.r);
     int nb = __shfl_sync(0xFFFFFFFFu, cr.sr, c.r + 1) - c.b0;
-    if (parts > 1) {  // a piece of the row (its only row)
+    if (SPLIT && parts > 1) {  // a piece of the row (its only row)
       const int lo = (int)((int64_t)nb * part / parts);
       nb = (int)((int64_t)nb * (part + 1) / parts) - lo;
       c.b0 += lo;
@@ -736,7 +738,7 @@ __global__ void __launch_bounds__(128) k_coupling_m(const MatDesc* __restrict__ 
     if ((cc.bt + 1) * CB >= cc.nslot) flush(cc.r);
     if (!advance(cc)) break;
   }
-  if (parts > 1) split_finish(D, ch, warp % VG, vbase, min(NVW, nv - vbase), lane);
+  if (SPLIT && parts > 1) split_finish(D, ch, warp % VG, vbase, min(NVW, nv - vbase), lane);
 }
 
 // any other k: the chunk's rows one after another, one block at a time
