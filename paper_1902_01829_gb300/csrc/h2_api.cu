@@ -1036,7 +1036,7 @@ h2_status h2_tune(h2_handle h, int32_t nv, const double* x, int64_t ldx, double*
   if ((s = mixed_configure(h, best_opt, best_cw, best_tree)) != H2_OK) return s;
   chosen[0] = best_cw;
   chosen[1] = kChunkOpts[best_opt];
-  chosen[2] = 1 << (h->q - std::max(0, h->tree_L - best_tree));  // leaves per tree CTA
+  chosen[2] = h2i::mixed_tree_leaves(h, nv);
   return H2_OK;
 }
 

@@ -52,6 +52,7 @@ struct MixedLaunch {
   const int2* jobs = nullptr;        // (matrix, subtree) per tree CTA
   int64_t njobs = 0;
   int tree_T = 0;                    // levels below the subtree roots of the deepest job
+  int depth = 0, warp_L = -1;        // a single matrix: its depth and the subtree level of tree_warps.cuh's kernels
   const int4* chunks = nullptr;      // coupling row chunks (mixed.cuh)
   int64_t nchunks = 0;
   bool split = false;                // some chunk is a piece of a long row
@@ -295,6 +296,8 @@ h2_status validate_desc(const h2_desc* d, bool s_values, bool d_values, int64_t*
 h2_status mixed_launch(int storage, const MixedLaunch& L, unsigned buckets, cudaStream_t st, const TcPass* tc = nullptr);
 // precision form: use coupling chunk target option `chunk_opt`, `cw` dense consumer warps and
 // tree subtrees at level (default level - tree_opt)
+// leaves per tree CTA in the first pass of a product of nv vectors
+int mixed_tree_leaves(const h2_matrix_s* h, int nv);
 h2_status mixed_configure(h2_matrix_s* h, int chunk_opt, int cw, int tree_opt);
 // passes of at least this many vectors use the tensor-core dense phase (panel-layout handles)
 constexpr int kTcMinVectors = 8;

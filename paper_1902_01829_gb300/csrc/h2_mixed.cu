@@ -16,6 +16,7 @@
 #include "h2_internal.h"
 #include "mixed.cuh"
 #include "tc_dense.cuh"
+#include "tree_warps.cuh"
 
 namespace h2i {
 
@@ -391,6 +392,12 @@ void tree_jobs(int mat, int L, std::vector<int2>* jobs) {
   for (int t = 0; t < 1 << (L + spread); t++) jobs->push_back(make_int2(mat, (t & ((1 << spread) - 1)) ? -1 : t >> spread));
 }
 
+int mixed_tree_leaves(const h2_matrix_s* h, int nv) {
+  const MixedData& M = h->mx;
+  const bool warps = h2::warp_tree(h->q, h->k, kBucketNV[bucket_of(std::min(nv, kPassVectors))], M.bases_fp32);
+  return 1 << (warps ? h->q - M.launch.warp_L : M.launch.tree_T);
+}
+
 h2_status mixed_configure(h2_matrix_s* h, int chunk_opt, int cw, int tree_opt) {
   MixedData& M = h->mx;
   if (chunk_opt < 0 || chunk_opt > 2 || tree_opt < 0 || tree_opt > 2 ||
@@ -416,6 +423,8 @@ h2_status mixed_configure(h2_matrix_s* h, int chunk_opt, int cw, int tree_opt) {
     M.launch.jobs = M.jobs_dev[tree_opt];
     M.launch.tree_T = h->q - L;
     M.launch.njobs = std::max<int64_t>((int64_t)1 << L, h2::kTreeCluster);
+    M.launch.depth = h->q;
+    M.launch.warp_L = h2::warp_tree_level(h->q, h->grid, tree_opt);
     M.tree_opt = tree_opt;
   }
   if (!M.chunk_dev[chunk_opt]) {

@@ -8,6 +8,7 @@
 #include "mixed.cuh"
 #include "mma_dense.cuh"
 #include "tc_dense.cuh"
+#include "tree_warps.cuh"
 
 namespace h2i {
 
@@ -63,6 +64,15 @@ void bucket_phase(const MixedLaunch& L, int phase, int nvlo, cudaStream_t st, bo
   const int entries = tree_block_entries(L.k, round_up((int64_t)L.k * L.k, 8), FB != kFormF32);
   const unsigned tsm = tree_smem<TreeOpM<FB>, NVB>(L.k, entries, L.tree_T).bytes;
   const int dentries = tree_down_entries(L.k, round_up((int64_t)L.k * L.k, 8), FB != kFormF32);
+  if constexpr (RPL == 1 && NVB <= kWarpTreeMaxVectors) {
+    if (phase != 1 && L.warp_L >= 0 && warp_tree(L.depth, L.k, NVB, FB == kFormF32)) {
+      static const bool shared = (prefer_max_shared(k_upsweep_warps<FB, NVB>), prefer_max_shared(k_downsweep_warps<FB, NVB>), true);
+      (void)shared;
+      if (phase == 0) k_upsweep_warps<FB, NVB><<<1u << L.warp_L, kWarpTreeWarps * 32, 0, st>>>(mats, L.warp_L, convert ? 1 : 0);
+      else k_downsweep_warps<FB, NVB><<<1u << L.warp_L, kWarpTreeWarps * 32, 0, st>>>(mats, L.warp_L, expand);
+      return;
+    }
+  }
   if (phase == 0 && L.njobs > 0) {
     if constexpr (NVB <= 4) {
       if (!convert) {  // beside the dense stream

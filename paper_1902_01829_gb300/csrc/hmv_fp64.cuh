@@ -194,15 +194,15 @@ struct TreeOp64 {
   static constexpr bool kParts = true;
   static __device__ __forceinline__ bool want_parts(const P& T) { return T.oz != 0; }
   static __device__ __forceinline__ unsigned abs_bits(float2 x) { return __float_as_uint(x.x) & 0x7FFFFFFFu; }
-  // leaf j's vectors xs ([point][vector], stride VS) as digits (mma_fp64.cuh); vmax: float bits of max |x| per vector
-  template <int VS, int TH>
-  static __device__ __forceinline__ void parts(const P& T, int64_t j, int s, const float2* xs, const unsigned* vmax) {
+  // leaf j's vectors as digits (mma_fp64.cuh); arguments as TreeOpM::parts
+  static __device__ __forceinline__ void parts(const P& T, int64_t j, int s, const float2* xs, int cs, int vs,
+                                               const unsigned* vmax, int tid, int threads) {
     const int nh = T.nv > 8 ? 2 : 1;
     unsigned char* chunk = T.xd + j * xd_chunk_bytes(T.xks, nh);
     // |x| 2^(54 - ex) <= 0x7F7F7F7F7F7F7F, the digits' range: the exponent of the largest |x|, one more where its
     // fraction leaves no room
     auto ex = [&](int v) { return max((int)(vmax[v] >> 23) - ((vmax[v] & 0x7FFFFFu) < 0x7D0000u ? 127 : 126), kXdMinExp); };
-    for (int i = threadIdx.x; i < ((s + 15) >> 4) * 32 * nh; i += TH) {
+    for (int i = tid; i < ((s + 15) >> 4) * 32 * nh; i += threads) {
       const int ln = i & 31, u = i >> 5, ks = nh == 2 ? u >> 1 : u, half = nh == 2 ? u & 1 : 0;
       const int v = (ln >> 2) + 8 * half, c0 = 16 * ks + (ln & 3);
       const float up = __int_as_float((127 - (v < T.nv ? ex(v) : 0)) << 23);  // 2^-ex; 2^(54 - ex) may be no float
@@ -210,7 +210,7 @@ struct TreeOp64 {
 #pragma unroll
       for (int q = 0; q < 4; q++) {
         const int c = c0 + 4 * q;
-        const float2 x = (v < T.nv && c < s) ? xs[c * VS + v] : make_float2(0.f, 0.f);
+        const float2 x = (v < T.nv && c < s) ? xs[c * cs + v * vs] : make_float2(0.f, 0.f);
         const long long n = __float2ll_rn(x.x * up * 0x1p54f) + __float2ll_rn(x.y * up * 0x1p54f) + 0x80808080808080LL;
         lo[q] = (uint32_t)n;
         hi[q] = (uint32_t)((unsigned long long)n >> 32);
@@ -223,9 +223,8 @@ struct TreeOp64 {
       for (int p = 0; p < kXdDigits; p++) dst[32 * p] = make_uint2(d0[p], d1[p]);
     }
     // (a chunk with an infinity or NaN: kXdNaN makes its vector's sums NaN)
-    if (threadIdx.x < 16)
-      reinterpret_cast<int*>(chunk)[threadIdx.x] =
-          threadIdx.x >= T.nv ? kXdMinExp : vmax[threadIdx.x] >= 0x7F800000u ? kXdNaN : ex(threadIdx.x);
+    if (tid < 16)
+      reinterpret_cast<int*>(chunk)[tid] = tid >= T.nv ? kXdMinExp : vmax[tid] >= 0x7F800000u ? kXdNaN : ex(tid);
   }
   static __device__ __forceinline__ int copy_bytes(int entries) { return 8 * entries; }
   static __device__ __forceinline__ const char* U(const P& T, const Leaf& l) { return T.dmat + l.uoff; }

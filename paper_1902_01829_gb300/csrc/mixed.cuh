@@ -356,15 +356,16 @@ struct TreeOpM {
     T.x4[l.xp * T.nv + v * sp + a] = x;
   }
   static constexpr bool kParts = true;
-  // leaf j's vectors xs ([point][vector], stride VS) as 16-bit parts; vmax: float bits of max |x| per vector
-  template <int VS, int TH>
-  static __device__ __forceinline__ void parts(const P& T, int64_t j, int s, const float* xs, const unsigned* vmax) {
+  // leaf j's vectors (entry (point c, vector v) at xs[c * cs + v * vs]) as 16-bit parts, by `threads` threads of which this
+  // is `tid`; vmax: float bits of max |x| per vector
+  static __device__ __forceinline__ void parts(const P& T, int64_t j, int s, const float* xs, int cs, int vs, const unsigned* vmax,
+                                               int tid, int threads) {
     const int nh = T.nv > 8 ? 2 : 1;
     unsigned char* chunk = T.D->xp + j * xp_chunk_bytes(T.D->xks, nh);
     const bool bf = T.D->code_form == kFormBf16;
     // x = 2^(e - 14) (hi + mid + lo); e from the exponent bits, at least -110 so that 2^(14 - e) is finite
     auto shift = [&](int v) { return bf ? 0 : 14 - max((int)(vmax[v] >> 23) - 126, -110); };
-    for (int i = threadIdx.x; i < ((s + 15) >> 4) * 32 * nh; i += TH) {
+    for (int i = tid; i < ((s + 15) >> 4) * 32 * nh; i += threads) {
       const int ln = i & 31, u = i >> 5, ks = nh == 2 ? u >> 1 : u, half = nh == 2 ? u & 1 : 0;
       const int v = (ln >> 2) + 8 * half, c0 = 16 * ks + (ln & 3);
       const float up = __int_as_float((127 + (v < T.nv ? shift(v) : 0)) << 23);
@@ -372,7 +373,7 @@ struct TreeOpM {
 #pragma unroll
       for (int q = 0; q < 4; q++) {
         const int c = c0 + 4 * q;
-        x[q] = (v < T.nv && c < s) ? xs[c * VS + v] * up : 0.f;
+        x[q] = (v < T.nv && c < s) ? xs[c * cs + v * vs] * up : 0.f;
       }
       const bool finite = v >= T.nv || vmax[v] < 0x7F800000u;
       uint2* dst = reinterpret_cast<uint2*>(chunk + kXpScale + u * 768 + ln * 8);
@@ -397,8 +398,8 @@ struct TreeOpM {
         dst[32 * p] = make_uint2(w[0], w[1]);
       }
     }
-    if (threadIdx.x < 16) {
-      const int v = threadIdx.x;
+    if (tid < 16) {
+      const int v = tid;
       reinterpret_cast<float*>(chunk)[v] = v < T.nv ? __int_as_float((127 - shift(v)) << 23) : 0.f;
     }
   }
@@ -417,11 +418,13 @@ struct TreeOpM {
   }
 };
 
-// copy n floats (n a multiple of 4, both ends 16-byte aligned) into the warp's staging buffer
+// copy n floats (n a multiple of 4, both ends 16-byte aligned) into the warp's staging buffer; CG: read through L2 (written
+// by another CTA of the launch)
+template <bool CG = false>
 __device__ __forceinline__ void stage_vectors(float* __restrict__ dst, const float* __restrict__ src, int n, int lane) {
   const float4* s4 = reinterpret_cast<const float4*>(src);
   float4* d4 = reinterpret_cast<float4*>(dst);
-  for (int i = lane; i < n / 4; i += 32) d4[i] = s4[i];
+  for (int i = lane; i < n / 4; i += 32) d4[i] = CG ? __ldcg(s4 + i) : s4[i];
   __syncwarp();
 }
 

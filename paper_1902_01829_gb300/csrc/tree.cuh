@@ -376,7 +376,7 @@ __device__ __forceinline__ void tree_up(const typename Op::P& P, int64_t sub, bo
     };
     if (S.nbuf == 2) fetch_next(buf = cur ^ 1);
     if constexpr (Op::kParts) {
-      if (parts && !climbing && d == 0) Op::template parts<VS, TH>(P, j0 + t, C, x0, vmax + 16 * (t % 3));
+      if (parts && !climbing && d == 0) Op::parts(P, j0 + t, C, x0, VS, 1, vmax + 16 * (t % 3), threadIdx.x, TH);
     }
     const typename Op::A* A = reinterpret_cast<const typename Op::A*>(tree_dyn + cur * S.block);
 #pragma unroll 1
