@@ -457,7 +457,8 @@ cudaError_t set_pass_smem() {
     constexpr int CW = h2::dense_consumer_warps(NVB);
     cudaError_t e = cudaSuccess;
     if constexpr (NVB > 4) {
-      e = cudaFuncSetAttribute(h2::k_dense_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, h2::kOzSmem);
+      for (const void* f : {(const void*)h2::k_dense_oz<false>, (const void*)h2::k_dense_oz<true>})
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, h2::kOzSmem);
     } else {
       e = cudaFuncSetAttribute(h2::k_dense_stream<NVB, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                h2::stream_smem_bytes(NVB, CW));
@@ -555,7 +556,8 @@ h2_status run_pass(h2_matrix_s* h, int nv, const double* x, int64_t ldx, double*
       P.xd = h->xd;
       P.x2 = h->x2;
       P.xks = T.xks;
-      k_dense_oz<<<h->grid, (kOzWarps + 1) * 32, kOzSmem, st>>>(P);
+      if (h->wide) k_dense_oz<true><<<h->grid, (kOzWarps + 1) * 32, kOzSmem, st>>>(P);
+      else k_dense_oz<false><<<h->grid, (kOzWarps + 1) * 32, kOzSmem, st>>>(P);
     } else {
       StreamParams P{};
       common(P);
@@ -779,6 +781,7 @@ h2_status build_device(h2_matrix_s* h, const h2_desc* d) {
       if ((st = upload(h, &h->eY, R.eY.data(), h->leaves)) != H2_OK) return st;
     }
     // the digits' tables (see mma_fp64.cuh), per item = per dense block
+    for (char w : R.d_wide) h->wide = h->wide || w;
     if ((st = upload(h, &h->item_exp, R.d_exp.data(), h->nD)) != H2_OK) return st;
     if ((st = upload(h, &h->item_leaf, d->D_colidx, h->nD)) != H2_OK) return st;
     if ((st = dalloc(h, &h->xd, h->leaves * h2::xd_chunk_bytes((h->m_max + 15) / 16, 2))) != H2_OK) return st;

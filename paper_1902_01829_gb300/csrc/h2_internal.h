@@ -217,6 +217,7 @@ struct h2_matrix_s {
   int32_t* oE = nullptr;
   int2* Sco = nullptr;
   // passes of more than four vectors: the dense phase by digits (k_dense_oz)
+  bool wide = false;                  // some dense block is wide (mma_fp64.cuh)
   int* item_exp = nullptr;            // per dense item: its block's exponent and column leaf
   int* item_leaf = nullptr;
   unsigned char* xd = nullptr;        // digits of the pass's vectors

@@ -290,42 +290,51 @@ __device__ __forceinline__ void mma_block(uint32_t base, int cb, uint32_t X, int
     for (int e = 0; e < 4; e++) run[i][e] = fmaf(s0 * sc[e >> 1], hi[i][e] + lo[i][e], run[i][e]);
 }
 
-// The same of a wide block, in FP32: codes at `codes`, vectors X ([vector][vs points]); n = 2t + (e & 1), its four rows
-// from row rows[e & 1], tile i the i-th of them. Bound by issue slots like the streams: 1,500 cycles an SM for a 64 x 64
-// block.
-template <int F>
+// The same of a wide block, in FP32, for up to 8 NH vectors: codes at `codes`, vectors X ([vector][vs points]); n = 2t +
+// (e & 1), its four rows from row rows[e & 1], tile i the i-th of them (rows past R are not stored). Bound by issue slots
+// like the streams (2D n = 50,001, int16, every block wide: dense phase of 8 / 16 vectors 105 / 131 us; rows loaded one by
+// one and both halves whatever the count: 188 / 190; the stream with as many vectors 166 / 217).
+// FOUR: a column's four rows are one aligned load.
+template <int F, int NH, bool FOUR>
 __device__ __forceinline__ void mma_wide_block(const unsigned char* codes, bool panel, const float* X, int vs, int C, int R,
                                                const int (&rows)[2], float scale, int nv, float (&run)[4][4]) {
-  using T = typename CodeT<F>::T;
   const int g = (threadIdx.x & 31) >> 2;
-  float acc[4][4];
+  float acc[4][2 * NH];
 #pragma unroll
   for (int i = 0; i < 4; i++)
 #pragma unroll
-    for (int e = 0; e < 4; e++) acc[i][e] = 0.f;
-  const T* A[2];
+    for (int e = 0; e < 2 * NH; e++) acc[i][e] = 0.f;
+  const uint16_t* A[2];
 #pragma unroll
   for (int u = 0; u < 2; u++)
-    A[u] = reinterpret_cast<const T*>(codes) + (panel ? (rows[u] >> 3) * (panel_stride(C) / 2) + (rows[u] & 7) : rows[u]);
+    A[u] = reinterpret_cast<const uint16_t*>(codes) + (panel ? (rows[u] >> 3) * (panel_stride(C) / 2) + (rows[u] & 7) : rows[u]);
   const int cs = panel ? 8 : code_stride(R);
-#pragma unroll 2
+#pragma unroll 4
   for (int c = 0; c < C; c++) {
-    float x[2];
+    float x[NH];
 #pragma unroll
-    for (int b = 0; b < 2; b++) x[b] = g + 8 * b < nv ? X[(g + 8 * b) * vs + c] : 0.f;
+    for (int b = 0; b < NH; b++) x[b] = g + 8 * b < nv ? X[(g + 8 * b) * vs + c] : 0.f;
 #pragma unroll
-    for (int u = 0; u < 2; u++)
+    for (int u = 0; u < 2; u++) {
+      float a[4];
+      if constexpr (FOUR) {
+        const uint2 w = *reinterpret_cast<const uint2*>(A[u] + c * cs);
+        const float2 lo = codes_to_f2<F>(w.x), hi = codes_to_f2<F>(w.y);
+        a[0] = lo.x, a[1] = lo.y, a[2] = hi.x, a[3] = hi.y;
+      } else {
 #pragma unroll
-      for (int i = 0; i < 4; i++) {
-        const float a = rows[u] + i < R ? code_to_f<F>(A[u][c * cs + i]) : 0.f;
-#pragma unroll
-        for (int b = 0; b < 2; b++) acc[i][u + 2 * b] = fmaf(a, x[b], acc[i][u + 2 * b]);
+        for (int i = 0; i < 4; i++) a[i] = rows[u] + i < R ? code_to_f<F>(A[u][c * cs + i]) : 0.f;
       }
+#pragma unroll
+      for (int i = 0; i < 4; i++)
+#pragma unroll
+        for (int b = 0; b < NH; b++) acc[i][u + 2 * b] = fmaf(a[i], x[b], acc[i][u + 2 * b]);
+    }
   }
 #pragma unroll
   for (int i = 0; i < 4; i++)
 #pragma unroll
-    for (int e = 0; e < 4; e++) run[i][e] = fmaf(scale, acc[i][e], run[i][e]);
+    for (int e = 0; e < 2 * NH; e++) run[i][e] = fmaf(scale, acc[i][e], run[i][e]);
 }
 
 // (WIDE in every launch: 32 matrices of 1024 .. 16384 points, fp16, 667 -> 674 us with no wide block among them)
@@ -371,8 +380,13 @@ __global__ void __launch_bounds__((kMmaWarps + 1) * 32, 1) k_dense_mma(MixedStre
         const int moff = min(bh.z, kStageMat - 16) & ~15, voff = min(bh.y, kMmaArea - 16) & ~15;
         if (WIDE && ((bh.x >> 18) & 1)) {
           const int n0 = two ? 8 * 2 * t + 4 * (turn & 1) : 4 * 2 * t, rows[2] = {n0, n0 + (two ? 8 : 4)};
-          mma_wide_block<F>(stage + kMixedHeader + moff, panel, reinterpret_cast<const float*>(stage + kMixedHeader + voff),
-                            min((int)((unsigned)bh.x >> 24), 64), C, R, rows, __int_as_float(bh.w), nv, run);
+          const unsigned char* wc = stage + kMixedHeader + moff;
+          const float* wx = reinterpret_cast<const float*>(stage + kMixedHeader + voff);
+          const int vs = min((int)((unsigned)bh.x >> 24), 64);
+          const bool four = panel || (code_stride(R) & 3) == 0;
+          if (four && nh == 1) mma_wide_block<F, 1, true>(wc, panel, wx, vs, C, R, rows, __int_as_float(bh.w), nv, run);
+          else if (four) mma_wide_block<F, 2, true>(wc, panel, wx, vs, C, R, rows, __int_as_float(bh.w), nv, run);
+          else mma_wide_block<F, 2, false>(wc, panel, wx, vs, C, R, rows, __int_as_float(bh.w), nv, run);
           continue;
         }
         const uint32_t codes = smem_addr(stage + kMixedHeader) + moff, X = smem_addr(stage + kMixedHeader) + voff;

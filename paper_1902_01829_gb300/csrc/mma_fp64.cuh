@@ -23,7 +23,7 @@
 // about 800 issue slots, and its 32 KB 1,400 at the copy bandwidth. Measured, 2D n = 50,001 (48- and 49-point leaves),
 // 16 vectors: six digits 837 -> 404 us in the dense phase, error against 64 bits 2.6e-14 -> 2.1e-14 (weight 6 left
 // out: 7e-14; the sums joined without the third exact step: 1e-13); seven digits with the vectors' fragments loaded
-// one at a time (76 bytes of spills less) 682 -> 669 us in the product, error 2.0e-14. About 5,000 cycles a block are
+// one at a time (60 bytes of spills less) 397 -> 375 us, error 2.0e-14. About 4,600 cycles a block are
 // still the chain of slicing, loads and MMAs of three warps a scheduler, not a pipe.
 //
 // Y^T = X^T D^T as in mma_dense.cuh: the vectors' digits are the A operand, written in fragment order by
@@ -116,6 +116,7 @@ struct OzParams {
 };
 
 // Producer warp. Stage header (ints): R, C, flags, row, ea, vector stride of a wide block.
+template <bool WIDE>
 __device__ __forceinline__ void oz_produce(const OzParams& P, const StreamShared& S, int ib, int ie) {
   const int lane = threadIdx.x & 31;
   const uint64_t pol = policy_evict_first();
@@ -154,7 +155,7 @@ __device__ __forceinline__ void oz_produce(const OzParams& P, const StreamShared
         unsigned char* stage = S.stage0 + s * kOzStage;
         int* h = reinterpret_cast<int*>(stage);
         const int C = (int)((shape >> 8) & 0xFF), vs = (int)((shape >> 16) & 0xFF);
-        const bool wide = (flags & kItemFlagWide) != 0;
+        const bool wide = WIDE && (flags & kItemFlagWide) != 0;
         h[0] = (int)(shape & 0xFF);
         h[1] = C;
         h[2] = flags;
@@ -255,33 +256,68 @@ __device__ __forceinline__ void oz_block(const double* A, uint32_t X, int R, int
   }
 }
 
-// The same quarter of a wide block in double-float: the block split with its offset o, the vectors' pairs X
-// ([vector][vs points]); acc[i][e] of rows r = 16 quarter + 4 t + 2 (e & 1) + i and vectors g (e < 2) and g + 8.
-__device__ __forceinline__ void oz_wide_block(const double* A, const float2* X, int R, int C, int vs, int r, int o, int nv,
-                                              float2 (&acc)[2][4]) {
-  const int g = (threadIdx.x & 31) >> 2;
+// (s, c) added to a running pair (fresh: the first)
+__device__ __forceinline__ void oz_put(float2* slot, bool fresh, float s, float c) {
+  float2 p = fresh ? make_float2(0.f, 0.f) : *slot;
+  df_add(p.x, p.y, s, c);
+  *slot = p;
+}
+
+// The same quarter of a wide block in double-float: the block split with its offset o, the vectors' pairs X ([vector][vs
+// points]), the sums added to the warp's running pairs. A lane has rows r, r + 1 (r = 16 quarter + 2 (lane % 8)) and four
+// vectors; with up to eight vectors (CS = 2) the half-warps take every second column and join their sums at the end.
+// Bound by issue slots like the double-float stream (2D n = 50,001, every block wide: dense phase of 8 / 16 vectors 516 /
+// 873 us, the stream's 506 / 820; with four rows and two vectors a lane, whatever the count, 909 / 917). Not inlined: its
+// registers would be oz_block's.
+template <int CS>
+__device__ __noinline__ void oz_wide_block(const double* A, const float2* X, int R, int C, int vs, int quarter, int o, int nv,
+                                           float2* mine, bool fresh) {
+  __builtin_assume(__isShared(A) && __isShared(X) && __isShared(mine));
+  const int lane = threadIdx.x & 31, r = 16 * quarter + 2 * (lane & 7), v0 = 4 * ((lane >> 3) & (CS == 2 ? 1 : 3));
+  const int c0 = CS == 2 ? lane >> 4 : 0, Cr = r < R ? C : 0;
+  float2 acc[2][4];
 #pragma unroll
   for (int i = 0; i < 2; i++)
 #pragma unroll
-    for (int e = 0; e < 4; e++) acc[i][e] = make_float2(0.f, 0.f);
-#pragma unroll 1
-  for (int c = 0; c < C; c++) {
-    float2 x[2];
+    for (int v = 0; v < 4; v++) acc[i][v] = make_float2(0.f, 0.f);
+  const bool pair = (R & 1) == 0;
+#pragma unroll 2
+  for (int c = c0; c < Cr; c += CS) {
+    const double* src = A + r + R * c;
+    double a[2];
+    if (pair) {
+      const double2 d = *reinterpret_cast<const double2*>(src);
+      a[0] = d.x;
+      a[1] = d.y;
+    } else {
+      a[0] = src[0];
+      a[1] = r + 1 < R ? src[1] : 0.0;
+    }
+    float h[2], l[2];
 #pragma unroll
-    for (int b = 0; b < 2; b++) x[b] = g + 8 * b < nv ? X[(g + 8 * b) * vs + c] : make_float2(0.f, 0.f);
+    for (int i = 0; i < 2; i++) split_f64(a[i], o, h[i], l[i]);
 #pragma unroll
-    for (int q = 0; q < 4; q++) {
-      float h, l;
-      split_f64(r + q < R ? A[r + q + R * c] : 0.0, o, h, l);
+    for (int v = 0; v < 4; v++) {
+      const float2 x = v0 + v < nv ? X[(v0 + v) * vs + c] : make_float2(0.f, 0.f);
 #pragma unroll
-      for (int b = 0; b < 2; b++) {
-        float2& p = acc[q & 1][(q >> 1) + 2 * b];
-        df_fma(p.x, p.y, h, l, x[b].x, x[b].y);
-      }
+      for (int i = 0; i < 2; i++) df_fma(acc[i][v].x, acc[i][v].y, h[i], l[i], x.x, x.y);
     }
   }
+  __syncwarp();  // (a digit block's pairs are other lanes')
+#pragma unroll
+  for (int i = 0; i < 2; i++)
+#pragma unroll
+    for (int v = 0; v < 4; v++) {
+      if constexpr (CS == 2)
+        df_add(acc[i][v].x, acc[i][v].y, __shfl_xor_sync(0xFFFFFFFFu, acc[i][v].x, 16), __shfl_xor_sync(0xFFFFFFFFu, acc[i][v].y, 16));
+      if (CS == 1 || i == c0)  // (half-warp i stores row i of the joined sums)
+        oz_put(mine + (v0 + v) * kOzRedStride + (r & 15) + i, fresh, acc[i][v].x, acc[i][v].y);
+    }
+  __syncwarp();
 }
 
+// WIDE: the handle has wide blocks (with their code inlined in the only kernel: 407 us at 2D n = 50,001, 375 without it)
+template <bool WIDE>
 __global__ void __launch_bounds__((kOzWarps + 1) * 32, 1) k_dense_oz(OzParams P) {
   extern __shared__ __align__(1024) unsigned char smem[];
   const StreamShared S = stream_shared<kOzStages, kOzStage>(smem);
@@ -289,7 +325,7 @@ __global__ void __launch_bounds__((kOzWarps + 1) * 32, 1) k_dense_oz(OzParams P)
   const int ib = P.cta_begin[blockIdx.x], ie = P.cta_begin[blockIdx.x + 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   if (warp == kOzWarps) {
-    oz_produce(P, S, ib, ie);
+    oz_produce<WIDE>(P, S, ib, ie);
     return;
   }
   StreamParams W{};
@@ -315,21 +351,12 @@ __global__ void __launch_bounds__((kOzWarps + 1) * 32, 1) k_dense_oz(OzParams P)
         const int shift = item_offset(flags);  // the row's output exponent (o of its blocks)
         const double* A = reinterpret_cast<const double*>(stage + kStageHeader);
         const unsigned char* xs = stage + kStageHeader + kStageMat;
-        // the lane's sums are added to its slots: tile i, element e are row 4 t + 2 (e & 1) + i, vector g + 8 (e >> 1)
-        auto put = [&](int i, int e, float s, float c) {
-          float2* slot = mine + (g + 8 * (e >> 1)) * kOzRedStride + 2 * (2 * t + (e & 1)) + i;
-          float2 p = fresh ? make_float2(0.f, 0.f) : *slot;
-          df_add(p.x, p.y, s, c);
-          *slot = p;
-        };
-        if (flags & kItemFlagWide) {
-          float2 acc[2][4];
-          oz_wide_block(A, reinterpret_cast<const float2*>(xs), R, C, min(h[5], 64), 16 * turn + 4 * t, shift, nv, acc);
+        if (WIDE && (flags & kItemFlagWide)) {
           if (fresh && !(ok = open_row())) break;
-#pragma unroll
-          for (int i = 0; i < 2; i++)
-#pragma unroll
-            for (int e = 0; e < 4; e++) put(i, e, acc[i][e].x, acc[i][e].y);
+          const float2* X = reinterpret_cast<const float2*>(xs);
+          const int vs = min(h[5], 64);
+          if (nh == 1) oz_wide_block<2>(A, X, R, C, vs, turn, shift, nv, mine, fresh);
+          else oz_wide_block<1>(A, X, R, C, vs, turn, shift, nv, mine, fresh);
           fresh = false;
           continue;
         }
@@ -355,7 +382,8 @@ __global__ void __launch_bounds__((kOzWarps + 1) * 32, 1) k_dense_oz(OzParams P)
             two_sum(s1, acc[i][2][e] * 0x1p-38f, s2, e2);
             two_sum(s2, acc[i][3][e] * 0x1p-46f, s3, e3);
             const float fb = f[e >> 1];
-            put(i, e, s3 * fb, (((e1 + e2) + e3) + tail) * fb);
+            // tile i, element e: row 4 t + 2 (e & 1) + i, vector g + 8 (e >> 1)
+            oz_put(mine + (g + 8 * (e >> 1)) * kOzRedStride + 4 * t + 2 * (e & 1) + i, fresh, s3 * fb, (((e1 + e2) + e3) + tail) * fb);
           }
         fresh = false;
       }
