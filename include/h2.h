@@ -402,6 +402,8 @@ h2_status h2_batch_matvec(h2_batch b, const int32_t* nv, const double* const* x,
  *                           four vectors)
  *   coupling row chunks:    about 64, 128 or 256 coupling blocks per warp
  *   tree jobs:              subtrees of 16, 32 or 64 leaves per group of eight CTAs
+ *                           (per CTA where a warp takes a node: k <= 16, up to eight
+ *                           vectors, 2^14 leaves in all)
  * (one warm-up and two timed batched products each, arguments as for
  * h2_batch_matvec), then the split of the dense work items over the CTAs:
  * each leaf row weighed by its bytes (its cycles in passes of more than four

@@ -52,7 +52,12 @@ struct MixedLaunch {
   const int2* jobs = nullptr;        // (matrix, subtree) per tree CTA
   int64_t njobs = 0;
   int tree_T = 0;                    // levels below the subtree roots of the deepest job
-  int depth = 0, warp_L = -1;        // a single matrix: its depth and the subtree level of tree_warps.cuh's kernels
+  // tree_warps.cuh: the vector-count buckets that take its kernels, and their (matrix, subtree) per CTA (null: one matrix)
+  // and levels of a CTA's subtree
+  unsigned warp_buckets = 0;
+  const int2* warp_jobs = nullptr;
+  int64_t warp_njobs = 0;
+  int warp_T = 0;
   const int4* chunks = nullptr;      // coupling row chunks (mixed.cuh)
   int64_t nchunks = 0;
   bool split = false;                // some chunk is a piece of a long row
@@ -319,6 +324,8 @@ struct h2_batch_s {
   bool chunk_split[3] = {false, false, false};
   int2* jobs_dev[3] = {nullptr, nullptr, nullptr};
   int64_t jobs_n[3] = {0, 0, 0};
+  int2* wjobs_dev[3] = {nullptr, nullptr, nullptr};
+  int64_t wjobs_n[3] = {0, 0, 0};
   h2i::Profiler prof;
   int64_t n_items = 0, device_bytes = 0;
   std::vector<void*> allocs;

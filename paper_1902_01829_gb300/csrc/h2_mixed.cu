@@ -394,8 +394,8 @@ void tree_jobs(int mat, int L, std::vector<int2>* jobs) {
 
 int mixed_tree_leaves(const h2_matrix_s* h, int nv) {
   const MixedData& M = h->mx;
-  const bool warps = h2::warp_tree(h->q, h->k, kBucketNV[bucket_of(std::min(nv, kPassVectors))], M.bases_fp32);
-  return 1 << (warps ? h->q - M.launch.warp_L : M.launch.tree_T);
+  const bool warps = (M.launch.warp_buckets >> bucket_of(std::min(nv, kPassVectors))) & 1u;
+  return 1 << (warps ? M.launch.warp_T : M.launch.tree_T);
 }
 
 h2_status mixed_configure(h2_matrix_s* h, int chunk_opt, int cw, int tree_opt) {
@@ -423,8 +423,11 @@ h2_status mixed_configure(h2_matrix_s* h, int chunk_opt, int cw, int tree_opt) {
     M.launch.jobs = M.jobs_dev[tree_opt];
     M.launch.tree_T = h->q - L;
     M.launch.njobs = std::max<int64_t>((int64_t)1 << L, h2::kTreeCluster);
-    M.launch.depth = h->q;
-    M.launch.warp_L = h2::warp_tree_level(h->q, h->grid, tree_opt);
+    M.launch.warp_T = h2::warp_tree_levels(h->q, h->grid, tree_opt);
+    M.launch.warp_njobs = (int64_t)1 << (h->q - M.launch.warp_T);
+    M.launch.warp_buckets = 0;
+    for (int b = 0; b < kBuckets; b++)
+      if (h2::warp_tree(h->q, h->k, kBucketNV[b], M.bases_fp32)) M.launch.warp_buckets |= 1u << b;
     M.tree_opt = tree_opt;
   }
   if (!M.chunk_dev[chunk_opt]) {
@@ -1204,6 +1207,22 @@ h2_status batch_configure(h2_batch_s* b, int chunk_opt, int tree_opt, int cw) {
     if ((st = balloc(b, &b->jobs_dev[tree_opt], (int64_t)jobs.size(), jobs.data())) != H2_OK) return st;
     b->jobs_n[tree_opt] = (int64_t)jobs.size();
   }
+  // (a CTA of tree_warps.cuh takes as many leaves as a cluster of tree.cuh)
+  const int wT = T + h2::kTreeClusterLog;
+  int64_t leaves = 0;
+  for (const h2_matrix_s* h : b->hs) leaves += h->leaves;
+  const bool warps = h2::warp_tree_batch(leaves, L.k);
+  if (warps && !b->wjobs_dev[tree_opt]) {
+    std::vector<int2> jobs;
+    for (int64_t i = 0; i < count; i++)
+      for (int t = 0; t < 1 << std::max(0, b->hs[(size_t)i]->q - wT); t++) jobs.push_back(make_int2((int)i, t));
+    if ((st = balloc(b, &b->wjobs_dev[tree_opt], (int64_t)jobs.size(), jobs.data())) != H2_OK) return st;
+    b->wjobs_n[tree_opt] = (int64_t)jobs.size();
+  }
+  L.warp_buckets = warps ? 15u : 0u;
+  L.warp_jobs = b->wjobs_dev[tree_opt];
+  L.warp_njobs = b->wjobs_n[tree_opt];
+  L.warp_T = wT;
   if (!L.mats || tree_opt != b->tree_opt) {  // the descriptors carry each member's subtree level
     std::vector<h2::MatDesc> descs((size_t)count);
     for (int64_t i = 0, r0 = 0; i < count; r0 += b->hs[(size_t)i]->leaves, i++) {

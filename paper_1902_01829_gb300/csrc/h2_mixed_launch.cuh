@@ -65,11 +65,13 @@ void bucket_phase(const MixedLaunch& L, int phase, int nvlo, cudaStream_t st, bo
   const unsigned tsm = tree_smem<TreeOpM<FB>, NVB>(L.k, entries, L.tree_T).bytes;
   const int dentries = tree_down_entries(L.k, round_up((int64_t)L.k * L.k, 8), FB != kFormF32);
   if constexpr (RPL == 1 && NVB <= kWarpTreeMaxVectors) {
-    if (phase != 1 && L.warp_L >= 0 && warp_tree(L.depth, L.k, NVB, FB == kFormF32)) {
+    constexpr int B = NVB == 1 ? 0 : NVB == 2 ? 1 : NVB == 4 ? 2 : 3;  // (the bucket)
+    if (phase != 1 && ((L.warp_buckets >> B) & 1u)) {
       static const bool shared = (prefer_max_shared(k_upsweep_warps<FB, NVB>), prefer_max_shared(k_downsweep_warps<FB, NVB>), true);
       (void)shared;
-      if (phase == 0) k_upsweep_warps<FB, NVB><<<1u << L.warp_L, kWarpTreeWarps * 32, 0, st>>>(mats, L.warp_L, convert ? 1 : 0);
-      else k_downsweep_warps<FB, NVB><<<1u << L.warp_L, kWarpTreeWarps * 32, 0, st>>>(mats, L.warp_L, expand);
+      const unsigned grid = (unsigned)L.warp_njobs, threads = kWarpTreeWarps * 32;
+      if (phase == 0) k_upsweep_warps<FB, NVB><<<grid, threads, 0, st>>>(mats, L.warp_jobs, nvlo, L.warp_T, convert ? 1 : 0);
+      else k_downsweep_warps<FB, NVB><<<grid, threads, 0, st>>>(mats, L.warp_jobs, nvlo, L.warp_T, expand);
       return;
     }
   }

@@ -5,10 +5,10 @@
 // its block from global memory straight into registers and keeps only the vectors in shared memory (256 bytes a
 // vector), with no barrier inside a level; a CTA of tree.cuh takes one node at a time with all its warps, needs
 // 10 KB a CTA for its blocks (four CTAs beside the dense stream) and idles half of its warps where a step has fewer
-// tasks than warps (k = 16, up to eight vectors). One launch per phase; CTA b owns the subtree of node b of level L,
+// tasks than warps (k = 16, up to eight vectors). One launch per phase; a CTA owns a subtree of T levels,
 // the nodes above it are climbed with a ticket per level, the second CTA to arrive at a parent taking it.
 // 2D n = 2^20, int16 with FP32 bases, phases in order, tree.cuh -> here: upsweep / downsweep of one vector 118 / 86 -> 84 /
-// 48 us, of four 228 / 150 -> 112 / 70, of eight 297 / 183 -> 208 / 157.
+// 48 us, of four 228 / 150 -> 112 / 70, of eight 297 / 183 -> 175 / 165.
 #pragma once
 #include <algorithm>
 
@@ -22,18 +22,34 @@ constexpr int kWarpTreeWarps = 8, kWarpTreeMaxVectors = 8;
 //   vectors             1                      2                      4                       8
 //   depth 10     105/112  100/135       118/133  114/149      149/145  151/170        188/223   166/210
 //   depth 11     143/147  150/180       164/174  163/192      231/194  238/221        308/325   260/291
-//   depth 12     217/209  234/242       254/247  254/256      391/299  400/318        537/505   445/432
-//   depth 14     686/643  756/741       846/790  856/831    1292/1036 1331/1068     1812/1697 1432/1347
+//   depth 12     217/209  234/242       254/247  254/256      391/299  400/318        537/499   445/422
+//   depth 14     686/643  756/741       846/790  856/831    1292/1036 1331/1058     1812/1671 1432/1331
 // k = 9: 270 -> 260 at depth 12, one vector; k = 25: 576 -> 625 (above 16 rows a warp takes one column at a time).
 inline bool warp_tree(int q, int k, int nvb, bool bases_fp32) {
   if (k > 16 || nvb > kWarpTreeMaxVectors) return false;
   return q >= (nvb == 4 ? 11 : nvb <= 2 && !bases_fp32 ? 13 : 12);
 }
-// level of the CTAs' subtrees: two CTAs an SM; opt: the tuner's choice (one or two levels higher)
-inline int warp_tree_level(int q, int sms, int opt) {
+// The same for a batch, all of whose members' trees count. fp16, 32-point leaves, product in us, tree.cuh / these: 64
+// members of 4,096 .. 32,768 points (some 40,000 leaves), 1, 2, 4, 8 vectors 2539/2459, 2812/2766, 3078/2928, 2530/2075;
+// 128 members of 4,096 .. 131,072, 1 to 16 vectors 13853/12352. The tree phases of 32 members of 1,024 .. 16,384 (some
+// 8,000 leaves) took as long a warp per node as they do here.
+constexpr int64_t kWarpTreeBatchLeaves = 1 << 14;
+inline bool warp_tree_batch(int64_t leaves, int k) { return k <= 16 && leaves >= kWarpTreeBatchLeaves; }
+// levels of the CTAs' subtrees: two CTAs an SM; opt: the tuner's choice (one or two levels more)
+inline int warp_tree_levels(int q, int sms, int opt) {
   int L = 0;
   while ((1 << L) < 2 * sms) L++;
-  return std::max(0, std::min(L, q) - opt);
+  return q - std::max(0, std::min(L, q) - opt);
+}
+
+// leaf j's 16-bit parts for passes of up to four vectors (a batch's; a function of its own: few launches want them, and its
+// registers would be the projection's; as a call in the variant of eight vectors it took 40 us more at 2D n = 2^20)
+template <int F>
+__device__ __noinline__ void leaf_parts_w(const MatDesc* D, int64_t j, int s, const float* xs, int spad, const unsigned* vmax) {
+  TreeParamsM P{};
+  P.nv = D->nv;
+  P.D = D;
+  TreeOpM<F>::parts(P, j, s, xs, 1, spad, vmax, threadIdx.x & 31, 32);
 }
 
 // the leaf's x (convert: from the product's own x, whose FP32 copy and 16-bit parts are left here) times V_j^T
@@ -53,7 +69,7 @@ __device__ __forceinline__ void project_leaf_w(const TreeParamsM& P, int LR, int
         const int a = lane + 32 * h;
         xr[v][h] = (v < P.nv && a < sj) ? x_load(P.x, P.xy32, off + v * P.ldx + a) : 0.f;  // padding is zero
       }
-    const bool parts = NVB > 4 && TreeOpM<F>::want_parts(P);
+    const bool parts = TreeOpM<F>::want_parts(P);  // (in a batch also for members of few vectors)
 #pragma unroll
     for (int v = 0; v < NVB; v++) {
       if (v >= P.nv) break;
@@ -71,7 +87,11 @@ __device__ __forceinline__ void project_leaf_w(const TreeParamsM& P, int LR, int
       }
     }
     __syncwarp();
-    if (parts) TreeOpM<F>::parts(P, j, sj, wbuf, 1, spad, vmax, lane, 32);
+    if constexpr (NVB > 4) {
+      if (parts) TreeOpM<F>::parts(P, j, sj, wbuf, 1, spad, vmax, lane, 32);
+    } else {
+      if (parts) leaf_parts_w<F>(P.D, j, sj, wbuf, spad, vmax);
+    }
   } else {
     stage_vectors(wbuf, xj, P.nv * spad, lane);  // the FP32 copy of x(j), padding zero
   }
@@ -100,16 +120,20 @@ __device__ __forceinline__ void up_node_w(const TreeParamsM& P, int LR, int64_t 
   store_node_m<1, NVB, false>(P.xhat + (p * P.nv + v0) * P.kp, P.k, P.kp, LR, nw, acc, lane);
 }
 
-// leaf projection and the whole upsweep (Alg. 2, Eq. 2) of a single matrix
+// leaf projection and the whole upsweep (Alg. 2, Eq. 2): CTA b works on subtree jobs[b].y of matrix jobs[b].x (without jobs:
+// subtree b of the only matrix); the matrices of fewer than nvlo or more than NVB vectors are left to another launch
 template <int F, int NVB>
-__global__ void __launch_bounds__(kWarpTreeWarps * 32) k_upsweep_warps(const MatDesc* __restrict__ mats, int L, int convert) {
+__global__ void __launch_bounds__(kWarpTreeWarps * 32, NVB == 2 ? 4 : 0) k_upsweep_warps(const MatDesc* __restrict__ mats,
+                                                                        const int2* __restrict__ jobs, int nvlo, int Tmax, int convert) {
   __shared__ __align__(16) float wstage[kWarpTreeWarps][NVB * 64];
   __shared__ unsigned vmax[kWarpTreeWarps][16];
   __shared__ int second;
-  const TreeParamsM P = tree_params(mats[0]);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, LR = mats[0].LR, T = P.q - L;
+  const int2 job = jobs ? jobs[blockIdx.x] : make_int2(0, (int)blockIdx.x);
+  const TreeParamsM P = tree_params(mats[job.x]);
+  if (P.nv < nvlo || P.nv > NVB) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, LR = P.D->LR, T = min(Tmax, P.q), L = P.q - T;
   float* wbuf = wstage[warp];
-  const int64_t sub = blockIdx.x;
+  const int64_t sub = job.y;
   for (int t = warp; t < 1 << T; t += kWarpTreeWarps)
     project_leaf_w<F, NVB>(P, LR, (sub << T) + t, lane, wbuf, vmax[warp], convert != 0);
   __syncthreads();
@@ -201,15 +225,18 @@ __device__ __forceinline__ void expand_leaf_w(const TreeParamsM& P, int64_t j, i
   __syncwarp();  // wbuf is reused by the warp's next leaf
 }
 
-// the whole downsweep (Alg. 4, Eq. 5) of a single matrix; expand as tree_down
+// the whole downsweep (Alg. 4, Eq. 5); expand as tree_down
 template <int F, int NVB>
-__global__ void __launch_bounds__(kWarpTreeWarps * 32, NVB == 8 ? 3 : 4) k_downsweep_warps(const MatDesc* __restrict__ mats, int L, int expand) {
+__global__ void __launch_bounds__(kWarpTreeWarps * 32, NVB == 8 ? 3 : 4) k_downsweep_warps(const MatDesc* __restrict__ mats,
+                                                                        const int2* __restrict__ jobs, int nvlo, int Tmax, int expand) {
   __shared__ float path[2][NVB][64];
   __shared__ __align__(16) float wstage[kWarpTreeWarps][NVB * 64];
-  const TreeParamsM P = tree_params(mats[0]);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, LR = mats[0].LR, T = P.q - L;
+  const int2 job = jobs ? jobs[blockIdx.x] : make_int2(0, (int)blockIdx.x);
+  const TreeParamsM P = tree_params(mats[job.x]);
+  if (P.nv < nvlo || P.nv > NVB) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, LR = P.D->LR, T = min(Tmax, P.q), L = P.q - T;
   float* wbuf = wstage[warp];
-  const int64_t sub = blockIdx.x, root = ((int64_t)1 << L) - 1 + sub;
+  const int64_t sub = job.y, root = ((int64_t)1 << L) - 1 + sub;
   // the path from the root to the subtree's root, recomputed by every CTA, a warp per vector (only the subtree's
   // own root is stored: the nodes above belong to several CTAs)
   if (L > 0 && warp < P.nv) {

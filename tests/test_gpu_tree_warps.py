@@ -59,3 +59,30 @@ def test_large_trees(h2, shape, form, bases):
             check(oracle.rel_l2(y.cpu().numpy(), ref), acc_tol(A), (shape, form, "tuner's last candidate"))
             assert chosen["tree_leaves"] in [1 << (A.q - L) for L in (9, 8, 7)]
     M.close()
+
+
+@pytest.mark.parametrize("form, bases", FORMS)
+def test_batch_of_many_leaves(h2, form, bases):
+    """A batch of more than 2^14 leaves takes these kernels for all its members of up to eight vectors, shallow ones and
+    single leaves too, beside members of more vectors and of none."""
+    sizes = [(32767, 4, 1), (20000, 2, 3), (10, 16, 2), (100, 32, 8), (2000, 2, 7), (300, 4, 16), (64, 64, 1), (5000, 40, 0)]
+    As = [h2gen.generate(dim=1, n=n, m=m, p=16, eta=0.9, kernel="exp", ell=0.2, seed=45 + i) for i, (n, m, _) in enumerate(sizes)]
+    assert sum(A.leaves for A in As) >= 1 << 14 and min(A.q for A in As) == 0
+    B = h2.H2Batch([h2.H2Matrix.from_generator(A, storage=form, bases_fp32=bases) for A in As])
+    xs = [h2gen.vectors(980 + i, A.n, max(nv, 1)) for i, (A, (_, _, nv)) in enumerate(zip(As, sizes))]
+    refs = [oracle.matvec(A, x, **quant.dequantized_arrays(A, form, bases)) for A, x in zip(As, xs)]
+    xd = [to_dev(x) if nv else None for x, (_, _, nv) in zip(xs, sizes)]
+    narrow = [x[:, :4] if x is not None else None for x in xd]  # up to four vectors: beside the dense stream
+    for tuned in (False, True):
+        for vectors in (xd, narrow):
+            ys = [torch.full((x.shape[1] if x is not None else 1, A.n), float("nan"), dtype=torch.float64, device="cuda:0").t()
+                  for A, x in zip(As, vectors)]
+            if tuned:
+                B.tune(vectors, ys)
+            for _ in range(2):  # the tickets return to zero
+                B.matvec(vectors, ys)
+                B.check()
+                for A, x, y, ref in zip(As, vectors, ys, refs):
+                    if x is not None:
+                        check(oracle.rel_l2(y.cpu().numpy(), ref[:, :x.shape[1]]), acc_tol(A), (A.n, form, x.shape[1], tuned))
+    B.close()
