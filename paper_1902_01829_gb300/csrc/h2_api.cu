@@ -676,8 +676,10 @@ h2_status build_device(h2_matrix_s* h, const h2_desc* d) {
   CUDA_TRY(cudaDeviceGetAttribute(&h->grid, cudaDevAttrMultiProcessorCount, dev));
 
   if ((st = upload(h, &h->leaf_off, lo, h->leaves + 1)) != H2_OK) return st;
-  if ((st = upload(h, &h->Srow, d->S_rowptr, h->n_nodes + 1)) != H2_OK) return st;
-  if ((st = upload(h, &h->Scol, d->S_colidx, h->nS)) != H2_OK) return st;
+  if (h->storage != H2_FP64) {  // (the FP64 coupling reads its segments and Sco)
+    if ((st = upload(h, &h->Srow, d->S_rowptr, h->n_nodes + 1)) != H2_OK) return st;
+    if ((st = upload(h, &h->Scol, d->S_colidx, h->nS)) != H2_OK) return st;
+  }
   if ((st = dalloc(h, &h->err, 1)) != H2_OK) return st;
   CUDA_TRY(cudaMemset(h->err, 0, sizeof(int)));
   if ((st = dalloc(h, &h->ticket, h->n_nodes)) != H2_OK) return st;

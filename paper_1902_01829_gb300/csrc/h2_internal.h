@@ -232,7 +232,7 @@ struct h2_matrix_s {
   const void* csegs = nullptr;        // coupling segments (h2::CouplingSeg), and the split rows' partial sums
   int64_t ncsegs = 0;
   float2* cpart = nullptr;            // [slot][v][kp]
-  int* cticket = nullptr;             // one counter per split row (at its first slot), zero between products
+  int* cticket = nullptr;             // [slot][4]: a split row's counter per slice of four vectors at its first slot, zero between products
   int* vexp = nullptr;                // per vector of the current pass: x scaled by 2^-vexp[v]
   unsigned long long* vpart = nullptr;  // per-block maxima of the scale pass
   unsigned* vticket = nullptr;        // last-block ticket of the scale pass, zero between products

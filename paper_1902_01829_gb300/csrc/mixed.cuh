@@ -7,8 +7,9 @@
 //   int16  offset binary: code = q + 32768, q in [-32767, 32767]
 // The phases are those of the FP64 form (hmv_fp64.cuh, stream_fp64.cuh):
 // fused leaf projection + upsweep (Eq. 2), coupling over all levels (Eq. 3),
-// fused downsweep (Eq. 5), and the TMA-streamed dense blocks fused with the
-// leaf expansion (Sec. 2.2, Eq. 4). Vectors x, xhat, yhat are FP32 with
+// downsweep (Eq. 5) with the leaf expansion (Eq. 4), and the dense blocks
+// (Sec. 2.2): TMA-streamed for up to four vectors, MMA tiles (mma_dense.cuh)
+// or tcgen05 (tc_dense.cuh) for more. Vectors x, xhat, yhat are FP32 with
 // strides rounded up to multiples of 4 (16-byte chunks for the bulk copies).
 #pragma once
 #include <type_traits>
@@ -74,7 +75,7 @@ struct __align__(16) MixedBlock {
   float scale;
   unsigned short cols;  // C
   unsigned char vs;     // vector stride (>= C, multiple of 4)
-  unsigned char src;    // bit 0: vector from the second source (yhat); bit 1: FP32 entries (not codes);
+  unsigned char src;    // bit 0: a leaf basis U_i (its vector is yhat); bit 1: FP32 entries (not codes; U_i only);
                         // bit 2: panel layout (below); bit 3: a wide block of fp16 or int16 codes
 };
 // A dense block is wide if an fp16 code is below 2^-10 (a block's largest is 1) or an int16 code below 256 (of 32767),
@@ -948,12 +949,7 @@ __global__ void __launch_bounds__(128, RPL == 1 ? 6 : 4) k_coupling_kf(const Mat
   if (parts > 1) split_finish(D, ch, 0, 0, nv, lane);
 }
 
-// ---------------------------------------------------------------- dense near field + expansion (TMA stream)
-// Per-block side information of the dense stream, 16 bytes.
-
-
-
-
+// ---------------------------------------------------------------- dense near field (TMA stream)
 constexpr int kMixedMaxBlocks = 8;   // blocks of one row per work item
 constexpr int kMixedVecCols = 256;   // vector columns of one work item (sum of its blocks' vs)
 constexpr int kMixedHeader = 256;
@@ -996,7 +992,7 @@ struct MixedStreamParams {
 // Stage header (ints): [0] R, [1] nb, [2] row, [3] flags, [4] uniform (1: every block a full 64 x 64
 // column-major block of 16-bit codes with 64 vector columns, 2: the same in the panel layout; the
 // blocks' codes and vector chunks then follow each other at fixed strides); block t at 8 + 4 t:
-// cols | FP32-entries flag << 16, vs, matrix offset in bytes, scale (bits);
+// cols | panel << 17, vs, matrix offset in bytes, scale (bits);
 // [40 + t] block t's vector offset in bytes; [48] nv; [50..51] y; [52..53] ldy.
 constexpr int kHdVoff = 40, kHdNv = 48, kHdXy32 = 49, kHdY = 50, kHdLdy = 52;
 template <int NST, int SB, int VAREA>
@@ -1030,7 +1026,6 @@ __device__ __forceinline__ void mixed_produce(const MixedStreamParams& P, const 
     // each lane fetches the matrix fields of its own item
     const char* l_dmat = nullptr;
     const float* l_x4 = nullptr;
-    const float* l_yhat = nullptr;
     double* l_y = nullptr;
     long long l_ldy = 0;
     int l_nv = 0, l_xy32 = 0;
@@ -1038,7 +1033,6 @@ __device__ __forceinline__ void mixed_produce(const MixedStreamParams& P, const 
       const MatDesc& D = P.mats[d1.w >> 8];
       l_dmat = D.dmat;
       l_x4 = D.x4;
-      l_yhat = D.yhat;
       l_y = D.y;
       l_ldy = D.ldy;
       l_nv = D.nv;
@@ -1068,7 +1062,6 @@ __device__ __forceinline__ void mixed_produce(const MixedStreamParams& P, const 
       const long long b0 = (long long)(((unsigned long long)b_hi << 32) | b_lo);
       const char* dmat = reinterpret_cast<const char*>(__shfl_sync(0xFFFFFFFFu, (unsigned long long)l_dmat, t));
       const float* x4 = reinterpret_cast<const float*>(__shfl_sync(0xFFFFFFFFu, (unsigned long long)l_x4, t));
-      const float* yh = reinterpret_cast<const float*>(__shfl_sync(0xFFFFFFFFu, (unsigned long long)l_yhat, t));
       const unsigned long long ydst = __shfl_sync(0xFFFFFFFFu, (unsigned long long)l_y, t);
       const long long ldy = (long long)__shfl_sync(0xFFFFFFFFu, (unsigned long long)l_ldy, t);
       const int nv = __shfl_sync(0xFFFFFFFFu, l_nv, t);
@@ -1099,10 +1092,10 @@ __device__ __forceinline__ void mixed_produce(const MixedStreamParams& P, const 
       voff -= vbytes;
       // uniform item: every block full 64 x 64 16-bit codes in one layout, 64 vector columns each
       const int panel0 = __shfl_sync(0xFFFFFFFFu, (int)((mb.src >> 2) & 1), 0);
-      const bool full = lane >= nb || (!(mb.src & 2) && mb.cols == 64 && mb.vs == 64 && (int)((mb.src >> 2) & 1) == panel0);
+      const bool full = lane >= nb || (mb.cols == 64 && mb.vs == 64 && (int)((mb.src >> 2) & 1) == panel0);
       const int uniform = (__all_sync(0xFFFFFFFFu, full) && R == 64) ? 1 + panel0 : 0;
       if (lane < nb) {
-        hd[8 + 4 * lane] = mb.cols | ((mb.src & 2) << 15) | ((mb.src & 4) << 15);
+        hd[8 + 4 * lane] = mb.cols | ((mb.src & 4) << 15);
         hd[9 + 4 * lane] = mb.vs;
         hd[10 + 4 * lane] = moff;
         hd[11 + 4 * lane] = __float_as_int(mb.scale);
@@ -1126,10 +1119,8 @@ __device__ __forceinline__ void mixed_produce(const MixedStreamParams& P, const 
                         S.full + s, pol);
       }
       __syncwarp();
-      if (lane < nb && vbytes > 0) {  // a matrix multiplies no vectors in this product: matrix bytes only
-        const float* src = (mb.src & 1) ? yh : x4;
-        bulk_g2s(stage + kMixedHeader + kStageMat + voff, src + mb.voff * nv, vbytes, S.full + s);
-      }
+      if (lane < nb && vbytes > 0)  // (a matrix may multiply no vectors in this product: matrix bytes only)
+        bulk_g2s(stage + kMixedHeader + kStageMat + voff, x4 + mb.voff * nv, vbytes, S.full + s);
       __syncwarp();
       issued = it + 1;
     }
@@ -1161,14 +1152,11 @@ __device__ __forceinline__ void consume_item(const unsigned char* stage, const i
     const bool even = (R & 1) == 0;
     int base = 0;
     for (int t = 0; t < nb; t++) {
-      const int cw = hd[8 + 4 * t];
-      const bool f32 = (cw >> 16) & 1;
-      const int C = min(cw & 0xFFFF, 64), vs = min(hd[9 + 4 * t], 64);
+      const int C = min(hd[8 + 4 * t] & 0xFFFF, 64), vs = min(hd[9 + 4 * t], 64);
       const int moff = min(hd[10 + 4 * t], kStageMat - 16) & ~15;
       const float scale = __int_as_float(hd[11 + 4 * t]);
       const int voff = min(hd[kHdVoff + t], VAREA - 16) & ~15;
       const uint16_t* A = reinterpret_cast<const uint16_t*>(stage + kMixedHeader + moff);
-      const float* A32 = reinterpret_cast<const float*>(stage + kMixedHeader + moff);
       const float* X = reinterpret_cast<const float*>(stage + kMixedHeader + kStageMat + voff);
       const int G = (C + 3) >> 2;
       int first = hw - (base % HW);
@@ -1183,9 +1171,6 @@ __device__ __forceinline__ void consume_item(const unsigned char* stage, const i
           const int col = c + j;
           if (col >= C) {
             a[j] = make_float2(0.f, 0.f);
-          } else if (f32) {
-            a[j].x = A32[r0 + R * col];
-            a[j].y = (r0 + 1 < R) ? A32[r0 + 1 + R * col] : 0.f;
           } else if (even) {
             a[j] = codes_to_f2<F>(*reinterpret_cast<const uint32_t*>(A + r0 + R * col));
           } else {
