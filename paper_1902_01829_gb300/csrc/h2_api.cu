@@ -687,8 +687,8 @@ h2_status build_device(h2_matrix_s* h, const h2_desc* d) {
   // subtree roots of the tree kernels: up to 128 CTAs of one leaf; then four leaves per CTA, whose three
   // inner steps cost less than two more climbed levels (2D n = 2^16, 16 vectors, up + down: four leaves
   // 73 us, two 85, eight 94); from 2^13 leaves on the CTAs outnumber the SMs many times and each repeats
-  // the path from the root, so they take up to 16 (2D n = 2^20, upsweep of 8 vectors: 16 leaves 290 us, eight
-  // 320, four 373)
+  // the path from the root, so they take up to 16 (2D n = 2^20, upsweep of 8 vectors of the scaled forms, which have
+  // tree_warps.cuh's kernels for it now: 16 leaves 290 us, eight 320, four 373)
   h->tree_L = h->q <= 7 ? h->q : h->q <= 9 ? 7 : h->q <= 12 ? h->q - 2 : std::max(10, h->q - 4);
   if (h->storage != H2_FP64) return mixed_build(h, d);
 

@@ -18,10 +18,11 @@
 //    of up to 32 clusters below a node computes the levels up to it, its CTAs sharing each level's
 //    nodes. One ticket per level (fence, atomic, reload through L2) cost 2.5 us a level.
 //  - the downsweep's path from the root to the subtree is recomputed by every CTA.
-// Measured (upsweep / downsweep with expansion, us; one warp per node and a ticket per level before):
-// 2D n = 50,001 FP64, 16 vectors 297 / 188 -> 82 / 31; 2D n = 2^16 int16, 16 vectors 60 / 41 -> 40 / 33;
-// 3D n = 2^14 bf16, k = 64, 16 vectors 154 / 62 -> 75 / 41; 3D n = 2^16 int16, 8 vectors 194 / 159 -> 73 / 58;
-// 3D n = 2^14 FP64, one vector 172 / 70 -> 87 / 37. A step is still bound by the length of its instruction
+// Measured (upsweep with the vectors' conversion / downsweep with expansion, phases in order, us; one warp per node and a
+// ticket per level before): 2D n = 50,001 FP64, 16 vectors 294 / 184 -> 89 / 55; 2D n = 2^16 int16, 16 vectors 68 / 41 ->
+// 46 / 35; 3D n = 2^14 bf16, k = 64, 16 vectors 160 / 62 -> 77 / 41; 3D n = 2^16 int16, 8 vectors 203 / 157 -> 78 / 58;
+// 3D n = 2^14 FP64, one vector 169 / 69 -> 83 / 49. Where the nodes outnumber the chip's warps a warp per node is the better
+// one: tree_warps.cuh, for the scaled forms. A step is still bound by the length of its instruction
 // chain (about 4.5 cycles an instruction, one warp per scheduler): 2,000 cycles.
 #pragma once
 #include <cooperative_groups.h>
