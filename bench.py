@@ -159,8 +159,9 @@ TRAFFIC_KERNEL = {("fp64", False): "k_dense_stream", ("int16", True): "k_dense_s
 # digit products per product of two FP64 entries in the FP64 form's dense phase at more than four vectors
 # (seven 8-bit digits each: the 21 pairs of weight <= 5 and the seven of weight 6)
 DIGIT_PAIRS = 28
-# mma.sync FP16 rate of the chip, TFLOP/s (a loop of m16n8k16: 8 cycles each per SM quarter)
-MMA_SYNC_TFLOPS = 600.0
+# mma.sync FP16 rate of the chip, TFLOP/s, as measured (profiles/mma_and_tree_kernels.md: a loop of m16n8k16, 8 cycles
+# each per SM quarter)
+MMA_SYNC_TFLOPS = 606.0
 
 
 def dense_kernel_bytes(info: dict, A, nv: int, storage: str = "fp64", bases_fp32: bool = False) -> int:

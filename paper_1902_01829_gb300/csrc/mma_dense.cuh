@@ -26,7 +26,7 @@
 // Measured, dense phase: 2D n = 2^16 int16, 16 vectors 126 -> 75 us; 32 matrices of 1024 .. 16384 points, 32-point
 // leaves, fp16, 1 to 16 vectors 599 -> 203 us; 3D n = 2^16 int16, 8 vectors 393 -> 325 us. The K steps are now
 // bound by their chain (loads, permutes, MMAs: about 800 cycles with three warps a scheduler), not by the tensor
-// pipe (a quarter busy).
+// pipe (42% busy).
 //
 // A CTA per SM, persistent over its items (the dense stream's, h2_mixed.cu): a producer warp copies each
 // item's codes and its blocks' vector chunks into a ring of stages; twelve consumer warps take the blocks

@@ -23,7 +23,7 @@
 // about 800 issue slots, and its 32 KB 1,400 at the copy bandwidth. Measured, 2D n = 50,001 (48- and 49-point leaves),
 // 16 vectors: six digits 837 -> 404 us in the dense phase, error against 64 bits 2.6e-14 -> 2.1e-14 (weight 6 left
 // out: 7e-14; the sums joined without the third exact step: 1e-13); seven digits with the vectors' fragments loaded
-// one at a time (60 bytes of spills less) 397 -> 375 us, error 2.0e-14. About 4,600 cycles a block are
+// one at a time (60 bytes of spills less) 397 -> 375 us, error 2.0e-14. 4,200 cycles a block are
 // still the chain of slicing, loads and MMAs of three warps a scheduler, not a pipe.
 //
 // Y^T = X^T D^T as in mma_dense.cuh: the vectors' digits are the A operand, written in fragment order by
