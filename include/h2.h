@@ -217,6 +217,8 @@ h2_status h2_create_generated(const h2_desc* d, const h2_coupling_kernel* kc, co
  * 2^-46 of itself): the error of a row stays below 2^-38 of sum_j |a_ij||x_j|
  * for any vector and near 2^-46 of it where a row's entries are alike, and the
  * last bits of a column may differ between a call of four vectors and of five.
+ * A row's near-field and far-field parts are each rounded to the type of y and
+ * added there, so both have to lie in its range.
  * Errors: H2_ERR_INVALID (NULL, nv < 1, ld < n), H2_ERR_CUDA (launch failed).
  */
 h2_status h2_matvec(h2_handle h, int32_t nv, const double* x, int64_t ldx, double* y, int64_t ldy, void* stream);

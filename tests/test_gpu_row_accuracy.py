@@ -6,7 +6,8 @@ import types
 import numpy as np
 import pytest
 
-from oracle import quant
+import h2gen
+from oracle import construct, quant
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -126,4 +127,24 @@ def test_scaled_rows(h2, form, kind, sizes, nv):
     ref, bound = product(A, quant.dequantized_arrays(A, form)["D_val"], x.astype(np.float64))
     worst = np.max(np.abs(y - ref) / bound)
     assert worst <= FP32_TOL, (kind, np.log2(worst))
+    M.close()
+
+
+@pytest.mark.parametrize("form", ["int16", "fp16"])
+def test_generated_wide_blocks(h2, form):
+    """Dense blocks generated on the device carry the mark of wide blocks too: every leaf pair a block, so short a
+    correlation length that most rows see their own point alone, vectors that span 2^40 within a leaf; more than four
+    vectors against the same codes times four (the streams: FP32 entry by entry)."""
+    A = h2gen.generate(dim=2, n=700, m=32, p=4, eta=0.0, kernel="exp", ell=0.002, seed=61, coupling_values=False, dense_values=False)
+    D = construct.dense_blocks(A.leaf_offset, A.D_rowptr, A.D_colidx, A.points, A.kernel, A.ell)
+    A.keys = [(i, int(j)) for i in range(A.leaves) for j in A.D_colidx[A.D_rowptr[i]:A.D_rowptr[i + 1]]]
+    rng = np.random.default_rng(62)
+    x = (rng.uniform(0.5, 1.0, (A.n, 16)) * np.ldexp(1.0, -rng.integers(0, 41, (A.n, 16)))).astype(np.float32)
+    _, bound = product(A, quant.dequantize_blocks(D, np.asarray(A.D_valoff), form), x.astype(np.float64))
+    M = h2.H2Matrix.from_generator(A, storage=form, bases_fp32=True, coupling="kernel", dense="generated")
+    four = M.matvec_f32(to_dev(x[:, :4])).cpu().numpy().astype(np.float64)
+    for nv in (7, 16):
+        y = M.matvec_f32(to_dev(x[:, :nv])).cpu().numpy().astype(np.float64)[:, :4]
+        assert np.max(np.abs(y - four) / bound[:, :4]) <= 2 * FP32_TOL, (form, nv)
+    M.check()
     M.close()
