@@ -209,8 +209,8 @@ h2_status h2_create_generated(const h2_desc* d, const h2_coupling_kernel* kc, co
  * tensor cores, whatever the leaves and bases. Other passes of more than four
  * vectors run the dense blocks on MMA tiles: the scaled forms with the vectors
  * split into three 16-bit parts (fp16 and int16 codes: down to 2^-38
- * of the largest entry of a leaf, where a block's codes span at most 2^10, int16
- * 2^7, without zeros; else as FP32), the FP64 form by exact products of 8-bit
+ * of the largest entry of a leaf, where a block's codes span at most 2^10 without
+ * zeros; else as FP32), the FP64 form by exact products of 8-bit
  * digits where a dense block has no zeros and its entries span less than 2^9,
  * else in double-float. Digits hold a block's entries to 2^-55 of its largest
  * and a vector's to 2^-54 of the largest of its leaf (double-float: each to

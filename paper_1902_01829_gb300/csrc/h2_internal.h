@@ -65,7 +65,7 @@ struct MixedLaunch {
   const int* cta_begin = nullptr;    // [grid + 1]
   const int* mma_begin = nullptr;    // the same for passes of more than four vectors (k_dense_mma)
   const void* blk = nullptr;         // h2::MixedBlock records
-  bool wide = false;                 // some dense block is wide (mixed.cuh)
+  bool wide = false;                 // some dense block is kBlockWide or kBlockLow (mixed.cuh)
   int grid = 0;
   int* err = nullptr;
   long long budget = kWaitBudget;

@@ -83,14 +83,14 @@ float quantize(const double* a, int64_t cnt, int form, uint16_t* codes) {
   return sigma;
 }
 
-// kBlockWide if some code of a dense block is (mixed.cuh), else 0
+// a dense block's kBlockWide and kBlockLow (mixed.cuh) from its codes
 unsigned char wide_flag(const uint16_t* codes, int64_t cnt, int form) {
-  bool w = false;
+  int w = 0;
   if (form == h2::kFormFp16)
     for (int64_t i = 0; i < cnt; i++) w |= h2::wide_code<h2::kFormFp16>(codes[i]);
   else if (form == h2::kFormInt16)
     for (int64_t i = 0; i < cnt; i++) w |= h2::wide_code<h2::kFormInt16>(codes[i]);
-  return w ? h2::kBlockWide : 0;
+  return (unsigned char)w;
 }
 
 // quantize then transpose a rows x cols column-major block into cols x rows codes
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(256) k_gen_dense(GenDense a) {
     const float sigma = F == h2::kFormInt16 ? (float)(m / 32767.0) : (float)m;
     uint16_t* dst = reinterpret_cast<uint16_t*>(a.dmat + a.bbyte[t]);
     const int ps2 = h2::panel_stride(sj) / 2, cs = h2::code_stride(si);
-    bool wide = false;
+    int wide = 0;
 #pragma unroll
     for (int u = 0; u < 16; u++) {
       const int e = threadIdx.x + 256 * u;
@@ -287,13 +287,17 @@ __global__ void __launch_bounds__(256) k_gen_dense(GenDense a) {
     }
     if (threadIdx.x == 0) a.blk[a.bglob[t]].scale = sigma;
     if constexpr (F != h2::kFormBf16) {
-      wide = __any_sync(0xFFFFFFFFu, wide);
+      wide = __reduce_or_sync(0xFFFFFFFFu, wide);
       if (lane == 0) wwide[warp] = wide;
     }
     __syncthreads();  // xs and wmax are reused by the next block
     if constexpr (F != h2::kFormBf16) {
-      if (threadIdx.x < 32 && __any_sync(0xFFFFFFFFu, lane < 8 && wwide[lane & 7]) && lane == 0)
-        a.blk[a.bglob[t]].src |= h2::kBlockWide;
+      if (threadIdx.x == 0) {
+        int w = 0;
+#pragma unroll
+        for (int u = 0; u < 8; u++) w |= wwide[u];
+        a.blk[a.bglob[t]].src |= (unsigned char)w;
+      }
     }
   }
 }
@@ -838,7 +842,7 @@ h2_status mixed_build(h2_matrix_s* h, const h2_desc* d) {
     for (int64_t g = 0; g < nblk; g++) {
       float& mx = (blk[g].src & 1) ? M.umax : M.dmax;
       mx = std::max(mx, blk[g].scale);
-      M.launch.wide = M.launch.wide || (blk[g].src & h2::kBlockWide);
+      M.launch.wide = M.launch.wide || (blk[g].src & (h2::kBlockWide | h2::kBlockLow));
     }
 
     // work items: consecutive dense blocks of one row, at most kMixedMaxBlocks blocks, 32 KB of

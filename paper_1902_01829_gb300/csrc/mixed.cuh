@@ -76,16 +76,20 @@ struct __align__(16) MixedBlock {
   unsigned short cols;  // C
   unsigned char vs;     // vector stride (>= C, multiple of 4)
   unsigned char src;    // bit 0: a leaf basis U_i (its vector is yhat); bit 1: FP32 entries (not codes; U_i only);
-                        // bit 2: panel layout (below); bit 3: a wide block of fp16 or int16 codes
+                        // bit 2: panel layout (below); bits 3, 4: kBlockWide, kBlockLow
 };
-// A dense block is wide if an fp16 code is below 2^-10 (a block's largest is 1) or an int16 code below 256 (of 32767),
-// zeros among them: what k_dense_mma's split leaves out could then show in a row of small codes (mma_dense.cuh).
-constexpr int kBlockWide = 8;
+// Dense blocks whose smallest code is far below the largest (1 in fp16, 32767 in int16), zeros among them, where what
+// k_dense_mma's split leaves out could show in a row of small codes (mma_dense.cuh): wide below 2^-10 (32 in int16);
+// int16 blocks with codes of 32 to 255 only want the product of the low parts too.
+constexpr int kBlockWide = 8, kBlockLow = 16;
 template <int F>
-__host__ __device__ __forceinline__ bool wide_code(uint16_t c) {
-  if (F == kFormFp16) return (c & 0x7FFFu) < 0x1400u;
-  if (F == kFormInt16) return c > 32768 - 256 && c < 32768 + 256;
-  return false;
+__host__ __device__ __forceinline__ int wide_code(uint16_t c) {
+  if (F == kFormFp16) return (c & 0x7FFFu) < 0x1400u ? kBlockWide : 0;
+  if (F == kFormInt16) {
+    const int q = c < 32768 ? 32768 - c : c - 32768;
+    return q < 32 ? kBlockWide : q < 256 ? kBlockLow : 0;
+  }
+  return 0;
 }
 
 // Panel layout of a block of codes (64 rows, C columns): eight panels of 8 rows,

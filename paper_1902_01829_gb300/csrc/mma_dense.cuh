@@ -11,13 +11,14 @@
 //   x_v = hi + mid + lo in bf16 (all 24 bits of any FP32).
 // A code is a B entry as it is (fp16, bf16); an int16 code q = 256 (h + l) with h = q >> 8 and l = the low
 // byte / 256, both exact in fp16, times hi, mid (and lo): l lo is left out, below 2^-23 of its product where |q| >= 256
-// (with it 5 MMAs become 6: 2D n = 2^18, 8 vectors, dense phase 261 -> 313 us). The leading products h hi and the rest
-// accumulate apart, in FP32, and a block's sums enter the row's after sigma 2^(e - 14) is applied, so nothing is
-// rounded to 16 bits and no chain is longer than a block. Blocks with smaller int16 codes, or with fp16 codes below
-// 2^-10, zeros among them ("wide"), are multiplied in FP32 by the same warps (mma_wide_block) with the vectors as they
-// are: a row of such a block may see small codes or small vector entries alone. In the others every row weighs the
-// leaf's largest entry with 2^-10 (int16: 2^-7) at least, so what the parts cut off is below 64 2^10 2^-38 of
-// sum_j |d_ij| |x_j| for any vector, in most cases below FP32's rounding of the sum.
+// (with it 5 MMAs become 6: 2D n = 2^18, 8 vectors, dense phase 261 -> 313 us), and taken in blocks with smaller codes
+// (kBlockLow). The leading products h hi and the rest accumulate apart, in FP32, and a block's sums enter the row's
+// after sigma 2^(e - 14) is applied, so nothing is rounded to 16 bits and no chain is longer than a block. Blocks with a
+// code below 2^-10 of the largest, zeros among them (kBlockWide), are multiplied in FP32 by the same warps
+// (mma_wide_block) with the vectors as they are: a row of such a block may see small vector entries alone. In the others
+// every row weighs the leaf's largest entry with 2^-10 at least, so what the parts cut off is below 64 2^10 2^-38 of
+// sum_j |d_ij| |x_j| for any vector, in most cases below FP32's rounding of the sum. (Small int16 matrices feel a wide
+// block's latency: with blocks of codes below 256 wide too, 2D n = 1,000 took 64 us for 16 vectors, 52 so.)
 //
 // What bounds it: at 16 vectors the FP32 pipes spent 2048 FMAs of a warp on a 64 x 64 block (1360 cycles an
 // SM with its loads); 3 (int16: 5) MMAs per tile and K step take 192 (320) and the codes' loads from shared
@@ -70,8 +71,8 @@ __device__ __forceinline__ uint32_t int16_low(uint32_t c) {
 
 // Producer warp: as mixed_produce, with the blocks' vector chunks in the parts' layout (a wide block's in FP32).
 // Stage header (ints): [0] R, [1] nb, [2] row, [3] flags, [4] vector halves (1 or 2); block t at 8 + 4 t:
-// columns | panel << 17 | wide << 18 | vector stride << 24, vector offset, matrix offset, scale; [48] nv, [49] xy32, [50..51] y, [52..53] ldy.
-// WIDE: the launch's matrices have wide blocks.
+// columns | panel << 17 | wide << 18 | low << 19 | vector stride << 24, vector offset, matrix offset, scale; [48] nv, [49] xy32, [50..51] y, [52..53] ldy.
+// WIDE: the launch's matrices have wide or low blocks.
 template <bool WIDE>
 __device__ __forceinline__ void mma_produce(const MixedStreamParams& P, const StreamShared& S, int ib, int ie,
                                             MixedBlock* blkbuf) {
@@ -152,7 +153,7 @@ __device__ __forceinline__ void mma_produce(const MixedStreamParams& P, const St
       moff -= codes;
       voff += m_bytes - vbytes;  // the vectors' chunks follow the codes
       if (lane < nb) {
-        hd[8 + 4 * lane] = mb.cols | ((mb.src & (4 | kBlockWide)) << 15) | (mb.vs << 24);
+        hd[8 + 4 * lane] = mb.cols | ((mb.src & (4 | kBlockWide | kBlockLow)) << 15) | (mb.vs << 24);
         hd[9 + 4 * lane] = voff;
         hd[10 + 4 * lane] = moff;
         hd[11 + 4 * lane] = __float_as_int(mb.scale);
@@ -211,7 +212,7 @@ __device__ __forceinline__ uint32_t lds16(uint32_t addr) {
 // rows are one aligned 8-byte load; 1: the same with the last K step's columns tested (tested in every case, 64-point
 // blocks took 318 us for 301: 2D n = 65,536, 64 vectors); 0: every code is tested and loaded by itself.
 template <int F, int LOAD>
-__device__ __forceinline__ void mma_block(uint32_t base, int cb, uint32_t X, int C, int rows, float scale, int nh,
+__device__ __forceinline__ void mma_block(uint32_t base, int cb, uint32_t X, int C, int rows, float scale, int nh, bool low,
                                           float (&run)[4][4]) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   float hi[4][4], lo[4][4];
@@ -279,6 +280,10 @@ __device__ __forceinline__ void mma_block(uint32_t base, int cb, uint32_t X, int
       for (int p = 0; p < 2; p++)
 #pragma unroll
         for (int i = 0; i < 4; i++) mma_m16n8k16(lo[i], a[p], bl[i][0], bl[i][1], bf);
+    if (digits && low) {
+#pragma unroll
+      for (int i = 0; i < 4; i++) mma_m16n8k16(lo[i], a[2], bl[i][0], bl[i][1], bf);
+    }
   }
   float sc[2];
   asm volatile("ld.shared.f32 %0, [%1];" : "=f"(sc[0]) : "r"(X + 4 * g));
@@ -393,10 +398,10 @@ __global__ void __launch_bounds__((kMmaWarps + 1) * 32, 1) k_dense_mma(MixedStre
         const int r = two ? 8 * g + 4 * (turn & 1) : 4 * g, cb = panel ? 16 : 2 * code_stride(R);
         // (in the column-major layout the last lanes' rows may lie past R: they read what follows, unused)
         const uint32_t base = codes + (panel ? (r >> 3) * panel_stride(C) + 2 * (r & 7) : 2 * r);
-        const bool wide = panel || (code_stride(R) & 3) == 0;
-        if (wide && (C & 15) == 0) mma_block<F, 2>(base, cb, X, C, 4, __int_as_float(bh.w), nh, run);
-        else if (wide) mma_block<F, 1>(base, cb, X, C, 4, __int_as_float(bh.w), nh, run);
-        else mma_block<F, 0>(base, cb, X, C, R - r, __int_as_float(bh.w), nh, run);
+        const bool wide = panel || (code_stride(R) & 3) == 0, low = WIDE && ((bh.x >> 19) & 1);
+        if (wide && (C & 15) == 0) mma_block<F, 2>(base, cb, X, C, 4, __int_as_float(bh.w), nh, low, run);
+        else if (wide) mma_block<F, 1>(base, cb, X, C, 4, __int_as_float(bh.w), nh, low, run);
+        else mma_block<F, 0>(base, cb, X, C, R - r, __int_as_float(bh.w), nh, low, run);
       }
       turn -= nb << two;
     }
